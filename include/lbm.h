@@ -192,11 +192,15 @@ lbm_status lbm_init(lbm_ctx* ctx, const lbm_init_spec* init);
 /* Advances n time steps, asynchronously on the context's stream (captured into a CUDA
  * graph on first use).  Each step: density (Sec. 2.1); solid-node densities (Eq. 15);
  * chemical potential (Eq. 12); nonideal force (Eq. 9) with exact-difference forcing
- * (Eqs. 13-14), collision (Eq. 4) and streaming (Eq. 5) fused in one kernel; then every cut
- * link by Eq. 16 (q < 1/2) or Eq. 17 (q >= 1/2) with the per-node compensation of Eq. 18
- * accumulated in FP64.  The density pass of the next state overlaps the links on a second
- * stream the context creates on first use (ordered with the context's stream by events; no
- * device memory is allocated); to the caller the work is on the context's stream. */
+ * (Eqs. 13-14), collision (Eq. 4) and streaming (Eq. 5); then every cut link by Eq. 16
+ * (q < 1/2) or Eq. 17 (q >= 1/2) with the per-node compensation of Eq. 18 accumulated in FP64.
+ * FP32 lattices on two population lattices with an equation of state (not slabs) run the fused
+ * step: one pass over the populations, then the links, then the solid layers.  Others, and a
+ * lattice whose kernels the caller chose (lbm_set_collide_kernel, lbm_set_mu_kernel), run the
+ * separate passes, the density pass of the next state overlapping the links on a second stream
+ * the context creates on first use (ordered with the context's stream by events).  Both give the
+ * same values, bit for bit.  No device memory is allocated; to the caller the work is on the
+ * context's stream. */
 lbm_status lbm_step(lbm_ctx* ctx, int64_t n);
 
 /* Captures and instantiates the step graphs that lbm_step(n) will launch from the current state,
@@ -267,8 +271,8 @@ lbm_status lbm_last_dM(lbm_ctx* ctx, double* dM);
  * waits for the stream. */
 lbm_status lbm_last_dM_async(lbm_ctx* ctx, double* dM);
 
-/* Advances n steps like lbm_step, launching the five phases one by one with CUDA events on
- * the context's stream between them, and adds each phase's device time (ms) to ms5:
+/* Advances n steps like lbm_step, launching the five phases of the separate passes one by one
+ * (the same values, bit for bit) with CUDA events on the context's stream between them, and adds each phase's device time (ms) to ms5:
  * [0] density, [1] solid layers (Eq. 15), [2] chemical potential, [3] force + collision +
  * streaming, [4] boundary links (Eqs. 16-18).  Synchronises after every step. */
 lbm_status lbm_profile_steps(lbm_ctx* ctx, int64_t n, double* ms5);
@@ -294,18 +298,21 @@ lbm_status lbm_launches_per_step(lbm_ctx* ctx, int64_t* n);
  * encode the tensor maps (FP32 with a driver that has the encoder) and the lattice gives each
  * persistent block at least 16 tiles, kind 0 otherwise; kind 2 runs only when set (on GB300 its
  * added density work slows a collide kernel that is already bound by instruction issue more
- * than the separate density pass costs).  Setting a kind the lattice cannot run returns
+ * than the separate density pass costs).  Setting a kind, the current one too, makes lbm_step run
+ * the separate passes instead of the fused step.  Setting a kind the lattice cannot run returns
  * LBM_EINVAL.  Call after lbm_build_links; the step graphs are captured again.  A
  * bounded wait of kind 1 or 2 that gives up is reported as LBM_ETIMEOUT by the next lbm_mass. */
 lbm_status lbm_set_collide_kernel(lbm_ctx* ctx, int32_t kind);
-/* The collide kernel lbm_step runs now (0 plain, 1 TMA-pipelined, 2 column sweeps). */
+/* The collide kernel of the separate passes (0 plain, 1 TMA-pipelined, 2 column sweeps): the one
+ * lbm_step runs unless it runs the fused step. */
 lbm_status lbm_get_collide_kernel(lbm_ctx* ctx, int32_t* kind);
 
 /* The chemical-potential pass (Eq. 12) of the chemical-potential force model: 0 one node a
  * thread, 1 four (FP64: two) consecutive nodes of a row a thread from 16-byte loads, 2 (FP32
  * only) row sweeps, a thread walking down a column of four-node groups with the stencil's rows
  * in registers.  The default is 2 for FP32 lattices of at least four 512 x 16-node blocks per
- * SM, else 1.  All three give the same bits.  Call
+ * SM, else 1.  All three give the same bits.  Setting a kind makes lbm_step run the separate
+ * passes instead of the fused step.  Call
  * after lbm_build_links; the step graphs are captured again.  LBM_EINVAL for another value or
  * for 2 on an FP64 lattice. */
 lbm_status lbm_set_mu_kernel(lbm_ctx* ctx, int32_t kind);

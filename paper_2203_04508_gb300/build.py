@@ -22,6 +22,7 @@ COMMON = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-ffp-contract=o
 UNITS = [
     ("lbm_api.cu", []),
     ("lbm_step.cu", []),
+    ("lbm_fused.cu", []),
     ("lbm_geometry.cu", ["-fmad=false"]),
     ("lbm_eos.cpp", ["-x", "cu"]),
     ("lbm_noalloc.cu", []),

@@ -60,8 +60,8 @@ struct Layout {
   // set-up scratch (which use the idle second lattice otherwise), `bmom` the boundary nodes'
   // saved moments
   size_t stage, bmom;
-  size_t lq64, lq, ldir, lx2f, bnode, bstart, carry, rhob;
-  size_t s1node, s1mask, s1winv, s1nb, s2node, s2mask, s2winv;
+  size_t lq64, lq, ldir, lx2f, bnode, bstart, carry, rhob, bnd, bmask, bq;
+  size_t s1node, s1mask, s1winv, s1nb, s2node, s2mask, s2winv, s2nb;
   size_t cyl, drops, partials, counter, step_ctr, scalars, kerr, dm_ring, block_sums, totals;
   size_t total;
 };
@@ -101,6 +101,10 @@ Layout make_layout(const lbm_config* c) {
   L.lx2f = take(L.cap.links);
   L.bnode = take(L.cap.bnodes * 4);
   L.bstart = take((L.cap.bnodes + 1) * 4);
+  const bool by_node = L.sz == 4;        // the fused step's links by boundary node
+  L.bnd = take(by_node ? L.cap.bnodes * 8 : 0);
+  L.bmask = take(by_node ? L.cap.bnodes * 2 : 0);
+  L.bq = take(by_node ? L.cap.bnodes * 8 * L.sz : 0);
   L.carry = take(L.cap.bnodes * 8);
   L.rhob = take(L.cap.bnodes * L.sz);
   L.bmom = take(aa ? 3 * L.cap.bnodes * L.sz : 0);
@@ -111,6 +115,7 @@ Layout make_layout(const lbm_config* c) {
   L.s2node = take(L.cap.s2 * 4);
   L.s2mask = take(L.cap.s2);
   L.s2winv = take(L.cap.s2 * L.sz);
+  L.s2nb = take(L.cap.s2 * 8 * 4);
   // fluid nodes whose chemical-potential stencil reaches a solid or boundary node: each solid-layer
   // or boundary node is in the stencils of at most 9 nodes
   L.near = take((size_t)9 * (L.cap.bnodes + L.cap.s1 + L.cap.s2) * 4);
@@ -121,7 +126,7 @@ Layout make_layout(const lbm_config* c) {
   L.cyl = take((size_t)(c->n_cyl > 0 ? c->n_cyl : 1) * 4 * 8);
   L.drops = take((size_t)MAX_DROPS * 5 * 8);
   size_t nparts = 2 * (size_t)mass_blocks();
-  size_t bparts = (size_t)((L.cap.bnodes + 255) / 256) + 1;
+  size_t bparts = (size_t)((L.cap.bnodes + 255) / 256 + 1) * 8;   // one per block, or per warp of 32
   L.partials = take(8 * (nparts > bparts ? nparts : bparts));
   L.counter = take(16);
   L.step_ctr = take(16);
@@ -172,6 +177,9 @@ struct lbm_ctx {
   int collide_kind = 1;
   long long spin_limit = 1LL << 22;   // polls before a pipelined kernel's wait gives up
   int mu_kind = -1;                   // chemical-potential pass (-1: the precision's default)
+  bool collide_set = false;           // lbm_set_collide_kernel was called
+  bool fused_ok = false;              // the fused step's kernels can run on this device
+  int fused_rows = 0;                 // rows a warp of the fused step walks
   long long n_near = 0;               // entries of the near list, built where the fused density +
   bool near_built = false;            // mu pass is selected (lbm_build_links, lbm_set_mu_kernel)
   lbm_status sticky = LBM_OK;
@@ -285,6 +293,8 @@ void fill_lattice(lbm_ctx* c, Lattice<real>& L) {
   L.RT = (real)RT;
   L.a = (real)g.a;
   L.b = (real)g.b;
+  L.b4 = (real)(g.b / 4.0);
+  L.pr_nk = (real)(-g.a * c->eos.alpha / (2.0 * M_SQRT2 * g.b));
   L.aalpha = (real)(g.a * c->eos.alpha);
   L.k2 = (real)(g.k * g.k);
   L.kappa = (real)g.kappa;
@@ -299,9 +309,18 @@ void fill_lattice(lbm_ctx* c, Lattice<real>& L) {
     const double P0 = 8.0 * eta0 - 9.0 * eta0 * eta0 + 3.0 * eta0 * eta0 * eta0;
     L.cs_r0[k] = r0;
     L.cs_inv_r0[k] = (real)(1.0 / r0d);
-    L.cs_eta0[k] = (real)eta0;
-    L.cs_a0[k] = (real)a0;
-    L.cs_p0a3[k] = (real)(P0 / (a0 * a0 * a0));
+    const double p3 = P0 / (a0 * a0 * a0);
+    // N(eta) = n0 + n1 eta + n2 eta^2, shifted to h = eta - eta0
+    const double n0 = 8.0 - 9.0 * eta0 + 3.0 * eta0 * eta0 + p3 * (a0 * a0 + a0 + 1.0);
+    const double n1 = -9.0 + 3.0 * eta0 - p3 * (a0 + 2.0), n2 = 3.0 + p3;
+    L.cs_m0[k] = (real)(n0 + n1 * eta0 + n2 * eta0 * eta0);
+    L.cs_m1[k] = (real)(n1 + 2.0 * n2 * eta0);
+    L.cs_m2[k] = (real)n2;
+    const double x0 = g.b * r0d, aal = g.a * c->eos.alpha;
+    L.pr_kb[k] = (real)(2.0 * M_SQRT2 * g.b / (M_SQRT2 - 1.0 + x0));
+    L.pr_x0[k] = (real)x0;
+    L.pr_rtb[k] = (real)(RT * g.b / (1.0 - x0));
+    L.pr_naD[k] = (real)(-aal / (1.0 + 2.0 * x0 - x0 * x0));
     L.cs_c0[k] = (real)(eos_mu(g.eos, g.a, g.b, RT, g.a * c->eos.alpha, r0d) - c->eos.mu_sat);
   }
   L.rho_ref = (real)c->rho_ref;
@@ -311,11 +330,10 @@ void fill_lattice(lbm_ctx* c, Lattice<real>& L) {
   L.s_eps = (real)g.s_eps;
   L.s_q = (real)g.s_q;
   L.s_nu = (real)g.s_nu;
-  // in the storage precision, as a kernel would form them
-  L.keep_e = real(1) - L.s_e;
-  L.keep_eps = real(1) - L.s_eps;
-  L.keep_q = real(1) - L.s_q;
-  L.keep_nu = real(1) - L.s_nu;
+  L.nke36 = (real)((g.s_e - 1.0) / 36.0);
+  L.kp36 = (real)((1.0 - g.s_eps) / 36.0);
+  L.kq12 = (real)((1.0 - g.s_q) / 12.0);
+  L.kn4 = (real)((1.0 - g.s_nu) / 4.0);
   L.gx = (real)g.gx;
   L.gy = (real)g.gy;
   L.bc = g.bc;
@@ -328,6 +346,10 @@ void fill_lattice(lbm_ctx* c, Lattice<real>& L) {
   L.ldir = (const uint8_t*)(w + y.ldir);
   L.lq = (const real*)(w + y.lq);
   L.lx2f = (const uint8_t*)(w + y.lx2f);
+  L.bnd = (const int2*)(w + y.bnd);
+  L.bmask = (const unsigned short*)(w + y.bmask);
+  L.bq = (const real*)(w + y.bq);
+  L.bcap = (int)y.cap.bnodes;
   L.carry = (double*)(w + y.carry);
   L.n_s1 = (int)c->n_s1;
   L.n_s2 = (int)c->n_s2;
@@ -338,6 +360,11 @@ void fill_lattice(lbm_ctx* c, Lattice<real>& L) {
   L.s2node = (const int*)(w + y.s2node);
   L.s2mask = (const uint8_t*)(w + y.s2mask);
   L.s2winv = (const real*)(w + y.s2winv);
+  L.s2nb = (const int*)(w + y.s2nb);
+  // planes the fused step leaves free
+  L.fx = (real*)(w + y.psip);
+  L.fy = (real*)(w + (c->cfg.force_model == LBM_FORCE_PSEUDO ? y.rho2 : y.mu2));
+  L.rho_next = nullptr;
   L.partials = (double*)(w + y.partials);
   L.counter = (unsigned int*)(w + y.counter);
   L.dM_ring = (double*)(w + y.dm_ring);
@@ -416,6 +443,22 @@ lbm_status validate(const lbm_config* g, char* msg) {
   return LBM_OK;
 }
 
+// Does lbm_step run the fused step?  FP32 on two population lattices with an equation of state,
+// unless the caller chose kernels of the separate passes; slabs hand their neighbours planes that
+// only the separate passes keep.
+bool fused(const lbm_ctx* c) {
+  return c->fused_ok && !c->fp64 && c->cfg.layout == LBM_LAYOUT_AB && c->cfg.eos != LBM_EOS_NONE && !c->slab.on &&
+         c->mu_kind < 0 && !c->collide_set;
+}
+
+// From the fused step to the separate passes: those start from the density planes, and find the
+// walls' chemical potential in the second mu plane too, which the fused step keeps forces in.
+cudaError_t leave_fused(lbm_ctx* c) {
+  c->rho_ok = false;
+  if (c->cfg.force_model == LBM_FORCE_PSEUDO) return cudaSuccess;
+  return cudaMemcpyAsync(c->ws + c->lay.mu2, c->ws + c->lay.mu, c->lay.plane * c->lay.sz, cudaMemcpyDeviceToDevice, c->stream);
+}
+
 // descriptors of a step from lattice `cur`: its density in plane `cur`, the boundary densities
 // into rho_b, and the next state's density plane
 template <typename real>
@@ -434,6 +477,29 @@ void step_lattices(const lbm_ctx* c, const Lattice<real>& L, int cur, Lattice<re
   Ln = Lt;
   Ln.rho = planes[cur ^ 1];
   if (alt) Ln.mu = (real*)(c->ws + (cur ? c->lay.mu : c->lay.mu2));
+}
+
+// The descriptor of the fused step from lattice `cur`: its density (pseudopotential force: psi) in
+// plane `cur`, the next state's in the other.
+Lattice<float> fused_lattice(const lbm_ctx* c, const Lattice<float>& L, int cur) {
+  Lattice<float> F = L;
+  F.rho_b = (float*)(c->ws + c->lay.rhob);
+  const bool pp = c->cfg.force_model == LBM_FORCE_PSEUDO;
+  float* planes[2] = {(float*)(c->ws + (pp ? c->lay.mu : c->lay.rho)), (float*)(c->ws + (pp ? c->lay.mu2 : c->lay.rho2))};
+  (pp ? F.mu : F.rho) = planes[cur];
+  F.rho_next = planes[cur ^ 1];
+  return F;
+}
+
+// Issues one step from lattice `cur` on the context's stream.
+template <typename real>
+cudaError_t issue_step(lbm_ctx* c, const Lattice<real>& L, int cur) {
+  if constexpr (sizeof(real) == 4) {
+    if (fused(c)) return launch_fused_step(fused_lattice(c, L, cur), cur, c->fused_rows, c->stream);
+  }
+  Lattice<real> Lt, Ln;
+  step_lattices(c, L, cur, Lt, Ln);
+  return launch_step_overlap(Lt, Ln, cur, c->stream, c->side, c->ev_fork, c->ev_join);
 }
 
 // Steps in the longest step graph (even, so that a launch keeps the lattice parity): fewer
@@ -456,14 +522,10 @@ template <typename real>
 lbm_status step_graph(lbm_ctx* c, const Lattice<real>& L, int p, int steps, cudaGraphExec_t* out) {
   cudaGraphExec_t& slot = c->graph[(steps == 2 ? 0 : steps == 1 ? 2 : 4) + p];
   if (!slot) {
-    Lattice<real> Lt, Ln;
     cudaGraph_t g;
     CUDA_OK(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e1 = cudaSuccess;
-    for (int k = 0; k < steps && e1 == cudaSuccess; ++k) {
-      step_lattices(c, L, p ^ (k & 1), Lt, Ln);
-      e1 = launch_step_overlap(Lt, Ln, p ^ (k & 1), c->stream, c->side, c->ev_fork, c->ev_join);
-    }
+    for (int k = 0; k < steps && e1 == cudaSuccess; ++k) e1 = issue_step(c, L, p ^ (k & 1));
     cudaError_t e3 = cudaStreamEndCapture(c->stream, &g);
     if (e1 != cudaSuccess || e3 != cudaSuccess)
       return fail(c, LBM_ECUDA, "graph capture failed: %s", cudaGetErrorString(e1 != cudaSuccess ? e1 : e3));
@@ -495,9 +557,13 @@ lbm_status do_step(lbm_ctx* c, const Lattice<real>& L, long long n) {
   if (n <= 0) return LBM_OK;
   lbm_status sst = step_streams(c);
   if (sst != LBM_OK) return sst;
-  Lattice<real> Lt, Ln;
+  if (!c->rho_ok && fused(c)) {
+    if constexpr (sizeof(real) == 4) CUDA_OK(c, launch_fused_prepare(fused_lattice(c, L, c->cur ^ 1), c->cur, c->stream));
+    c->rho_ok = true;
+  }
   if (!c->rho_ok) {
     // density of the current lattice and its solid layers, which the overlapped step expects
+    Lattice<real> Lt, Ln;
     step_lattices(c, L, c->cur, Lt, Ln);
     CUDA_OK(c, launch_phase(Lt, c->cur, 0, c->stream));
     CUDA_OK(c, launch_phase(Lt, c->cur, 1, c->stream));
@@ -529,8 +595,7 @@ lbm_status do_step(lbm_ctx* c, const Lattice<real>& L, long long n) {
     n = 0;
   }
   for (long long k = 0; k < n; ++k) {
-    step_lattices(c, L, c->cur, Lt, Ln);
-    CUDA_OK(c, launch_step_overlap(Lt, Ln, c->cur, c->stream, c->side, c->ev_fork, c->ev_join));
+    CUDA_OK(c, issue_step(c, L, c->cur));
     c->cur ^= 1;
   }
   return LBM_OK;
@@ -960,9 +1025,14 @@ lbm_status lbm_build_links(lbm_ctx* c) {
   o.kind = (uint8_t*)(w + y.kind);
   o.bnode = (int*)(w + y.bnode); o.bstart = (int*)(w + y.bstart); o.ldir = (uint8_t*)(w + y.ldir);
   o.lq64 = (double*)(w + y.lq64); o.lx2f = (uint8_t*)(w + y.lx2f); o.lq = w + y.lq;
+  if (!c->fp64) {
+    o.bnd = (int2*)(w + y.bnd); o.bmask = (unsigned short*)(w + y.bmask); o.bq = w + y.bq;
+    o.bcap = (int)y.cap.bnodes;
+  }
   o.s1node = (int*)(w + y.s1node); o.s1mask = (uint8_t*)(w + y.s1mask); o.s1winv = w + y.s1winv;
   o.s1nb = (int*)(w + y.s1nb);
   o.s2node = (int*)(w + y.s2node); o.s2mask = (uint8_t*)(w + y.s2mask); o.s2winv = w + y.s2winv;
+  o.s2nb = (int*)(w + y.s2nb);
   o.mu = w + y.mu;
   o.fp64 = c->fp64;
   o.n_bnodes = (int)c->n_bnodes;
@@ -1005,8 +1075,13 @@ lbm_status lbm_build_links(lbm_ctx* c) {
     const long long tiles = (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8);
     c->collide_kind = (c->tma_ok && tiles >= 16LL * c->tma.blocks[g.force_model == LBM_FORCE_PSEUDO ? 1 : 0]) ? 1 : 0;
     refresh(c);
-    // the list of nodes the fused density + mu pass leaves to k_mu_near, where that pass runs
-    if (c->Lf.mu_kernel == 3) {
+    int dev = 0, sms = 0;
+    c->fused_ok = cudaGetDevice(&dev) == cudaSuccess &&
+                  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && fused_setup();
+    if (!c->fused_ok) (void)cudaGetLastError();
+    c->fused_rows = fused_rows(g.nx, g.ny, sms);
+    // the list of nodes the combined density + mu pass leaves to k_mu_near, where that pass runs
+    if (c->Lf.mu_kernel == 3 && !fused(c)) {
       lbm_status st = near_list(c);
       if (st != LBM_OK) return st;
       refresh(c);
@@ -1127,7 +1202,16 @@ lbm_status lbm_set_collide_kernel(lbm_ctx* c, int32_t kind) {
     return fail(c, LBM_EINVAL,
                 "the column sweeps need the chemical-potential force with an equation of state, nx a multiple of 32 "
                 "and ny of 8, and a whole lattice of two population lattices");
-  if (kind == c->collide_kind) return LBM_OK;
+  if (kind == c->collide_kind && c->collide_set) return LBM_OK;
+  if (!c->collide_set) {
+    const bool was = fused(c);
+    c->collide_set = true;
+    if (was) CUDA_OK(c, leave_fused(c));
+    if (!c->fp64 && c->Lf.mu_kernel == 3 && !c->near_built) {
+      lbm_status st = near_list(c);
+      if (st != LBM_OK) return st;
+    }
+  }
   c->collide_kind = kind;
   // captured launches carry the old kernel: capture again
   for (auto& gr : c->graph)
@@ -1158,8 +1242,9 @@ lbm_status lbm_set_mu_kernel(lbm_ctx* c, int32_t kind) {
     return fail(c, LBM_EINVAL, "the fused chemical-potential kernel needs the chemical-potential force");
   if (kind == 3 && c->cfg.layout == LBM_LAYOUT_AA)
     return fail(c, LBM_EINVAL, "the fused chemical-potential kernel needs two population lattices");
+  if (fused(c)) CUDA_OK(c, leave_fused(c));
   c->mu_kind = kind;
-  c->rho_ok = false;   // a change to or from the fused pass moves where mu is kept
+  c->rho_ok = false;   // a change to or from the combined pass moves where mu is kept
   if (kind == 3 && !c->near_built) {
     lbm_status st = near_list(c);
     if (st != LBM_OK) return st;
@@ -1181,7 +1266,7 @@ lbm_status lbm_get_collide_kernel(lbm_ctx* c, int32_t* kind) {
 
 lbm_status lbm_launches_per_step(lbm_ctx* c, int64_t* n) {
   if (!c || !c->built || !n) return LBM_ESTATE;
-  *n = c->fp64 ? launches_per_step_overlap(c->Ld) : launches_per_step_overlap(c->Lf);
+  *n = fused(c) ? fused_launches(c->Lf) : c->fp64 ? launches_per_step_overlap(c->Ld) : launches_per_step_overlap(c->Lf);
   return LBM_OK;
 }
 

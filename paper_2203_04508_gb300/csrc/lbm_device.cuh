@@ -39,6 +39,9 @@ struct Lattice {
   real* rho_b;                  // if set: the boundary phase leaves the density of each
                                 // boundary node's final populations here (one per node)
   real* mu;                     // chemical potential minus k^2 mu_sat (constant at solids)
+  real* rho_next;               // fused step (FP32): the next state's density (psi) plane
+  real* fx;                     // fused step (FP32): the force at nodes next to solids, left by
+  real* fy;                     // the pass for the boundary phase
   real* psip;                   // if set: psi'(rho) - mu_sat of every fluid node, left by the
                                 // density pass for the chemical-potential pass (single lattices)
   const uint8_t* kind;
@@ -49,14 +52,18 @@ struct Lattice {
   real RT, a, b, aalpha, k2, kappa, mu_sat;
   real rho_split;                // sqrt(rho_g rho_l): below it mu is evaluated against rho_g
   // CS, per reference density rho0 in {rho_g, rho_l} (index 0 gas, 1 liquid), storage-rounded:
-  // rho0, 1/rho0, eta0 = b rho0/4, a0 = 1 - eta0, P(eta0)/a0^3, psi'(rho0) - mu_sat (FP64 on host)
-  real cs_r0[2], cs_inv_r0[2], cs_eta0[2], cs_a0[2], cs_p0a3[2], cs_c0[2];
+  // rho0, 1/rho0, the coefficients of N(h) (psi_prime_cs), psi'(rho0) - mu_sat (FP64 on the host)
+  real b4;                       // b / 4
+  real cs_r0[2], cs_inv_r0[2], cs_m0[2], cs_m1[2], cs_m2[2], cs_c0[2];
+  // PR, besides rho0, 1/rho0 and psi'(rho0) - mu_sat: -K; 2 sqrt 2 b/(c1+x0), x0, RT b/(1-x0),
+  // -a alpha/D0 (psi_prime_pr)
+  real pr_nk, pr_kb[2], pr_x0[2], pr_rtb[2], pr_naD[2];
   real rho_ref;
   // collision, Eqs. 3-4
   int coll;
   real omega;                   // 1 / tau (BGK)
   real s_e, s_eps, s_q, s_nu;
-  real keep_e, keep_eps, keep_q, keep_nu;   // 1 - s_k, formed once in the storage precision
+  real nke36, kp36, kq12, kn4;  // (s_e - 1)/36, (1 - s_eps)/36, (1 - s_q)/12, (1 - s_nu)/4
   real gx, gy;
   int bc;
   // pseudopotential force model (instead of Eqs. 9 and 12): mu holds psi, the solid layers
@@ -71,6 +78,12 @@ struct Lattice {
   const uint8_t* ldir;
   const real* lq;
   const uint8_t* lx2f;
+  // the same by boundary node (FP32): node and column; bits 0-7 the directions 1-8 it cuts, bits
+  // 8-15 whether x2 is fluid there; q of direction i at bq[(i - 1) bcap + b]
+  const int2* bnd;
+  const unsigned short* bmask;
+  const real* bq;
+  int bcap;
   // first and second solid layers for Eq. 15
   int n_s1, n_s2;
   const int* s1node;
@@ -78,6 +91,8 @@ struct Lattice {
   const int* s1nb;              // per first-layer entry, 8 ints: the boundary-node index of each
                                 // contributing neighbour (-1 elsewhere)
   const real* s1winv;
+  const int* s2nb;              // per second-layer entry, 8 ints: the first-layer index of each
+                                // contributing neighbour (-1 elsewhere)
   const int* s2node;
   const uint8_t* s2mask;
   const real* s2winv;
@@ -151,60 +166,172 @@ __device__ __forceinline__ void load_pops(const Lattice<real>& L, int c, int x, 
 // the EOS terms, the force and mu are assembled through these, so that every kernel that
 // evaluates them (density, scatter, chemical potential, collide, boundary, read-out, batched)
 // gets the same bits.
+// The same functions on float2 take two nodes at once in sm_103a's packed FP32 instructions
+// (add / sub / mul / fma .f32x2), each half rounded like the scalar operation: half the issue
+// slots, the same bits.
+// One difference: ptxas fuses a packed product with a packed sum that follows, rounding spelled
+// out or not, so shared code hands a product to fma_rn or another product, never to add_rn or sub_rn.
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+#define LBMGB_PACKED(name, op)                                                            \
+  __device__ __forceinline__ float2 name(float2 a, float2 b) {                           \
+    float2 d;                                                                            \
+    asm(op ".rn.f32x2 %0, %1, %2;"                                                       \
+        : "=l"(reinterpret_cast<unsigned long long&>(d))                                 \
+        : "l"(reinterpret_cast<const unsigned long long&>(a)),                           \
+          "l"(reinterpret_cast<const unsigned long long&>(b)));                          \
+    return d;                                                                            \
+  }
+LBMGB_PACKED(add_rn, "add")
+LBMGB_PACKED(sub_rn, "sub")
+LBMGB_PACKED(mul_rn, "mul")
+#undef LBMGB_PACKED
+__device__ __forceinline__ float2 fma_rn(float2 a, float2 b, float2 c) {
+  float2 d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;"
+      : "=l"(reinterpret_cast<unsigned long long&>(d))
+      : "l"(reinterpret_cast<const unsigned long long&>(a)), "l"(reinterpret_cast<const unsigned long long&>(b)),
+        "l"(reinterpret_cast<const unsigned long long&>(c)));
+  return d;
+}
+// the same value in every half
+template <typename V> struct SplatOf;
+template <> struct SplatOf<float> { static __device__ __forceinline__ float of(float a) { return a; } };
+template <> struct SplatOf<double> { static __device__ __forceinline__ double of(double a) { return a; } };
+template <> struct SplatOf<float2> { static __device__ __forceinline__ float2 of(float a) { return make_float2(a, a); } };
+template <typename V, typename T>
+__device__ __forceinline__ V splat(T a) { return SplatOf<V>::of(a); }
+// the scalar type of a value of one or two nodes
+template <typename V> struct ScalarOf { using type = V; };
+template <> struct ScalarOf<float2> { using type = float; };
+
+// FP32 reciprocal, square root and log1p without branches, so that the instructions around them
+// interleave (the compiler's division and log1pf test for special arguments and branch): the
+// hardware approximation and one Newton step each, within an ulp for normal arguments; an
+// argument of zero gives NaN.
+__device__ __forceinline__ float approx_rcp(float a) { float y; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(a)); return y; }
+__device__ __forceinline__ float2 approx_rcp(float2 a) { return make_float2(approx_rcp(a.x), approx_rcp(a.y)); }
+template <typename V>
+__device__ __forceinline__ V recip(V a) {
+  const V y = approx_rcp(a);
+  return fma_rn(y, fma_rn(mul_rn(splat<V>(-1.0f), a), y, splat<V>(1.0f)), y);
+}
+template <>
+__device__ __forceinline__ double recip<double>(double a) { return 1.0 / a; }
+// sqrt of positive values
+__device__ __forceinline__ float approx_rsqrt(float a) { float y; asm("rsqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(a)); return y; }
+__device__ __forceinline__ float2 approx_rsqrt(float2 a) { return make_float2(approx_rsqrt(a.x), approx_rsqrt(a.y)); }
+template <typename V>
+__device__ __forceinline__ V root(V a) {
+  const V y = approx_rsqrt(a), q = mul_rn(a, y);
+  return fma_rn(fma_rn(mul_rn(splat<V>(-1.0f), q), q, a), mul_rn(splat<V>(0.5f), y), q);
+}
+template <>
+__device__ __forceinline__ double root<double>(double a) { return sqrt(a); }
+// log(1 + a b).  2^e is the power of two that brings 1 + a b into [sqrt(1/2), sqrt(2)), f = (1 +
+// a b) 2^-e - 1 (one rounding: 2^-e - 1 is exact), log = e ln 2 + f + f^2 Q(f) with Q the
+// weighted minimax polynomial of degree 8 on that range (fitted for this file by iterated least
+// squares; relative error 4e-9, with FP32 rounding at most 0.6 ulp).  NaN unless 1 + a b > 0.
+__device__ __forceinline__ int log_exponent(float u) { return (__float_as_int(u) - 0x3f3504f3) & (int)0xff800000; }
+__device__ __forceinline__ float log_or_nan(float u, float v) { return u > 0.0f ? v : __int_as_float(0x7fffffff); }
+struct LogParts {   // k: e 2^23, s: 2^-e
+  static __device__ __forceinline__ void of(float u, float& k, float& s) {
+    const int i = log_exponent(u);
+    k = (float)i;
+    s = __int_as_float(0x3f800000 - i);
+  }
+  static __device__ __forceinline__ void of(float2 u, float2& k, float2& s) {
+    of(u.x, k.x, s.x);
+    of(u.y, k.y, s.y);
+  }
+  static __device__ __forceinline__ float checked(float u, float v) { return log_or_nan(u, v); }
+  static __device__ __forceinline__ float2 checked(float2 u, float2 v) {
+    return make_float2(log_or_nan(u.x, v.x), log_or_nan(u.y, v.y));
+  }
+};
+template <typename V>
+__device__ __forceinline__ V log1p_product(V a, V b) {
+  auto K = [](float c) { return splat<V>(c); };
+  const V u = fma_rn(a, b, K(1.0f)), z = mul_rn(a, b);
+  V k, s;
+  LogParts::of(u, k, s);
+  const V f = fma_rn(z, s, sub_rn(s, K(1.0f)));
+  V q = fma_rn(K(-0.0762307197f), f, K(0.1290552169f));
+  q = fma_rn(q, f, K(-0.1324298531f));
+  q = fma_rn(q, f, K(0.1418163329f));
+  q = fma_rn(q, f, K(-0.1660905629f));
+  q = fma_rn(q, f, K(0.2000198513f));
+  q = fma_rn(q, f, K(-0.2500158549f));
+  q = fma_rn(q, f, K(0.3333332539f));
+  q = fma_rn(q, f, K(-0.4999998808f));
+  const V r = fma_rn(mul_rn(f, f), q, f);
+  return LogParts::checked(u, fma_rn(k, K(8.26295829e-8f), r));   // ln 2 / 2^23
+}
+template <>
+__device__ __forceinline__ double log1p_product<double>(double a, double b) { return log1p(__dmul_rn(a, b)); }
+// hi where r > split, else lo
+__device__ __forceinline__ float pick(float r, float split, float lo, float hi) { return r > split ? hi : lo; }
+__device__ __forceinline__ double pick(double r, double split, double lo, double hi) { return r > split ? hi : lo; }
+__device__ __forceinline__ float2 pick(float2 r, float split, float lo, float hi) {
+  return make_float2(r.x > split ? hi : lo, r.y > split ? hi : lo);
+}
 
 // ---------------------------------------------------------------------------------------
 // Equation of state: bulk chemical potential psi'(rho) minus its coexistence value.
 //   CS: psi' = RT [ln rho + (8 eta - 9 eta^2 + 3 eta^3)/(1-eta)^3] - 2 a rho,  eta = b rho/4
 //   PR: Eq. 11 without the gradient term.
 // ---------------------------------------------------------------------------------------
-__device__ __forceinline__ float dev_log(float x) { return logf(x); }
-__device__ __forceinline__ double dev_log(double x) { return log(x); }
-
-__device__ __forceinline__ float dev_log1p(float x) { return log1pf(x); }
-__device__ __forceinline__ double dev_log1p(double x) { return log1p(x); }
 
 // CS: psi'(rho) - mu_sat evaluated against the nearer coexistence density rho0 (gas below
 // sqrt(rho_g rho_l), liquid above), where psi'(rho0) = mu_sat:
 //   RT ln(rho/rho0) + RT [G(eta) - G(eta0)] - 2a (rho - rho0) + c0,
 //   G(eta) = P(eta)/(1-eta)^3,  P = 8 eta - 9 eta^2 + 3 eta^3,
 // with ln(rho/rho0) = log1p((rho - rho0)/rho0) and the exact factorisation
-//   G(eta) - G(eta0) = h { [8 - 9(eta+eta0) + 3(eta^2 + eta eta0 + eta0^2)] / b^3
-//                          + P(eta0) (a^2 + a b + b^2) / (a^3 b^3) },
-//   h = eta - eta0, a = 1 - eta0, b = 1 - eta,
-// so that every term vanishes with rho - rho0 (which is exact near rho0) instead of cancelling
-// between terms of size RT ln rho.  c0 = psi'(rho0) - mu_sat of the storage-rounded rho0 is
-// computed in FP64 on the host, so both branches meet the same function.  One division.
-template <typename real>
-__device__ __forceinline__ real psi_prime_shifted(const Lattice<real>& L, real r) {
-  if (L.eos == EOS_CS) {
-    const int k = r > L.rho_split ? 1 : 0;
-    const real dr = r - L.cs_r0[k];
-    const real eta0 = L.cs_eta0[k], a = L.cs_a0[k];
-    const real eta = mul_rn(mul_rn(L.b, r), real(0.25));
-    const real h = mul_rn(mul_rn(L.b, dr), real(0.25));
-    const real bb = real(1) - eta;
-    const real ib = real(1) / bb;
-    const real ib3 = mul_rn(mul_rn(ib, ib), ib);
-    // 8 - 9 (eta + eta0) + 3 (eta^2 + eta eta0 + eta0^2),  P(eta0) (a^2 + a b + b^2) / (a^3 b^3)
-    const real sq = fma_rn(eta, eta, fma_rn(eta, eta0, mul_rn(eta0, eta0)));
-    const real q1 = fma_rn(real(3), sq, fma_rn(real(-9), eta + eta0, real(8)));
-    const real q2 = mul_rn(L.cs_p0a3[k], fma_rn(a, a, fma_rn(a, bb, mul_rn(bb, bb))));
-    const real t1 = mul_rn(L.RT, dev_log1p(mul_rn(dr, L.cs_inv_r0[k])));
-    const real t2 = mul_rn(mul_rn(L.RT, h), mul_rn(q1 + q2, ib3));
-    return (t1 + t2) + fma_rn(mul_rn(real(-2), L.a), dr, L.cs_c0[k]);
-  }
-  // Peng-Robinson, Eq. 11 without the gradient term
-  const real s2 = real(1.4142135623730951);
-  const real br = mul_rn(L.b, r);
-  const real om = real(1) - br;
-  const real t1 = mul_rn(L.RT, dev_log(r / om));
-  const real t2 = mul_rn(L.aalpha / mul_rn(real(2) * s2, L.b), dev_log((s2 - real(1) + br) / (s2 + real(1) - br)));
-  const real t4 = mul_rn(L.aalpha, r) / fma_rn(-br, br, fma_rn(real(2), br, real(1)));
-  return (((t1 - t2) + L.RT / om) - t4) - L.mu_sat;
+//   G(eta) - G(eta0) = h N(h) / (1-eta)^3,  h = eta - eta0,  a = 1 - eta0,
+//   N = 8 - 9(eta+eta0) + 3(eta^2 + eta eta0 + eta0^2) + (P(eta0)/a^3) (a^2 + a (1-eta) + (1-eta)^2),
+// a quadratic m0 + m1 h + m2 h^2 in h whose coefficients belong to rho0, so that every term
+// vanishes with rho - rho0 (which is exact near rho0) instead of cancelling between terms of size
+// RT ln rho.  c0 = psi'(rho0) - mu_sat of the storage-rounded rho0 and the m's are computed in
+// FP64 on the host, so both branches meet the same function.  One reciprocal.
+template <typename V, typename real>
+__device__ __forceinline__ V psi_prime_cs(const Lattice<real>& L, V r) {
+  auto K = [](real c) { return splat<V>(c); };
+  auto C = [&](const real (&c)[2]) { return pick(r, L.rho_split, c[0], c[1]); };
+  const V dr = sub_rn(r, C(L.cs_r0));
+  const V h = mul_rn(K(L.b4), dr);
+  const V ib = recip(fma_rn(K(-L.b4), r, K(1)));
+  const V ib3 = mul_rn(mul_rn(ib, ib), ib);
+  const V N = fma_rn(fma_rn(C(L.cs_m2), h, C(L.cs_m1)), h, C(L.cs_m0));
+  const V lg = log1p_product(dr, C(L.cs_inv_r0));
+  return fma_rn(K(L.RT), lg, fma_rn(mul_rn(K(L.RT), h), mul_rn(N, ib3), fma_rn(K(real(-2) * L.a), dr, C(L.cs_c0))));
+}
+// Peng-Robinson, Eq. 11 without the gradient term,
+//   RT ln(rho/(1-x)) - K ln((c1+x)/(c2-x)) + RT/(1-x) - a alpha rho/D - mu_sat,
+//   x = b rho, c1,2 = sqrt 2 -+ 1, D = 1 + 2x - x^2 = (c1+x)(c2-x), K = a alpha/(2 sqrt 2 b),
+// against the nearer coexistence density likewise: the differences from rho0 are, exactly,
+//   ln: log1p(dr / (rho0 (1-x))) and log1p(2 sqrt 2 b dr / ((c1+x0)(c2-x))),
+//   RT b dr / ((1-x0)(1-x)),  a alpha dr (1 + x x0) / (D0 D).
+template <typename V, typename real>
+__device__ __forceinline__ V psi_prime_pr(const Lattice<real>& L, V r) {
+  auto K = [](real c) { return splat<V>(c); };
+  auto C = [&](const real (&c)[2]) { return pick(r, L.rho_split, c[0], c[1]); };
+  const V dr = sub_rn(r, C(L.cs_r0)), x = mul_rn(K(L.b), r);
+  const V iom = recip(fma_rn(K(-L.b), r, K(1))), ic2 = recip(fma_rn(K(-L.b), r, K(real(2.414213562373095))));
+  const V iD = mul_rn(ic2, recip(fma_rn(K(L.b), r, K(real(0.41421356237309503)))));
+  const V l1 = log1p_product(dr, mul_rn(C(L.cs_inv_r0), iom)), l2 = log1p_product(dr, mul_rn(C(L.pr_kb), ic2));
+  const V t = mul_rn(mul_rn(C(L.pr_naD), fma_rn(x, C(L.pr_x0), K(1))), iD);
+  const V S = fma_rn(C(L.pr_rtb), iom, t);
+  return fma_rn(K(L.RT), l1, fma_rn(K(L.pr_nk), l2, fma_rn(dr, S, C(L.cs_c0))));
+}
+template <typename V, typename real>
+__device__ __forceinline__ V psi_prime_shifted(const Lattice<real>& L, V r) {
+  return L.eos == EOS_CS ? psi_prime_cs(L, r) : psi_prime_pr(L, r);
 }
 
 // Fourth-order central first derivatives and Laplacian along the lattice axes.
@@ -241,9 +368,9 @@ __device__ __forceinline__ Stencil stencil_at(const Lattice<real>& L, int x, int
 
 // Undivided fourth-order differences D(p) = 8 (p_1 - p_-1) - (p_2 - p_-2) = 12 dp/dx along
 // each axis (8 x exact, so fused or not it rounds the same).
-template <typename real>
-__device__ __forceinline__ real diff4_of(real p1, real pm1, real p2, real pm2) {
-  return real(8) * (p1 - pm1) - (p2 - pm2);
+template <typename V>
+__device__ __forceinline__ V diff4_of(V p1, V pm1, V p2, V pm2) {
+  return fma_rn(splat<V>(typename ScalarOf<V>::type(8)), sub_rn(p1, pm1), sub_rn(pm2, p2));
 }
 template <typename real>
 __device__ __forceinline__ void diff4(const real* __restrict__ p, const Stencil& s, real& dx, real& dy) {
@@ -262,12 +389,17 @@ __device__ __forceinline__ void grad4(const real* __restrict__ p, const Stencil&
 // (16 [(p1 - c) + (p-1 - c)] - [(p2 - c) + (p-2 - c)])/12: inside a bulk phase the
 // differences are exact (Sterbenz), so FP32 keeps the Laplacian's relative accuracy there
 // instead of losing it to cancellation between terms of size 30 rho.
-template <typename real>
-__device__ __forceinline__ real lap4_of(real c, real xp1, real xm1, real xp2, real xm2, real yp1, real ym1, real yp2,
-                                        real ym2) {
-  real lx = real(16) * ((xp1 - c) + (xm1 - c)) - ((xp2 - c) + (xm2 - c));
-  real ly = real(16) * ((yp1 - c) + (ym1 - c)) - ((yp2 - c) + (ym2 - c));
-  return (lx + ly) * real(1.0 / 12.0);
+// the Laplacian from the second differences over one node and the negated ones over two, x and y
+template <typename V>
+__device__ __forceinline__ V lap4_diff(V x1, V nx2, V y1, V ny2) {
+  using real = typename ScalarOf<V>::type;
+  const V c16 = splat<V>(real(16));
+  return mul_rn(add_rn(fma_rn(c16, x1, nx2), fma_rn(c16, y1, ny2)), splat<V>(real(1.0 / 12.0)));
+}
+template <typename V>
+__device__ __forceinline__ V lap4_of(V c, V xp1, V xm1, V xp2, V xm2, V yp1, V ym1, V yp2, V ym2) {
+  return lap4_diff(add_rn(sub_rn(xp1, c), sub_rn(xm1, c)), add_rn(sub_rn(c, xp2), sub_rn(c, xm2)),
+                   add_rn(sub_rn(yp1, c), sub_rn(ym1, c)), add_rn(sub_rn(c, yp2), sub_rn(c, ym2)));
 }
 template <typename real>
 __device__ __forceinline__ real lap4(const real* __restrict__ p, int n, const Stencil& s) {
@@ -276,18 +408,20 @@ __device__ __forceinline__ real lap4(const real* __restrict__ p, int n, const St
 
 
 // Eq. 12 in mesh units, shifted: mu~ = k^2 (psi'(rho) - mu_sat) - kappa^ lap(rho)
-template <typename real>
-__device__ __forceinline__ real mu_of(const Lattice<real>& L, real psip, real lap) {
-  return fma_rn(L.k2, psip, -mul_rn(L.kappa, lap));
+template <typename V, typename real>
+__device__ __forceinline__ V mu_of(const Lattice<real>& L, V psip, V lap) {
+  return fma_rn(splat<V>(L.k2), psip, mul_rn(splat<V>(-L.kappa), lap));
 }
 // delta rho / 36 to within an ulp: the product with the rounded reciprocal, corrected once
 // with its FMA residual
-__device__ __forceinline__ float div36(float d) {
-  const float c = 1.0f / 36.0f;
-  const float q = d * c;
-  return fmaf(fmaf(-36.0f, q, d), c, q);
+template <typename V>
+__device__ __forceinline__ V div36(V d) {
+  const V c = splat<V>(1.0f / 36.0f);
+  const V q = mul_rn(d, c);
+  return fma_rn(fma_rn(splat<V>(-36.0f), q, d), c, q);
 }
-__device__ __forceinline__ double div36(double d) { return d / 36.0; }
+template <>
+__device__ __forceinline__ double div36<double>(double d) { return d / 36.0; }
 
 // F = rho g - rho grad(mu) + c_s^2 grad(rho) (Eq. 9), one component, from the undivided
 // differences D(mu) and D(rho) of diff4 (grad = D/12, c_s^2 = 1/3):
@@ -297,49 +431,64 @@ __device__ __forceinline__ double div36(double d) { return d / 36.0; }
 // within an ulp: no rounded constant (1/12, 1/3) scales either term, because such a constant
 // biases the force the same way at every node and step, and that bias builds up in the flow
 // where unbiased rounding errors do not.
-template <typename real>
-__device__ __forceinline__ real force_cp(real r, real g, real dmu, real drho) {
-  const real p = mul_rn(r, dmu);
-  const real e = fma_rn(r, dmu, -p);
-  const real G = fma_rn(real(-3), e, fma_rn(real(-3), p, drho));
-  return fma_rn(r, g, div36(G));
+template <typename V, typename real>
+__device__ __forceinline__ V force_cp(V r, real g, V dmu, V drho) {
+  const V pn = mul_rn(mul_rn(splat<V>(real(-1)), r), dmu);   // -r D(mu)
+  const V e = fma_rn(r, dmu, pn);
+  const V G = fma_rn(splat<V>(real(-3)), e, fma_rn(splat<V>(real(3)), pn, drho));
+  return fma_rn(r, splat<V>(g), div36(G));
 }
 // F = rho g + c a, the pseudopotential force of centre value c and sum a, one component
-template <typename real>
-__device__ __forceinline__ real force_pp(real r, real g, real c, real a) {
-  return fma_rn(c, a, mul_rn(r, g));
+template <typename V, typename real>
+__device__ __forceinline__ V force_pp(V r, real g, V c, V a) {
+  return fma_rn(c, a, mul_rn(r, splat<V>(g)));
 }
 
 // Pseudopotential of the pseudopotential force model, psi = [2 (rho c_s^2 - k^2 p0(rho))]^(1/2)
 // clamped at zero (rho c_s^2 + (G/2) psi^2 = k^2 p0 with G = -1), p0 the CS or PR pressure.
+// As 2 rho w with w = 1/3 - k^2 p0 / rho.
+template <typename V, typename real>
+__device__ __forceinline__ V psi_cs(const Lattice<real>& L, V r) {
+  auto K = [](real c) { return splat<V>(c); };
+  const V om = fma_rn(K(-L.b4), r, K(1)), eta = mul_rn(K(L.b4), r);
+  const V ib = recip(om);
+  const V poly = fma_rn(eta, fma_rn(eta, om, K(1)), K(1));   // 1 + eta + eta^2 - eta^3
+  const V t = fma_rn(mul_rn(K(L.RT), poly), mul_rn(mul_rn(ib, ib), ib), mul_rn(K(-L.a), r));
+  const V w = fma_rn(K(-L.k2), t, K(real(1.0 / 3.0)));
+  return mul_rn(mul_rn(K(2), r), w);
+}
+__device__ __forceinline__ float positive_root(float a, float q) { return a > 0.0f ? q : 0.0f; }
+__device__ __forceinline__ double positive_root(double a, double q) { return a > 0.0 ? q : 0.0; }
+__device__ __forceinline__ float2 positive_root(float2 a, float2 q) {
+  return make_float2(positive_root(a.x, q.x), positive_root(a.y, q.y));
+}
+template <typename real>
+__device__ __forceinline__ real psi_pr(const Lattice<real>& L, real r) {
+  const real br = mul_rn(L.b, r);
+  const real p0 = mul_rn(r, L.RT) / (real(1) - br) - mul_rn(mul_rn(L.aalpha, r), r) / fma_rn(br, real(2) - br, real(1));
+  return mul_rn(real(2), fma_rn(r, real(1.0 / 3.0), -mul_rn(L.k2, p0)));
+}
 template <typename real>
 __device__ __forceinline__ real psi_of(const Lattice<real>& L, real r) {
-  real p0;
-  if (L.eos == EOS_CS) {
-    const real eta = mul_rn(mul_rn(L.b, r), real(0.25));
-    const real om = real(1) - eta;
-    const real poly = fma_rn(eta, fma_rn(eta, real(1) - eta, real(1)), real(1));   // 1 + eta + eta^2 - eta^3
-    p0 = mul_rn(mul_rn(r, L.RT), poly) / mul_rn(mul_rn(om, om), om) - mul_rn(mul_rn(L.a, r), r);
-  } else {
-    const real br = mul_rn(L.b, r);
-    p0 = mul_rn(r, L.RT) / (real(1) - br) - mul_rn(mul_rn(L.aalpha, r), r) / fma_rn(br, real(2) - br, real(1));
-  }
-  const real arg = mul_rn(real(2), fma_rn(r, real(1.0 / 3.0), -mul_rn(L.k2, p0)));
-  return arg > real(0) ? sqrt(arg) : real(0);
+  const real arg = L.eos == EOS_CS ? psi_cs(L, r) : psi_pr(L, r);
+  return positive_root(arg, root(arg));
+}
+__device__ __forceinline__ float2 psi_of(const Lattice<float>& L, float2 r) {
+  const float2 arg = L.eos == EOS_CS ? psi_cs(L, r) : make_float2(psi_pr(L, r.x), psi_pr(L, r.y));
+  return positive_root(arg, root(arg));
 }
 
 // Adds the pseudopotential force -G psi(x) sum_i w_i psi(x + e_i) e_i (G = -1, w = 1/3 on the
 // axes, 1/12 on the diagonals) from the centre value c and the eight neighbours, as
 // differences of opposite neighbours (exact inside a bulk phase).
-template <typename real>
-__device__ __forceinline__ void pp_sums(real e, real n, real w, real s, real ne, real nw, real sw, real se, real& ax,
-                                        real& ay) {
-  const real d1 = ne - sw, d2 = se - nw;
-  const real third = real(1.0 / 3.0), twelfth = real(1.0 / 12.0);
-  ax = (e - w) * third + (d1 + d2) * twelfth;
-  ay = (n - s) * third + (d1 - d2) * twelfth;
+template <typename V>
+__device__ __forceinline__ void pp_sums(V e, V n, V w, V s, V ne, V nw, V sw, V se, V& ax, V& ay) {
+  using real = typename ScalarOf<V>::type;
+  const V d1 = sub_rn(ne, sw), d2 = sub_rn(se, nw);
+  const V third = splat<V>(real(1.0 / 3.0)), twelfth = splat<V>(real(1.0 / 12.0));
+  ax = fma_rn(sub_rn(e, w), third, mul_rn(add_rn(d1, d2), twelfth));
+  ay = fma_rn(sub_rn(n, s), third, mul_rn(sub_rn(d1, d2), twelfth));
 }
-
 
 // Nonideal force of Eq. 9 in mesh units, F = -rho grad(mu^) + c_s^2 grad(rho), plus rho g;
 // with PSEUDO the pseudopotential force from the psi plane instead.
@@ -374,32 +523,36 @@ __device__ __forceinline__ void force_at(const Lattice<real>& L, int x, int y, r
 //   w_i rho [3 e.du + 4.5 (e.du)(e.(2u+du)) - 1.5 du.(2u+du)].
 template <typename real>
 __device__ __forceinline__ real edm_term(int i, real r, real ux, real uy, real dux, real duy) {
-  real edu = real(ex(i)) * dux + real(ey(i)) * duy;
-  real e2u = real(ex(i)) * (real(2) * ux + dux) + real(ey(i)) * (real(2) * uy + duy);
-  real du2u = dux * (real(2) * ux + dux) + duy * (real(2) * uy + duy);
-  return real(wgt(i)) * r * (real(3) * edu + real(4.5) * edu * e2u - real(1.5) * du2u);
+  // (products rounded explicitly: every kernel that evaluates a link gets the same bits)
+  const real ax = real(2) * ux + dux, ay = real(2) * uy + duy;
+  const real edu = real(ex(i)) * dux + real(ey(i)) * duy;
+  const real e2u = real(ex(i)) * ax + real(ey(i)) * ay;
+  const real du2u = fma_rn(dux, ax, mul_rn(duy, ay));
+  const real t = fma_rn(real(3), edu, fma_rn(mul_rn(real(4.5), edu), e2u, mul_rn(real(-1.5), du2u)));
+  return mul_rn(mul_rn(real(wgt(i)), r), t);
 }
 
 // Moments of a node's offset populations: delta rho = sum_i (f_i - w_i rho_ref) and
 // j = sum_i f_i e_i.  j is summed as differences of opposite populations, which are exact in
 // floating point near equilibrium (Sterbenz), so the momentum keeps its relative accuracy
 // although it is a small difference of populations of size ~rho/9.
-template <typename real>
-__device__ __forceinline__ real density_sum(const real (&f)[9]) {
-  return f[0] + (((f[1] + f[3]) + (f[2] + f[4])) + ((f[5] + f[7]) + (f[6] + f[8])));
+template <typename V>
+__device__ __forceinline__ V density_sum(const V (&f)[9]) {
+  return add_rn(f[0], add_rn(add_rn(add_rn(f[1], f[3]), add_rn(f[2], f[4])), add_rn(add_rn(f[5], f[7]), add_rn(f[6], f[8]))));
 }
 
-template <typename real>
-__device__ __forceinline__ void moments(const real (&f)[9], real& drho, real& jx, real& jy) {
+template <typename V>
+__device__ __forceinline__ void moments(const V (&f)[9], V& drho, V& jx, V& jy) {
   drho = density_sum(f);
-  jx = (f[1] - f[3]) + ((f[5] - f[7]) + (f[8] - f[6]));
-  jy = (f[2] - f[4]) + ((f[5] - f[7]) + (f[6] - f[8]));
+  const V d57 = sub_rn(f[5], f[7]), d86 = sub_rn(f[8], f[6]);
+  jx = add_rn(sub_rn(f[1], f[3]), add_rn(d57, d86));
+  jy = add_rn(sub_rn(f[2], f[4]), sub_rn(d57, d86));
 }
 
 // Density as the read-out pass and the sweep store it (the same sum, in the same order).
-template <typename real>
-__device__ __forceinline__ real density_of(const Lattice<real>& L, const real (&f)[9]) {
-  return L.rho_ref + density_sum(f);
+template <typename V, typename real>
+__device__ __forceinline__ V density_of(const Lattice<real>& L, const V (&f)[9]) {
+  return add_rn(splat<V>(L.rho_ref), density_sum(f));
 }
 
 // Collision (Eq. 4) of offset populations with the exact-difference term (Eq. 13).
@@ -417,103 +570,102 @@ __device__ __forceinline__ real density_of(const Lattice<real>& L, const real (&
 // from rho/9 and rho/36 times u = J/rho: the rounded constants and 1/rho would scale the
 // momentum the collision passes on by a fixed factor every step, and at a steady state such a
 // bias builds up where unbiased rounding does not.
-template <typename real>
-__device__ __forceinline__ void odd_split(real Jx, real Jy, real& px, real& py, real& pd, real& pa) {
+template <typename V>
+__device__ __forceinline__ void odd_split(V Jx, V Jy, V& px, V& py, V& pd, V& pa) {
   // w_i rho 3 e_i.u for e = (1,1) and (-1,1) is (Jx + Jy)/12 and (Jy - Jx)/12; the axis terms
   // take what is left of J/2, so that the first moment of the odd parts is J up to rounding of
   // the sums, whatever the rounding of 1/12
-  pd = mul_rn(Jx + Jy, real(1.0 / 12.0));
-  pa = mul_rn(Jy - Jx, real(1.0 / 12.0));
-  px = fma_rn(real(0.5), Jx, pa - pd);
-  py = fma_rn(real(0.5), Jy, -(pd + pa));
+  using real = typename ScalarOf<V>::type;
+  const V c12 = splat<V>(real(1.0 / 12.0)), n12 = splat<V>(real(-1.0 / 12.0)), half = splat<V>(real(0.5));
+  const V s = add_rn(Jx, Jy), d = sub_rn(Jy, Jx);
+  const V npd = mul_rn(s, n12);
+  pd = mul_rn(s, c12);
+  pa = mul_rn(d, c12);
+  px = fma_rn(half, Jx, fma_rn(d, c12, npd));
+  py = fma_rn(half, Jy, fma_rn(d, n12, npd));
 }
 
-// The parts added for the odd moments and the BGK branch round every product that meets a sum
-// explicitly (mul_rn / fma_rn), so that no kernel's compiler fuses them differently: all kernels
-// that collide a node get the same bits.
-template <typename real>
-__device__ __forceinline__ void collide_node(const Lattice<real>& L, real (&f)[9], real r, real drho,
-                                             real jx, real jy, real Fx, real Fy) {
-  const real inv_r = real(1) / r;
-  const real ux = jx * inv_r, uy = jy * inv_r;
-  const real vx = ux + Fx * inv_r, vy = uy + Fy * inv_r;
-  const real q36 = div36(drho);
-  real neq[9];
+// The second-order part w_i rho (4.5 (e_i.v)^2 - 1.5 v^2) of f^eq from X = Jx vx, Y = Jy vy,
+// Z = Jx vy (J = rho v): X/3 - Y/6 and Y/3 - X/6 on the axes, (X + Y)/12 +- Z/4 on the two
+// diagonals, -2 (X + Y)/3 at rest; the rounded constants are exact multiples of one another, so
+// the parts sum to zero.
+//
+// Every operation is rounded explicitly (add_rn ... fma_rn), so that no kernel's compiler fuses
+// them differently, and no product enters a plain sum (ptxas fuses mul.rn.f32x2 with a following
+// add.rn.f32x2): all kernels that collide a node, or two at once, get the same bits.
+// Opposite directions share their even and odd parts, f~_i = w_i delta rho + (even +- odd).
+template <typename V, typename real>
+__device__ __forceinline__ void collide_node(const Lattice<real>& L, V (&f)[9], V r, V drho, V jx, V jy, V Fx, V Fy) {
+  auto K = [](real c) { return splat<V>(c); };
+  const real third = real(1.0 / 3.0), sixth = real(1.0 / 6.0), twelfth = real(1.0 / 12.0), twothirds = real(2.0 / 3.0);
+  const V inv_r = recip(r);
+  const V q36 = div36(drho);
+  const V ux = mul_rn(jx, inv_r), uy = mul_rn(jy, inv_r);
+  const V Jx = add_rn(jx, Fx), Jy = add_rn(jy, Fy);
+  const V vx = mul_rn(Jx, inv_r), vy = mul_rn(Jy, inv_r);
+  const V X = mul_rn(Jx, vx), Y = mul_rn(Jy, vy), Z = mul_rn(Jx, vy);
+  const V S = fma_rn(Jx, vx, Y);
+  V px, py, pd, pa;
+  odd_split(Jx, Jy, px, py, pd, pa);
+  // even parts of the rest, x, y, diagonal (5, 7) and antidiagonal (6, 8) directions, odd parts
+  V n0, nx, ny, nd, na, ox, oy, od, oa;
   if (L.coll == COLL_MRT) {
-    const real s13 = f[1] + f[3], s24 = f[2] + f[4], s57 = f[5] + f[7], s68 = f[6] + f[8];
-    const real s1234 = s13 + s24, s5678 = s57 + s68;
-    const real d13 = f[1] - f[3], d24 = f[2] - f[4];
-    const real j2r = (jx * jx + jy * jy) * inv_r;
-    // non-equilibrium moments, scaled by 1 - s_k
-    const real e = ((real(-4) * f[0] - s1234 + real(2) * s5678) + (real(2) * drho - real(3) * j2r)) * L.keep_e;
-    const real eps = ((real(4) * f[0] - real(2) * s1234 + s5678) - (drho - real(3) * j2r)) * L.keep_eps;
-    const real qx = ((jx - real(3) * d13) + jx) * L.keep_q;
-    const real qy = ((jy - real(3) * d24) + jy) * L.keep_q;
-    const real pxx = ((s13 - s24) - (jx * jx - jy * jy) * inv_r) * L.keep_nu;
-    const real pxy = ((s57 - s68) - jx * jy * inv_r) * L.keep_nu;
-    const real e36 = e * real(1.0 / 36.0), e18 = e * real(1.0 / 18.0);
-    const real s36 = eps * real(1.0 / 36.0), s18 = eps * real(1.0 / 18.0);
-    const real qx6 = qx * real(1.0 / 6.0), qy6 = qy * real(1.0 / 6.0);
-    const real qx12 = qx * real(1.0 / 12.0), qy12 = qy * real(1.0 / 12.0);
-    const real pxx4 = pxx * real(0.25), pxy4 = pxy * real(0.25);
-    const real a14 = -e36 - s18, a58 = e18 + s36;
-    neq[0] = real(4) * (s36 - e36);
-    neq[1] = a14 - qx6 + pxx4;
-    neq[2] = a14 - qy6 - pxx4;
-    neq[3] = a14 + qx6 + pxx4;
-    neq[4] = a14 + qy6 - pxx4;
-    neq[5] = a58 + qx12 + qy12 + pxy4;
-    neq[6] = a58 - qx12 + qy12 - pxy4;
-    neq[7] = a58 - qx12 - qy12 + pxy4;
-    neq[8] = a58 + qx12 - qy12 - pxy4;
+    const V s13 = add_rn(f[1], f[3]), s24 = add_rn(f[2], f[4]), s57 = add_rn(f[5], f[7]), s68 = add_rn(f[6], f[8]);
+    const V sa = add_rn(s13, s24), sd = add_rn(s57, s68);
+    const V njx = mul_rn(K(-1), jx);
+    const V j2 = fma_rn(jx, ux, mul_rn(jy, uy));   // j.j / rho
+    // non-equilibrium moments; the factors (1 - s_k) over the norms of M's rows follow
+    const V me = fma_rn(K(-3), j2, fma_rn(K(2), drho, sub_rn(add_rn(sd, sd), fma_rn(K(4), f[0], sa))));
+    const V mp = fma_rn(K(3), j2, sub_rn(fma_rn(K(4), f[0], fma_rn(K(-2), sa, sd)), drho));
+    const V qx = add_rn(fma_rn(K(-3), sub_rn(f[1], f[3]), jx), jx);
+    const V qy = add_rn(fma_rn(K(-3), sub_rn(f[2], f[4]), jy), jy);
+    const V pxx = fma_rn(jy, uy, fma_rn(njx, ux, sub_rn(s13, s24)));
+    const V pxy = fma_rn(njx, uy, sub_rn(s57, s68));
+    const V a14 = fma_rn(K(L.nke36), me, mul_rn(K(real(-2) * L.kp36), mp));
+    const V a58 = fma_rn(K(real(-2) * L.nke36), me, mul_rn(K(L.kp36), mp));
+    n0 = fma_rn(K(real(4) * L.nke36), me, mul_rn(K(real(4) * L.kp36), mp));
+    nx = fma_rn(K(L.kn4), pxx, a14);
+    ny = fma_rn(K(-L.kn4), pxx, a14);
+    nd = fma_rn(K(L.kn4), pxy, a58);
+    na = fma_rn(K(-L.kn4), pxy, a58);
+    ox = fma_rn(K(real(-2) * L.kq12), qx, px);
+    oy = fma_rn(K(real(-2) * L.kq12), qy, py);
+    od = fma_rn(K(L.kq12), add_rn(qx, qy), pd);
+    oa = fma_rn(K(L.kq12), sub_rn(qy, qx), pa);
   } else {
+    // (1 - 1/tau) (f - f^eq(rho, u)), as half sums and half differences of opposite directions
     const real keep = real(1) - L.omega;
-    const real usq = mul_rn(real(1.5), fma_rn(ux, ux, mul_rn(uy, uy)));
-    real ox, oy, od, oa;
-    odd_split(jx, jy, ox, oy, od, oa);
-    const real r9 = mul_rn(r, real(1.0 / 9.0)), r36 = mul_rn(r, real(1.0 / 36.0));
-    const real ud = ux + uy, ua = uy - ux;
-    const real ex_ = fma_rn(mul_rn(real(4.5), ux), ux, -usq), ey_ = fma_rn(mul_rn(real(4.5), uy), uy, -usq);
-    const real ed = fma_rn(mul_rn(real(4.5), ud), ud, -usq), ea = fma_rn(mul_rn(real(4.5), ua), ua, -usq);
-    neq[0] = mul_rn(keep, (f[0] - real(16) * q36) + real(4) * mul_rn(r9, usq));
-    neq[1] = mul_rn(keep, (f[1] - real(4) * q36) - fma_rn(r9, ex_, ox));
-    neq[3] = mul_rn(keep, (f[3] - real(4) * q36) - fma_rn(r9, ex_, -ox));
-    neq[2] = mul_rn(keep, (f[2] - real(4) * q36) - fma_rn(r9, ey_, oy));
-    neq[4] = mul_rn(keep, (f[4] - real(4) * q36) - fma_rn(r9, ey_, -oy));
-    neq[5] = mul_rn(keep, (f[5] - q36) - fma_rn(r36, ed, od));
-    neq[7] = mul_rn(keep, (f[7] - q36) - fma_rn(r36, ed, -od));
-    neq[6] = mul_rn(keep, (f[6] - q36) - fma_rn(r36, ea, oa));
-    neq[8] = mul_rn(keep, (f[8] - q36) - fma_rn(r36, ea, -oa));
+    const real kh = real(0.5) * keep;
+    const V x0 = mul_rn(jx, ux), y0 = mul_rn(jy, uy), z0 = mul_rn(jx, uy), s0 = fma_rn(jx, ux, y0);
+    V bx, by, bd, ba;
+    odd_split(jx, jy, bx, by, bd, ba);
+    auto even = [&](V a, V b, V q, V ne) {   // keep ((f_a + f_b)/2 + q + ne), -q the share of delta rho
+      return mul_rn(K(keep), fma_rn(K(0.5), add_rn(add_rn(a, q), add_rn(b, q)), ne));
+    };
+    const V m4q = mul_rn(K(-4), q36), m1q = mul_rn(K(-1), q36);
+    n0 = mul_rn(K(keep), fma_rn(K(twothirds), s0, fma_rn(K(-16), q36, f[0])));
+    nx = even(f[1], f[3], m4q, fma_rn(K(-third), x0, mul_rn(K(sixth), y0)));
+    ny = even(f[2], f[4], m4q, fma_rn(K(-third), y0, mul_rn(K(sixth), x0)));
+    nd = even(f[5], f[7], m1q, fma_rn(K(-0.25), z0, mul_rn(K(-twelfth), s0)));
+    na = even(f[6], f[8], m1q, fma_rn(K(0.25), z0, mul_rn(K(-twelfth), s0)));
+    ox = fma_rn(K(kh), sub_rn(f[1], f[3]), fma_rn(K(-keep), bx, px));
+    oy = fma_rn(K(kh), sub_rn(f[2], f[4]), fma_rn(K(-keep), by, py));
+    od = fma_rn(K(kh), sub_rn(f[5], f[7]), fma_rn(K(-keep), bd, pd));
+    oa = fma_rn(K(kh), sub_rn(f[6], f[8]), fma_rn(K(-keep), ba, pa));
   }
-  // f~_i = w_i delta rho + w_i rho (3 e.u' + 4.5 (e.u')^2 - 1.5 u'^2) + neq_i, opposite
-  // directions sharing the even part
-  const real vsq = mul_rn(real(1.5), fma_rn(vx, vx, mul_rn(vy, vy)));
-  const real r9 = mul_rn(r, real(1.0 / 9.0)), r36 = mul_rn(r, real(1.0 / 36.0));
-  // odd parts from the post-collision momentum rho u' = j + F
-  real px, py, pd, pa;
-  odd_split(jx + Fx, jy + Fy, px, py, pd, pa);
-  auto even_of = [&](real ev) { return fma_rn(mul_rn(real(4.5), ev), ev, -vsq); };
-  f[0] = real(16) * q36 + (real(-4) * mul_rn(r9, vsq) + neq[0]);
-  {
-    const real even = even_of(vx);
-    f[1] = real(4) * q36 + (fma_rn(r9, even, px) + neq[1]);
-    f[3] = real(4) * q36 + (fma_rn(r9, even, -px) + neq[3]);
-  }
-  {
-    const real even = even_of(vy);
-    f[2] = real(4) * q36 + (fma_rn(r9, even, py) + neq[2]);
-    f[4] = real(4) * q36 + (fma_rn(r9, even, -py) + neq[4]);
-  }
-  {
-    const real even = even_of(vx + vy);
-    f[5] = q36 + (fma_rn(r36, even, pd) + neq[5]);
-    f[7] = q36 + (fma_rn(r36, even, -pd) + neq[7]);
-  }
-  {
-    const real even = even_of(vy - vx);
-    f[6] = q36 + (fma_rn(r36, even, pa) + neq[6]);
-    f[8] = q36 + (fma_rn(r36, even, -pa) + neq[8]);
-  }
+  nx = fma_rn(K(third), X, fma_rn(K(-sixth), Y, nx));
+  ny = fma_rn(K(third), Y, fma_rn(K(-sixth), X, ny));
+  nd = fma_rn(K(0.25), Z, fma_rn(K(twelfth), S, nd));
+  na = fma_rn(K(-0.25), Z, fma_rn(K(twelfth), S, na));
+  f[0] = fma_rn(K(16), q36, fma_rn(K(-twothirds), S, n0));
+  f[1] = fma_rn(K(4), q36, add_rn(nx, ox));
+  f[3] = fma_rn(K(4), q36, sub_rn(nx, ox));
+  f[2] = fma_rn(K(4), q36, add_rn(ny, oy));
+  f[4] = fma_rn(K(4), q36, sub_rn(ny, oy));
+  f[5] = add_rn(q36, add_rn(nd, od));
+  f[7] = add_rn(q36, sub_rn(nd, od));
+  f[6] = add_rn(q36, add_rn(na, oa));
+  f[8] = add_rn(q36, sub_rn(na, oa));
 }
 
 // Eqs. 16-17 (present scheme) and their variants for one link.
@@ -524,19 +676,15 @@ __device__ __forceinline__ void collide_node(const Lattice<real>& L, real (&f)[9
 template <typename real>
 __device__ __forceinline__ real link_rule(int bc, real q, int x2_fluid, real a, real b2, real c, real Fi) {
   if (bc == BC_HBB) return a;
-  const bool with_force = bc == BC_PRESENT;
-  if (q < real(0.5)) {
-    if (!x2_fluid) return a;
-    real w = real(1) - real(2) * q;
-    real v = real(2) * q * a + w * b2;
-    if (with_force) v += w * Fi;
-    return v;
-  }
-  real inv = real(1) / (real(2) * q);
-  real w = (real(2) * q - real(1)) * inv;
-  real v = a * inv + w * c;
-  if (with_force) v += w * Fi;
-  return v;
+  // v = A a + W (b2 or c) [+ W Fi]
+  const bool low = q < real(0.5);
+  if (low && !x2_fluid) return a;
+  const real q2 = mul_rn(real(2), q);
+  const real inv = recip(low ? real(1) : q2);
+  const real A = low ? q2 : inv;
+  const real W = low ? real(1) - q2 : mul_rn(q2 - real(1), inv);
+  const real v = fma_rn(A, a, mul_rn(W, low ? b2 : c));
+  return bc == BC_PRESENT ? fma_rn(W, Fi, v) : v;
 }
 
 // Deterministic block sum of one double per thread (fixed shuffle tree, then warps in order).

@@ -1,0 +1,896 @@
+// The fused step (FP32, two population lattices, an equation of state): chemical potential, force,
+// collision, streaming and the next state's density in ONE pass over the populations (k_walk on
+// large lattices, k_tile on the others), then the cut links (k_bc_fused) and the solid layers
+// (k_solids), instead of a density, a chemical-potential, a collide, a boundary and two layer
+// kernels and a scatter that hand planes to one another through memory.  The values are those of
+// the separate passes, bit for bit.
+//
+// A warp works on rows of FW = 64 columns, two adjacent ones a lane, in sm_103a's packed FP32
+// arithmetic (float2: the separate collide kernel was bound by instruction issue as much as by
+// bytes).  It forms what the OUT = 56 inner columns receive: the columns beyond belong to the
+// neighbouring strips and are collided again here, so that every store is an aligned pair of its
+// own (the shifted directions go through the neighbouring lane) and each node's density can be
+// summed from registers as the populations streaming into it are formed.  That costs 64/56 = 14 %
+// of the arithmetic and of the L2 traffic, nothing of the DRAM traffic: 36 + 36 bytes of
+// populations, 4 + 4 of density and the node's class are read and written once.
+//
+// Slots of boundary nodes whose source is solid are left to k_bc_fused, which finds the force of
+// those nodes in two planes (the pass stores it in the rows next to solids).  The densities of
+// boundary nodes come from k_bc_fused, those of the solid layers from k_solids.
+//
+// On the 2048 x 4096 impact lattice a step takes 0.133 ms against 0.192 ms for the separate passes
+// (1024 x 1024 with 16 drops 33 against 45 us, 131 x 97 9.3 against 29 us); the pass itself 0.13 ms,
+// 661 MB of DRAM traffic.  What was tried on the way there: the density formed from the populations
+// at the start of the same pass instead of the end of the previous one (72 instead of 80 bytes a
+// node, but the populations of four more rows wait in shared memory for their collision: 10 warps
+// an SM instead of 12, 0.19 ms); 8-byte cp.async through L1 instead of 16-byte ones past it (the
+// L1 lines left beside 200 KB of shared memory bound the loads in flight: 0.20 against 0.15 ms);
+// one row an iteration, conditions inside (0.22 ms: divergent branches and short chains).
+#include "lbm_fused.cuh"
+
+#include "lbm_internal.h"
+#include "lbm_phases.cuh"
+
+namespace lbmgb {
+
+namespace {
+
+constexpr int FW = 64;                 // columns a warp holds
+constexpr int FD = 4;                  // rows of populations (and densities) requested ahead
+constexpr int ROW_F = 9 * FW * 4;      // bytes of one row's populations in shared memory
+constexpr int HX = 4;                  // columns held on each side of the strip's outputs
+constexpr int OUT = FW - 2 * HX;       // output columns
+constexpr int SP = FW / 2 + 4;         // pairs of a density or chemical-potential row: two more each side
+constexpr int RHO_ROWS = 16, MU_ROWS = 8;   // rows of the two rings (psi: RHO_ROWS)
+constexpr int RHO_CHUNKS = SP / 2;     // 16-byte pieces of a density row
+
+// LEAD: rows between the newest density row and the collision
+template <bool PSEUDO> struct Reach {
+  static constexpr int LEAD = PSEUDO ? 1 : 4;
+  static constexpr int BYTES = FD * ROW_F + (RHO_ROWS + (PSEUDO ? 0 : MU_ROWS)) * SP * 8;
+};
+
+__device__ __forceinline__ void cp4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
+
+// stores under a condition, as predicated instructions: the strip's end lanes would otherwise
+// cost a divergent branch for each direction
+__device__ __forceinline__ void store_if(bool p, char* at, float2 v) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.s32 p, %0, 0;\n @p st.global.v2.f32 [%1], {%2, %3};\n}\n" ::"r"((int)p), "l"(at),
+               "f"(v.x), "f"(v.y)
+               : "memory");
+}
+__device__ __forceinline__ void store_if(bool p, char* at, float v) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.s32 p, %0, 0;\n @p st.global.f32 [%1], %2;\n}\n" ::"r"((int)p), "l"(at), "f"(v)
+               : "memory");
+}
+
+// Programmatic dependent launch: a kernel of the step may start while the one before it still runs
+// (grid_launch there), and reads or writes nothing that one touches before grid_wait, which waits
+// for it to finish.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// column c of a lattice of nx columns, wrapped (c within one lattice of the range, or clamped)
+__device__ __forceinline__ int wrap_col(int c, int nx) {
+  c %= nx;
+  return c < 0 ? c + nx : c;
+}
+
+// The walk: one warp takes a strip up through a band of rows.  At row r it forms the chemical
+// potential of row r - 2, whose stencil is complete then, collides row r - 4 and completes the
+// density of row r - 5.  Rows arrive by cp.async FD rows ahead; densities and chemical potentials
+// live in rings in shared memory that no other warp reads, so one __syncwarp a row is all the
+// synchronisation.
+//
+// One warp: the populations streaming into the output columns of strip `strip` in rows [ya, yb),
+// and those nodes' density (psi), from the state in lattice `cur`.
+template <bool PSEUDO>
+__device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip, int ya, int yb, char* smem) {
+  using R = Reach<PSEUDO>;
+  constexpr int LEAD = R::LEAD;
+  const int lane = threadIdx.x & 31;
+  const int x0 = strip * OUT, c = x0 - HX + 2 * lane;   // this lane's columns c, c + 1
+  const bool mine = lane >= HX / 2 && lane < 32 - HX / 2;
+  const bool out1 = mine && c + 1 < L.nx, one = mine && c + 1 == L.nx;   // both outputs; the first only
+  const int ca = wrap_col(c, L.nx), cb = wrap_col(c + 1, L.nx);   // inside the lattice
+  // Rows arrive in 16-byte pieces of four columns, straight into shared memory (not through L1,
+  // which would bound the rows in flight).  With nx a multiple of four a wrapped piece stays one
+  // aligned piece; otherwise the strips at the edges (split) load their columns one by one.
+  const bool split = (L.nx & 3) != 0 && (x0 - 2 * HX < 0 || x0 + OUT + 2 * HX > L.nx);
+  const int p4 = wrap_col(x0 - HX + 4 * (lane & 15), L.nx);                 // this lane's piece of a population row
+  const int q4 = wrap_col(x0 - 2 * HX + 4 * lane, L.nx);                    // ... of a density row (18 lanes)
+  const float* __restrict__ fin = L.f[cur];
+  float* __restrict__ fout = L.f[cur ^ 1];
+  const float* __restrict__ rin = PSEUDO ? L.mu : L.rho;   // the state's density (psi)
+  float* __restrict__ rout = L.rho_next;                   // the next state's
+  const float2* const fs = reinterpret_cast<const float2*>(smem) + lane;          // own pair: + (row, i) * 32
+  float2* const rs = reinterpret_cast<float2*>(smem + FD * ROW_F) + HX / 2 + lane;   // density (psi): + row * SP
+  float2* const ms = rs + RHO_ROWS * SP;                                          // chemical potential
+  auto rslot = [](int r) { return (r & (RHO_ROWS - 1)) * SP; };
+  auto mslot = [](int r) { return (r & (MU_ROWS - 1)) * SP; };
+  auto fslot = [](int y) { return (y & (FD - 1)) * (9 * 32); };
+
+  // row r inside the lattice: wrapped, or (walls) clamped to a wall row, whose values no fluid
+  // node's stencil reaches
+  auto row_of = [&](int r) {
+    if (L.walls) return min(max(r, 0), L.ny - 1);
+    return r < 0 ? r + L.ny : (r >= L.ny ? r - L.ny : r);
+  };
+  auto load_rho = [&](int r) {
+    const int n = row_of(r) * L.pitch;
+    char* const d = smem + FD * ROW_F + rslot(r) * 8;
+    if (!split) {
+      if (lane < RHO_CHUNKS) cp16(d + 16 * lane, reinterpret_cast<const char*>(rin) + 4u * (unsigned)(n + q4));
+    } else {
+      for (int e = lane; e < 4 * RHO_CHUNKS; e += 32) cp4(d + 4 * e, rin + n + wrap_col(x0 - 2 * HX + e, L.nx));
+    }
+  };
+  auto load_f = [&](int y) {
+    const int n = row_of(y) * L.pitch;
+    char* const d = smem + fslot(y) * 8;
+    if (!split) {
+      // a warp's 32 pieces are two directions' rows
+      const char* base = reinterpret_cast<const char*>(fin + (lane >> 4) * (long long)L.plane) + 4u * (unsigned)(n + p4);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) cp16(d + 512 * k + 16 * lane, base + 8ll * k * L.plane);
+      if (lane < 16) cp16(d + 2048 + 16 * lane, base + 32ll * L.plane);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        cp4(d + 256 * i + 8 * lane, fin + i * L.plane + n + ca);
+        cp4(d + 256 * i + 8 * lane + 4, fin + i * L.plane + n + cb);
+      }
+    }
+  };
+  // rows collided: ya - 1 .. yb; the newest density row r runs from rb to re
+  const int rb = PSEUDO ? ya : ya - 1, re = yb + LEAD;
+  // density row r + FD and the populations of the row FD above the one collided with row r
+  auto request = [&](int r) {
+    if (r + FD <= re) load_rho(r + FD);
+    const int y = r - LEAD + FD;
+    if (y >= ya - 1 && y <= yb) load_f(y);
+    cp_commit();
+  };
+  // the classes of columns c and c + 1 of the row, in bytes 0 and 1
+  auto kind_row = [&](int r) -> unsigned {
+    const uint8_t* k = L.kind + row_of(r) * L.pitch;
+    if ((L.nx & 1) == 0) return *reinterpret_cast<const unsigned short*>(k + ca);
+    return k[ca] | ((unsigned)k[cb] << 8);
+  };
+  // bit 0 / 1: column c / c + 1 is fluid
+  auto fluid_bits = [](unsigned k) {
+    return ((k & 0xffu) == KIND_FLUID ? 1u : 0u) | ((k >> 8) == KIND_FLUID ? 2u : 0u);
+  };
+  auto load_pops = [&](int y, float2 (&v)[9]) {
+    const float2* d = fs + fslot(y);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) v[i] = d[i * 32];
+  };
+  // the undivided x differences of Eq. 9 from a pair and its neighbour pairs
+  auto dx_of = [](float2 l, float2 C, float2 g) {
+    return fma_rn(splat<float2>(8.0f), make_float2(sub_rn(C.y, l.y), sub_rn(g.x, C.x)), sub_rn(l, g));
+  };
+  // mu from the densities of its row (left, own, right pair) and of the rows around it
+  auto mu_at = [&](float2 l, float2 C, float2 g, float2 u1, float2 u2, float2 d1, float2 d2) {
+    // (x+1 - c) + (x-1 - c): within the pair the two differences are +-(C.y - C.x)
+    const float t = sub_rn(C.y, C.x);
+    const float2 x1 = make_float2(add_rn(t, sub_rn(l.y, C.x)), add_rn(sub_rn(g.x, C.y), -t));
+    const float2 lap = lap4_diff(x1, add_rn(sub_rn(C, g), sub_rn(C, l)), add_rn(sub_rn(u1, C), sub_rn(d1, C)),
+                                 add_rn(sub_rn(C, u2), sub_rn(C, d2)));
+    return mu_of(L, psi_prime_shifted(L, C), lap);
+  };
+  auto force_pp_at = [&](float2 rho, int y, float2& Fx, float2& Fy) {
+    const float2* u = rs + rslot(y + 1);
+    const float2* q = rs + rslot(y);
+    const float2* d = rs + rslot(y - 1);
+    const float2 C = q[0], U = u[0], D = d[0];
+    float2 ax, ay;
+    pp_sums(make_float2(C.y, q[1].x), U, make_float2(q[-1].y, C.x), D, make_float2(U.y, u[1].x), make_float2(u[-1].y, U.x),
+            make_float2(d[-1].y, D.x), make_float2(D.y, d[1].x), ax, ay);
+    Fx = force_pp(rho, L.gx, C, ax);
+    Fy = force_pp(rho, L.gy, C, ay);
+  };
+  // What the rows collided so far stream into row y (the next one collided) and the row below it:
+  // that row's density is complete once row y is collided.
+  struct Incoming {
+    float2 c0, s13;          // row y - 1: at rest, and along x
+    float2 d2, d5, d6;       // into row y - 1 from row y - 2
+    float2 e2, e5, e6;       // into row y from row y - 1
+  } in;
+  {
+    const float2 z = make_float2(0.f, 0.f);
+    in = {z, z, z, z, z, z, z, z};
+  }
+  const unsigned at_c = 4u * (unsigned)c;
+  const bool odd = (L.nx & 1) != 0;
+  // Streaming of row y's post-collision populations: every pair of outputs receives columns c - 1, c
+  // (moving right) or c + 1, c + 2 (moving left) through the neighbouring lane, so that all stores
+  // are aligned pairs.  Slots whose source is solid get a meaningless value; the boundary phase
+  // rewrites those of fluid nodes, nothing reads the others.
+  auto stream_row = [&](const float2 (&v)[9], int y) {
+    auto right = [](float2 a) { return make_float2(__shfl_up_sync(0xffffffffu, a.y, 1), a.x); };
+    auto left = [](float2 a) { return make_float2(a.y, __shfl_down_sync(0xffffffffu, a.x, 1)); };
+    const float2 r1 = right(v[1]), r5 = right(v[5]), r8 = right(v[8]);
+    const float2 l3 = left(v[3]), l6 = left(v[6]), l7 = left(v[7]);
+    // byte offsets of row y and its neighbours in a plane; one outside [ya, yb) is not stored to
+    const unsigned at = 4u * (unsigned)(y * L.pitch) + at_c, au = at + 4u * (unsigned)L.pitch, ad = at - 4u * (unsigned)L.pitch;
+    auto put = [&](bool ok, int i, unsigned off, float2 a) {
+      char* p = reinterpret_cast<char*>(fout + (long long)i * L.plane) + off;
+      store_if(ok && out1, p, a);
+      if (odd) store_if(ok && one, p, a.x);
+    };
+    const bool mid = y >= ya && y < yb, up = y + 1 < yb, dn = y > ya;
+    put(mid, 0, at, v[0]);
+    put(mid, 1, at, r1);
+    put(mid, 3, at, l3);
+    put(up, 2, au, v[2]);
+    put(up, 5, au, r5);
+    put(up, 6, au, l6);
+    put(dn, 4, ad, v[4]);
+    put(dn, 7, ad, l7);
+    put(dn, 8, ad, r8);
+    // row y - 1: density_sum's order
+    const float2 sum = add_rn(in.c0, add_rn(add_rn(in.s13, add_rn(in.d2, v[4])),
+                                            add_rn(add_rn(in.d5, l7), add_rn(in.d6, r8))));
+    float2 q = add_rn(splat<float2>(L.rho_ref), sum);
+    if (PSEUDO) q = psi_of(L, q);
+    char* p = reinterpret_cast<char*>(rout) + ad;
+    store_if(dn && out1, p, q);
+    if (odd) store_if(dn && one, p, q.x);
+    in.c0 = v[0];
+    in.s13 = add_rn(r1, l3);
+    in.d2 = in.e2;
+    in.d5 = in.e5;
+    in.d6 = in.e6;
+    in.e2 = v[2];
+    in.e5 = r5;
+    in.e6 = l6;
+  };
+
+  // density rows below rb, then the first FD requests
+#pragma unroll
+  for (int k = 1; k <= (PSEUDO ? 2 : 4); ++k) load_rho(rb - k);
+#pragma unroll
+  for (int k = 0; k < FD; ++k) {
+    cp_commit();                       // (the group of walls that precedes a request is empty here)
+    request(rb - FD + k);
+  }
+  unsigned k0 = kind_row(rb), k1 = kind_row(rb + 1);   // of rows r, r + 1
+  unsigned bits = 0;                   // fluid bits of this lane, two per row, the newest row lowest
+  unsigned solid = 0, none = 0;        // per row: some column of the warp is not fluid / none is
+  // the two rows below the first: their classes decide about walls, and about the force rows
+#pragma unroll
+  for (int k = 2; k >= 1; --k) {
+    const unsigned fl = fluid_bits(kind_row(rb - k));
+    bits = (bits << 2) | fl;
+    solid = (solid << 1) | (__all_sync(0xffffffffu, fl == 3u) ? 0u : 1u);
+    none = (none << 1) | (__any_sync(0xffffffffu, fl != 0u) ? 0u : 1u);
+    if (!PSEUDO && fl != 3u) {
+      // (they take part in the first collisions: their walls now)
+      const float* m = L.mu + row_of(rb - k) * L.pitch;
+      float2* const w = ms + mslot(rb - k);
+      if (!(fl & 1u)) w->x = m[ca];
+      if (!(fl & 2u)) w->y = m[cb];
+    }
+  }
+  for (int r = rb; r <= re;) {
+    const int y = r - LEAD;
+    const bool all0 = __all_sync(0xffffffffu, k0 == 0u), all1 = __all_sync(0xffffffffu, k1 == 0u);   // (fluid is 0)
+    // groups are committed in the order walls(r - 2), request(r - 2), walls(r - 1), request(r - 1)
+    if (r < re && y >= ya - 1 && all0 && all1 && !(solid & ((2u << LEAD) - 1u))) {
+      // Rows y - 1 .. r + 1 hold no solid node: the chemical potentials of rows r - 2 and r - 1 and
+      // the collisions of rows y and y + 1 in one run of instructions without branches, whose chains
+      // overlap.
+      bits = (bits << 4) | 15u;
+      solid <<= 2;
+      none <<= 2;
+      k0 = kind_row(min(r + 2, re));
+      k1 = kind_row(min(r + 3, re));
+      cp_wait<4>();                    // density rows r, r + 1 and population rows y, y + 1 are in
+      __syncwarp();
+      // the populations into registers; their slots take the rows FD above at once, which have two
+      // iterations' time to arrive
+      float2 w0[9], w1[9];
+      load_pops(y, w0);
+      load_pops(y + 1, w1);
+      cp_commit();
+      request(r);
+      cp_commit();
+      request(r + 1);
+      auto collide_stream = [&](float2 (&w)[9], int yy, auto&& force) {
+        float2 drho, jx, jy, Fx, Fy;
+        moments(w, drho, jx, jy);
+        const float2 rho = add_rn(splat<float2>(L.rho_ref), drho);
+        force(rho, Fx, Fy);
+        collide_node(L, w, rho, drho, jx, jy, Fx, Fy);
+        stream_row(w, yy);
+      };
+      if constexpr (PSEUDO) {
+        collide_stream(w0, y, [&](float2 rho, float2& Fx, float2& Fy) { force_pp_at(rho, y, Fx, Fy); });
+        collide_stream(w1, y + 1, [&](float2 rho, float2& Fx, float2& Fy) { force_pp_at(rho, y + 1, Fx, Fy); });
+      } else {
+        const float2 p6 = rs[rslot(r - 6)], p5 = rs[rslot(r - 5)], t0 = rs[rslot(r)], t1 = rs[rslot(r + 1)];
+        const float2* q4 = rs + rslot(r - 4);
+        const float2* q3 = rs + rslot(r - 3);
+        const float2* q2 = rs + rslot(r - 2);
+        const float2* q1 = rs + rslot(r - 1);
+        const float2 p4 = q4[0], p3 = q3[0], p2 = q2[0], p1 = q1[0];
+        const float2 mu0 = mu_at(q2[-1], p2, q2[1], p1, t0, p3, p4);
+        const float2 mu1 = mu_at(q1[-1], p1, q1[1], t0, t1, p2, p3);
+        const float2 m6 = ms[mslot(r - 6)], m5 = ms[mslot(r - 5)];
+        const float2* z4 = ms + mslot(r - 4);
+        const float2* z3 = ms + mslot(r - 3);
+        const float2 m4 = z4[0], m3 = z3[0];
+        const float2 dm0 = dx_of(z4[-1], m4, z4[1]), dr0 = dx_of(q4[-1], p4, q4[1]);
+        const float2 dm1 = dx_of(z3[-1], m3, z3[1]), dr1 = dx_of(q3[-1], p3, q3[1]);
+        ms[mslot(r - 2)] = mu0;
+        ms[mslot(r - 1)] = mu1;
+        collide_stream(w0, y, [&](float2 rho, float2& Fx, float2& Fy) {
+          Fx = force_cp(rho, L.gx, dm0, dr0);
+          Fy = force_cp(rho, L.gy, diff4_of(m3, m5, mu0, m6), diff4_of(p3, p5, p2, p6));
+        });
+        collide_stream(w1, y + 1, [&](float2 rho, float2& Fx, float2& Fy) {
+          Fx = force_cp(rho, L.gx, dm1, dr1);
+          Fy = force_cp(rho, L.gy, diff4_of(mu0, m4, mu1, m5), diff4_of(p2, p4, p1, p5));
+        });
+      }
+      r += 2;
+      continue;
+    }
+    // ---- one row, solids anywhere
+    const unsigned fl = fluid_bits(k0);
+    k0 = k1;
+    k1 = kind_row(min(r + 2, re));
+    bits = (bits << 2) | fl;
+    solid = (solid << 1) | (all0 ? 0u : 1u);
+    none = (none << 1) | (__any_sync(0xffffffffu, fl != 0u) ? 0u : 1u);
+    cp_wait<3>();                      // density row r, population row y, the walls of row r - 2
+    __syncwarp();
+    if (!PSEUDO) {
+      if (!all0) {
+        // the walls' chemical potential into row r's place in the ring
+        const float* m = L.mu + row_of(r) * L.pitch;
+        float2* const w = ms + mslot(r);
+        if (!(fl & 1u)) cp4(&w->x, m + ca);
+        if (!(fl & 2u)) cp4(&w->y, m + cb);
+      }
+      if (!(none & 4u)) {
+        // chemical potential of row r - 2
+        const float2* q = rs + rslot(r - 2);
+        const float2 mu = mu_at(q[-1], q[0], q[1], rs[rslot(r - 1)], rs[rslot(r)], rs[rslot(r - 3)], rs[rslot(r - 4)]);
+        float2* const w = ms + mslot(r - 2);
+        if (bits & (1u << 4)) w->x = mu.x;
+        if (bits & (2u << 4)) w->y = mu.y;
+      }
+    }
+    cp_commit();
+    // collision and streaming of row y
+    if (y >= ya - 1 && !(none & (1u << LEAD))) {
+      float2 v[9];
+      load_pops(y, v);
+      float2 drho, jx, jy, Fx, Fy;
+      moments(v, drho, jx, jy);
+      const float2 rho = add_rn(splat<float2>(L.rho_ref), drho);
+      if constexpr (PSEUDO) {
+        force_pp_at(rho, y, Fx, Fy);
+      } else {
+        const float2* q = rs + rslot(y);
+        const float2* z = ms + mslot(y);
+        Fx = force_cp(rho, L.gx, dx_of(z[-1], z[0], z[1]), dx_of(q[-1], q[0], q[1]));
+        Fy = force_cp(rho, L.gy, diff4_of(ms[mslot(y + 1)], ms[mslot(y - 1)], ms[mslot(y + 2)], ms[mslot(y - 2)]),
+                      diff4_of(rs[rslot(y + 1)], rs[rslot(y - 1)], rs[rslot(y + 2)], rs[rslot(y - 2)]));
+      }
+      if ((solid & (7u << (LEAD - 1))) && y >= ya && y < yb) {
+        // next to a solid: the force for the boundary phase
+        const unsigned fy = (bits >> (2 * LEAD)) & 3u;
+        const int n = y * L.pitch + c;
+        if ((out1 || one) && (fy & 1u)) { L.fx[n] = Fx.x; L.fy[n] = Fy.x; }
+        if (out1 && (fy & 2u)) { L.fx[n + 1] = Fx.y; L.fy[n + 1] = Fy.y; }
+      }
+      collide_node(L, v, rho, drho, jx, jy, Fx, Fy);
+      stream_row(v, y);
+    }
+    request(r);
+    ++r;
+  }
+  cp_wait<0>();
+}
+
+template <bool PSEUDO>
+__global__ void __launch_bounds__(32) k_walk(const __grid_constant__ Lattice<float> L, int cur, int strips, int rows) {
+  extern __shared__ __align__(16) char smem[];
+  const int band = blockIdx.x / strips, strip = blockIdx.x - band * strips;
+  const int ya = band * rows, yb = min(ya + rows, L.ny);
+  grid_wait();
+  grid_launch();
+  walk<PSEUDO>(L, cur, strip, ya, yb, smem);
+}
+
+// ---------------------------------------------------------------------------------------
+// The same pass by tiles: a block of W warps takes the OUT output columns of a strip in H rows; its
+// density rows (five more on each side) and population rows (one more) arrive together, then all
+// chemical-potential rows, all collisions and all densities are formed side by side.
+template <bool PSEUDO, int H>
+struct Tile {
+  static constexpr int MR = PSEUDO ? 0 : 3;              // chemical-potential rows beyond the outputs
+  static constexpr int RR = PSEUDO ? 2 : 5;              // density (psi) rows beyond the outputs
+  static constexpr int NC = H + 2, NM = H + 2 * MR, NR = H + 2 * RR;
+  static constexpr int F = 0, RHO = NC * ROW_F, MU = RHO + NR * SP * 8, FLAGS = MU + (PSEUDO ? 0 : NM * SP * 8);
+  static constexpr int BYTES = FLAGS + (H + 6) * 4;
+};
+
+template <bool PSEUDO, int H, int W, int MINB>
+__global__ void __launch_bounds__(32 * W, MINB) k_tile(const __grid_constant__ Lattice<float> L, int cur, int strips) {
+  extern __shared__ __align__(16) char smem[];
+  using T = Tile<PSEUDO, H>;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int band = blockIdx.x / strips, strip = blockIdx.x - band * strips;
+  const int ya = band * H, yb = min(ya + H, L.ny);
+  const int x0 = strip * OUT, c = x0 - HX + 2 * lane;
+  const bool mine = lane >= HX / 2 && lane < 32 - HX / 2;
+  const bool out1 = mine && c + 1 < L.nx, one = mine && c + 1 == L.nx;
+  const int ca = wrap_col(c, L.nx), cb = wrap_col(c + 1, L.nx);
+  const bool split = (L.nx & 3) != 0 && (x0 - 2 * HX < 0 || x0 + OUT + 2 * HX > L.nx);
+  const bool odd = (L.nx & 1) != 0;
+  const float* __restrict__ fin = L.f[cur];
+  float* __restrict__ fout = L.f[cur ^ 1];
+  const float* __restrict__ rin = PSEUDO ? L.mu : L.rho;
+  int* const flags = reinterpret_cast<int*>(smem + T::FLAGS);   // rows ya - 3 ..: 1 some column solid, 2 none fluid
+  auto row_of = [&](int r) {
+    if (L.walls) return min(max(r, 0), L.ny - 1);
+    return r < 0 ? r + L.ny : (r >= L.ny ? r - L.ny : r);
+  };
+  // rows of the tile's arrays by lattice row
+  auto rho_row = [&](int r) { return reinterpret_cast<float2*>(smem + T::RHO) + (r - ya + T::RR) * SP + HX / 2 + lane; };
+  auto mu_row = [&](int r) { return reinterpret_cast<float2*>(smem + T::MU) + (r - ya + T::MR) * SP + HX / 2 + lane; };
+  auto pop_row = [&](int y) { return reinterpret_cast<float2*>(smem + (y - ya + 1) * ROW_F) + lane; };
+  grid_wait();
+  grid_launch();
+  // ---- everything the tile reads
+  {
+    const int p4 = wrap_col(x0 - HX + 4 * (lane & 15), L.nx), q4 = wrap_col(x0 - 2 * HX + 4 * lane, L.nx);
+    for (int r = ya - T::RR + warp; r < yb + T::RR; r += W) {
+      const int n = row_of(r) * L.pitch;
+      char* const d = smem + T::RHO + (r - ya + T::RR) * SP * 8;
+      if (!split) {
+        if (lane < RHO_CHUNKS) cp16(d + 16 * lane, rin + n + q4);
+      } else {
+        for (int e = lane; e < 4 * RHO_CHUNKS; e += 32) cp4(d + 4 * e, rin + n + wrap_col(x0 - 2 * HX + e, L.nx));
+      }
+    }
+    for (int y = ya - 1 + warp; y <= yb; y += W) {
+      const int n = row_of(y) * L.pitch;
+      char* const d = smem + (y - ya + 1) * ROW_F;
+      if (!split) {
+        const float* base = fin + (lane >> 4) * (long long)L.plane + n + p4;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) cp16(d + 512 * k + 16 * lane, base + 2ll * k * L.plane);
+        if (lane < 16) cp16(d + 2048 + 16 * lane, base + 8ll * L.plane);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+          cp4(d + 256 * i + 8 * lane, fin + i * L.plane + n + ca);
+          cp4(d + 256 * i + 8 * lane + 4, fin + i * L.plane + n + cb);
+        }
+      }
+    }
+    cp_commit();
+  }
+  // node classes of this warp's chemical-potential rows (psi: of the rows the force flags need), and
+  // the walls' chemical potential where they are solid
+  constexpr int M0 = 3, NMR = (H + 6 + W - 1) / W;
+  unsigned fl[NMR];
+  float2 wall[NMR];
+#pragma unroll
+  for (int k = 0; k < NMR; ++k) {
+    const int m = ya - M0 + warp + k * W;
+    fl[k] = 0u;
+    if (m >= yb + M0) continue;
+    const uint8_t* kd = L.kind + row_of(m) * L.pitch;
+    fl[k] = (kd[ca] == KIND_FLUID ? 1u : 0u) | (kd[cb] == KIND_FLUID ? 2u : 0u);
+  }
+#pragma unroll
+  for (int k = 0; k < NMR; ++k) {
+    const int m = ya - M0 + warp + k * W;
+    if (m >= yb + M0) continue;
+    const float* w = L.mu + row_of(m) * L.pitch;
+    wall[k] = make_float2(0.f, 0.f);
+    if (!PSEUDO && !(fl[k] & 1u)) wall[k].x = w[ca];
+    if (!PSEUDO && !(fl[k] & 2u)) wall[k].y = w[cb];
+    const bool all = __all_sync(0xffffffffu, fl[k] == 3u), any = __any_sync(0xffffffffu, fl[k] != 0u);
+    if (lane == 0) flags[m - ya + M0] = (all ? 0 : 1) | (any ? 0 : 2);
+  }
+  cp_wait<0>();
+  __syncthreads();
+  // ---- chemical potentials
+  if (!PSEUDO) {
+#pragma unroll
+    for (int k = 0; k < NMR; ++k) {
+      const int m = ya - M0 + warp + k * W;
+      if (m >= yb + M0) continue;
+      const float2* q = rho_row(m);
+      const float2 C = q[0], l = q[-1], g = q[1], u1 = q[SP], u2 = q[2 * SP], d1 = q[-SP], d2 = q[-2 * SP];
+      const float t = sub_rn(C.y, C.x);
+      const float2 x1 = make_float2(add_rn(t, sub_rn(l.y, C.x)), add_rn(sub_rn(g.x, C.y), -t));
+      const float2 lap = lap4_diff(x1, add_rn(sub_rn(C, g), sub_rn(C, l)), add_rn(sub_rn(u1, C), sub_rn(d1, C)),
+                                   add_rn(sub_rn(C, u2), sub_rn(C, d2)));
+      const float2 mu = mu_of(L, psi_prime_shifted(L, C), lap);
+      *mu_row(m) = make_float2(fl[k] & 1u ? mu.x : wall[k].x, fl[k] & 2u ? mu.y : wall[k].y);
+    }
+    __syncthreads();
+  }
+  // ---- collisions and streaming
+  for (int y = ya - 1 + warp; y <= yb; y += W) {
+    const int* fg = flags + (y - ya + M0);
+    if (fg[0] & 2) continue;
+    float2 v[9];
+    float2* const pr = pop_row(y);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) v[i] = pr[32 * i];
+    float2 drho, jx, jy, Fx, Fy;
+    moments(v, drho, jx, jy);
+    const float2 rho = add_rn(splat<float2>(L.rho_ref), drho);
+    const float2* q = rho_row(y);
+    if constexpr (PSEUDO) {
+      const float2 C = q[0], U = q[SP], D = q[-SP];
+      float2 ax, ay;
+      pp_sums(make_float2(C.y, q[1].x), U, make_float2(q[-1].y, C.x), D, make_float2(U.y, q[SP + 1].x),
+              make_float2(q[SP - 1].y, U.x), make_float2(q[-SP - 1].y, D.x), make_float2(D.y, q[-SP + 1].x), ax, ay);
+      Fx = force_pp(rho, L.gx, C, ax);
+      Fy = force_pp(rho, L.gy, C, ay);
+    } else {
+      const float2* z = mu_row(y);
+      auto dx_of = [](const float2* p) {
+        const float2 l = p[-1], C = p[0], g = p[1];
+        return fma_rn(splat<float2>(8.0f), make_float2(sub_rn(C.y, l.y), sub_rn(g.x, C.x)), sub_rn(l, g));
+      };
+      Fx = force_cp(rho, L.gx, dx_of(z), dx_of(q));
+      Fy = force_cp(rho, L.gy, diff4_of(z[SP], z[-SP], z[2 * SP], z[-2 * SP]), diff4_of(q[SP], q[-SP], q[2 * SP], q[-2 * SP]));
+    }
+    const bool mid = y >= ya && y < yb, up = y + 1 < yb, dn = y > ya;
+    if (mid && ((fg[-1] | fg[0] | fg[1]) & 1)) {
+      // next to a solid: the force for the boundary phase (read at boundary nodes only)
+      const int n = y * L.pitch + c;
+      if (out1) {
+        *reinterpret_cast<float2*>(L.fx + n) = Fx;
+        *reinterpret_cast<float2*>(L.fy + n) = Fy;
+      } else if (one) {
+        L.fx[n] = Fx.x;
+        L.fy[n] = Fy.x;
+      }
+    }
+    collide_node(L, v, rho, drho, jx, jy, Fx, Fy);
+    auto right = [](float2 a) { return make_float2(__shfl_up_sync(0xffffffffu, a.y, 1), a.x); };
+    auto left = [](float2 a) { return make_float2(a.y, __shfl_down_sync(0xffffffffu, a.x, 1)); };
+    const float2 r1 = right(v[1]), r5 = right(v[5]), r8 = right(v[8]);
+    const float2 l3 = left(v[3]), l6 = left(v[6]), l7 = left(v[7]);
+    const unsigned at = 4u * (unsigned)(y * L.pitch) + 4u * (unsigned)c, au = at + 4u * (unsigned)L.pitch,
+                   ad = at - 4u * (unsigned)L.pitch;
+    auto put = [&](bool ok, int i, unsigned off, float2 a) {
+      char* p = reinterpret_cast<char*>(fout + (long long)i * L.plane) + off;
+      store_if(ok && out1, p, a);
+      if (odd) store_if(ok && one, p, a.x);
+    };
+    put(mid, 0, at, v[0]);
+    put(mid, 1, at, r1);
+    put(mid, 3, at, l3);
+    put(up, 2, au, v[2]);
+    put(up, 5, au, r5);
+    put(up, 6, au, l6);
+    put(dn, 4, ad, v[4]);
+    put(dn, 7, ad, l7);
+    put(dn, 8, ad, r8);
+    // what the densities of rows y - 1, y and y + 1 are summed from, in place of the populations
+    pr[0] = v[0];
+    pr[32] = add_rn(r1, l3);
+    pr[64] = v[2];
+    pr[96] = r5;
+    pr[128] = l6;
+    pr[160] = v[4];
+    pr[192] = l7;
+    pr[224] = r8;
+  }
+  __syncthreads();
+  // ---- densities (psi) of the outputs; rows next to solids hold meaningless values where a source
+  // is solid: the boundary phase forms the boundary nodes' densities
+  for (int y = ya + warp; y < yb; y += W) {
+    if (flags[y - ya + M0] & 2) continue;
+    const float2* o = pop_row(y);
+    const float2* d = o - 9 * 32;
+    const float2* u = o + 9 * 32;
+    const float2 sum = add_rn(o[0], add_rn(add_rn(o[32], add_rn(d[64], u[160])), add_rn(add_rn(d[96], u[192]), add_rn(d[128], u[224]))));
+    float2 q = add_rn(splat<float2>(L.rho_ref), sum);
+    if (PSEUDO) q = psi_of(L, q);
+    float* p = L.rho_next + y * L.pitch + c;
+    if (out1) *reinterpret_cast<float2*>(p) = q;
+    else if (one) *p = q.x;
+  }
+}
+
+// Cut links of one boundary node a thread (phase_bc's arithmetic, the force from the planes the
+// pass left).  Latency is all it costs, so the loads make two rounds: the node's record -- set up
+// with the geometry, and fetched before the pass it depends on has finished -- then everything
+// else at once.  The node's own populations stay in registers for its density.  Leaves one
+// compensation sum per warp; k_solids adds them up.
+constexpr int BC_BLOCK = 64;
+template <bool PSEUDO>
+__global__ void __launch_bounds__(BC_BLOCK) k_bc_fused(const __grid_constant__ Lattice<float> L, int cur) {
+  const int b = blockIdx.x * BC_BLOCK + threadIdx.x;
+  const bool live = b < L.n_bnodes;
+  const int2 nd = live ? L.bnd[b] : make_int2(0, 0);
+  const unsigned mask = live ? L.bmask[b] : 0u;
+  float q[8];
+#pragma unroll
+  for (int i = 1; i < 9; ++i) q[i - 1] = mask & (1u << (i - 1)) ? L.bq[(i - 1) * (long long)L.bcap + b] : 0.f;
+  grid_wait();
+  grid_launch();
+  double sum = 0.0;
+  if (live) {
+    const int n = nd.x, x = nd.y;
+    float* fout = L.f[cur ^ 1];
+    const float* __restrict__ fin = L.f[cur];
+    // offsets to the neighbours (periodic in x, and in y without walls)
+    const int xm = x == 0 ? L.nx - 1 : -1, xp = x == L.nx - 1 ? 1 - L.nx : 1;
+    const int ym = !L.walls && n < L.pitch ? L.plane - L.pitch : -L.pitch;
+    const int yp = !L.walls && n >= L.plane - L.pitch ? L.pitch - L.plane : L.pitch;
+    auto nb = [&](int dx, int dy) { return n + (dx < 0 ? xm : dx > 0 ? xp : 0) + (dy < 0 ? ym : dy > 0 ? yp : 0); };
+    float g[9], fl[9], a[8], cc[8];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) g[i] = fout[i * L.plane + n];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) fl[i] = fin[i * L.plane + n];
+    const float Fx = L.fx[n], Fy = L.fy[n];
+    const double carry = L.carry[b];
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+      a[i - 1] = cc[i - 1] = 0.f;
+      if (mask & (1u << (i - 1))) {
+        a[i - 1] = fout[i * L.plane + nb(ex(i), ey(i))];
+        cc[i - 1] = fout[opp(i) * L.plane + nb(-ex(i), -ey(i))];
+      }
+    }
+    float drho, jx, jy;
+    moments(fl, drho, jx, jy);
+    const float r = L.rho_ref + drho;
+    const float inv_r = 1.0f / r;
+    const float ux = jx * inv_r, uy = jy * inv_r, dux = Fx * inv_r, duy = Fy * inv_r;
+    float v[8];
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+      if (!(mask & (1u << (i - 1)))) continue;
+      const float Fi = edm_term<float>(i, r, ux, uy, dux, duy);
+      v[i - 1] = link_rule<float>(L.bc, q[i - 1], (mask >> (i + 7)) & 1u, a[i - 1], g[i], cc[i - 1], Fi);
+      sum += (double)a[i - 1] - (double)v[i - 1];
+    }
+    // (no link reads a slot another link of the node writes: b2 counts only where x2 is fluid)
+#pragma unroll
+    for (int i = 1; i < 9; ++i) {
+      if (!(mask & (1u << (i - 1)))) continue;
+      g[opp(i)] = v[i - 1];
+      fout[opp(i) * L.plane + n] = v[i - 1];
+    }
+    if (L.bc == BC_PRESENT || L.bc == BC_MIBC) {
+      const double t = (double)g[0] + sum + carry;
+      g[0] = (float)t;
+      L.carry[b] = t - (double)g[0];
+      fout[n] = g[0];
+    } else {
+      sum = 0.0;
+    }
+    const float rn = density_of(L, g);
+    L.rho_b[b] = rn;
+    L.rho_next[n] = PSEUDO ? psi_of(L, rn) : rn;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+  if ((threadIdx.x & 31) == 0) L.partials[b >> 5] = sum;
+}
+
+// Both solid layers from the boundary nodes' densities in rho_b (every fluid neighbour of a
+// first-layer node is a boundary node), into the density plane (psi with the wall factor into the
+// psi plane).  A second-layer node forms its first-layer neighbours' densities again, one a lane of
+// its eight lanes, and adds them in phase_solid's order.  The last block adds the links'
+// compensation sums in the order of k_bc's two-level sum, and steps the counter; steps == 0 leaves
+// that out (the layers of a new state).
+constexpr int SOLID_BLOCK = 256;
+template <bool PSEUDO>
+__global__ void __launch_bounds__(SOLID_BLOCK) k_solids(const __grid_constant__ Lattice<float> L, int blocks2, int blocks1,
+                                                        int steps) {
+  __shared__ double red[32];
+  const int blk = blockIdx.x;
+  auto first = [&](unsigned m, float winv, const int (&nb)[8]) {
+    float acc = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (m & (1u << i)) acc = fma_rn((float)wgt(i + 1), L.rho_b[nb[i]], acc);
+    return acc * winv;
+  };
+  auto record = [&](int k, unsigned& m, float& winv, int (&nb)[8]) {
+    m = L.s1mask[k];
+    winv = L.s1winv[k];
+    const int4 u = *reinterpret_cast<const int4*>(L.s1nb + 8 * k), w = *reinterpret_cast<const int4*>(L.s1nb + 8 * k + 4);
+    nb[0] = u.x; nb[1] = u.y; nb[2] = u.z; nb[3] = u.w;
+    nb[4] = w.x; nb[5] = w.y; nb[6] = w.z; nb[7] = w.w;
+  };
+  if (blk < blocks2) {
+    const int t = blk * SOLID_BLOCK + threadIdx.x, k = t >> 3, lane = t & 7;
+    unsigned m2 = 0, m = 0;
+    float winv2 = 0.f, winv = 0.f;
+    int nb[8], n = 0;
+    if (k < L.n_s2) {
+      m2 = L.s2mask[k];
+      winv2 = L.s2winv[k];
+      n = L.s2node[k];
+      if (m2 & (1u << lane)) record(L.s2nb[8 * k + lane], m, winv, nb);
+    }
+    grid_wait();
+    grid_launch();
+    const float v = first(m, winv, nb);
+    float acc = 0.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float vi = __shfl_sync(0xffffffffu, v, i, 8);
+      if (m2 & (1u << i)) acc = fma_rn((float)wgt(i + 1), vi, acc);
+    }
+    const float rs = acc * winv2;
+    if (k < L.n_s2 && lane == 0) L.rho_next[n] = PSEUDO ? psi_wall(L, n, rs) : rs;
+  } else if (blk < blocks2 + blocks1) {
+    const int k = (blk - blocks2) * SOLID_BLOCK + threadIdx.x;
+    unsigned m = 0;
+    float winv = 0.f;
+    int nb[8], n = 0;
+    if (k < L.n_s1) {
+      n = L.s1node[k];
+      record(k, m, winv, nb);
+    }
+    grid_wait();
+    grid_launch();
+    const float rs = first(m, winv, nb);
+    if (k < L.n_s1) L.rho_next[n] = PSEUDO ? psi_wall(L, n, rs) : rs;
+  } else {
+    grid_wait();
+    grid_launch();
+    if (steps) {
+      // k_bc's blocks of eight warps: their warps' sums in block_sum's tree, then the blocks'
+      const int warps = (L.n_bnodes + 31) / 32, chunks = (warps + 7) / 8;
+      double v = 0.0;
+      for (int k = threadIdx.x; k < chunks; k += SOLID_BLOCK) {
+        double w[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) w[j] = 8 * k + j < warps ? L.partials[8 * k + j] : 0.0;
+        v += ((w[0] + w[4]) + (w[2] + w[6])) + ((w[1] + w[5]) + (w[3] + w[7]));
+      }
+      const double total = block_sum(v, red);
+      if (threadIdx.x == 0) {
+        const unsigned long long st = *L.step_ctr;
+        L.dM_ring[st % DM_RING] = total;
+        L.dM_ring[DM_RING] = total;
+        *L.step_ctr = st + 1;
+      }
+    }
+  }
+}
+
+// A new state (set up, loaded or advanced by the separate passes) in lattice `cur`: the density
+// (psi) of its fluid nodes into rho_next, and of its boundary nodes into rho_b, from which k_solids
+// forms the solid layers.
+template <bool PSEUDO>
+__global__ void __launch_bounds__(128) k_density(Lattice<float> L, int cur) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, n = blockIdx.y * L.pitch + x;
+  if (x >= L.nx || L.kind[n] != KIND_FLUID) return;
+  const float* __restrict__ f = L.f[cur] + n;
+  float v[9];
+#pragma unroll
+  for (int i = 0; i < 9; ++i) v[i] = f[i * L.plane];
+  const float r = density_of(L, v);
+  L.rho_next[n] = PSEUDO ? psi_of(L, r) : r;
+}
+__global__ void __launch_bounds__(128) k_boundary_density(Lattice<float> L, int cur) {
+  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= L.n_bnodes) return;
+  const float* __restrict__ f = L.f[cur] + L.bnode[b];
+  float v[9];
+#pragma unroll
+  for (int i = 0; i < 9; ++i) v[i] = f[i * L.plane];
+  L.rho_b[b] = density_of(L, v);
+}
+
+// the two tile shapes: output rows, warps a block, blocks an SM
+constexpr int TH_S = 6, TW_S = 8, TB_S = 3;
+constexpr int TH_M = 14, TW_M = 8, TB_M = 3;
+inline unsigned blocks_for(int n, int b) { return (unsigned)((n + b - 1) / b); }
+
+}  // namespace
+
+// How the pass runs on a lattice of nx x ny: rows a warp walks (> 0), or which tiles (0: 14 rows,
+// -1: 6 rows).  Counted in tiles of 14 rows:
+//   below half a tile an SM the 6-row tiles spread a small lattice over more SMs (us a step, 6 rows
+//   against 14: 96 x 96 9.0 / 10.3, 192 x 160 9.3 / 10.8, but 300 x 300 12.2 / 10.5);
+//   from 28 tiles an SM on the walk wins, whose rows are formed twice only at the bands' ends and
+//   whose loads run through all of its rows (walk / tiles: 1024 x 1536 50.3 / 43.6, 1600 x 2048
+//   75.8 / 77.1, 2048 x 2048 90.6 / 94.5, 2048 x 4096 144 / 179).
+// A walk takes as many rows as give every SM 24 warps: two waves of what fits at once, so that the
+// warps whose rows hold solid nodes, which take longer, do not set the pass's time alone.
+int fused_rows(int nx, int ny, int sms) {
+  const long long strips = (nx + OUT - 1) / OUT;
+  const long long tiles = strips * ((ny + TH_M - 1) / TH_M);
+  if (2 * tiles < sms) return -1;
+  if (tiles < 28LL * sms) return 0;
+  const long long bands = 24LL * sms / strips;
+  const int rows = (int)((ny + bands - 1) / (bands > 0 ? bands : 1));
+  return rows < 16 ? 16 : rows;
+}
+
+bool fused_setup() {
+  auto allow = [](const void* k, int bytes) {
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
+  };
+  return allow((const void*)k_tile<false, TH_S, TW_S, TB_S>, Tile<false, TH_S>::BYTES) &&
+         allow((const void*)k_tile<true, TH_S, TW_S, TB_S>, Tile<true, TH_S>::BYTES) &&
+         allow((const void*)k_tile<false, TH_M, TW_M, TB_M>, Tile<false, TH_M>::BYTES) &&
+         allow((const void*)k_tile<true, TH_M, TW_M, TB_M>, Tile<true, TH_M>::BYTES) &&
+         allow((const void*)k_walk<false>, Reach<false>::BYTES) && allow((const void*)k_walk<true>, Reach<true>::BYTES);
+}
+
+// a launch that may overlap the end of the one before it in the stream
+template <typename... P, typename... A>
+static cudaError_t launch_after(void (*k)(P...), int grid, int block, int smem, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3((unsigned)grid);
+  c.blockDim = dim3((unsigned)block);
+  c.dynamicSmemBytes = (size_t)smem;
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = s ? 1 : 0;
+  return cudaLaunchKernelEx(&c, k, P(args)...);
+}
+static cudaError_t launch_solids(const Lattice<float>& L, int steps, cudaStream_t s) {
+  const int b2 = (int)blocks_for(8 * L.n_s2, SOLID_BLOCK), b1 = (int)blocks_for(L.n_s1, SOLID_BLOCK);
+  return launch_after(L.pseudo ? k_solids<true> : k_solids<false>, b2 + b1 + 1, SOLID_BLOCK, 0, s, L, b2, b1, steps);
+}
+
+cudaError_t launch_fused_prepare(const Lattice<float>& L, int cur, cudaStream_t s) {
+  const dim3 grid(blocks_for(L.nx, 128), (unsigned)L.ny);
+  if (L.pseudo) k_density<true><<<grid, 128, 0, s>>>(L, cur);
+  else k_density<false><<<grid, 128, 0, s>>>(L, cur);
+  if (L.n_bnodes > 0) k_boundary_density<<<blocks_for(L.n_bnodes, 128), 128, 0, s>>>(L, cur);
+  return launch_solids(L, 0, s);
+}
+
+template <int H, int W, int B>
+static cudaError_t launch_tiles(const Lattice<float>& L, int cur, cudaStream_t s) {
+  const int strips = (L.nx + OUT - 1) / OUT, bands = (L.ny + H - 1) / H;
+  return L.pseudo ? launch_after(k_tile<true, H, W, B>, strips * bands, 32 * W, Tile<true, H>::BYTES, s, L, cur, strips)
+                  : launch_after(k_tile<false, H, W, B>, strips * bands, 32 * W, Tile<false, H>::BYTES, s, L, cur, strips);
+}
+static cudaError_t launch_pass(const Lattice<float>& L, int cur, int rows, cudaStream_t s) {
+  if (rows < 0) return launch_tiles<TH_S, TW_S, TB_S>(L, cur, s);
+  if (rows == 0) return launch_tiles<TH_M, TW_M, TB_M>(L, cur, s);
+  const int strips = (L.nx + OUT - 1) / OUT, bands = (L.ny + rows - 1) / rows;
+  return L.pseudo ? launch_after(k_walk<true>, strips * bands, 32, Reach<true>::BYTES, s, L, cur, strips, rows)
+                  : launch_after(k_walk<false>, strips * bands, 32, Reach<false>::BYTES, s, L, cur, strips, rows);
+}
+
+cudaError_t launch_fused_step(const Lattice<float>& L, int cur, int rows, cudaStream_t s) {
+  cudaError_t e = launch_pass(L, cur, rows, s);
+  if (e == cudaSuccess && L.n_bnodes > 0)
+    e = launch_after(L.pseudo ? k_bc_fused<true> : k_bc_fused<false>, (int)blocks_for(L.n_bnodes, BC_BLOCK), BC_BLOCK, 0, s, L, cur);
+  return e == cudaSuccess ? launch_solids(L, 1, s) : e;
+}
+
+int fused_launches(const Lattice<float>& L) { return 2 + (L.n_bnodes > 0 ? 1 : 0); }
+
+}  // namespace lbmgb

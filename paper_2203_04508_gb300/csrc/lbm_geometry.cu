@@ -301,8 +301,8 @@ cudaError_t geom_classify_and_count(const GeomParams& g, const GeomScratch& s, u
 }
 
 // Each node's place in the lists: the boundary-node list (node, first link) and the two layer
-// lists (node), and the boundary index of every boundary node in the plane bidx (read back for
-// the first layer's neighbour table; other entries are never read).  The block offsets are the
+// lists (node), and the list index of every boundary node and first-layer node in the plane bidx
+// (read back for the layers' neighbour tables; other entries are never read).  The block offsets are the
 // scanned totals k_scan_lanes left.
 __global__ void __launch_bounds__(LIST_BLOCK) k_fill_nodes(GeomParams g, const uint8_t* kind, const int* offs, int nb,
                                                            GeomOut o, int* bidx) {
@@ -326,7 +326,11 @@ __global__ void __launch_bounds__(LIST_BLOCK) k_fill_nodes(GeomParams g, const u
       o.bstart[e] = lane_of_packed(ex, LANE_LINKS) + off[LANE_LINKS];
       bidx[n] = e;
     }
-    if (lane_of_packed(c[j], LANE_S1)) o.s1node[lane_of_packed(ex, LANE_S1) + off[LANE_S1]] = (int)n;
+    if (lane_of_packed(c[j], LANE_S1)) {
+      const int e = lane_of_packed(ex, LANE_S1) + off[LANE_S1];
+      o.s1node[e] = (int)n;
+      bidx[n] = e;
+    }
     if (lane_of_packed(c[j], LANE_S2)) o.s2node[lane_of_packed(ex, LANE_S2) + off[LANE_S2]] = (int)n;
     ex += c[j];
   }
@@ -341,6 +345,7 @@ __global__ void k_fill_links(GeomParams g, const uint8_t* kind, int n_bnodes, Ge
   const int n = o.bnode[b];
   const int x = n % g.pitch, y = n / g.pitch;
   int l = o.bstart[b];
+  unsigned mask = 0;
   const int nbodies = g.n_cyl + (g.walls ? 2 : 0);
   for (int i = 1; i < 9; ++i) {
     int m;
@@ -359,14 +364,22 @@ __global__ void k_fill_links(GeomParams g, const uint8_t* kind, int n_bnodes, Ge
     o.lq64[l] = qb;
     ((real*)o.lq)[l] = (real)qb;
     o.lx2f[l] = (ok2 && kind[m2] == KIND_FLUID) ? 1 : 0;
+    if (o.bnd) {
+      mask |= (1u << (i - 1)) | (o.lx2f[l] ? 1u << (i + 7) : 0u);
+      ((real*)o.bq)[(i - 1) * (long long)o.bcap + b] = (real)qb;
+    }
     ++l;
+  }
+  if (o.bnd) {
+    o.bnd[b] = make_int2(n, x);
+    o.bmask[b] = (unsigned short)mask;
   }
 }
 
 // Entry j of a solid-layer list (node[j] of class cls): the mask of its neighbours of class
-// `from`, 1 / sum of their weights, and (first layer) for each contributing neighbour -- all of
-// them boundary-fluid nodes -- its index in the boundary-node list, nb[8 j + i - 1], -1 where
-// bit i-1 of the mask is clear
+// `from`, 1 / sum of their weights, and for each contributing neighbour -- boundary-fluid nodes for
+// the first layer, first-layer nodes for the second -- its index in that list, nb[8 j + i - 1], -1
+// where bit i-1 of the mask is clear
 template <typename real>
 __global__ void k_fill_layer(GeomParams g, const uint8_t* kind, int count, uint8_t from, const int* node,
                              uint8_t* mask, real* winv, const int* bidx, int* nb) {
@@ -409,8 +422,8 @@ template <typename real>
 static cudaError_t fill_typed(const GeomParams& g, const GeomScratch& s, const GeomOut& o, cudaStream_t st) {
   const unsigned gn = (unsigned)((g.plane + 255) / 256);
   const int nb = (int)((g.plane + LIST_NODES - 1) / LIST_NODES);
-  // the block offsets geom_classify_and_count left in block_sums; the boundary index of each
-  // boundary node into the scratch plane `off`
+  // the block offsets geom_classify_and_count left in block_sums; the list index of each
+  // boundary and first-layer node into the scratch plane `off`
   int* bidx = s.off;
   k_fill_nodes<<<nb, LIST_BLOCK, 0, st>>>(g, o.kind, s.block_sums, nb, o, bidx);
   if (o.n_bnodes > 0) k_fill_links<real><<<(o.n_bnodes + 255) / 256, 256, 0, st>>>(g, o.kind, o.n_bnodes, o);
@@ -419,7 +432,7 @@ static cudaError_t fill_typed(const GeomParams& g, const GeomScratch& s, const G
                                                              (real*)o.s1winv, bidx, o.s1nb);
   if (o.n_s2 > 0)
     k_fill_layer<real><<<(o.n_s2 + 255) / 256, 256, 0, st>>>(g, o.kind, o.n_s2, KIND_SOLID1, o.s2node, o.s2mask,
-                                                             (real*)o.s2winv, nullptr, nullptr);
+                                                             (real*)o.s2winv, bidx, o.s2nb);
   k_wall_mu<real><<<gn, 256, 0, st>>>(g, o.kind, s.body, (real*)o.mu);
   return cudaGetLastError();
 }

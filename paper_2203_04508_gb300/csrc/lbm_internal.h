@@ -78,6 +78,17 @@ struct CollideTma {
 bool collide_tma_setup(CollideTma* T, const Lattice<float>& L, const void* rho0, const void* rho1, const void* mu1,
                        void* edge, char* err);
 
+// ---- the fused step (lbm_fused.cu): FP32, two population lattices, an equation of state
+// raises the kernels' shared-memory limit on the current device; false when the device refuses
+bool fused_setup();
+// how the pass runs on a lattice of nx x ny: rows a warp walks, or <= 0 for tiles
+int fused_rows(int nx, int ny, int sms);
+// the solid layers of a new state in lattice cur, where the fused step expects them
+cudaError_t launch_fused_prepare(const Lattice<float>& L, int cur, cudaStream_t s);
+// one step from lattice cur (L.rho_b, L.fx and L.fy set)
+cudaError_t launch_fused_step(const Lattice<float>& L, int cur, int rows, cudaStream_t s);
+int fused_launches(const Lattice<float>& L);
+
 // ---- halo messages of a y-slab (lbm_slab.cu)
 constexpr int SLAB_PLANES = 11;   // nine populations, density, psi'(rho) - mu_sat or psi
 struct SlabMsgLayout {
@@ -120,7 +131,9 @@ struct GeomOut {
   int* bnode; int* bstart; uint8_t* ldir; double* lq64; uint8_t* lx2f;
   int* s1node; uint8_t* s1mask; int* s2node; uint8_t* s2mask;
   int* s1nb;                                // 8 per first-layer entry: neighbours' boundary index
+  int* s2nb;                                // 8 per second-layer entry: neighbours' first-layer index
   void* lq;   void* s1winv; void* s2winv;   // precision-typed
+  int2* bnd; unsigned short* bmask; void* bq; int bcap;   // links by boundary node (FP32; null otherwise)
   void* mu;                                 // precision-typed plane
   int fp64;
   int n_bnodes, n_s1, n_s2;                 // list lengths (from the counts)

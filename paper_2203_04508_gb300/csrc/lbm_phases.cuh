@@ -35,7 +35,7 @@ __device__ __forceinline__ void phase_solid(const Lattice<real>& L, int layer, i
   real acc = real(0);
 #pragma unroll
   for (int i = 1; i < 9; ++i) {
-    if (m & (1u << (i - 1))) acc += real(wgt(i)) * L.rho[node_at(L, x + ex(i), y + ey(i))];
+    if (m & (1u << (i - 1))) acc = fma_rn(real(wgt(i)), L.rho[node_at(L, x + ex(i), y + ey(i))], acc);
   }
   L.rho[n] = acc * winv;
 }

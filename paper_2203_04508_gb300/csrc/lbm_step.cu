@@ -24,6 +24,7 @@
 #include <cstdio>
 
 #include "lbm_device.cuh"
+#include "lbm_fused.cuh"
 #include "lbm_internal.h"
 #include "lbm_phases.cuh"
 
@@ -73,14 +74,6 @@ template <typename real>
 __global__ void __launch_bounds__(NODE_BLOCK) k_bmom(Lattice<real> L, int cur) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b < L.n_bnodes) phase_bmom(L, cur, b);
-}
-
-// psi(rho_s) (1 + c_w) of a solid-layer node whose density is rho_s (pseudopotential force)
-template <typename real>
-__device__ __forceinline__ real psi_wall(const Lattice<real>& L, int n, real rs) {
-  const int b = L.body[n];
-  const double cw = b < L.n_cyl ? L.cyl[4 * b + 3] : L.cw_walls;
-  return psi_of(L, rs) * (real(1) + (real)cw);
 }
 
 // Eq. 15 for one solid layer; with the pseudopotential force also the layer's psi, so that the
@@ -588,8 +581,8 @@ __global__ void __launch_bounds__(NODE_BLOCK) k_collide_tma(Lattice<float> L, in
   const int lx = threadIdx.x % CT_X, ly = threadIdx.x / CT_X;
   auto f_of = [&](int s) { return reinterpret_cast<float*>(tma_smem + s * SB); };
   // mu (or psi) right after the populations, the density (chemical potential) after it
-  auto mu_of = [&](int s) { return reinterpret_cast<float*>(tma_smem + s * SB + FB); };
-  auto rho_of = [&](int s) { return reinterpret_cast<float*>(tma_smem + s * SB + FB + TMA_M_BYTES); };
+  auto mu_at = [&](int s) { return reinterpret_cast<float*>(tma_smem + s * SB + FB); };
+  auto rho_at = [&](int s) { return reinterpret_cast<float*>(tma_smem + s * SB + FB + TMA_M_BYTES); };
   float* ring = reinterpret_cast<float*>(tma_smem + TMA_STAGES * SB);
   uint8_t* rkind = tma_smem + TMA_STAGES * SB + SW_RING_BYTES;
   // this block's tiles k = 0 .. nt - 1, as tile coordinates (tx, ty) advanced without a division:
@@ -630,8 +623,8 @@ __global__ void __launch_bounds__(NODE_BLOCK) k_collide_tma(Lattice<float> L, in
     if (FMODE == 2) tma_load_3d(f_of(s), &M.f, x0 - TMA_POX, y0 - 1, 0, &bar[s]);
     else tma_load_3d(f_of(s), &M.f, x0, y0, 0, &bar[s]);
     if (h) {
-      tma_load_2d(mu_of(s), &M.mu, x0 - TMA_HOX, y0 - CT_H, &bar[s]);
-      if (!PSEUDO) tma_load_2d(rho_of(s), &M.rho, x0 - TMA_HOX, y0 - CT_H, &bar[s]);
+      tma_load_2d(mu_at(s), &M.mu, x0 - TMA_HOX, y0 - CT_H, &bar[s]);
+      if (!PSEUDO) tma_load_2d(rho_at(s), &M.rho, x0 - TMA_HOX, y0 - CT_H, &bar[s]);
     }
   };
   if (threadIdx.x == 0) {
@@ -653,8 +646,8 @@ __global__ void __launch_bounds__(NODE_BLOCK) k_collide_tma(Lattice<float> L, in
     // a wait that gives up is acted on at the block barrier below, once every thread has read
     // the stage (what a thread whose wait gave up read is never used)
     const bool ok = mbar_wait(&bar[s], (uint32_t)((k / TMA_STAGES) & 1), L.spin_limit);
-    float* sm = mu_of(s);
-    float* sr = rho_of(s);
+    float* sm = mu_at(s);
+    float* sr = rho_at(s);
     if (stencils && !(tile.z & 1)) {
       // the halo wraps around a periodic edge: plain wrap-aware loads, as k_collide stages it
       const int h = PSEUDO ? 1 : CT_H;
@@ -824,7 +817,7 @@ __global__ void __launch_bounds__(NODE_BLOCK) k_solid1_b(Lattice<real> L) {
   real acc = real(0);
 #pragma unroll
   for (int i = 1; i < 9; ++i) {
-    if (m & (1u << (i - 1))) acc += real(wgt(i)) * L.rho_b[L.s1nb[8 * j + i - 1]];
+    if (m & (1u << (i - 1))) acc = fma_rn(real(wgt(i)), L.rho_b[L.s1nb[8 * j + i - 1]], acc);
   }
   const real rs = acc * L.s1winv[j];
   L.rho[L.s1node[j]] = rs;
