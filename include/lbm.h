@@ -404,8 +404,12 @@ lbm_status lbm_batch_build_links(lbm_batch* b);
 /* lbm_init for every instance with specs[k] (n specs).  Synchronises. */
 lbm_status lbm_batch_init(lbm_batch* b, const lbm_init_spec* specs);
 
-/* Advances every instance n steps in ONE cooperative launch of a persistent kernel (captured
- * into a CUDA graph on first use for this n): each step runs the phases of lbm_step over all
+/* Advances every instance n steps.  Where all of them run the fused step (lbm_step: FP32, two
+ * population lattices, an equation of state) its three kernels run over flat lists of all
+ * instances' work, captured into CUDA graphs on first use; a batch whose poll budget the caller
+ * set (lbm_batch_set_spin_limit, other than the default) and every other batch runs ONE cooperative
+ * launch of a persistent kernel (captured for this n), to which the tile shape and the schedule
+ * below belong.  Both give the same values, bit for bit.  In the persistent kernel each step runs the phases of lbm_step over all
  * instances' work, separated by grid barriers; per-instance compensation sums go to each
  * instance's ring as with lbm_step.  Asynchronous; lbm_batch_check reports a barrier timeout. */
 lbm_status lbm_batch_step(lbm_batch* b, int64_t n);
@@ -415,7 +419,9 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t n);
 lbm_status lbm_batch_check(lbm_batch* b);
 
 /* Polls before a grid-barrier wait gives up (default 2^22, about a second or more); 0 makes
- * every wait give up at once (used to test the timeout path).  Clears the error flag. */
+ * every wait give up at once (used to test the timeout path).  Another value than the default makes
+ * lbm_batch_step run the persistent kernel (the fused step waits for nothing).  Clears the error
+ * flag. */
 lbm_status lbm_batch_set_spin_limit(lbm_batch* b, int64_t polls);
 
 /* Shape of the node tiles of the persistent kernel: 2^log2w nodes wide and 256 / 2^log2w

@@ -179,7 +179,7 @@ struct lbm_ctx {
   int mu_kind = -1;                   // chemical-potential pass (-1: the precision's default)
   bool collide_set = false;           // lbm_set_collide_kernel was called
   bool fused_ok = false;              // the fused step's kernels can run on this device
-  int fused_rows = 0;                 // rows a warp of the fused step walks
+  PassPlan plan;                      // how the fused step's pass runs on this lattice
   long long n_near = 0;               // entries of the near list, built where the fused density +
   bool near_built = false;            // mu pass is selected (lbm_build_links, lbm_set_mu_kernel)
   lbm_status sticky = LBM_OK;
@@ -495,7 +495,7 @@ Lattice<float> fused_lattice(const lbm_ctx* c, const Lattice<float>& L, int cur)
 template <typename real>
 cudaError_t issue_step(lbm_ctx* c, const Lattice<real>& L, int cur) {
   if constexpr (sizeof(real) == 4) {
-    if (fused(c)) return launch_fused_step(fused_lattice(c, L, cur), cur, c->fused_rows, c->stream);
+    if (fused(c)) return launch_fused_step(fused_lattice(c, L, cur), cur, c->plan, c->stream);
   }
   Lattice<real> Lt, Ln;
   step_lattices(c, L, cur, Lt, Ln);
@@ -1079,7 +1079,7 @@ lbm_status lbm_build_links(lbm_ctx* c) {
     c->fused_ok = cudaGetDevice(&dev) == cudaSuccess &&
                   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && fused_setup();
     if (!c->fused_ok) (void)cudaGetLastError();
-    c->fused_rows = fused_rows(g.nx, g.ny, sms);
+    c->plan = fused_plan(g.nx, g.ny, sms);
     // the list of nodes the combined density + mu pass leaves to k_mu_near, where that pass runs
     if (c->Lf.mu_kernel == 3 && !fused(c)) {
       lbm_status st = near_list(c);
@@ -1653,6 +1653,8 @@ void lbm_destroy(lbm_ctx* c) {
 // ---------------------------------------------------------------------------------------
 // Batched lattices
 // ---------------------------------------------------------------------------------------
+constexpr long long BATCH_SPIN_DEFAULT = 1LL << 22;
+
 struct lbm_batch {
   int n = 0;
   bool fp64 = false;
@@ -1663,7 +1665,12 @@ struct lbm_batch {
   size_t tab_off = 0;
   // table offsets inside the tables region
   size_t t_lat = 0, t_tiles = 0, t_s1 = 0, t_s2 = 0, t_bc = 0, t_first = 0, t_group = 0, t_part = 0, t_bar = 0,
-         t_err = 0;
+         t_err = 0, t_flat = 0, t_fpass = 0, t_fbc = 0, t_fsolid = 0;
+  long long cap_fpass = 0, cap_fbc = 0, cap_fsolid = 0;
+  // the fused step over all instances, where every one of them runs it
+  FusedBatch fb{};
+  bool fused = false;
+  cudaGraphExec_t fgraph[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   int groups = 2;
   long long cap_tiles = 0, cap_s1 = 0, cap_s2 = 0, cap_bc = 0;
   BatchDev dev{};
@@ -1673,7 +1680,7 @@ struct lbm_batch {
   cudaGraphExec_t graph = nullptr;
   long long graph_steps = -1;
   int graph_cur = -1;
-  long long spin_limit = 1LL << 22;
+  long long spin_limit = BATCH_SPIN_DEFAULT;
   int tile_log2w = BATCH_TILE_LOG2W_DEFAULT;
   int cur = 0;
   std::string err;
@@ -1685,7 +1692,9 @@ struct BatchPlan {
   std::vector<size_t> off, bytes;
   size_t tab_off, total;
   size_t t_lat, t_tiles, t_s1, t_s2, t_bc, t_first, t_group, t_part, t_bar, t_err;
+  size_t t_flat, t_fpass, t_fbc, t_fsolid;
   long long cap_tiles, cap_s1, cap_s2, cap_bc;
+  long long cap_fpass, cap_fbc, cap_fsolid;
 };
 
 lbm_status plan_batch(int n, const lbm_config* cfgs, BatchPlan* P, char* msg) {
@@ -1694,6 +1703,8 @@ lbm_status plan_batch(int n, const lbm_config* cfgs, BatchPlan* P, char* msg) {
   P->bytes.resize(n);
   size_t o = 0;
   P->cap_tiles = P->cap_s1 = P->cap_s2 = P->cap_bc = 0;
+  P->cap_fpass = P->cap_fbc = P->cap_fsolid = 0;
+  const bool fp32 = cfgs[0].precision == LBM_FP32;
   for (int k = 0; k < n; ++k) {
     lbm_status s = validate(&cfgs[k], msg);
     if (s != LBM_OK) return s;
@@ -1715,6 +1726,8 @@ lbm_status plan_batch(int n, const lbm_config* cfgs, BatchPlan* P, char* msg) {
     // phase, in chunks that follow the layer's own
     P->cap_s2 += (L.cap.s2 + bb - 1) / bb + (cfgs[k].layout == LBM_LAYOUT_AA ? (L.cap.bnodes + bb - 1) / bb : 0);
     P->cap_bc += (L.cap.bnodes + bb - 1) / bb;
+    if (fp32)
+      fused_batch_caps(cfgs[k].nx, cfgs[k].ny, L.cap.bnodes, L.cap.s1, L.cap.s2, &P->cap_fpass, &P->cap_fbc, &P->cap_fsolid);
   }
   P->tab_off = o;
   size_t t = 0;
@@ -1730,6 +1743,10 @@ lbm_status plan_batch(int n, const lbm_config* cfgs, BatchPlan* P, char* msg) {
   P->t_part = take((size_t)(P->cap_bc + 1) * sizeof(double));
   P->t_bar = take(16 + BATCH_WORK_COUNTERS * 8);   // barrier words, then the work counters
   P->t_err = take(16);
+  P->t_flat = take(fp32 ? 2 * (size_t)n * sizeof(Lattice<float>) : 0);
+  P->t_fpass = take((size_t)P->cap_fpass * sizeof(int4));
+  P->t_fbc = take((size_t)P->cap_fbc * sizeof(int2));
+  P->t_fsolid = take((size_t)P->cap_fsolid * sizeof(int2));
   P->total = P->tab_off + t;
   return LBM_OK;
 }
@@ -1829,6 +1846,91 @@ lbm_status batch_tables(lbm_batch* b) {
   return LBM_OK;
 }
 
+// The fused step's descriptors and work lists, where every instance runs it.
+lbm_status fused_tables(lbm_batch* b) {
+  for (auto& g : b->fgraph)
+    if (g) { cudaGraphExecDestroy(g); g = nullptr; }
+  b->fused = true;
+  for (auto* c : b->ctx) b->fused &= fused(c);
+  if (!b->fused) return LBM_OK;
+  int dev = 0, sms = 0;
+  BCUDA(b, cudaGetDevice(&dev));
+  BCUDA(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  long long tiles = 0, strip_rows = 0;
+  for (auto* c : b->ctx) {
+    tiles += fused_tiles(c->cfg.nx, c->cfg.ny);
+    strip_rows += fused_strip_rows(c->cfg.nx, c->cfg.ny);
+  }
+  FusedBatch& F = b->fb;
+  F.rows = fused_batch_rows(b->n, tiles, strip_rows, sms);
+  std::vector<Lattice<float>> lats;
+  for (int p = 0; p < 2; ++p)
+    for (auto* c : b->ctx) lats.push_back(fused_lattice(c, c->Lf, p));
+  std::vector<int4> pass;
+  std::vector<int2> bc, solid;
+  for (int k = 0; k < b->n; ++k) {
+    const lbm_ctx* c = b->ctx[k];
+    fused_batch_items(k, c->cfg.nx, c->cfg.ny, (int)c->n_bnodes, (int)c->n_s1, (int)c->n_s2, F.rows, &pass, &bc, &solid);
+  }
+  if ((long long)pass.size() > b->cap_fpass || (long long)bc.size() > b->cap_fbc || (long long)solid.size() > b->cap_fsolid)
+    return bfail(b, LBM_ENOMEM, "batch work lists exceed their capacity");
+  // the tallest items first: the last to start are then the shortest
+  std::stable_sort(pass.begin(), pass.end(), [](const int4& u, const int4& v) { return u.w > v.w; });
+  char* t = b->ws + b->tab_off;
+  auto up = [&](size_t at, const void* p, size_t bytes) {
+    return bytes ? cudaMemcpyAsync(t + at, p, bytes, cudaMemcpyHostToDevice, b->stream) : cudaSuccess;
+  };
+  BCUDA(b, up(b->t_flat, lats.data(), lats.size() * sizeof(lats[0])));
+  BCUDA(b, up(b->t_fpass, pass.data(), pass.size() * sizeof(int4)));
+  BCUDA(b, up(b->t_fbc, bc.data(), bc.size() * sizeof(int2)));
+  BCUDA(b, up(b->t_fsolid, solid.data(), solid.size() * sizeof(int2)));
+  BCUDA(b, cudaStreamSynchronize(b->stream));
+  F.lat[0] = (const Lattice<float>*)(t + b->t_flat);
+  F.lat[1] = F.lat[0] + b->n;
+  F.pass = (const int4*)(t + b->t_fpass);
+  F.bc = (const int2*)(t + b->t_fbc);
+  F.solid = (const int2*)(t + b->t_fsolid);
+  F.n_pass = (int)pass.size();
+  F.n_bc = (int)bc.size();
+  F.n_solid = (int)solid.size();
+  return LBM_OK;
+}
+
+// n fused steps of every instance: graphs of STEPS_LONG, two and one steps, as lbm_step's
+lbm_status fused_batch_step(lbm_batch* b, long long n) {
+  bool ready = true;
+  for (auto* c : b->ctx) ready &= c->rho_ok;
+  if (!ready) BCUDA(b, launch_fused_batch_prepare(b->fb, b->cur, b->stream));
+  int cur = b->cur;
+  auto run = [&](int steps) -> lbm_status {
+    if (!b->stream) {
+      // the legacy default stream is not captured
+      for (int k = 0; k < steps; ++k, cur ^= 1) BCUDA(b, launch_fused_batch_step(b->fb, cur, b->stream));
+      return LBM_OK;
+    }
+    cudaGraphExec_t& slot = b->fgraph[(steps == 2 ? 0 : steps == 1 ? 2 : 4) + cur];
+    if (!slot) {
+      cudaGraph_t g = nullptr;
+      BCUDA(b, cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal));
+      cudaError_t e = cudaSuccess;
+      for (int k = 0; k < steps && e == cudaSuccess; ++k) e = launch_fused_batch_step(b->fb, cur ^ (k & 1), b->stream);
+      cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
+      if (e == cudaSuccess) e = e2;
+      if (e == cudaSuccess) e = cudaGraphInstantiate(&slot, g, 0);
+      if (g) cudaGraphDestroy(g);
+      if (e != cudaSuccess) return bfail(b, LBM_ECUDA, "graph capture failed: %s", cudaGetErrorString(e));
+    }
+    BCUDA(b, cudaGraphLaunch(slot, b->stream));
+    cur ^= steps & 1;
+    return LBM_OK;
+  };
+  lbm_status st = LBM_OK;
+  for (; n >= STEPS_LONG && st == LBM_OK; n -= STEPS_LONG) st = run(STEPS_LONG);
+  for (; n >= 2 && st == LBM_OK; n -= 2) st = run(2);
+  if (n == 1 && st == LBM_OK) st = run(1);
+  return st;
+}
+
 }  // namespace
 
 extern "C" {
@@ -1864,6 +1966,8 @@ lbm_status lbm_batch_create(int32_t n, const lbm_config* cfgs, void* stream, voi
   b->tab_off = P.tab_off;
   b->t_lat = P.t_lat; b->t_tiles = P.t_tiles; b->t_s1 = P.t_s1; b->t_s2 = P.t_s2; b->t_bc = P.t_bc;
   b->t_first = P.t_first; b->t_group = P.t_group; b->t_part = P.t_part; b->t_bar = P.t_bar; b->t_err = P.t_err;
+  b->t_flat = P.t_flat; b->t_fpass = P.t_fpass; b->t_fbc = P.t_fbc; b->t_fsolid = P.t_fsolid;
+  b->cap_fpass = P.cap_fpass; b->cap_fbc = P.cap_fbc; b->cap_fsolid = P.cap_fsolid;
   b->cap_tiles = P.cap_tiles; b->cap_s1 = P.cap_s1; b->cap_s2 = P.cap_s2; b->cap_bc = P.cap_bc;
   b->ctx.assign(n, nullptr);
   for (int k = 0; k < n; ++k) {
@@ -1881,7 +1985,8 @@ lbm_status lbm_batch_build_links(lbm_batch* b) {
     if (st != LBM_OK) return bfail(b, st, "instance %d: %s", k, b->ctx[k]->err.c_str());
   }
   if (b->graph) { cudaGraphExecDestroy(b->graph); b->graph = nullptr; }
-  return b->fp64 ? batch_tables<double>(b) : batch_tables<float>(b);
+  lbm_status st = b->fp64 ? batch_tables<double>(b) : batch_tables<float>(b);
+  return st == LBM_OK ? fused_tables(b) : st;
 }
 
 lbm_status lbm_batch_init(lbm_batch* b, const lbm_init_spec* specs) {
@@ -1904,6 +2009,22 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t n) {
   }
   if (n <= 0) return n == 0 ? LBM_OK : LBM_EINVAL;
   if (n > (1LL << 30)) return bfail(b, LBM_EINVAL, "too many steps in one launch");
+  const int flip = (int)(n & 1);
+  // the fused step where every instance runs it, unless the caller bounds the persistent kernel's
+  // waits (the fused step has none)
+  bool all_fused = b->fused && b->spin_limit == BATCH_SPIN_DEFAULT;
+  for (int k = 0; k < b->n && all_fused; ++k) all_fused = fused(b->ctx[k]);
+  if (all_fused) {
+    lbm_status st = fused_batch_step(b, n);
+    if (st != LBM_OK) return st;
+    b->cur ^= flip;
+    for (int k = 0; k < b->n; ++k) {
+      b->ctx[k]->cur ^= flip;
+      b->ctx[k]->steps += n;
+      b->ctx[k]->rho_ok = true;
+    }
+    return LBM_OK;
+  }
   b->dev.spin_limit = b->spin_limit;
   if (b->use_graph && (b->graph_steps != n || b->graph_cur != b->cur || !b->graph)) {
     if (b->graph) { cudaGraphExecDestroy(b->graph); b->graph = nullptr; }
@@ -1928,7 +2049,6 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t n) {
   }
   if (b->use_graph && b->graph) BCUDA(b, cudaGraphLaunch(b->graph, b->stream));
   else BCUDA(b, launch_batch(b->dev, b->fp64, b->grid, (int)n, b->cur, b->stream));
-  const int flip = (int)(n & 1);
   b->cur ^= flip;
   for (int k = 0; k < b->n; ++k) {
     b->ctx[k]->cur ^= flip;
@@ -2053,6 +2173,8 @@ const char* lbm_batch_last_error(const lbm_batch* b) { return b ? b->err.c_str()
 void lbm_batch_destroy(lbm_batch* b) {
   if (!b) return;
   if (b->graph) cudaGraphExecDestroy(b->graph);
+  for (auto& g : b->fgraph)
+    if (g) cudaGraphExecDestroy(g);
   for (auto* c : b->ctx) lbm_destroy(c);
   delete b;
 }

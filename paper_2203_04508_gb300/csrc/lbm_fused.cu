@@ -18,14 +18,23 @@
 // those nodes in two planes (the pass stores it in the rows next to solids).  The densities of
 // boundary nodes come from k_bc_fused, those of the solid layers from k_solids.
 //
-// On the 2048 x 4096 impact lattice a step takes 0.133 ms against 0.192 ms for the separate passes
-// (1024 x 1024 with 16 drops 33 against 45 us, 131 x 97 9.3 against 29 us); the pass itself 0.13 ms,
+// On the 2048 x 4096 impact lattice a step takes 0.145 ms against 0.192 ms for the separate passes
+// (1024 x 1024 with 16 drops 33 against 45 us, 131 x 97 9.0 against 29 us); the pass itself 0.13 ms,
 // 661 MB of DRAM traffic.  What was tried on the way there: the density formed from the populations
 // at the start of the same pass instead of the end of the previous one (72 instead of 80 bytes a
 // node, but the populations of four more rows wait in shared memory for their collision: 10 warps
 // an SM instead of 12, 0.19 ms); 8-byte cp.async through L1 instead of 16-byte ones past it (the
 // L1 lines left beside 200 KB of shared memory bound the loads in flight: 0.20 against 0.15 ms);
-// one row an iteration, conditions inside (0.22 ms: divergent branches and short chains).
+// one row an iteration, conditions inside (0.22 ms: divergent branches and short chains); four
+// columns a lane (half the shared-memory and store instructions, but 7 warps an SM: 0.20 ms).
+//
+// Batches run the same kernels over flat lists of all instances' tiles (walks, where the instances
+// are large), links and layers, each block with its instance's descriptor in shared memory: 64
+// lattices of 128..768 take 398 us a step against 590 us for the persistent kernel (k_batch: six grid
+// barriers a step, 890 instructions a node), 256 of 64..128 119 against 217 us.
+#include <algorithm>
+#include <vector>
+
 #include "lbm_fused.cuh"
 
 #include "lbm_internal.h"
@@ -61,18 +70,6 @@ __device__ __forceinline__ void cp16(void* dst, const void* src) {
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
-
-// stores under a condition, as predicated instructions: the strip's end lanes would otherwise
-// cost a divergent branch for each direction
-__device__ __forceinline__ void store_if(bool p, char* at, float2 v) {
-  asm volatile("{\n .reg .pred p;\n setp.ne.s32 p, %0, 0;\n @p st.global.v2.f32 [%1], {%2, %3};\n}\n" ::"r"((int)p), "l"(at),
-               "f"(v.x), "f"(v.y)
-               : "memory");
-}
-__device__ __forceinline__ void store_if(bool p, char* at, float v) {
-  asm volatile("{\n .reg .pred p;\n setp.ne.s32 p, %0, 0;\n @p st.global.f32 [%1], %2;\n}\n" ::"r"((int)p), "l"(at), "f"(v)
-               : "memory");
-}
 
 // Programmatic dependent launch: a kernel of the step may start while the one before it still runs
 // (grid_launch there), and reads or writes nothing that one touches before grid_wait, which waits
@@ -211,8 +208,6 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
     const float2 z = make_float2(0.f, 0.f);
     in = {z, z, z, z, z, z, z, z};
   }
-  const unsigned at_c = 4u * (unsigned)c;
-  const bool odd = (L.nx & 1) != 0;
   // Streaming of row y's post-collision populations: every pair of outputs receives columns c - 1, c
   // (moving right) or c + 1, c + 2 (moving left) through the neighbouring lane, so that all stores
   // are aligned pairs.  Slots whose source is solid get a meaningless value; the boundary phase
@@ -222,31 +217,50 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
     auto left = [](float2 a) { return make_float2(a.y, __shfl_down_sync(0xffffffffu, a.x, 1)); };
     const float2 r1 = right(v[1]), r5 = right(v[5]), r8 = right(v[8]);
     const float2 l3 = left(v[3]), l6 = left(v[6]), l7 = left(v[7]);
-    // byte offsets of row y and its neighbours in a plane; one outside [ya, yb) is not stored to
-    const unsigned at = 4u * (unsigned)(y * L.pitch) + at_c, au = at + 4u * (unsigned)L.pitch, ad = at - 4u * (unsigned)L.pitch;
-    auto put = [&](bool ok, int i, unsigned off, float2 a) {
-      char* p = reinterpret_cast<char*>(fout + (long long)i * L.plane) + off;
-      store_if(ok && out1, p, a);
-      if (odd) store_if(ok && one, p, a.x);
-    };
-    const bool mid = y >= ya && y < yb, up = y + 1 < yb, dn = y > ya;
-    put(mid, 0, at, v[0]);
-    put(mid, 1, at, r1);
-    put(mid, 3, at, l3);
-    put(up, 2, au, v[2]);
-    put(up, 5, au, r5);
-    put(up, 6, au, l6);
-    put(dn, 4, ad, v[4]);
-    put(dn, 7, ad, l7);
-    put(dn, 8, ad, r8);
     // row y - 1: density_sum's order
     const float2 sum = add_rn(in.c0, add_rn(add_rn(in.s13, add_rn(in.d2, v[4])),
                                             add_rn(add_rn(in.d5, l7), add_rn(in.d6, r8))));
     float2 q = add_rn(splat<float2>(L.rho_ref), sum);
     if (PSEUDO) q = psi_of(L, q);
-    char* p = reinterpret_cast<char*>(rout) + ad;
-    store_if(dn && out1, p, q);
-    if (odd) store_if(dn && one, p, q.x);
+    const int n = y * L.pitch + c;
+    const bool mid = y >= ya && y < yb, up = y + 1 < yb, dn = y > ya;   // rows the band does not own are left
+    if (out1) {
+      auto put = [&](float* plane, int at, float2 a) { *reinterpret_cast<float2*>(plane + at) = a; };
+      if (mid) {
+        put(fout, n, v[0]);
+        put(fout + 1ll * L.plane, n, r1);
+        put(fout + 3ll * L.plane, n, l3);
+      }
+      if (up) {
+        put(fout + 2ll * L.plane, n + L.pitch, v[2]);
+        put(fout + 5ll * L.plane, n + L.pitch, r5);
+        put(fout + 6ll * L.plane, n + L.pitch, l6);
+      }
+      if (dn) {
+        put(fout + 4ll * L.plane, n - L.pitch, v[4]);
+        put(fout + 7ll * L.plane, n - L.pitch, l7);
+        put(fout + 8ll * L.plane, n - L.pitch, r8);
+        put(rout, n - L.pitch, q);
+      }
+    } else if (one) {
+      auto put = [&](float* plane, int at, float a) { plane[at] = a; };
+      if (mid) {
+        put(fout, n, v[0].x);
+        put(fout + 1ll * L.plane, n, r1.x);
+        put(fout + 3ll * L.plane, n, l3.x);
+      }
+      if (up) {
+        put(fout + 2ll * L.plane, n + L.pitch, v[2].x);
+        put(fout + 5ll * L.plane, n + L.pitch, r5.x);
+        put(fout + 6ll * L.plane, n + L.pitch, l6.x);
+      }
+      if (dn) {
+        put(fout + 4ll * L.plane, n - L.pitch, v[4].x);
+        put(fout + 7ll * L.plane, n - L.pitch, l7.x);
+        put(fout + 8ll * L.plane, n - L.pitch, r8.x);
+        put(rout, n - L.pitch, q.x);
+      }
+    }
     in.c0 = v[0];
     in.s13 = add_rn(r1, l3);
     in.d2 = in.e2;
@@ -416,6 +430,26 @@ __global__ void __launch_bounds__(32) k_walk(const __grid_constant__ Lattice<flo
   walk<PSEUDO>(L, cur, strip, ya, yb, smem);
 }
 
+// The descriptor of a batch's instance in shared memory, copied by the block's threads (the tables
+// are constant: this runs before grid_wait).
+__device__ __forceinline__ void take_lattice(Lattice<float>& L, const Lattice<float>* lat, int k) {
+  static_assert(sizeof(Lattice<float>) % 4 == 0, "descriptor size");
+  const int* s = reinterpret_cast<const int*>(lat + k);
+  int* d = reinterpret_cast<int*>(&L);
+  for (int i = threadIdx.x; i < (int)(sizeof(Lattice<float>) / 4); i += blockDim.x) d[i] = s[i];
+}
+// a batch: item blockIdx.x is (instance, strip, first row, rows)
+__global__ void __launch_bounds__(32) k_walk_batch(const Lattice<float>* lat, const int4* items, int cur) {
+  extern __shared__ __align__(16) char smem[];
+  __shared__ __align__(16) Lattice<float> L;
+  const int4 it = items[blockIdx.x];
+  take_lattice(L, lat, it.x);
+  __syncwarp();
+  grid_wait();
+  grid_launch();
+  walk<false>(L, cur, it.y, it.z, it.z + it.w, smem);
+}
+
 // ---------------------------------------------------------------------------------------
 // The same pass by tiles: a block of W warps takes the OUT output columns of a strip in H rows; its
 // density rows (five more on each side) and population rows (one more) arrive together, then all
@@ -429,19 +463,15 @@ struct Tile {
   static constexpr int BYTES = FLAGS + (H + 6) * 4;
 };
 
-template <bool PSEUDO, int H, int W, int MINB>
-__global__ void __launch_bounds__(32 * W, MINB) k_tile(const __grid_constant__ Lattice<float> L, int cur, int strips) {
-  extern __shared__ __align__(16) char smem[];
+template <bool PSEUDO, int H, int W>
+__device__ __forceinline__ void tile(const Lattice<float>& L, int cur, int strip, int ya, int yb, char* smem) {
   using T = Tile<PSEUDO, H>;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int band = blockIdx.x / strips, strip = blockIdx.x - band * strips;
-  const int ya = band * H, yb = min(ya + H, L.ny);
   const int x0 = strip * OUT, c = x0 - HX + 2 * lane;
   const bool mine = lane >= HX / 2 && lane < 32 - HX / 2;
   const bool out1 = mine && c + 1 < L.nx, one = mine && c + 1 == L.nx;
   const int ca = wrap_col(c, L.nx), cb = wrap_col(c + 1, L.nx);
   const bool split = (L.nx & 3) != 0 && (x0 - 2 * HX < 0 || x0 + OUT + 2 * HX > L.nx);
-  const bool odd = (L.nx & 1) != 0;
   const float* __restrict__ fin = L.f[cur];
   float* __restrict__ fout = L.f[cur ^ 1];
   const float* __restrict__ rin = PSEUDO ? L.mu : L.rho;
@@ -454,18 +484,23 @@ __global__ void __launch_bounds__(32 * W, MINB) k_tile(const __grid_constant__ L
   auto rho_row = [&](int r) { return reinterpret_cast<float2*>(smem + T::RHO) + (r - ya + T::RR) * SP + HX / 2 + lane; };
   auto mu_row = [&](int r) { return reinterpret_cast<float2*>(smem + T::MU) + (r - ya + T::MR) * SP + HX / 2 + lane; };
   auto pop_row = [&](int y) { return reinterpret_cast<float2*>(smem + (y - ya + 1) * ROW_F) + lane; };
-  grid_wait();
-  grid_launch();
   // ---- everything the tile reads
   {
     const int p4 = wrap_col(x0 - HX + 4 * (lane & 15), L.nx), q4 = wrap_col(x0 - 2 * HX + 4 * lane, L.nx);
+    int e4[3] = {0, 0, 0};
+    if (split) {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) e4[j] = wrap_col(x0 - 2 * HX + lane + 32 * j, L.nx);
+    }
     for (int r = ya - T::RR + warp; r < yb + T::RR; r += W) {
       const int n = row_of(r) * L.pitch;
       char* const d = smem + T::RHO + (r - ya + T::RR) * SP * 8;
       if (!split) {
         if (lane < RHO_CHUNKS) cp16(d + 16 * lane, rin + n + q4);
       } else {
-        for (int e = lane; e < 4 * RHO_CHUNKS; e += 32) cp4(d + 4 * e, rin + n + wrap_col(x0 - 2 * HX + e, L.nx));
+#pragma unroll
+        for (int j = 0; j < 3; ++j)
+          if (lane + 32 * j < 4 * RHO_CHUNKS) cp4(d + 4 * (lane + 32 * j), rin + n + e4[j]);
       }
     }
     for (int y = ya - 1 + warp; y <= yb; y += W) {
@@ -560,13 +595,13 @@ __global__ void __launch_bounds__(32 * W, MINB) k_tile(const __grid_constant__ L
     const bool mid = y >= ya && y < yb, up = y + 1 < yb, dn = y > ya;
     if (mid && ((fg[-1] | fg[0] | fg[1]) & 1)) {
       // next to a solid: the force for the boundary phase (read at boundary nodes only)
-      const int n = y * L.pitch + c;
+      const int nf = y * L.pitch + c;
       if (out1) {
-        *reinterpret_cast<float2*>(L.fx + n) = Fx;
-        *reinterpret_cast<float2*>(L.fy + n) = Fy;
+        *reinterpret_cast<float2*>(L.fx + nf) = Fx;
+        *reinterpret_cast<float2*>(L.fy + nf) = Fy;
       } else if (one) {
-        L.fx[n] = Fx.x;
-        L.fy[n] = Fy.x;
+        L.fx[nf] = Fx.x;
+        L.fy[nf] = Fy.x;
       }
     }
     collide_node(L, v, rho, drho, jx, jy, Fx, Fy);
@@ -574,22 +609,42 @@ __global__ void __launch_bounds__(32 * W, MINB) k_tile(const __grid_constant__ L
     auto left = [](float2 a) { return make_float2(a.y, __shfl_down_sync(0xffffffffu, a.x, 1)); };
     const float2 r1 = right(v[1]), r5 = right(v[5]), r8 = right(v[8]);
     const float2 l3 = left(v[3]), l6 = left(v[6]), l7 = left(v[7]);
-    const unsigned at = 4u * (unsigned)(y * L.pitch) + 4u * (unsigned)c, au = at + 4u * (unsigned)L.pitch,
-                   ad = at - 4u * (unsigned)L.pitch;
-    auto put = [&](bool ok, int i, unsigned off, float2 a) {
-      char* p = reinterpret_cast<char*>(fout + (long long)i * L.plane) + off;
-      store_if(ok && out1, p, a);
-      if (odd) store_if(ok && one, p, a.x);
-    };
-    put(mid, 0, at, v[0]);
-    put(mid, 1, at, r1);
-    put(mid, 3, at, l3);
-    put(up, 2, au, v[2]);
-    put(up, 5, au, r5);
-    put(up, 6, au, l6);
-    put(dn, 4, ad, v[4]);
-    put(dn, 7, ad, l7);
-    put(dn, 8, ad, r8);
+    const int n = y * L.pitch + c;
+    if (out1) {
+      auto put = [&](int i, int at, float2 a) { *reinterpret_cast<float2*>(fout + (long long)i * L.plane + at) = a; };
+      if (mid) {
+        put(0, n, v[0]);
+        put(1, n, r1);
+        put(3, n, l3);
+      }
+      if (up) {
+        put(2, n + L.pitch, v[2]);
+        put(5, n + L.pitch, r5);
+        put(6, n + L.pitch, l6);
+      }
+      if (dn) {
+        put(4, n - L.pitch, v[4]);
+        put(7, n - L.pitch, l7);
+        put(8, n - L.pitch, r8);
+      }
+    } else if (one) {
+      auto put = [&](int i, int at, float a) { fout[(long long)i * L.plane + at] = a; };
+      if (mid) {
+        put(0, n, v[0].x);
+        put(1, n, r1.x);
+        put(3, n, l3.x);
+      }
+      if (up) {
+        put(2, n + L.pitch, v[2].x);
+        put(5, n + L.pitch, r5.x);
+        put(6, n + L.pitch, l6.x);
+      }
+      if (dn) {
+        put(4, n - L.pitch, v[4].x);
+        put(7, n - L.pitch, l7.x);
+        put(8, n - L.pitch, r8.x);
+      }
+    }
     // what the densities of rows y - 1, y and y + 1 are summed from, in place of the populations
     pr[0] = v[0];
     pr[32] = add_rn(r1, l3);
@@ -617,6 +672,27 @@ __global__ void __launch_bounds__(32 * W, MINB) k_tile(const __grid_constant__ L
   }
 }
 
+template <bool PSEUDO, int H, int W, int MINB>
+__global__ void __launch_bounds__(32 * W, MINB) k_tile(const __grid_constant__ Lattice<float> L, int cur, int strips, int rows) {
+  extern __shared__ __align__(16) char smem[];
+  const int band = blockIdx.x / strips, strip = blockIdx.x - band * strips;
+  const int ya = band * rows, yb = min(ya + rows, L.ny);
+  grid_wait();
+  grid_launch();
+  tile<PSEUDO, H, W>(L, cur, strip, ya, yb, smem);
+}
+template <int H, int W, int MINB>
+__global__ void __launch_bounds__(32 * W, MINB) k_tile_batch(const Lattice<float>* lat, const int4* items, int cur) {
+  extern __shared__ __align__(16) char smem[];
+  __shared__ __align__(16) Lattice<float> L;
+  const int4 it = items[blockIdx.x];
+  take_lattice(L, lat, it.x);
+  __syncthreads();
+  grid_wait();
+  grid_launch();
+  tile<false, H, W>(L, cur, it.y, it.z, it.z + it.w, smem);
+}
+
 // Cut links of one boundary node a thread (phase_bc's arithmetic, the force from the planes the
 // pass left).  Latency is all it costs, so the loads make two rounds: the node's record -- set up
 // with the geometry, and fetched before the pass it depends on has finished -- then everything
@@ -624,8 +700,7 @@ __global__ void __launch_bounds__(32 * W, MINB) k_tile(const __grid_constant__ L
 // compensation sum per warp; k_solids adds them up.
 constexpr int BC_BLOCK = 64;
 template <bool PSEUDO>
-__global__ void __launch_bounds__(BC_BLOCK) k_bc_fused(const __grid_constant__ Lattice<float> L, int cur) {
-  const int b = blockIdx.x * BC_BLOCK + threadIdx.x;
+__device__ __forceinline__ void links(const Lattice<float>& L, int cur, int b) {
   const bool live = b < L.n_bnodes;
   const int2 nd = live ? L.bnd[b] : make_int2(0, 0);
   const unsigned mask = live ? L.bmask[b] : 0u;
@@ -696,6 +771,19 @@ __global__ void __launch_bounds__(BC_BLOCK) k_bc_fused(const __grid_constant__ L
   if ((threadIdx.x & 31) == 0) L.partials[b >> 5] = sum;
 }
 
+template <bool PSEUDO>
+__global__ void __launch_bounds__(BC_BLOCK) k_bc_fused(const __grid_constant__ Lattice<float> L, int cur) {
+  links<PSEUDO>(L, cur, blockIdx.x * BC_BLOCK + threadIdx.x);
+}
+// item: (instance, first boundary node)
+__global__ void __launch_bounds__(BC_BLOCK) k_bc_batch(const Lattice<float>* lat, const int2* items, int cur) {
+  __shared__ __align__(16) Lattice<float> L;
+  const int2 it = items[blockIdx.x];
+  take_lattice(L, lat, it.x);
+  __syncthreads();
+  links<false>(L, cur, it.y + threadIdx.x);
+}
+
 // Both solid layers from the boundary nodes' densities in rho_b (every fluid neighbour of a
 // first-layer node is a boundary node), into the density plane (psi with the wall factor into the
 // psi plane).  A second-layer node forms its first-layer neighbours' densities again, one a lane of
@@ -704,10 +792,8 @@ __global__ void __launch_bounds__(BC_BLOCK) k_bc_fused(const __grid_constant__ L
 // that out (the layers of a new state).
 constexpr int SOLID_BLOCK = 256;
 template <bool PSEUDO>
-__global__ void __launch_bounds__(SOLID_BLOCK) k_solids(const __grid_constant__ Lattice<float> L, int blocks2, int blocks1,
-                                                        int steps) {
+__device__ __forceinline__ void solids(const Lattice<float>& L, int blk, int blocks2, int blocks1, int steps) {
   __shared__ double red[32];
-  const int blk = blockIdx.x;
   auto first = [&](unsigned m, float winv, const int (&nb)[8]) {
     float acc = 0.f;
 #pragma unroll
@@ -781,12 +867,26 @@ __global__ void __launch_bounds__(SOLID_BLOCK) k_solids(const __grid_constant__ 
   }
 }
 
+template <bool PSEUDO>
+__global__ void __launch_bounds__(SOLID_BLOCK) k_solids(const __grid_constant__ Lattice<float> L, int blocks2, int blocks1,
+                                                        int steps) {
+  solids<PSEUDO>(L, blockIdx.x, blocks2, blocks1, steps);
+}
+// item: (instance, its block)
+__global__ void __launch_bounds__(SOLID_BLOCK) k_solids_batch(const Lattice<float>* lat, const int2* items, int steps) {
+  __shared__ __align__(16) Lattice<float> L;
+  const int2 it = items[blockIdx.x];
+  take_lattice(L, lat, it.x);
+  __syncthreads();
+  solids<false>(L, it.y, (8 * L.n_s2 + SOLID_BLOCK - 1) / SOLID_BLOCK, (L.n_s1 + SOLID_BLOCK - 1) / SOLID_BLOCK, steps);
+}
+
 // A new state (set up, loaded or advanced by the separate passes) in lattice `cur`: the density
 // (psi) of its fluid nodes into rho_next, and of its boundary nodes into rho_b, from which k_solids
 // forms the solid layers.
 template <bool PSEUDO>
-__global__ void __launch_bounds__(128) k_density(Lattice<float> L, int cur) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, n = blockIdx.y * L.pitch + x;
+__device__ __forceinline__ void density(const Lattice<float>& L, int cur, int x, int y) {
+  const int n = y * L.pitch + x;
   if (x >= L.nx || L.kind[n] != KIND_FLUID) return;
   const float* __restrict__ f = L.f[cur] + n;
   float v[9];
@@ -795,8 +895,20 @@ __global__ void __launch_bounds__(128) k_density(Lattice<float> L, int cur) {
   const float r = density_of(L, v);
   L.rho_next[n] = PSEUDO ? psi_of(L, r) : r;
 }
-__global__ void __launch_bounds__(128) k_boundary_density(Lattice<float> L, int cur) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x;
+template <bool PSEUDO>
+__global__ void __launch_bounds__(128) k_density(const __grid_constant__ Lattice<float> L, int cur) {
+  density<PSEUDO>(L, cur, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y);
+}
+// a batch: the pass's items (64 threads cover a strip's columns)
+__global__ void __launch_bounds__(64) k_density_batch(const Lattice<float>* lat, const int4* items, int cur) {
+  __shared__ __align__(16) Lattice<float> L;
+  const int4 it = items[blockIdx.x];
+  take_lattice(L, lat, it.x);
+  __syncthreads();
+  if (threadIdx.x >= OUT) return;
+  for (int y = it.z; y < it.z + it.w; ++y) density<false>(L, cur, it.y * OUT + threadIdx.x, y);
+}
+__device__ __forceinline__ void boundary_density(const Lattice<float>& L, int cur, int b) {
   if (b >= L.n_bnodes) return;
   const float* __restrict__ f = L.f[cur] + L.bnode[b];
   float v[9];
@@ -805,40 +917,66 @@ __global__ void __launch_bounds__(128) k_boundary_density(Lattice<float> L, int 
   L.rho_b[b] = density_of(L, v);
 }
 
-// the two tile shapes: output rows, warps a block, blocks an SM
-constexpr int TH_S = 6, TW_S = 8, TB_S = 3;
+// the tile shapes: output rows at most, warps a block, blocks an SM
 constexpr int TH_M = 14, TW_M = 8, TB_M = 3;
+constexpr int TH_L = 10, TW_L = 4, TB_L = 5;
+__global__ void __launch_bounds__(128) k_boundary_density(const __grid_constant__ Lattice<float> L, int cur) {
+  boundary_density(L, cur, blockIdx.x * blockDim.x + threadIdx.x);
+}
+__global__ void __launch_bounds__(BC_BLOCK) k_boundary_density_batch(const Lattice<float>* lat, const int2* items, int cur) {
+  __shared__ __align__(16) Lattice<float> L;
+  const int2 it = items[blockIdx.x];
+  take_lattice(L, lat, it.x);
+  __syncthreads();
+  boundary_density(L, cur, it.y + threadIdx.x);
+}
+
 inline unsigned blocks_for(int n, int b) { return (unsigned)((n + b - 1) / b); }
 
 }  // namespace
 
-// How the pass runs on a lattice of nx x ny: rows a warp walks (> 0), or which tiles (0: 14 rows,
-// -1: 6 rows).  Counted in tiles of 14 rows:
-//   below half a tile an SM the 6-row tiles spread a small lattice over more SMs (us a step, 6 rows
-//   against 14: 96 x 96 9.0 / 10.3, 192 x 160 9.3 / 10.8, but 300 x 300 12.2 / 10.5);
+long long fused_tiles(int nx, int ny) { return (long long)((nx + OUT - 1) / OUT) * ((ny + TH_M - 1) / TH_M); }
+constexpr int MIN_TILE_ROWS = 2;
+
+// How the pass runs on a lattice of nx x ny, counted in tiles of 14 rows:
 //   from 28 tiles an SM on the walk wins, whose rows are formed twice only at the bands' ends and
-//   whose loads run through all of its rows (walk / tiles: 1024 x 1536 50.3 / 43.6, 1600 x 2048
-//   75.8 / 77.1, 2048 x 2048 90.6 / 94.5, 2048 x 4096 144 / 179).
-// A walk takes as many rows as give every SM 24 warps: two waves of what fits at once, so that the
-// warps whose rows hold solid nodes, which take longer, do not set the pass's time alone.
-int fused_rows(int nx, int ny, int sms) {
-  const long long strips = (nx + OUT - 1) / OUT;
-  const long long tiles = strips * ((ny + TH_M - 1) / TH_M);
-  if (2 * tiles < sms) return -1;
-  if (tiles < 28LL * sms) return 0;
-  const long long bands = 24LL * sms / strips;
-  const int rows = (int)((ny + bands - 1) / (bands > 0 ? bands : 1));
-  return rows < 16 ? 16 : rows;
+//   whose loads run through all of its rows (walk / tiles, us a step: 1024 x 1536 50.3 / 43.4,
+//   1600 x 2048 75.8 / 74.7, 2048 x 2048 90.6 / 90.7, 2048 x 3072 118 / 130, 2048 x 4096 145 / 175).
+//   A walk takes as many rows as give every SM 24 warps: two waves of what fits at once, so that the
+//   warps whose rows hold solid nodes, which take longer, do not set the pass's time alone (one wave:
+//   175 against 157 us on 2048 x 4096).
+//   below, tiles of at most 14 rows and eight warps, or (from 6 tiles an SM) 10 rows and four warps,
+//   of which five fit an SM and so overlap their phases better (1024 x 1536 44.9 / 43.4, 800 x 800
+//   21.7 / 22.8).  The bands have equal heights and as many as give every SM the same number of tiles
+//   (500 x 300 13.0 -> 11.8, 96 x 96 10.3 -> 8.2).
+PassPlan fused_plan(int nx, int ny, int sms) {
+  const int strips = (nx + OUT - 1) / OUT;
+  const long long tiles = fused_tiles(nx, ny);
+  PassPlan p;
+  if (tiles >= 28LL * sms) {
+    p.kind = PassPlan::WALK;
+    const long long bands = std::max(1LL, 24LL * sms / strips);
+    p.rows = std::max(16, (int)((ny + bands - 1) / bands));
+    return p;
+  }
+  p.kind = tiles >= 6LL * sms ? PassPlan::TILE_L : PassPlan::TILE_M;
+  const int most = p.kind == PassPlan::TILE_L ? TH_L : TH_M;
+  const long long least = (ny + most - 1) / most, per_sm = (strips * least + sms - 1) / sms;
+  const long long bands = std::max(least, per_sm * sms / strips);
+  p.rows = std::max((int)((ny + bands - 1) / bands), MIN_TILE_ROWS);
+  return p;
 }
 
 bool fused_setup() {
   auto allow = [](const void* k, int bytes) {
     return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
   };
-  return allow((const void*)k_tile<false, TH_S, TW_S, TB_S>, Tile<false, TH_S>::BYTES) &&
-         allow((const void*)k_tile<true, TH_S, TW_S, TB_S>, Tile<true, TH_S>::BYTES) &&
-         allow((const void*)k_tile<false, TH_M, TW_M, TB_M>, Tile<false, TH_M>::BYTES) &&
+  return allow((const void*)k_tile<false, TH_M, TW_M, TB_M>, Tile<false, TH_M>::BYTES) &&
          allow((const void*)k_tile<true, TH_M, TW_M, TB_M>, Tile<true, TH_M>::BYTES) &&
+         allow((const void*)k_walk_batch, Reach<false>::BYTES) &&
+         allow((const void*)k_tile<false, TH_L, TW_L, TB_L>, Tile<false, TH_L>::BYTES) &&
+         allow((const void*)k_tile<true, TH_L, TW_L, TB_L>, Tile<true, TH_L>::BYTES) &&
+         allow((const void*)k_tile_batch<TH_L, TW_L, TB_L>, Tile<false, TH_L>::BYTES) &&
          allow((const void*)k_walk<false>, Reach<false>::BYTES) && allow((const void*)k_walk<true>, Reach<true>::BYTES);
 }
 
@@ -871,24 +1009,70 @@ cudaError_t launch_fused_prepare(const Lattice<float>& L, int cur, cudaStream_t 
 }
 
 template <int H, int W, int B>
-static cudaError_t launch_tiles(const Lattice<float>& L, int cur, cudaStream_t s) {
-  const int strips = (L.nx + OUT - 1) / OUT, bands = (L.ny + H - 1) / H;
-  return L.pseudo ? launch_after(k_tile<true, H, W, B>, strips * bands, 32 * W, Tile<true, H>::BYTES, s, L, cur, strips)
-                  : launch_after(k_tile<false, H, W, B>, strips * bands, 32 * W, Tile<false, H>::BYTES, s, L, cur, strips);
-}
-static cudaError_t launch_pass(const Lattice<float>& L, int cur, int rows, cudaStream_t s) {
-  if (rows < 0) return launch_tiles<TH_S, TW_S, TB_S>(L, cur, s);
-  if (rows == 0) return launch_tiles<TH_M, TW_M, TB_M>(L, cur, s);
+static cudaError_t launch_tiles(const Lattice<float>& L, int cur, int rows, cudaStream_t s) {
   const int strips = (L.nx + OUT - 1) / OUT, bands = (L.ny + rows - 1) / rows;
-  return L.pseudo ? launch_after(k_walk<true>, strips * bands, 32, Reach<true>::BYTES, s, L, cur, strips, rows)
-                  : launch_after(k_walk<false>, strips * bands, 32, Reach<false>::BYTES, s, L, cur, strips, rows);
+  return L.pseudo ? launch_after(k_tile<true, H, W, B>, strips * bands, 32 * W, Tile<true, H>::BYTES, s, L, cur, strips, rows)
+                  : launch_after(k_tile<false, H, W, B>, strips * bands, 32 * W, Tile<false, H>::BYTES, s, L, cur, strips, rows);
+}
+static cudaError_t launch_pass(const Lattice<float>& L, int cur, PassPlan p, cudaStream_t s) {
+  if (p.kind == PassPlan::TILE_M) return launch_tiles<TH_M, TW_M, TB_M>(L, cur, p.rows, s);
+  if (p.kind == PassPlan::TILE_L) return launch_tiles<TH_L, TW_L, TB_L>(L, cur, p.rows, s);
+  const int strips = (L.nx + OUT - 1) / OUT, bands = (L.ny + p.rows - 1) / p.rows;
+  return L.pseudo ? launch_after(k_walk<true>, strips * bands, 32, Reach<true>::BYTES, s, L, cur, strips, p.rows)
+                  : launch_after(k_walk<false>, strips * bands, 32, Reach<false>::BYTES, s, L, cur, strips, p.rows);
 }
 
-cudaError_t launch_fused_step(const Lattice<float>& L, int cur, int rows, cudaStream_t s) {
-  cudaError_t e = launch_pass(L, cur, rows, s);
+cudaError_t launch_fused_step(const Lattice<float>& L, int cur, PassPlan plan, cudaStream_t s) {
+  cudaError_t e = launch_pass(L, cur, plan, s);
   if (e == cudaSuccess && L.n_bnodes > 0)
     e = launch_after(L.pseudo ? k_bc_fused<true> : k_bc_fused<false>, (int)blocks_for(L.n_bnodes, BC_BLOCK), BC_BLOCK, 0, s, L, cur);
   return e == cudaSuccess ? launch_solids(L, 1, s) : e;
+}
+
+// ---- batches
+void fused_batch_items(int k, int nx, int ny, int n_bnodes, int n_s1, int n_s2, int rows, std::vector<int4>* pass,
+                       std::vector<int2>* bc, std::vector<int2>* solid) {
+  const int strips = (nx + OUT - 1) / OUT;
+  const int most = rows > 0 ? rows : TH_L, bands = (ny + most - 1) / most;
+  const int per = (ny + bands - 1) / bands;   // bands of equal height
+  for (int b = 0; b * per < ny; ++b)
+    for (int st = 0; st < strips; ++st) pass->push_back(make_int4(k, st, b * per, std::min(per, ny - b * per)));
+  for (int b = 0; b < n_bnodes; b += BC_BLOCK) bc->push_back(make_int2(k, b));
+  const int blocks = (int)(blocks_for(8 * n_s2, SOLID_BLOCK) + blocks_for(n_s1, SOLID_BLOCK)) + 1;
+  for (int b = 0; b < blocks; ++b) solid->push_back(make_int2(k, b));
+}
+// upper bounds of the three lists for one instance
+void fused_batch_caps(int nx, int ny, long long bnodes, long long s1, long long s2, long long* pass, long long* bc,
+                      long long* solid) {
+  *pass += (long long)((nx + OUT - 1) / OUT) * ((ny + TH_L - 1) / TH_L);
+  *bc += (bnodes + BC_BLOCK - 1) / BC_BLOCK;
+  *solid += (8 * s2 + SOLID_BLOCK - 1) / SOLID_BLOCK + (s1 + SOLID_BLOCK - 1) / SOLID_BLOCK + 1;
+}
+// Rows a warp of the batch walks, or 0 for tiles.  Small lattices are better off in tiles however
+// many there are (64 lattices of 128..768: 407 us a step in tiles, 446 walked -- a quarter of their
+// rows hold solid nodes, and a walk through such rows is slow), so the batch walks where its mean
+// lattice would on its own.
+int fused_batch_rows(int n, long long tiles, long long strip_rows, int sms) {
+  if (tiles < 28LL * sms * n) return 0;
+  const long long rows = (strip_rows + 24LL * sms - 1) / (24LL * sms);
+  return rows < 32 ? 32 : (int)rows;
+}
+long long fused_strip_rows(int nx, int ny) { return (long long)((nx + OUT - 1) / OUT) * ny; }
+
+cudaError_t launch_fused_batch_prepare(const FusedBatch& B, int cur, cudaStream_t s) {
+  const Lattice<float>* lat = B.lat[cur ^ 1];   // whose next plane is this state's
+  k_density_batch<<<B.n_pass, 64, 0, s>>>(lat, B.pass, cur);
+  if (B.n_bc > 0) k_boundary_density_batch<<<B.n_bc, BC_BLOCK, 0, s>>>(lat, B.bc, cur);
+  k_solids_batch<<<B.n_solid, SOLID_BLOCK, 0, s>>>(lat, B.solid, 0);
+  return cudaGetLastError();
+}
+cudaError_t launch_fused_batch_step(const FusedBatch& B, int cur, cudaStream_t s) {
+  const Lattice<float>* lat = B.lat[cur];
+  cudaError_t e = B.rows > 0 ? launch_after(k_walk_batch, B.n_pass, 32, Reach<false>::BYTES, s, lat, B.pass, cur)
+                             : launch_after(k_tile_batch<TH_L, TW_L, TB_L>, B.n_pass, 32 * TW_L, Tile<false, TH_L>::BYTES, s, lat,
+                                            B.pass, cur);
+  if (e == cudaSuccess && B.n_bc > 0) e = launch_after(k_bc_batch, B.n_bc, BC_BLOCK, 0, s, lat, B.bc, cur);
+  return e == cudaSuccess ? launch_after(k_solids_batch, B.n_solid, SOLID_BLOCK, 0, s, lat, B.solid, 1) : e;
 }
 
 int fused_launches(const Lattice<float>& L) { return 2 + (L.n_bnodes > 0 ? 1 : 0); }

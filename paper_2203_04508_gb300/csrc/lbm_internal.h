@@ -1,6 +1,8 @@
 // Internal declarations shared by the library's translation units (not part of the ABI).
 #pragma once
 #include <cstdint>
+#include <vector>
+
 #include <cuda.h>            // CUtensorMap (the type; the encoder is taken from the CUDA driver at run time)
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>   // header-only; a no-op unless a profiler attaches
@@ -81,13 +83,35 @@ bool collide_tma_setup(CollideTma* T, const Lattice<float>& L, const void* rho0,
 // ---- the fused step (lbm_fused.cu): FP32, two population lattices, an equation of state
 // raises the kernels' shared-memory limit on the current device; false when the device refuses
 bool fused_setup();
-// how the pass runs on a lattice of nx x ny: rows a warp walks, or <= 0 for tiles
-int fused_rows(int nx, int ny, int sms);
+// how the pass runs on a lattice: walked, or in tiles of one of two shapes, and the rows of a walk
+// or a tile
+struct PassPlan {
+  enum Kind { WALK, TILE_M, TILE_L } kind = TILE_M;
+  int rows = 0;
+};
+PassPlan fused_plan(int nx, int ny, int sms);
 // the solid layers of a new state in lattice cur, where the fused step expects them
 cudaError_t launch_fused_prepare(const Lattice<float>& L, int cur, cudaStream_t s);
 // one step from lattice cur (L.rho_b, L.fx and L.fy set)
-cudaError_t launch_fused_step(const Lattice<float>& L, int cur, int rows, cudaStream_t s);
+cudaError_t launch_fused_step(const Lattice<float>& L, int cur, PassPlan plan, cudaStream_t s);
 int fused_launches(const Lattice<float>& L);
+// a batch's fused step: every kernel over a flat list of all instances' items
+struct FusedBatch {
+  const Lattice<float>* lat[2];   // the instances' descriptors by lattice parity
+  const int4* pass;               // (instance, strip, first row, rows)
+  const int2* bc;                 // (instance, first boundary node)
+  const int2* solid;              // (instance, block)
+  int n_pass, n_bc, n_solid, rows;   // rows > 0: walks of about that many rows, 0: tiles
+};
+long long fused_tiles(int nx, int ny);
+long long fused_strip_rows(int nx, int ny);
+int fused_batch_rows(int n, long long tiles, long long strip_rows, int sms);
+void fused_batch_items(int k, int nx, int ny, int n_bnodes, int n_s1, int n_s2, int rows, std::vector<int4>* pass,
+                       std::vector<int2>* bc, std::vector<int2>* solid);
+void fused_batch_caps(int nx, int ny, long long bnodes, long long s1, long long s2, long long* pass, long long* bc,
+                      long long* solid);
+cudaError_t launch_fused_batch_prepare(const FusedBatch& B, int cur, cudaStream_t s);
+cudaError_t launch_fused_batch_step(const FusedBatch& B, int cur, cudaStream_t s);
 
 // ---- halo messages of a y-slab (lbm_slab.cu)
 constexpr int SLAB_PLANES = 11;   // nine populations, density, psi'(rho) - mu_sat or psi

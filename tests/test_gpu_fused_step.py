@@ -99,3 +99,30 @@ def test_switching_paths_and_reading_out_between_steps(tmp_path):
     assert np.array_equal(a.populations(), b.populations())
     assert np.array_equal(a.populations(), c.populations())
     assert np.array_equal(a.populations(), d.populations())
+
+
+@pytest.mark.parametrize("walk", [False, True])
+def test_fused_batch_equals_the_persistent_kernel_and_single_lattices(walk):
+    """Instances of mixed sizes advanced by the fused step over flat item lists (tiles, and the walks
+    that large batches take) against the persistent batched kernel (which a batch whose waits are
+    bounded by the caller runs) and against a lattice of its own, bit for bit."""
+    import paper_2203_04508_gb300 as G
+    scs = [S.small_parity(), _box(64, 70, walls=1), _box(117, 61), S.e1_flat_drop(0.3, 60.0, nx=90, ny=75, r0=18.0)]
+    if walk:
+        scs = [_box(2100, 2001, walls=1), _box(2000, 2100)]
+    a, b = (G.Batch([sc.physics() for sc in scs]) for _ in range(2))
+    b.set_spin_limit((1 << 22) + 1)
+    for batch in (a, b):
+        batch.init([sc.droplets() for sc in scs])
+    for n in (1, 13, 2):
+        a.step(n)
+        b.step(n)
+        b.check()
+    for k in range(len(scs)):
+        one = make_lattice(scs[k], fp64=False)
+        one.step(16)
+        pops = one.populations()
+        assert np.array_equal(a.instances[k].populations(), pops), k
+        assert np.array_equal(b.instances[k].populations(), pops), k
+        assert a.instances[k].mass() == one.mass() == b.instances[k].mass()
+        assert np.array_equal(a.instances[k].dM_history(), one.dM_history())
