@@ -216,6 +216,11 @@ lbm_status lbm_prepare_steps(lbm_ctx* ctx, int64_t n);
  * by the read-out kernel directly, others through device staging memory and copies). */
 lbm_status lbm_fields(lbm_ctx* ctx, void* rho, void* vx, void* vy, int32_t on_device);
 
+/* lbm_fields into device arrays that belong to another stream (cudaStream_t): the read-out runs on
+ * the context's stream after the work queued on `stream` so far, and the work queued on `stream`
+ * next runs after it.  Does not synchronise. */
+lbm_status lbm_fields_on_stream(lbm_ctx* ctx, void* rho, void* vx, void* vy, void* stream);
+
 /* Checkpoint / resume.  lbm_save writes the state of an initialised context to `path`: a
  * header (magic "LBMGBCK1", format version, a hash of the configuration, lattice size,
  * precision, step count, lattice parity, M0), then the current lattice's populations as stored

@@ -60,6 +60,7 @@ _SIGS = {
     "lbm_step": (I32, [P, I64]),
     "lbm_prepare_steps": (I32, [P, I64]),
     "lbm_fields": (I32, [P, P, P, P, I32]),
+    "lbm_fields_on_stream": (I32, [P, P, P, P, P]),
     "lbm_populations": (I32, [P, P, I32]),
     "lbm_set_populations": (I32, [P, P, I32]),
     "lbm_mass": (I32, [P, C.POINTER(D), C.POINTER(D), C.POINTER(D)]),

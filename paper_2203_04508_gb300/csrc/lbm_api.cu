@@ -159,6 +159,7 @@ struct lbm_ctx {
   bool rho_ok = false;
   cudaStream_t side = nullptr;                      // second stream of the overlapped step
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  cudaEvent_t ev_user = nullptr;                    // orders a read-out with a stream of the caller's
   long long steps = 0;
   long long n_links = 0, n_bnodes = 0, n_s1 = 0, n_s2 = 0, n_fluid = 0;
   Lattice<float> Lf{};
@@ -1280,6 +1281,30 @@ void* mapped_host(void* p) {
   return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
 }
 
+}  // extern "C"
+
+namespace {
+
+// Queues the fields of the current state into device-writable arrays: from the planes the fused step
+// keeps (formed first for a new state) in one launch, or through the separate passes.  The arrays of
+// a pair of columns are written together where they are 8-byte aligned.
+cudaError_t queue_fields(lbm_ctx* c, void* r, void* u, void* v) {
+  if (fused(c) && (((uintptr_t)r | (uintptr_t)u | (uintptr_t)v) & 7) == 0) {
+    if (!c->rho_ok) {
+      cudaError_t e = launch_fused_prepare(fused_lattice(c, c->Lf, c->cur ^ 1), c->cur, c->stream);
+      if (e != cudaSuccess) return e;
+      c->rho_ok = true;
+    }
+    return launch_fused_fields(fused_lattice(c, c->Lf, c->cur), c->cur, (float*)r, (float*)u, (float*)v, c->stream);
+  }
+  if (c->fp64) return launch_fields(c->Ld, c->cur, (double*)r, (double*)u, (double*)v, c->stream);
+  return launch_fields(c->Lf, c->cur, (float*)r, (float*)u, (float*)v, c->stream);
+}
+
+}  // namespace
+
+extern "C" {
+
 lbm_status lbm_fields(lbm_ctx* c, void* rho, void* vx, void* vy, int32_t on_device) {
   LBM_RANGE("lbm_fields");
   if (!c || !c->inited) return LBM_ESTATE;
@@ -1287,30 +1312,41 @@ lbm_status lbm_fields(lbm_ctx* c, void* rho, void* vx, void* vy, int32_t on_devi
   if (!rho || !vx || !vy) return fail(c, LBM_EINVAL, "null output");
   const long long dn = (long long)c->cfg.nx * c->cfg.ny;
   const size_t sz = c->lay.sz;
-  if (!on_device) {
-    // page-locked host arrays: the read-out kernel writes them directly, no staging copies
-    void* hr = mapped_host(rho);
-    void* hu = mapped_host(vx);
-    void* hv = mapped_host(vy);
-    if (hr && hu && hv) {
-      if (c->fp64) CUDA_OK(c, launch_fields(c->Ld, c->cur, (double*)hr, (double*)hu, (double*)hv, c->stream));
-      else CUDA_OK(c, launch_fields(c->Lf, c->cur, (float*)hr, (float*)hu, (float*)hv, c->stream));
-      CUDA_OK(c, cudaStreamSynchronize(c->stream));
-      return LBM_OK;
-    }
+  if (on_device) {
+    CUDA_OK(c, queue_fields(c, rho, vx, vy));
+    return LBM_OK;
+  }
+  // page-locked host arrays: the read-out kernel writes them directly, no staging copies
+  void* hr = mapped_host(rho);
+  void* hu = mapped_host(vx);
+  void* hv = mapped_host(vy);
+  if (hr && hu && hv) {
+    CUDA_OK(c, queue_fields(c, hr, hu, hv));
+    CUDA_OK(c, cudaStreamSynchronize(c->stream));
+    return LBM_OK;
   }
   char* stage = stage_area(c);
-  char* r = on_device ? (char*)rho : stage;
-  char* u = on_device ? (char*)vx : stage + dn * sz;
-  char* v = on_device ? (char*)vy : stage + 2 * dn * sz;
-  if (c->fp64) CUDA_OK(c, launch_fields(c->Ld, c->cur, (double*)r, (double*)u, (double*)v, c->stream));
-  else CUDA_OK(c, launch_fields(c->Lf, c->cur, (float*)r, (float*)u, (float*)v, c->stream));
-  if (!on_device) {
-    CUDA_OK(c, cudaMemcpyAsync(rho, r, dn * sz, cudaMemcpyDeviceToHost, c->stream));
-    CUDA_OK(c, cudaMemcpyAsync(vx, u, dn * sz, cudaMemcpyDeviceToHost, c->stream));
-    CUDA_OK(c, cudaMemcpyAsync(vy, v, dn * sz, cudaMemcpyDeviceToHost, c->stream));
-    CUDA_OK(c, cudaStreamSynchronize(c->stream));
-  }
+  const size_t step = (dn * sz + 7) / 8 * 8;   // (three planes hold it: a plane's rows are padded, or a multiple of 128 bytes)
+  CUDA_OK(c, queue_fields(c, stage, stage + step, stage + 2 * step));
+  CUDA_OK(c, cudaMemcpyAsync(rho, stage, dn * sz, cudaMemcpyDeviceToHost, c->stream));
+  CUDA_OK(c, cudaMemcpyAsync(vx, stage + step, dn * sz, cudaMemcpyDeviceToHost, c->stream));
+  CUDA_OK(c, cudaMemcpyAsync(vy, stage + 2 * step, dn * sz, cudaMemcpyDeviceToHost, c->stream));
+  CUDA_OK(c, cudaStreamSynchronize(c->stream));
+  return LBM_OK;
+}
+
+lbm_status lbm_fields_on_stream(lbm_ctx* c, void* rho, void* vx, void* vy, void* stream) {
+  if (!c || !c->inited) return LBM_ESTATE;
+  if (c->sticky != LBM_OK) return c->sticky;
+  cudaStream_t s = (cudaStream_t)stream;
+  if (s == c->stream) return lbm_fields(c, rho, vx, vy, 1);
+  if (!c->ev_user) CUDA_OK(c, cudaEventCreateWithFlags(&c->ev_user, cudaEventDisableTiming));
+  CUDA_OK(c, cudaEventRecord(c->ev_user, s));
+  CUDA_OK(c, cudaStreamWaitEvent(c->stream, c->ev_user, 0));
+  lbm_status st = lbm_fields(c, rho, vx, vy, 1);
+  if (st != LBM_OK) return st;
+  CUDA_OK(c, cudaEventRecord(c->ev_user, c->stream));
+  CUDA_OK(c, cudaStreamWaitEvent(s, c->ev_user, 0));
   return LBM_OK;
 }
 
@@ -1641,7 +1677,8 @@ void lbm_destroy(lbm_ctx* c) {
   for (auto& g : c->graph)
     if (g) cudaGraphExecDestroy(g);
   for (auto& a : c->adj_graphs) cudaGraphExecDestroy(a.exec);
-  for (cudaEvent_t e : {c->ev_start, c->ev_rec[0], c->ev_rec[1], c->ev_rev[0], c->ev_rev[1], c->ev_fork, c->ev_join})
+  for (cudaEvent_t e : {c->ev_start, c->ev_rec[0], c->ev_rec[1], c->ev_rev[0], c->ev_rev[1], c->ev_fork, c->ev_join,
+                        c->ev_user})
     if (e) cudaEventDestroy(e);
   if (c->aux) cudaStreamDestroy(c->aux);
   if (c->side) cudaStreamDestroy(c->side);

@@ -881,6 +881,107 @@ __global__ void __launch_bounds__(SOLID_BLOCK) k_solids_batch(const Lattice<floa
   solids<false>(L, it.y, (8 * L.n_s2 + SOLID_BLOCK - 1) / SOLID_BLOCK, (L.n_s1 + SOLID_BLOCK - 1) / SOLID_BLOCK, steps);
 }
 
+// ---------------------------------------------------------------------------------------
+// Read-out of a state whose density (psi) plane is current, in one launch: density and v = u +
+// F/(2 rho) into dense nx x ny arrays (k_fields' values).  A block forms the chemical potentials its
+// rows' forces need from the staged density rows; the populations go straight to registers.
+constexpr int RO_H = 8, RO_W = 4;
+template <bool PSEUDO>
+__global__ void __launch_bounds__(32 * RO_W) k_fields_fused(const __grid_constant__ Lattice<float> L, int cur, int strips,
+                                                            float* __restrict__ rho_out, float* __restrict__ vx_out,
+                                                            float* __restrict__ vy_out) {
+  constexpr int MR = 2, RR = PSEUDO ? 1 : 4;   // chemical-potential and density rows beyond the outputs
+  __shared__ __align__(16) float2 s_rho[(RO_H + 2 * RR) * SP];
+  __shared__ __align__(16) float2 s_mu[PSEUDO ? 1 : (RO_H + 2 * MR) * SP];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int band = blockIdx.x / strips, strip = blockIdx.x - band * strips;
+  const int ya = band * RO_H, yb = min(ya + RO_H, L.ny);
+  const int x0 = strip * OUT, c = x0 - HX + 2 * lane;
+  const bool mine = lane >= HX / 2 && lane < 32 - HX / 2;
+  const int ca = wrap_col(c, L.nx), cb = wrap_col(c + 1, L.nx);
+  const float* __restrict__ rin = PSEUDO ? L.mu : L.rho;
+  auto row_at = [&](int r) {
+    if (L.walls) r = min(max(r, 0), L.ny - 1);
+    else r = r < 0 ? r + L.ny : (r >= L.ny ? r - L.ny : r);
+    return r * L.pitch;
+  };
+  int e[3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) e[j] = wrap_col(x0 - 2 * HX + lane + 32 * j, L.nx);
+  for (int r = ya - RR + warp; r < yb + RR; r += RO_W) {
+    float* const d = reinterpret_cast<float*>(s_rho + (r - ya + RR) * SP);
+    const float* const q = rin + row_at(r);
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      if (lane + 32 * j < 2 * SP) d[lane + 32 * j] = q[e[j]];
+  }
+  __syncthreads();
+  if (!PSEUDO) {
+    for (int m = ya - MR + warp; m < yb + MR; m += RO_W) {
+      const float2* q = s_rho + (m - ya + RR) * SP + HX / 2 + lane;
+      const float2 C = q[0], l = q[-1], g = q[1], u1 = q[SP], u2 = q[2 * SP], d1 = q[-SP], d2 = q[-2 * SP];
+      const float t = sub_rn(C.y, C.x);
+      const float2 x1 = make_float2(add_rn(t, sub_rn(l.y, C.x)), add_rn(sub_rn(g.x, C.y), -t));
+      const float2 lap = lap4_diff(x1, add_rn(sub_rn(C, g), sub_rn(C, l)), add_rn(sub_rn(u1, C), sub_rn(d1, C)),
+                                   add_rn(sub_rn(C, u2), sub_rn(C, d2)));
+      float2 mu = mu_of(L, psi_prime_shifted(L, C), lap);
+      const int n = row_at(m);
+      if (L.kind[n + ca] != KIND_FLUID) mu.x = L.mu[n + ca];
+      if (L.kind[n + cb] != KIND_FLUID) mu.y = L.mu[n + cb];
+      s_mu[(m - ya + MR) * SP + HX / 2 + lane] = mu;
+    }
+    __syncthreads();
+  }
+  for (int y = ya + warp; y < yb; y += RO_W) {
+    const int n = y * L.pitch;
+    const bool f0 = L.kind[n + ca] == KIND_FLUID, f1 = L.kind[n + cb] == KIND_FLUID;
+    float2 r = make_float2(0.f, 0.f), vx = r, vy = r;
+    if (f0 || f1) {
+      const float* __restrict__ f = L.f[cur] + n;
+      float2 v[9], drho, jx, jy, Fx, Fy;
+#pragma unroll
+      for (int i = 0; i < 9; ++i) v[i] = make_float2(f[i * (long long)L.plane + ca], f[i * (long long)L.plane + cb]);
+      moments(v, drho, jx, jy);
+      const float2 rho = add_rn(splat<float2>(L.rho_ref), drho);
+      const float2* q = s_rho + (y - ya + RR) * SP + HX / 2 + lane;
+      if constexpr (PSEUDO) {
+        const float2 C = q[0], U = q[SP], D = q[-SP];
+        float2 ax, ay;
+        pp_sums(make_float2(C.y, q[1].x), U, make_float2(q[-1].y, C.x), D, make_float2(U.y, q[SP + 1].x),
+                make_float2(q[SP - 1].y, U.x), make_float2(q[-SP - 1].y, D.x), make_float2(D.y, q[-SP + 1].x), ax, ay);
+        Fx = force_pp(rho, L.gx, C, ax);
+        Fy = force_pp(rho, L.gy, C, ay);
+      } else {
+        const float2* z = s_mu + (y - ya + MR) * SP + HX / 2 + lane;
+        auto dx_of = [](const float2* p) {
+          const float2 l = p[-1], C = p[0], g = p[1];
+          return fma_rn(splat<float2>(8.0f), make_float2(sub_rn(C.y, l.y), sub_rn(g.x, C.x)), sub_rn(l, g));
+        };
+        Fx = force_cp(rho, L.gx, dx_of(z), dx_of(q));
+        Fy = force_cp(rho, L.gy, diff4_of(z[SP], z[-SP], z[2 * SP], z[-2 * SP]), diff4_of(q[SP], q[-SP], q[2 * SP], q[-2 * SP]));
+      }
+      if (f0) { r.x = rho.x; vx.x = fmaf(0.5f, Fx.x, jx.x) / rho.x; vy.x = fmaf(0.5f, Fy.x, jy.x) / rho.x; }
+      if (f1) { r.y = rho.y; vx.y = fmaf(0.5f, Fx.y, jx.y) / rho.y; vy.y = fmaf(0.5f, Fy.y, jy.y) / rho.y; }
+    }
+    if (!mine || c >= L.nx) continue;
+    const long long d = (long long)y * L.nx + c;
+    if (c + 1 < L.nx && (d & 1) == 0) {
+      *reinterpret_cast<float2*>(rho_out + d) = r;
+      *reinterpret_cast<float2*>(vx_out + d) = vx;
+      *reinterpret_cast<float2*>(vy_out + d) = vy;
+    } else {
+      rho_out[d] = r.x;
+      vx_out[d] = vx.x;
+      vy_out[d] = vy.x;
+      if (c + 1 < L.nx) {
+        rho_out[d + 1] = r.y;
+        vx_out[d + 1] = vx.y;
+        vy_out[d + 1] = vy.y;
+      }
+    }
+  }
+}
+
 // A new state (set up, loaded or advanced by the separate passes) in lattice `cur`: the density
 // (psi) of its fluid nodes into rho_next, and of its boundary nodes into rho_b, from which k_solids
 // forms the solid layers.
@@ -1073,6 +1174,13 @@ cudaError_t launch_fused_batch_step(const FusedBatch& B, int cur, cudaStream_t s
                                             B.pass, cur);
   if (e == cudaSuccess && B.n_bc > 0) e = launch_after(k_bc_batch, B.n_bc, BC_BLOCK, 0, s, lat, B.bc, cur);
   return e == cudaSuccess ? launch_after(k_solids_batch, B.n_solid, SOLID_BLOCK, 0, s, lat, B.solid, 1) : e;
+}
+
+cudaError_t launch_fused_fields(const Lattice<float>& L, int cur, float* r, float* vx, float* vy, cudaStream_t s) {
+  const int strips = (L.nx + OUT - 1) / OUT, bands = (L.ny + RO_H - 1) / RO_H;
+  if (L.pseudo) k_fields_fused<true><<<strips * bands, 32 * RO_W, 0, s>>>(L, cur, strips, r, vx, vy);
+  else k_fields_fused<false><<<strips * bands, 32 * RO_W, 0, s>>>(L, cur, strips, r, vx, vy);
+  return cudaGetLastError();
 }
 
 int fused_launches(const Lattice<float>& L) { return 2 + (L.n_bnodes > 0 ? 1 : 0); }

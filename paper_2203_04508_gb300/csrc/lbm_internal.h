@@ -95,6 +95,8 @@ cudaError_t launch_fused_prepare(const Lattice<float>& L, int cur, cudaStream_t 
 // one step from lattice cur (L.rho_b, L.fx and L.fy set)
 cudaError_t launch_fused_step(const Lattice<float>& L, int cur, PassPlan plan, cudaStream_t s);
 int fused_launches(const Lattice<float>& L);
+// density and velocity of the state in lattice cur, whose density (psi) plane L names (L.rho or L.mu)
+cudaError_t launch_fused_fields(const Lattice<float>& L, int cur, float* r, float* vx, float* vy, cudaStream_t s);
 // a batch's fused step: every kernel over a flat list of all instances' items
 struct FusedBatch {
   const Lattice<float>* lat[2];   // the instances' descriptors by lattice parity

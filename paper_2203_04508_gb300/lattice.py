@@ -137,11 +137,11 @@ class Lattice:
             self._c(self.lib.lbm_fields(self.ctx, *[C.c_void_p(t.data_ptr()) for t in out], 0))
             return tuple(out)
         if on_device:
-            out = [torch.empty((self.ny, self.nx), dtype=self.tdtype, device="cuda") for _ in range(3)]
-            self.stream.wait_stream(torch.cuda.current_stream())
-            self._c(self.lib.lbm_fields(self.ctx, *[C.c_void_p(t.data_ptr()) for t in out], 1))
-            torch.cuda.current_stream().wait_stream(self.stream)
-            return tuple(out)
+            out = tuple(torch.empty((self.ny, self.nx), dtype=self.tdtype, device="cuda") for _ in range(3))
+            # queued after the current stream's work and before its next
+            self._c(self.lib.lbm_fields_on_stream(self.ctx, *[t.data_ptr() for t in out],
+                                                  torch.cuda.current_stream().cuda_stream))
+            return out
         out = [np.zeros((self.ny, self.nx), self.dtype) for _ in range(3)]
         self._c(self.lib.lbm_fields(self.ctx, *[o.ctypes.data for o in out], 0))
         return tuple(out)
