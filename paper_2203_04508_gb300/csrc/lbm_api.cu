@@ -180,7 +180,7 @@ struct lbm_ctx {
   int mu_kind = -1;                   // chemical-potential pass (-1: the precision's default)
   bool collide_set = false;           // lbm_set_collide_kernel was called
   bool fused_ok = false;              // the fused step's kernels can run on this device
-  PassPlan plan;                      // how the fused step's pass runs on this lattice
+  PassPlan plan, tile_plan;           // how the fused step's pass runs on this lattice; without the walk
   long long n_near = 0;               // entries of the near list, built where the fused density +
   bool near_built = false;            // mu pass is selected (lbm_build_links, lbm_set_mu_kernel)
   lbm_status sticky = LBM_OK;
@@ -194,6 +194,10 @@ struct lbm_ctx {
     cudaGraphExec_t exec;
   };
   std::vector<AdjGraph> adj_graphs;
+  // the (workspace, steps, spacing) of the last reverse sweep: a sweep is issued launch by launch the
+  // first time, and captured when it is repeated
+  const char* adj_ws = nullptr;
+  long long adj_n = 0, adj_every = 0;
   // second stream and events of the reverse sweep (created on its first use)
   cudaStream_t aux = nullptr;
   cudaEvent_t ev_start = nullptr, ev_rec[2] = {nullptr, nullptr}, ev_rev[2] = {nullptr, nullptr};
@@ -366,6 +370,7 @@ void fill_lattice(lbm_ctx* c, Lattice<real>& L) {
   L.fx = (real*)(w + y.psip);
   L.fy = (real*)(w + (c->cfg.force_model == LBM_FORCE_PSEUDO ? y.rho2 : y.mu2));
   L.rho_next = nullptr;
+  L.mu_out = nullptr;
   L.partials = (double*)(w + y.partials);
   L.counter = (unsigned int*)(w + y.counter);
   L.dM_ring = (double*)(w + y.dm_ring);
@@ -1081,6 +1086,7 @@ lbm_status lbm_build_links(lbm_ctx* c) {
                   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && fused_setup();
     if (!c->fused_ok) (void)cudaGetLastError();
     c->plan = fused_plan(g.nx, g.ny, sms);
+    c->tile_plan = fused_tile_plan(g.nx, g.ny, sms);
     // the list of nodes the combined density + mu pass leaves to k_mu_near, where that pass runs
     if (c->Lf.mu_kernel == 3 && !fused(c)) {
       lbm_status st = near_list(c);
@@ -2230,7 +2236,7 @@ namespace {
 // restore the forward state afterwards.
 struct AdjLayout {
   long long n, every, nseg;
-  size_t ckpt, ckcarry, seg, segrho, segmu, lam0, lam1, lam_bc, lrj, lamF, Lmu, Lrho, bct, ring, ctr, carry, grad;
+  size_t ckpt, ckcarry, seg, segrho, segmu, lam0, lam1, lam_bc, lrj, lamF, Lmu, Lrho, winv, dqdc, bct, ring, ctr, carry, grad;
   size_t state;   // bytes of one population lattice (9 planes)
   size_t total;
 };
@@ -2252,7 +2258,7 @@ AdjLayout make_adj_layout(const lbm_ctx* c, long long n, long long every) {
   A.ckcarry = take((size_t)A.nseg * (size_t)y.cap.bnodes * 8);
   // two sets of segment buffers: one is recomputed while the other is swept backwards
   A.seg = take(2 * (size_t)(every + 1) * A.state);
-  A.segrho = take(2 * (size_t)every * pl);
+  A.segrho = take(2 * (size_t)(every + 1) * pl);   // (the fused recomputation forms one more)
   A.segmu = take(2 * (size_t)every * pl);
   A.lam0 = take(9 * pl);
   A.lam1 = take(9 * pl);
@@ -2261,6 +2267,8 @@ AdjLayout make_adj_layout(const lbm_ctx* c, long long n, long long every) {
   A.lamF = take(2 * pl);
   A.Lmu = take(pl);
   A.Lrho = take(pl);
+  A.winv = take(c->fp64 ? 0 : pl);
+  A.dqdc = take(c->fp64 || c->cfg.n_cyl == 0 ? 0 : (size_t)y.cap.bnodes * 8 * 16);
   A.bct = take((size_t)y.plane);
   A.ring = take((size_t)(DM_RING + 1) * 8);
   A.ctr = take(16);
@@ -2362,6 +2370,11 @@ lbm_status adjoint(lbm_ctx* c, const Lattice<real>& L, const void* drho, const v
   B.lamF = w + A.lamF;
   B.Lmu = w + A.Lmu;
   B.Lrho = w + A.Lrho;
+  B.winv = w + A.winv;
+  if constexpr (sizeof(real) == 4) {
+    B.dqdc = (const double2*)(w + A.dqdc);
+    CUDA_OK(c, adj_geometry(L, (float*)(w + A.winv), (double2*)(w + A.dqdc), c->cfg.n_cyl, st));
+  }
   B.bct = (const uint8_t*)(w + A.bct);
   B.grad = (double*)(w + A.grad);
   B.n_cyl = c->cfg.n_cyl;
@@ -2375,17 +2388,19 @@ lbm_status adjoint(lbm_ctx* c, const Lattice<real>& L, const void* drho, const v
   }
   cudaStream_t aux = c->aux;
   auto seg_at = [&](int buf, long long i) { return w + A.seg + ((size_t)buf * (A.every + 1) + i) * A.state; };
-  auto rho_at = [&](int buf, long long i) { return w + A.segrho + ((size_t)buf * A.every + i) * pl; };
+  auto rho_at = [&](int buf, long long i) { return w + A.segrho + ((size_t)buf * (A.every + 1) + i) * pl; };
   auto mu_at = [&](int buf, long long i) { return w + A.segmu + ((size_t)buf * A.every + i) * pl; };
   auto seg_len = [&](long long s) { return s + 1 < A.nseg ? A.every : A.n - s * A.every; };
-  // the chemical potential of the solid layers is constant: every step's plane starts as a
-  // copy of the lattice's own plane, whose fluid values the recomputation overwrites
-  for (int buf = 0; buf < 2; ++buf)
+  // The recomputation runs the fused step where there is one (whose lattice runs it), which
+  // leaves each step's density and chemical potential in its planes; otherwise the separate passes,
+  // whose chemical potential leaves the solid layers' constant one alone: every step's plane starts
+  // as a copy of the lattice's own.
+  const bool fused_re = fused(c);
+  for (int buf = 0; buf < 2 && !fused_re; ++buf)
     for (long long i = 0; i < A.every; ++i)
       CUDA_OK(c, cudaMemcpyAsync(mu_at(buf, i), L.mu, pl, cudaMemcpyDeviceToDevice, st));
   CUDA_OK(c, cudaMemsetAsync(w + A.Lrho, 0, pl, st));
 
-  // the graphs the sweep needs, captured before any of them runs
   auto find = [&](int kind, int buf, long long k, int par) -> cudaGraphExec_t {
     for (auto& a : c->adj_graphs)
       if (a.ws == w && a.n == A.n && a.every == A.every && a.kind == kind && a.buf == buf && a.k == k &&
@@ -2393,10 +2408,8 @@ lbm_status adjoint(lbm_ctx* c, const Lattice<real>& L, const void* drho, const v
         return a.exec;
     return nullptr;
   };
-  auto capture = [&](int kind, int buf, long long k, int par) -> lbm_status {
-    if (find(kind, buf, k, par)) return LBM_OK;
-    cudaGraph_t gr;
-    CUDA_OK(c, cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+  // one segment's recomputation (kind 0) or reverse steps (kind 1) on stream q
+  auto issue = [&](int kind, int buf, long long k, int par, cudaStream_t q) -> cudaError_t {
     cudaError_t e = cudaSuccess;
     Lattice<real> Lc = L;
     auto at = [&](long long i) {
@@ -2404,13 +2417,28 @@ lbm_status adjoint(lbm_ctx* c, const Lattice<real>& L, const void* drho, const v
       Lc.f[1] = (real*)seg_at(buf, i + 1);
       Lc.rho = (real*)rho_at(buf, i);
       Lc.mu = (real*)mu_at(buf, i);
-      Lc.psip = nullptr;   // the recomputation evaluates psi' in its own chemical-potential pass
+      Lc.psip = nullptr;   // the separate passes' recomputation evaluates psi' with mu
     };
     if (kind == 0) {
       // the segment's states (and each step's rho, mu) from slot 0
       for (long long i = 0; i < k && e == cudaSuccess; ++i) {
         at(i);
-        e = launch_step(Lc, 0, st);
+        if constexpr (sizeof(real) == 4) {
+          if (fused_re) {
+            Lattice<float> F = Lc;
+            F.mu = L.mu;   // the walls'
+            F.rho_b = (float*)(c->ws + c->lay.rhob);
+            if (i == 0) {
+              F.rho_next = F.rho;
+              e = launch_fused_prepare(F, 0, q);
+            }
+            F.rho_next = (float*)rho_at(buf, i + 1);
+            F.mu_out = (float*)mu_at(buf, i);
+            if (e == cudaSuccess) e = launch_fused_step(F, 0, c->tile_plan, q);
+            continue;
+          }
+        }
+        e = launch_step(Lc, 0, q);
       }
     } else {
       // its reverse steps: step i reads f^i from slot i and the values its links used from
@@ -2421,10 +2449,18 @@ lbm_status adjoint(lbm_ctx* c, const Lattice<real>& L, const void* drho, const v
         AdjBuffers Bi = B;
         Bi.lam_in = lam[pp];
         Bi.lam_out = lam[pp ^ 1];
-        e = adj_step(Lc, Bi, st);
+        Bi.first = i == k - 1;
+        e = adj_step(Lc, Bi, q);
         pp ^= 1;
       }
     }
+    return e;
+  };
+  auto capture = [&](int kind, int buf, long long k, int par) -> lbm_status {
+    if (find(kind, buf, k, par)) return LBM_OK;
+    cudaGraph_t gr;
+    CUDA_OK(c, cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
+    cudaError_t e = issue(kind, buf, k, par, st);
     cudaError_t e2 = cudaStreamEndCapture(st, &gr);
     if (e != cudaSuccess || e2 != cudaSuccess)
       return fail(c, LBM_ECUDA, "reverse-sweep capture failed: %s", cudaGetErrorString(e != cudaSuccess ? e : e2));
@@ -2435,7 +2471,14 @@ lbm_status adjoint(lbm_ctx* c, const Lattice<real>& L, const void* drho, const v
     c->adj_graphs.push_back({w, A.n, A.every, k, kind, buf, par, g});
     return LBM_OK;
   };
-  {
+  // a repeated sweep replays graphs, captured before any of them runs; the first is issued launch by
+  // launch (capturing and instantiating costs more host time than issuing once)
+  const bool again = !st || (c->adj_ws == w && c->adj_n == A.n && c->adj_every == A.every);   // (the default
+                                                                       // stream takes no capture: refused)
+  c->adj_ws = w;
+  c->adj_n = A.n;
+  c->adj_every = A.every;
+  if (again) {
     int p = 0;
     for (long long s = A.nseg - 1; s >= 0; --s) {
       const long long k = seg_len(s);
@@ -2446,6 +2489,10 @@ lbm_status adjoint(lbm_ctx* c, const Lattice<real>& L, const void* drho, const v
       p ^= (int)(k & 1);
     }
   }
+  auto run = [&](int kind, int buf, long long k, int par, cudaStream_t q) -> cudaError_t {
+    cudaGraphExec_t g = find(kind, buf, k, par);
+    return g ? cudaGraphLaunch(g, q) : issue(kind, buf, k, par, q);
+  };
   // recomputation of segment s into buffer set s & 1, on the second stream
   auto recompute = [&](long long s) -> lbm_status {
     const int buf = (int)(s & 1);
@@ -2453,7 +2500,7 @@ lbm_status adjoint(lbm_ctx* c, const Lattice<real>& L, const void* drho, const v
     if (c->n_bnodes > 0)
       CUDA_OK(c, cudaMemcpyAsync(L.carry, w + A.ckcarry + s * (size_t)y.cap.bnodes * 8, (size_t)c->n_bnodes * 8,
                                  cudaMemcpyDeviceToDevice, aux));
-    CUDA_OK(c, cudaGraphLaunch(find(0, buf, seg_len(s), 0), aux));
+    CUDA_OK(c, run(0, buf, seg_len(s), 0, aux));
     CUDA_OK(c, cudaEventRecord(c->ev_rec[buf], aux));
     return LBM_OK;
   };
@@ -2472,7 +2519,7 @@ lbm_status adjoint(lbm_ctx* c, const Lattice<real>& L, const void* drho, const v
       if (rs != LBM_OK) return rs;
     }
     CUDA_OK(c, cudaStreamWaitEvent(st, c->ev_rec[buf], 0));
-    CUDA_OK(c, cudaGraphLaunch(find(1, buf, k, p), st));
+    CUDA_OK(c, run(1, buf, k, p, st));
     CUDA_OK(c, cudaEventRecord(c->ev_rev[buf], st));
     p ^= (int)(k & 1);
   }

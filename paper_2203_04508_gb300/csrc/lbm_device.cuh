@@ -40,6 +40,7 @@ struct Lattice {
                                 // boundary node's final populations here (one per node)
   real* mu;                     // chemical potential minus k^2 mu_sat (constant at solids)
   real* rho_next;               // fused step (FP32): the next state's density (psi) plane
+  real* mu_out;                 // ... if set (tiles): this state's chemical potential is kept here
   real* fx;                     // fused step (FP32): the force at nodes next to solids, left by
   real* fy;                     // the pass for the boundary phase
   real* psip;                   // if set: psi'(rho) - mu_sat of every fluid node, left by the

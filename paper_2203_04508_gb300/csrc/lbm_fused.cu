@@ -560,7 +560,13 @@ __device__ __forceinline__ void tile(const Lattice<float>& L, int cur, int strip
       const float2 lap = lap4_diff(x1, add_rn(sub_rn(C, g), sub_rn(C, l)), add_rn(sub_rn(u1, C), sub_rn(d1, C)),
                                    add_rn(sub_rn(C, u2), sub_rn(C, d2)));
       const float2 mu = mu_of(L, psi_prime_shifted(L, C), lap);
-      *mu_row(m) = make_float2(fl[k] & 1u ? mu.x : wall[k].x, fl[k] & 2u ? mu.y : wall[k].y);
+      const float2 v = make_float2(fl[k] & 1u ? mu.x : wall[k].x, fl[k] & 2u ? mu.y : wall[k].y);
+      *mu_row(m) = v;
+      if (L.mu_out && m >= ya && m < yb) {
+        float* p = L.mu_out + m * L.pitch + c;
+        if (out1) *reinterpret_cast<float2*>(p) = v;
+        else if (one) *p = v.x;
+      }
     }
     __syncthreads();
   }
@@ -1065,6 +1071,15 @@ PassPlan fused_plan(int nx, int ny, int sms) {
   const long long least = (ny + most - 1) / most, per_sm = (strips * least + sms - 1) / sms;
   const long long bands = std::max(least, per_sm * sms / strips);
   p.rows = std::max((int)((ny + bands - 1) / bands), MIN_TILE_ROWS);
+  return p;
+}
+
+// the same without the walk (whose kernel keeps no chemical potential)
+PassPlan fused_tile_plan(int nx, int ny, int sms) {
+  PassPlan p = fused_plan(nx, ny, sms);
+  if (p.kind != PassPlan::WALK) return p;
+  p.kind = PassPlan::TILE_L;
+  p.rows = TH_L;
   return p;
 }
 

@@ -90,6 +90,7 @@ struct PassPlan {
   int rows = 0;
 };
 PassPlan fused_plan(int nx, int ny, int sms);
+PassPlan fused_tile_plan(int nx, int ny, int sms);
 // the solid layers of a new state in lattice cur, where the fused step expects them
 cudaError_t launch_fused_prepare(const Lattice<float>& L, int cur, cudaStream_t s);
 // one step from lattice cur (L.rho_b, L.fx and L.fy set)
@@ -216,6 +217,9 @@ struct AdjBuffers {
   void* lamF;           // 2 planes: dJ/dF (zero off the fluid)
   void* Lmu;            // dJ/dmu
   void* Lrho;           // dJ/drho (the density plane); between steps the density share of lambda
+  bool first;           // FP32: the step follows work other than a reverse step: nothing of it starts early
+  const void* winv;     // FP32: 1 / sum of Eq. 15's weights at second-layer nodes, by node
+  const double2* dqdc;  // FP32: dq/dc of the link of boundary node b in direction i at (i - 1) bcap + b
   const uint8_t* bct;   // per node: bit 0 lam_bc may be non-zero, bit 1 boundary node
   double* grad;         // dJ/d dmu per cylinder, dJ/d dmu of the walls, dJ/d(cx, cy) per cylinder
   int n_cyl;
@@ -223,6 +227,8 @@ struct AdjBuffers {
 // blocks of the objective's reduction over a plane of `plane` nodes (at most one per 256
 // nodes): it leaves 4 partial sums per block in `red`
 unsigned objective_blocks(long long plane);
+// FP32: winv and dqdc of a sweep
+cudaError_t adj_geometry(const Lattice<float>& L, float* winv, double2* dqdc, int n_cyl, cudaStream_t s);
 template <typename real> cudaError_t adj_flags(const Lattice<real>& L, uint8_t* bct, cudaStream_t s);
 template <typename real>
 cudaError_t objective_sums(const Lattice<real>& L, int cur, int body, uint8_t* touch, double* red, double rg,
