@@ -23,6 +23,7 @@ UNITS = [
     ("lbm_api.cu", []),
     ("lbm_step.cu", []),
     ("lbm_fused.cu", []),
+    ("lbm_fp64.cu", []),
     ("lbm_geometry.cu", ["-fmad=false"]),
     ("lbm_eos.cpp", ["-x", "cu"]),
     ("lbm_noalloc.cu", []),

@@ -19,16 +19,13 @@
 // populations), is not added to the nine planes: lambda^t is kept as (nine planes, Lrho) and the
 // next reverse step adds Lrho where it reads lambda.  The forward quantities of step t (rho,
 // solid rho, mu) are those the recomputation of the segment stored for that step.
+#include "lbm_fused.cuh"
 #include "lbm_internal.h"
 #include "lbm_phases.cuh"
 
 namespace lbmgb {
 
 constexpr int ADJ_BLOCK = 256;
-
-// programmatic dependent launch (see the fused step)
-__device__ __forceinline__ void adj_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void adj_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename real>
 __device__ __forceinline__ bool is_field_node(uint8_t k) {
@@ -423,8 +420,8 @@ __global__ void __launch_bounds__(AL_BLOCK) k_adj_links(const __grid_constant__ 
     dc[i - 1] = bd[i - 1] >= 0 && bd[i - 1] < A.n_cyl ? A.dqdc[(i - 1) * (long long)L.bcap + b] : make_double2(0.0, 0.0);
   }
   if (live) node_state(L, x, y, f, r, drho, jx, jy, Fx, Fy);
-  adj_wait();
-  adj_launch();
+  grid_wait();
+  grid_launch();
   if (!live) return;
   const float* lin = static_cast<const float*>(A.lam_in);
   const float lrn = static_cast<const float*>(A.Lrho)[n];   // density share of lambda^{t+1} at x1
@@ -526,8 +523,8 @@ __global__ void __launch_bounds__(AC_BLOCK) k_adj_nodes(const __grid_constant__ 
     }
     node_state(L, x, y, f, r, drho, jx, jy, Fx, Fy);
   }
-  adj_wait();
-  adj_launch();
+  grid_wait();
+  grid_launch();
   if (!live) return;
   const float* lin = static_cast<const float*>(A.lam_in);
   const float* lrp = static_cast<const float*>(A.Lrho);   // density share of lambda^{t+1}
@@ -605,8 +602,8 @@ __global__ void __launch_bounds__(AT_THREADS) k_adj_fields(const __grid_constant
     if (kd == KIND_FLUID) fluid |= 1u << k;
     if (r >= 2 && r < AT_FR - 2 && in) S.mu[r - 2][c] = L.mu[row(y) + xw];
   }
-  adj_wait();
-  adj_launch();
+  grid_wait();
+  grid_launch();
   const float* lF = static_cast<const float*>(A.lamF);
   float* Lrho = static_cast<float*>(A.Lrho);
 #pragma unroll
@@ -701,8 +698,8 @@ __global__ void __launch_bounds__(ADJ_BLOCK) k_adj_layers(const __grid_constant_
       }
     }
   }
-  adj_wait();
-  adj_launch();
+  grid_wait();
+  grid_launch();
   if (j >= L.n_s1) return;
   float v = Lrho[n];
 #pragma unroll
@@ -886,21 +883,6 @@ cudaError_t adj_export(const Lattice<real>& L, const real* lam, const real* Lrho
   return cudaGetLastError();
 }
 
-// a launch that may overlap the end of the one before it in the stream, if `early`
-template <typename... P, typename... A>
-static cudaError_t launch_after(void (*k)(P...), dim3 grid, int block, bool early, cudaStream_t s, A... args) {
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t c{};
-  c.gridDim = grid;
-  c.blockDim = dim3((unsigned)block);
-  c.stream = s;
-  c.attrs = &at;
-  c.numAttrs = early && s ? 1 : 0;
-  return cudaLaunchKernelEx(&c, k, P(args)...);
-}
-
 cudaError_t adj_geometry(const Lattice<float>& L, float* winv, double2* dqdc, int n_cyl, cudaStream_t s) {
   const int n = L.n_s2 > L.n_bnodes ? L.n_s2 : L.n_bnodes;
   if (n > 0) k_adj_geometry<<<list_grid(n), ADJ_BLOCK, 0, s>>>(L, winv, dqdc, n_cyl);
@@ -914,13 +896,19 @@ cudaError_t adj_step(const Lattice<real>& L, const AdjBuffers& A, cudaStream_t s
   if constexpr (sizeof(real) == 4) {
     cudaError_t e = cudaSuccess;
     const auto blocks = [](int n, int per) { return dim3((unsigned)((n + per - 1) / per)); };
-    if (L.n_bnodes > 0) e = launch_after(k_adj_links, blocks(L.n_bnodes, AL_BLOCK), AL_BLOCK, !A.first, s, L, A);
+    bool first = A.first;   // the step's first kernel follows other work: an ordinary launch
+    if (L.n_bnodes > 0) {
+      if (first) k_adj_links<<<blocks(L.n_bnodes, AL_BLOCK), AL_BLOCK, 0, s>>>(L, A);
+      else e = launch_after(k_adj_links, blocks(L.n_bnodes, AL_BLOCK), AL_BLOCK, 0, s, L, A);
+      first = false;
+    }
     const dim3 nodes((unsigned)((L.nx + AC_BLOCK - 1) / AC_BLOCK), (unsigned)L.ny);
-    if (e == cudaSuccess) e = launch_after(k_adj_nodes, nodes, AC_BLOCK, !A.first || L.n_bnodes > 0, s, L, A);
+    if (first) k_adj_nodes<<<nodes, AC_BLOCK, 0, s>>>(L, A);
+    else if (e == cudaSuccess) e = launch_after(k_adj_nodes, nodes, AC_BLOCK, 0, s, L, A);
     const int strips = (L.nx + AT_OUT - 1) / AT_OUT, bands = (L.ny + AT_H - 1) / AT_H;
-    if (e == cudaSuccess) e = launch_after(k_adj_fields, dim3((unsigned)(strips * bands)), AT_THREADS, true, s, L, A, strips);
-    if (e == cudaSuccess && L.n_s1 > 0) e = launch_after(k_adj_layers, blocks(L.n_s1, ADJ_BLOCK), ADJ_BLOCK, true, s, L, A);
-    return e;
+    if (e == cudaSuccess) e = launch_after(k_adj_fields, dim3((unsigned)(strips * bands)), AT_THREADS, 0, s, L, A, strips);
+    if (e == cudaSuccess && L.n_s1 > 0) e = launch_after(k_adj_layers, blocks(L.n_s1, ADJ_BLOCK), ADJ_BLOCK, 0, s, L, A);
+    return e == cudaSuccess ? cudaGetLastError() : e;
   } else {
     if (L.n_bnodes > 0) k_adj_bc<real><<<list_grid(L.n_bnodes), ADJ_BLOCK, 0, s>>>(L, A);
     k_adj_collide<real><<<adj_grid(L), ADJ_BLOCK, 0, s>>>(L, A);

@@ -101,10 +101,9 @@ Layout make_layout(const lbm_config* c) {
   L.lx2f = take(L.cap.links);
   L.bnode = take(L.cap.bnodes * 4);
   L.bstart = take((L.cap.bnodes + 1) * 4);
-  const bool by_node = L.sz == 4;        // the fused step's links by boundary node
-  L.bnd = take(by_node ? L.cap.bnodes * 8 : 0);
-  L.bmask = take(by_node ? L.cap.bnodes * 2 : 0);
-  L.bq = take(by_node ? L.cap.bnodes * 8 * L.sz : 0);
+  L.bnd = take(L.cap.bnodes * 8);        // the links by boundary node (fused and FP64 steps)
+  L.bmask = take(L.cap.bnodes * 2);
+  L.bq = take(L.cap.bnodes * 8 * L.sz);
   L.carry = take(L.cap.bnodes * 8);
   L.rhob = take(L.cap.bnodes * L.sz);
   L.bmom = take(aa ? 3 * L.cap.bnodes * L.sz : 0);
@@ -457,6 +456,14 @@ bool fused(const lbm_ctx* c) {
          c->mu_kind < 0 && !c->collide_set;
 }
 
+// The FP64 step (lbm_fp64.cu) is the default of FP64 lattices with two population lattices, the
+// chemical-potential force and an equation of state, whole and not slabs; a caller that names a
+// chemical-potential pass or a collide kernel gets the separate passes.  Both leave the same planes.
+bool step64(const lbm_ctx* c) {
+  return c->fp64 && c->cfg.layout == LBM_LAYOUT_AB && c->cfg.eos != LBM_EOS_NONE &&
+         c->cfg.force_model == LBM_FORCE_CHEMPOT && !c->slab.on && c->mu_kind < 0 && !c->collide_set;
+}
+
 // From the fused step to the separate passes: those start from the density planes, and find the
 // walls' chemical potential in the second mu plane too, which the fused step keeps forces in.
 cudaError_t leave_fused(lbm_ctx* c) {
@@ -505,6 +512,9 @@ cudaError_t issue_step(lbm_ctx* c, const Lattice<real>& L, int cur) {
   }
   Lattice<real> Lt, Ln;
   step_lattices(c, L, cur, Lt, Ln);
+  if constexpr (sizeof(real) == 8) {
+    if (step64(c)) return launch_fp64_step(Lt, Ln.rho, cur, c->stream);
+  }
   return launch_step_overlap(Lt, Ln, cur, c->stream, c->side, c->ev_fork, c->ev_join);
 }
 
@@ -1031,10 +1041,8 @@ lbm_status lbm_build_links(lbm_ctx* c) {
   o.kind = (uint8_t*)(w + y.kind);
   o.bnode = (int*)(w + y.bnode); o.bstart = (int*)(w + y.bstart); o.ldir = (uint8_t*)(w + y.ldir);
   o.lq64 = (double*)(w + y.lq64); o.lx2f = (uint8_t*)(w + y.lx2f); o.lq = w + y.lq;
-  if (!c->fp64) {
-    o.bnd = (int2*)(w + y.bnd); o.bmask = (unsigned short*)(w + y.bmask); o.bq = w + y.bq;
-    o.bcap = (int)y.cap.bnodes;
-  }
+  o.bnd = (int2*)(w + y.bnd); o.bmask = (unsigned short*)(w + y.bmask); o.bq = w + y.bq;
+  o.bcap = (int)y.cap.bnodes;
   o.s1node = (int*)(w + y.s1node); o.s1mask = (uint8_t*)(w + y.s1mask); o.s1winv = w + y.s1winv;
   o.s1nb = (int*)(w + y.s1nb);
   o.s2node = (int*)(w + y.s2node); o.s2mask = (uint8_t*)(w + y.s2mask); o.s2winv = w + y.s2winv;
@@ -1273,7 +1281,7 @@ lbm_status lbm_get_collide_kernel(lbm_ctx* c, int32_t* kind) {
 
 lbm_status lbm_launches_per_step(lbm_ctx* c, int64_t* n) {
   if (!c || !c->built || !n) return LBM_ESTATE;
-  *n = fused(c) ? fused_launches(c->Lf) : c->fp64 ? launches_per_step_overlap(c->Ld) : launches_per_step_overlap(c->Lf);
+  *n = fused(c) ? fused_launches(c->Lf) : step64(c) ? launches_fp64(c->Ld) : c->fp64 ? launches_per_step_overlap(c->Ld) : launches_per_step_overlap(c->Lf);
   return LBM_OK;
 }
 
@@ -1302,6 +1310,13 @@ cudaError_t queue_fields(lbm_ctx* c, void* r, void* u, void* v) {
       c->rho_ok = true;
     }
     return launch_fused_fields(fused_lattice(c, c->Lf, c->cur), c->cur, (float*)r, (float*)u, (float*)v, c->stream);
+  }
+  if (step64(c) && c->rho_ok) {
+    // the planes of the current state are complete but for its chemical potential
+    Lattice<double> Lt, Ln;
+    step_lattices(c, c->Ld, c->cur, Lt, Ln);
+    cudaError_t e = launch_fp64_mu(Lt, c->stream);
+    return e == cudaSuccess ? launch_fields_of(Lt, c->cur, (double*)r, (double*)u, (double*)v, c->stream) : e;
   }
   if (c->fp64) return launch_fields(c->Ld, c->cur, (double*)r, (double*)u, (double*)v, c->stream);
   return launch_fields(c->Lf, c->cur, (float*)r, (float*)u, (float*)v, c->stream);

@@ -71,12 +71,6 @@ __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_grou
 template <int N>
 __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
 
-// Programmatic dependent launch: a kernel of the step may start while the one before it still runs
-// (grid_launch there), and reads or writes nothing that one touches before grid_wait, which waits
-// for it to finish.
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // column c of a lattice of nx columns, wrapped (c within one lattice of the range, or clamped)
 __device__ __forceinline__ int wrap_col(int c, int nx) {
   c %= nx;
@@ -699,87 +693,10 @@ __global__ void __launch_bounds__(32 * W, MINB) k_tile_batch(const Lattice<float
   tile<false, H, W>(L, cur, it.y, it.z, it.z + it.w, smem);
 }
 
-// Cut links of one boundary node a thread (phase_bc's arithmetic, the force from the planes the
-// pass left).  Latency is all it costs, so the loads make two rounds: the node's record -- set up
-// with the geometry, and fetched before the pass it depends on has finished -- then everything
-// else at once.  The node's own populations stay in registers for its density.  Leaves one
-// compensation sum per warp; k_solids adds them up.
 constexpr int BC_BLOCK = 64;
 template <bool PSEUDO>
-__device__ __forceinline__ void links(const Lattice<float>& L, int cur, int b) {
-  const bool live = b < L.n_bnodes;
-  const int2 nd = live ? L.bnd[b] : make_int2(0, 0);
-  const unsigned mask = live ? L.bmask[b] : 0u;
-  float q[8];
-#pragma unroll
-  for (int i = 1; i < 9; ++i) q[i - 1] = mask & (1u << (i - 1)) ? L.bq[(i - 1) * (long long)L.bcap + b] : 0.f;
-  grid_wait();
-  grid_launch();
-  double sum = 0.0;
-  if (live) {
-    const int n = nd.x, x = nd.y;
-    float* fout = L.f[cur ^ 1];
-    const float* __restrict__ fin = L.f[cur];
-    // offsets to the neighbours (periodic in x, and in y without walls)
-    const int xm = x == 0 ? L.nx - 1 : -1, xp = x == L.nx - 1 ? 1 - L.nx : 1;
-    const int ym = !L.walls && n < L.pitch ? L.plane - L.pitch : -L.pitch;
-    const int yp = !L.walls && n >= L.plane - L.pitch ? L.pitch - L.plane : L.pitch;
-    auto nb = [&](int dx, int dy) { return n + (dx < 0 ? xm : dx > 0 ? xp : 0) + (dy < 0 ? ym : dy > 0 ? yp : 0); };
-    float g[9], fl[9], a[8], cc[8];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) g[i] = fout[i * L.plane + n];
-#pragma unroll
-    for (int i = 0; i < 9; ++i) fl[i] = fin[i * L.plane + n];
-    const float Fx = L.fx[n], Fy = L.fy[n];
-    const double carry = L.carry[b];
-#pragma unroll
-    for (int i = 1; i < 9; ++i) {
-      a[i - 1] = cc[i - 1] = 0.f;
-      if (mask & (1u << (i - 1))) {
-        a[i - 1] = fout[i * L.plane + nb(ex(i), ey(i))];
-        cc[i - 1] = fout[opp(i) * L.plane + nb(-ex(i), -ey(i))];
-      }
-    }
-    float drho, jx, jy;
-    moments(fl, drho, jx, jy);
-    const float r = L.rho_ref + drho;
-    const float inv_r = 1.0f / r;
-    const float ux = jx * inv_r, uy = jy * inv_r, dux = Fx * inv_r, duy = Fy * inv_r;
-    float v[8];
-#pragma unroll
-    for (int i = 1; i < 9; ++i) {
-      if (!(mask & (1u << (i - 1)))) continue;
-      const float Fi = edm_term<float>(i, r, ux, uy, dux, duy);
-      v[i - 1] = link_rule<float>(L.bc, q[i - 1], (mask >> (i + 7)) & 1u, a[i - 1], g[i], cc[i - 1], Fi);
-      sum += (double)a[i - 1] - (double)v[i - 1];
-    }
-    // (no link reads a slot another link of the node writes: b2 counts only where x2 is fluid)
-#pragma unroll
-    for (int i = 1; i < 9; ++i) {
-      if (!(mask & (1u << (i - 1)))) continue;
-      g[opp(i)] = v[i - 1];
-      fout[opp(i) * L.plane + n] = v[i - 1];
-    }
-    if (L.bc == BC_PRESENT || L.bc == BC_MIBC) {
-      const double t = (double)g[0] + sum + carry;
-      g[0] = (float)t;
-      L.carry[b] = t - (double)g[0];
-      fout[n] = g[0];
-    } else {
-      sum = 0.0;
-    }
-    const float rn = density_of(L, g);
-    L.rho_b[b] = rn;
-    L.rho_next[n] = PSEUDO ? psi_of(L, rn) : rn;
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
-  if ((threadIdx.x & 31) == 0) L.partials[b >> 5] = sum;
-}
-
-template <bool PSEUDO>
 __global__ void __launch_bounds__(BC_BLOCK) k_bc_fused(const __grid_constant__ Lattice<float> L, int cur) {
-  links<PSEUDO>(L, cur, blockIdx.x * BC_BLOCK + threadIdx.x);
+  links<PSEUDO, true>(L, cur, blockIdx.x * BC_BLOCK + threadIdx.x);
 }
 // item: (instance, first boundary node)
 __global__ void __launch_bounds__(BC_BLOCK) k_bc_batch(const Lattice<float>* lat, const int2* items, int cur) {
@@ -787,96 +704,14 @@ __global__ void __launch_bounds__(BC_BLOCK) k_bc_batch(const Lattice<float>* lat
   const int2 it = items[blockIdx.x];
   take_lattice(L, lat, it.x);
   __syncthreads();
-  links<false>(L, cur, it.y + threadIdx.x);
+  links<false, true>(L, cur, it.y + threadIdx.x);
 }
 
-// Both solid layers from the boundary nodes' densities in rho_b (every fluid neighbour of a
-// first-layer node is a boundary node), into the density plane (psi with the wall factor into the
-// psi plane).  A second-layer node forms its first-layer neighbours' densities again, one a lane of
-// its eight lanes, and adds them in phase_solid's order.  The last block adds the links'
-// compensation sums in the order of k_bc's two-level sum, and steps the counter; steps == 0 leaves
-// that out (the layers of a new state).
 constexpr int SOLID_BLOCK = 256;
-template <bool PSEUDO>
-__device__ __forceinline__ void solids(const Lattice<float>& L, int blk, int blocks2, int blocks1, int steps) {
-  __shared__ double red[32];
-  auto first = [&](unsigned m, float winv, const int (&nb)[8]) {
-    float acc = 0.f;
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-      if (m & (1u << i)) acc = fma_rn((float)wgt(i + 1), L.rho_b[nb[i]], acc);
-    return acc * winv;
-  };
-  auto record = [&](int k, unsigned& m, float& winv, int (&nb)[8]) {
-    m = L.s1mask[k];
-    winv = L.s1winv[k];
-    const int4 u = *reinterpret_cast<const int4*>(L.s1nb + 8 * k), w = *reinterpret_cast<const int4*>(L.s1nb + 8 * k + 4);
-    nb[0] = u.x; nb[1] = u.y; nb[2] = u.z; nb[3] = u.w;
-    nb[4] = w.x; nb[5] = w.y; nb[6] = w.z; nb[7] = w.w;
-  };
-  if (blk < blocks2) {
-    const int t = blk * SOLID_BLOCK + threadIdx.x, k = t >> 3, lane = t & 7;
-    unsigned m2 = 0, m = 0;
-    float winv2 = 0.f, winv = 0.f;
-    int nb[8], n = 0;
-    if (k < L.n_s2) {
-      m2 = L.s2mask[k];
-      winv2 = L.s2winv[k];
-      n = L.s2node[k];
-      if (m2 & (1u << lane)) record(L.s2nb[8 * k + lane], m, winv, nb);
-    }
-    grid_wait();
-    grid_launch();
-    const float v = first(m, winv, nb);
-    float acc = 0.f;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float vi = __shfl_sync(0xffffffffu, v, i, 8);
-      if (m2 & (1u << i)) acc = fma_rn((float)wgt(i + 1), vi, acc);
-    }
-    const float rs = acc * winv2;
-    if (k < L.n_s2 && lane == 0) L.rho_next[n] = PSEUDO ? psi_wall(L, n, rs) : rs;
-  } else if (blk < blocks2 + blocks1) {
-    const int k = (blk - blocks2) * SOLID_BLOCK + threadIdx.x;
-    unsigned m = 0;
-    float winv = 0.f;
-    int nb[8], n = 0;
-    if (k < L.n_s1) {
-      n = L.s1node[k];
-      record(k, m, winv, nb);
-    }
-    grid_wait();
-    grid_launch();
-    const float rs = first(m, winv, nb);
-    if (k < L.n_s1) L.rho_next[n] = PSEUDO ? psi_wall(L, n, rs) : rs;
-  } else {
-    grid_wait();
-    grid_launch();
-    if (steps) {
-      // k_bc's blocks of eight warps: their warps' sums in block_sum's tree, then the blocks'
-      const int warps = (L.n_bnodes + 31) / 32, chunks = (warps + 7) / 8;
-      double v = 0.0;
-      for (int k = threadIdx.x; k < chunks; k += SOLID_BLOCK) {
-        double w[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) w[j] = 8 * k + j < warps ? L.partials[8 * k + j] : 0.0;
-        v += ((w[0] + w[4]) + (w[2] + w[6])) + ((w[1] + w[5]) + (w[3] + w[7]));
-      }
-      const double total = block_sum(v, red);
-      if (threadIdx.x == 0) {
-        const unsigned long long st = *L.step_ctr;
-        L.dM_ring[st % DM_RING] = total;
-        L.dM_ring[DM_RING] = total;
-        *L.step_ctr = st + 1;
-      }
-    }
-  }
-}
-
 template <bool PSEUDO>
 __global__ void __launch_bounds__(SOLID_BLOCK) k_solids(const __grid_constant__ Lattice<float> L, int blocks2, int blocks1,
                                                         int steps) {
-  solids<PSEUDO>(L, blockIdx.x, blocks2, blocks1, steps);
+  solids<PSEUDO, SOLID_BLOCK>(L, blockIdx.x, blocks2, blocks1, steps);
 }
 // item: (instance, its block)
 __global__ void __launch_bounds__(SOLID_BLOCK) k_solids_batch(const Lattice<float>* lat, const int2* items, int steps) {
@@ -884,7 +719,7 @@ __global__ void __launch_bounds__(SOLID_BLOCK) k_solids_batch(const Lattice<floa
   const int2 it = items[blockIdx.x];
   take_lattice(L, lat, it.x);
   __syncthreads();
-  solids<false>(L, it.y, (8 * L.n_s2 + SOLID_BLOCK - 1) / SOLID_BLOCK, (L.n_s1 + SOLID_BLOCK - 1) / SOLID_BLOCK, steps);
+  solids<false, SOLID_BLOCK>(L, it.y, (8 * L.n_s2 + SOLID_BLOCK - 1) / SOLID_BLOCK, (L.n_s1 + SOLID_BLOCK - 1) / SOLID_BLOCK, steps);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1003,8 +838,9 @@ __device__ __forceinline__ void density(const Lattice<float>& L, int cur, int x,
   L.rho_next[n] = PSEUDO ? psi_of(L, r) : r;
 }
 template <bool PSEUDO>
-__global__ void __launch_bounds__(128) k_density(const __grid_constant__ Lattice<float> L, int cur) {
-  density<PSEUDO>(L, cur, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y);
+__global__ void __launch_bounds__(128) k_density(const __grid_constant__ Lattice<float> L, int cur, int per_row) {
+  const int y = blockIdx.x / per_row;
+  density<PSEUDO>(L, cur, (blockIdx.x - y * per_row) * 128 + threadIdx.x, y);
 }
 // a batch: the pass's items (64 threads cover a strip's columns)
 __global__ void __launch_bounds__(64) k_density_batch(const Lattice<float>* lat, const int4* items, int cur) {
@@ -1096,30 +932,15 @@ bool fused_setup() {
          allow((const void*)k_walk<false>, Reach<false>::BYTES) && allow((const void*)k_walk<true>, Reach<true>::BYTES);
 }
 
-// a launch that may overlap the end of the one before it in the stream
-template <typename... P, typename... A>
-static cudaError_t launch_after(void (*k)(P...), int grid, int block, int smem, cudaStream_t s, A... args) {
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t c{};
-  c.gridDim = dim3((unsigned)grid);
-  c.blockDim = dim3((unsigned)block);
-  c.dynamicSmemBytes = (size_t)smem;
-  c.stream = s;
-  c.attrs = &at;
-  c.numAttrs = s ? 1 : 0;
-  return cudaLaunchKernelEx(&c, k, P(args)...);
-}
 static cudaError_t launch_solids(const Lattice<float>& L, int steps, cudaStream_t s) {
   const int b2 = (int)blocks_for(8 * L.n_s2, SOLID_BLOCK), b1 = (int)blocks_for(L.n_s1, SOLID_BLOCK);
-  return launch_after(L.pseudo ? k_solids<true> : k_solids<false>, b2 + b1 + 1, SOLID_BLOCK, 0, s, L, b2, b1, steps);
+  return launch_after(L.pseudo ? k_solids<true> : k_solids<false>, dim3((unsigned)(b2 + b1 + 1)), SOLID_BLOCK, 0, s, L, b2, b1, steps);
 }
 
 cudaError_t launch_fused_prepare(const Lattice<float>& L, int cur, cudaStream_t s) {
-  const dim3 grid(blocks_for(L.nx, 128), (unsigned)L.ny);
-  if (L.pseudo) k_density<true><<<grid, 128, 0, s>>>(L, cur);
-  else k_density<false><<<grid, 128, 0, s>>>(L, cur);
+  const unsigned per_row = blocks_for(L.nx, 128), grid = per_row * (unsigned)L.ny;
+  if (L.pseudo) k_density<true><<<grid, 128, 0, s>>>(L, cur, (int)per_row);
+  else k_density<false><<<grid, 128, 0, s>>>(L, cur, (int)per_row);
   if (L.n_bnodes > 0) k_boundary_density<<<blocks_for(L.n_bnodes, 128), 128, 0, s>>>(L, cur);
   return launch_solids(L, 0, s);
 }
@@ -1127,21 +948,21 @@ cudaError_t launch_fused_prepare(const Lattice<float>& L, int cur, cudaStream_t 
 template <int H, int W, int B>
 static cudaError_t launch_tiles(const Lattice<float>& L, int cur, int rows, cudaStream_t s) {
   const int strips = (L.nx + OUT - 1) / OUT, bands = (L.ny + rows - 1) / rows;
-  return L.pseudo ? launch_after(k_tile<true, H, W, B>, strips * bands, 32 * W, Tile<true, H>::BYTES, s, L, cur, strips, rows)
-                  : launch_after(k_tile<false, H, W, B>, strips * bands, 32 * W, Tile<false, H>::BYTES, s, L, cur, strips, rows);
+  return L.pseudo ? launch_after(k_tile<true, H, W, B>, dim3((unsigned)(strips * bands)), 32 * W, Tile<true, H>::BYTES, s, L, cur, strips, rows)
+                  : launch_after(k_tile<false, H, W, B>, dim3((unsigned)(strips * bands)), 32 * W, Tile<false, H>::BYTES, s, L, cur, strips, rows);
 }
 static cudaError_t launch_pass(const Lattice<float>& L, int cur, PassPlan p, cudaStream_t s) {
   if (p.kind == PassPlan::TILE_M) return launch_tiles<TH_M, TW_M, TB_M>(L, cur, p.rows, s);
   if (p.kind == PassPlan::TILE_L) return launch_tiles<TH_L, TW_L, TB_L>(L, cur, p.rows, s);
   const int strips = (L.nx + OUT - 1) / OUT, bands = (L.ny + p.rows - 1) / p.rows;
-  return L.pseudo ? launch_after(k_walk<true>, strips * bands, 32, Reach<true>::BYTES, s, L, cur, strips, p.rows)
-                  : launch_after(k_walk<false>, strips * bands, 32, Reach<false>::BYTES, s, L, cur, strips, p.rows);
+  return L.pseudo ? launch_after(k_walk<true>, dim3((unsigned)(strips * bands)), 32, Reach<true>::BYTES, s, L, cur, strips, p.rows)
+                  : launch_after(k_walk<false>, dim3((unsigned)(strips * bands)), 32, Reach<false>::BYTES, s, L, cur, strips, p.rows);
 }
 
 cudaError_t launch_fused_step(const Lattice<float>& L, int cur, PassPlan plan, cudaStream_t s) {
   cudaError_t e = launch_pass(L, cur, plan, s);
   if (e == cudaSuccess && L.n_bnodes > 0)
-    e = launch_after(L.pseudo ? k_bc_fused<true> : k_bc_fused<false>, (int)blocks_for(L.n_bnodes, BC_BLOCK), BC_BLOCK, 0, s, L, cur);
+    e = launch_after(L.pseudo ? k_bc_fused<true> : k_bc_fused<false>, dim3(blocks_for(L.n_bnodes, BC_BLOCK)), BC_BLOCK, 0, s, L, cur);
   return e == cudaSuccess ? launch_solids(L, 1, s) : e;
 }
 
@@ -1184,8 +1005,8 @@ cudaError_t launch_fused_batch_prepare(const FusedBatch& B, int cur, cudaStream_
 }
 cudaError_t launch_fused_batch_step(const FusedBatch& B, int cur, cudaStream_t s) {
   const Lattice<float>* lat = B.lat[cur];
-  cudaError_t e = B.rows > 0 ? launch_after(k_walk_batch, B.n_pass, 32, Reach<false>::BYTES, s, lat, B.pass, cur)
-                             : launch_after(k_tile_batch<TH_L, TW_L, TB_L>, B.n_pass, 32 * TW_L, Tile<false, TH_L>::BYTES, s, lat,
+  cudaError_t e = B.rows > 0 ? launch_after(k_walk_batch, dim3((unsigned)B.n_pass), 32, Reach<false>::BYTES, s, lat, B.pass, cur)
+                             : launch_after(k_tile_batch<TH_L, TW_L, TB_L>, dim3((unsigned)B.n_pass), 32 * TW_L, Tile<false, TH_L>::BYTES, s, lat,
                                             B.pass, cur);
   if (e == cudaSuccess && B.n_bc > 0) e = launch_after(k_bc_batch, B.n_bc, BC_BLOCK, 0, s, lat, B.bc, cur);
   return e == cudaSuccess ? launch_after(k_solids_batch, B.n_solid, SOLID_BLOCK, 0, s, lat, B.solid, 1) : e;
@@ -1193,8 +1014,8 @@ cudaError_t launch_fused_batch_step(const FusedBatch& B, int cur, cudaStream_t s
 
 cudaError_t launch_fused_fields(const Lattice<float>& L, int cur, float* r, float* vx, float* vy, cudaStream_t s) {
   const int strips = (L.nx + OUT - 1) / OUT, bands = (L.ny + RO_H - 1) / RO_H;
-  if (L.pseudo) k_fields_fused<true><<<strips * bands, 32 * RO_W, 0, s>>>(L, cur, strips, r, vx, vy);
-  else k_fields_fused<false><<<strips * bands, 32 * RO_W, 0, s>>>(L, cur, strips, r, vx, vy);
+  if (L.pseudo) k_fields_fused<true><<<dim3((unsigned)(strips * bands)), 32 * RO_W, 0, s>>>(L, cur, strips, r, vx, vy);
+  else k_fields_fused<false><<<dim3((unsigned)(strips * bands)), 32 * RO_W, 0, s>>>(L, cur, strips, r, vx, vy);
   return cudaGetLastError();
 }
 

@@ -42,6 +42,9 @@ cudaError_t launch_step_overlap(const Lattice<real>& Lt, const Lattice<real>& Ln
 template <typename real> int launches_per_step_overlap(const Lattice<real>& L);
 // one double into page-locked host memory (its device address dst), in stream order
 cudaError_t launch_copy8(const double* src, double* dst, cudaStream_t s);
+// density and velocity of a state whose density and chemical potential are in L's planes
+template <typename real>
+cudaError_t launch_fields_of(const Lattice<real>& L, int cur, real* rho, real* vx, real* vy, cudaStream_t s);
 template <typename real> cudaError_t launch_fields(const Lattice<real>& L, int cur, real* r, real* vx, real* vy, cudaStream_t s);
 // populations i0 <= i < i1 of the current state, population i into dense plane i - i0 of out
 template <typename real>
@@ -91,6 +94,12 @@ struct PassPlan {
 };
 PassPlan fused_plan(int nx, int ny, int sms);
 PassPlan fused_tile_plan(int nx, int ny, int sms);
+// ---- the FP64 step (lbm_fp64.cu): chemical-potential force, an equation of state, two lattices
+// one step from lattice cur, whose density plane is L.rho (and psi' in L.psip); the next into rho_next
+cudaError_t launch_fp64_step(const Lattice<double>& L, double* rho_next, int cur, cudaStream_t s);
+// the chemical potential of such a state
+cudaError_t launch_fp64_mu(const Lattice<double>& L, cudaStream_t s);
+int launches_fp64(const Lattice<double>& L);
 // the solid layers of a new state in lattice cur, where the fused step expects them
 cudaError_t launch_fused_prepare(const Lattice<float>& L, int cur, cudaStream_t s);
 // one step from lattice cur (L.rho_b, L.fx and L.fy set)

@@ -1558,11 +1558,15 @@ cudaError_t launch_macro(const Lattice<real>& L, int cur, cudaStream_t s) {
 }
 
 template <typename real>
-cudaError_t launch_fields(const Lattice<real>& L, int cur, real* r, real* vx, real* vy, cudaStream_t s) {
-  cudaError_t e = launch_macro(L, cur, s);
-  if (e != cudaSuccess) return e;
+cudaError_t launch_fields_of(const Lattice<real>& L, int cur, real* r, real* vx, real* vy, cudaStream_t s) {
   k_fields<real><<<grid_for(L.plane, NODE_BLOCK), NODE_BLOCK, 0, s>>>(L, cur, r, vx, vy);
   return cudaGetLastError();
+}
+
+template <typename real>
+cudaError_t launch_fields(const Lattice<real>& L, int cur, real* r, real* vx, real* vy, cudaStream_t s) {
+  cudaError_t e = launch_macro(L, cur, s);
+  return e == cudaSuccess ? launch_fields_of(L, cur, r, vx, vy, s) : e;
 }
 
 template <typename real>
@@ -1618,6 +1622,7 @@ cudaError_t launch_init(const Lattice<real>& L, const double* drops, int n_drop,
   template cudaError_t launch_step_overlap<real>(const Lattice<real>&, const Lattice<real>&, int, cudaStream_t, \
                                                  cudaStream_t, cudaEvent_t, cudaEvent_t);                  \
   template int launches_per_step_overlap<real>(const Lattice<real>&);                                   \
+  template cudaError_t launch_fields_of<real>(const Lattice<real>&, int, real*, real*, real*, cudaStream_t); \
   template cudaError_t launch_fields<real>(const Lattice<real>&, int, real*, real*, real*, cudaStream_t); \
   template cudaError_t launch_populations<real>(const Lattice<real>&, int, real*, int, int, cudaStream_t); \
   template cudaError_t launch_column<real>(const Lattice<real>&, int, int, int, int, double*, cudaStream_t); \
