@@ -41,6 +41,8 @@ struct Lattice {
   real* mu;                     // chemical potential minus k^2 mu_sat (constant at solids)
   real* rho_next;               // fused step (FP32): the next state's density (psi) plane
   real* mu_out;                 // ... if set (tiles): this state's chemical potential is kept here
+  real* aa_edge;                // ... in AA order, walked: what the strips left and right of a boundary between
+                                // two hand on of their outermost columns, 2 x 8 values a row, by boundary
   real* fx;                     // fused step (FP32): the force at nodes next to solids, left by
   real* fy;                     // the pass for the boundary phase
   real* psip;                   // if set: psi'(rho) - mu_sat of every fluid node, left by the

@@ -85,7 +85,7 @@ __device__ __forceinline__ int wrap_col(int c, int nx) {
 //
 // One warp: the populations streaming into the output columns of strip `strip` in rows [ya, yb),
 // and those nodes' density (psi), from the state in lattice `cur`.
-template <bool PSEUDO>
+template <bool PSEUDO, int AA = 0>
 __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip, int ya, int yb, char* smem) {
   using R = Reach<PSEUDO>;
   constexpr int LEAD = R::LEAD;
@@ -102,11 +102,17 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
   const int q4 = wrap_col(x0 - 2 * HX + 4 * lane, L.nx);                    // ... of a density row (18 lanes)
   const float* __restrict__ fin = L.f[cur];
   float* __restrict__ fout = L.f[cur ^ 1];
+  float* const fone = L.f[0];                              // (AA: the one lattice)
   const float* __restrict__ rin = PSEUDO ? L.mu : L.rho;   // the state's density (psi)
   float* __restrict__ rout = L.rho_next;                   // the next state's
   const float2* const fs = reinterpret_cast<const float2*>(smem) + lane;          // own pair: + (row, i) * 32
   float2* const rs = reinterpret_cast<float2*>(smem + FD * ROW_F) + HX / 2 + lane;   // density (psi): + row * SP
   float2* const ms = rs + RHO_ROWS * SP;                                          // chemical potential
+  const int cm = c == 0 ? L.nx - 1 : c - 1, c1 = c + 1 == L.nx ? 0 : c + 1, c2 = c1 + 1 == L.nx ? 0 : c1 + 1;   // (AA 2)
+  // AA: this lane's part of aa_edge if it holds an outermost column with a strip beside it
+  float* edge = nullptr;
+  if (AA && lane == HX / 2 && strip > 0) edge = L.aa_edge + (strip - 1) * 16ll * L.ny + 8;
+  if (AA && lane == 31 - HX / 2 && x0 + OUT < L.nx) edge = L.aa_edge + strip * 16ll * L.ny;
   auto rslot = [](int r) { return (r & (RHO_ROWS - 1)) * SP; };
   auto mslot = [](int r) { return (r & (MU_ROWS - 1)) * SP; };
   auto fslot = [](int y) { return (y & (FD - 1)) * (9 * 32); };
@@ -129,7 +135,22 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
   auto load_f = [&](int y) {
     const int n = row_of(y) * L.pitch;
     char* const d = smem + fslot(y) * 8;
-    if (!split) {
+    if constexpr (AA == 2) {
+      // direction i from plane opp(i), row y - e_y
+      const int nm = row_of(y - 1) * L.pitch, np = row_of(y + 1) * L.pitch;
+      auto from = [&](int i) { return fin + opp(i) * (long long)L.plane + (ey(i) == 0 ? n : ey(i) > 0 ? nm : np); };
+      if (!split) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) cp16(d + 512 * k + 16 * lane, (lane & 16 ? from(2 * k + 1) : from(2 * k)) + p4);
+        if (lane < 16) cp16(d + 2048 + 16 * lane, from(8) + p4);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+          cp4(d + 256 * i + 8 * lane, from(i) + ca);
+          cp4(d + 256 * i + 8 * lane + 4, from(i) + cb);
+        }
+      }
+    } else if (!split) {
       // a warp's 32 pieces are two directions' rows
       const char* base = reinterpret_cast<const char*>(fin + (lane >> 4) * (long long)L.plane) + 4u * (unsigned)(n + p4);
 #pragma unroll
@@ -143,13 +164,14 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
       }
     }
   };
-  // rows collided: ya - 1 .. yb; the newest density row r runs from rb to re
-  const int rb = PSEUDO ? ya : ya - 1, re = yb + LEAD;
+  // rows collided: ya - 1 .. yb (AA: the band's own); the newest density row r runs from rb to re
+  const int ylo = AA ? ya : ya - 1, yhi = AA ? yb - 1 : yb;
+  const int rb = ylo + (PSEUDO ? 1 : 0), re = yhi + LEAD;
   // density row r + FD and the populations of the row FD above the one collided with row r
   auto request = [&](int r) {
     if (r + FD <= re) load_rho(r + FD);
     const int y = r - LEAD + FD;
-    if (y >= ya - 1 && y <= yb) load_f(y);
+    if (y >= ylo && y <= yhi) load_f(y);
     cp_commit();
   };
   // the classes of columns c and c + 1 of the row, in bytes 0 and 1
@@ -165,7 +187,14 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
   auto load_pops = [&](int y, float2 (&v)[9]) {
     const float2* d = fs + fslot(y);
 #pragma unroll
-    for (int i = 0; i < 9; ++i) v[i] = d[i * 32];
+    for (int i = 0; i < 9; ++i) {
+      if (AA == 2 && ex(i) != 0) {
+        const float* p = reinterpret_cast<const float*>(d + i * 32) - ex(i);
+        v[i] = make_float2(p[0], p[1]);
+      } else {
+        v[i] = d[i * 32];
+      }
+    }
   };
   // the undivided x differences of Eq. 9 from a pair and its neighbour pairs
   auto dx_of = [](float2 l, float2 C, float2 g) {
@@ -202,11 +231,15 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
     const float2 z = make_float2(0.f, 0.f);
     in = {z, z, z, z, z, z, z, z};
   }
+  struct {
+    float h, o1, o5, n5;     // AA, outermost columns: received and sent along x in row y - 1; sent into
+  } out = {0.f, 0.f, 0.f, 0.f};   // the column beside in row y - 1 and row y from the row below each
   // Streaming of row y's post-collision populations: every pair of outputs receives columns c - 1, c
   // (moving right) or c + 1, c + 2 (moving left) through the neighbouring lane, so that all stores
   // are aligned pairs.  Slots whose source is solid get a meaningless value; the boundary phase
   // rewrites those of fluid nodes, nothing reads the others.
-  auto stream_row = [&](const float2 (&v)[9], int y) {
+  // fl: this lane's fluid bits of the row
+  auto stream_row = [&](const float2 (&v)[9], int y, unsigned fl) {
     auto right = [](float2 a) { return make_float2(__shfl_up_sync(0xffffffffu, a.y, 1), a.x); };
     auto left = [](float2 a) { return make_float2(a.y, __shfl_down_sync(0xffffffffu, a.x, 1)); };
     const float2 r1 = right(v[1]), r5 = right(v[5]), r8 = right(v[8]);
@@ -218,7 +251,51 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
     if (PSEUDO) q = psi_of(L, q);
     const int n = y * L.pitch + c;
     const bool mid = y >= ya && y < yb, up = y + 1 < yb, dn = y > ya;   // rows the band does not own are left
-    if (out1) {
+    if constexpr (AA != 0) {
+      // (the density of a band's outermost rows and a strip's outermost columns: k_layers_aa)
+      if (y >= ya + 2 && out1) {
+        const bool first = c == x0, last = c + 1 == x0 + OUT - 1 || c + 1 == L.nx - 1;
+        float* const p = rout + n - L.pitch;
+        if (!first && !last) *reinterpret_cast<float2*>(p) = q;
+        else if (!first) *p = q.x;
+        else if (!last) p[1] = q.y;
+      }
+      if (edge) {
+        // row y - 1's record: what the outermost column has received from the strip, and what it
+        // has sent into the column beside it
+        const bool lo = lane == HX / 2;
+        auto at = [&](float2 a, float2 b) { return lo ? a.x : b.y; };
+        const float2 f24 = add_rn(in.d2, v[4]);
+        if (y >= ya + 2) {
+          float4* const p = reinterpret_cast<float4*>(edge + 16 * (y - 1));
+          p[0] = make_float4(at(in.c0, in.c0), out.h, at(f24, f24), at(in.d6, in.d5));
+          p[1] = make_float4(at(l7, r8), out.o1, out.o5, at(v[7], v[8]));
+        }
+        out.o5 = out.n5;
+        out.h = at(l3, r1);
+        out.o1 = at(v[3], v[1]);
+        out.n5 = at(v[6], v[5]);
+      }
+      if constexpr (AA == 1) {
+        // each node's own slot opp(i)
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+          float* const p = fone + opp(i) * (long long)L.plane + n;
+          if (out1) *reinterpret_cast<float2*>(p) = v[i];
+          else if (one) *p = v[i].x;
+        }
+      } else {
+        // slot i of x + e_i: the slots read
+        const int nm = row_of(y - 1) * L.pitch, n0 = y * L.pitch, np = row_of(y + 1) * L.pitch;
+        const bool w0 = (out1 || one) && (fl & 1u), w1 = out1 && (fl & 2u);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+          float* const p = fone + i * (long long)L.plane + (ey(i) == 0 ? n0 : ey(i) > 0 ? np : nm);
+          if (w0) p[ex(i) == 0 ? c : ex(i) > 0 ? c1 : cm] = v[i].x;
+          if (w1) p[ex(i) == 0 ? c1 : ex(i) > 0 ? c2 : c] = v[i].y;
+        }
+      }
+    } else if (out1) {
       auto put = [&](float* plane, int at, float2 a) { *reinterpret_cast<float2*>(plane + at) = a; };
       if (mid) {
         put(fout, n, v[0]);
@@ -295,7 +372,7 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
     const int y = r - LEAD;
     const bool all0 = __all_sync(0xffffffffu, k0 == 0u), all1 = __all_sync(0xffffffffu, k1 == 0u);   // (fluid is 0)
     // groups are committed in the order walls(r - 2), request(r - 2), walls(r - 1), request(r - 1)
-    if (r < re && y >= ya - 1 && all0 && all1 && !(solid & ((2u << LEAD) - 1u))) {
+    if (r < re && y >= ylo && all0 && all1 && !(solid & ((2u << LEAD) - 1u))) {
       // Rows y - 1 .. r + 1 hold no solid node: the chemical potentials of rows r - 2 and r - 1 and
       // the collisions of rows y and y + 1 in one run of instructions without branches, whose chains
       // overlap.
@@ -321,7 +398,7 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
         const float2 rho = add_rn(splat<float2>(L.rho_ref), drho);
         force(rho, Fx, Fy);
         collide_node(L, w, rho, drho, jx, jy, Fx, Fy);
-        stream_row(w, yy);
+        stream_row(w, yy, 3u);
       };
       if constexpr (PSEUDO) {
         collide_stream(w0, y, [&](float2 rho, float2& Fx, float2& Fy) { force_pp_at(rho, y, Fx, Fy); });
@@ -383,7 +460,7 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
     }
     cp_commit();
     // collision and streaming of row y
-    if (y >= ya - 1 && !(none & (1u << LEAD))) {
+    if (y >= ylo && !(none & (1u << LEAD))) {
       float2 v[9];
       load_pops(y, v);
       float2 drho, jx, jy, Fx, Fy;
@@ -406,7 +483,7 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
         if (out1 && (fy & 2u)) { L.fx[n + 1] = Fx.y; L.fy[n + 1] = Fy.y; }
       }
       collide_node(L, v, rho, drho, jx, jy, Fx, Fy);
-      stream_row(v, y);
+      stream_row(v, y, (bits >> (2 * LEAD)) & 3u);
     }
     request(r);
     ++r;
@@ -414,14 +491,14 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
   cp_wait<0>();
 }
 
-template <bool PSEUDO>
+template <bool PSEUDO, int AA = 0>
 __global__ void __launch_bounds__(32) k_walk(const __grid_constant__ Lattice<float> L, int cur, int strips, int rows) {
   extern __shared__ __align__(16) char smem[];
   const int band = blockIdx.x / strips, strip = blockIdx.x - band * strips;
   const int ya = band * rows, yb = min(ya + rows, L.ny);
   grid_wait();
   grid_launch();
-  walk<PSEUDO>(L, cur, strip, ya, yb, smem);
+  walk<PSEUDO, AA>(L, cur, strip, ya, yb, smem);
 }
 
 // The descriptor of a batch's instance in shared memory, copied by the block's threads (the tables
@@ -457,7 +534,12 @@ struct Tile {
   static constexpr int BYTES = FLAGS + (H + 6) * 4;
 };
 
-template <bool PSEUDO, int H, int W>
+// One population lattice in AA order (AA: the state's slot order plus one, pop_index): a tile collides
+// its own nodes only.  Each reads and writes nine slots that no other node touches -- its own
+// (natural order), or slot opp(i) of x - e_i (shifted), from aligned rows in shared memory read one
+// column aside -- but what streams into the tile's outermost rows and columns comes from other
+// tiles, so the density of those nodes is left to k_layers_aa.
+template <bool PSEUDO, int H, int W, int AA = 0>
 __device__ __forceinline__ void tile(const Lattice<float>& L, int cur, int strip, int ya, int yb, char* smem) {
   using T = Tile<PSEUDO, H>;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -468,6 +550,7 @@ __device__ __forceinline__ void tile(const Lattice<float>& L, int cur, int strip
   const bool split = (L.nx & 3) != 0 && (x0 - 2 * HX < 0 || x0 + OUT + 2 * HX > L.nx);
   const float* __restrict__ fin = L.f[cur];
   float* __restrict__ fout = L.f[cur ^ 1];
+  float* const fin1 = L.f[0];   // (AA: the one lattice)
   const float* __restrict__ rin = PSEUDO ? L.mu : L.rho;
   int* const flags = reinterpret_cast<int*>(smem + T::FLAGS);   // rows ya - 3 ..: 1 some column solid, 2 none fluid
   auto row_of = [&](int r) {
@@ -497,10 +580,26 @@ __device__ __forceinline__ void tile(const Lattice<float>& L, int cur, int strip
           if (lane + 32 * j < 4 * RHO_CHUNKS) cp4(d + 4 * (lane + 32 * j), rin + n + e4[j]);
       }
     }
-    for (int y = ya - 1 + warp; y <= yb; y += W) {
+    const int y0 = AA ? ya : ya - 1, y1 = AA ? yb : yb + 1;   // rows collided
+    for (int y = y0 + warp; y < y1; y += W) {
       const int n = row_of(y) * L.pitch;
       char* const d = smem + (y - ya + 1) * ROW_F;
-      if (!split) {
+      if constexpr (AA == 2) {
+        // direction i from plane opp(i), row y - e_y
+        const int nm = row_of(y - 1) * L.pitch, np = row_of(y + 1) * L.pitch;
+        auto from = [&](int i) { return fin + opp(i) * (long long)L.plane + (ey(i) == 0 ? n : ey(i) > 0 ? nm : np); };
+        if (!split) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) cp16(d + 512 * k + 16 * lane, (lane & 16 ? from(2 * k + 1) : from(2 * k)) + p4);
+          if (lane < 16) cp16(d + 2048 + 16 * lane, from(8) + p4);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 9; ++i) {
+            cp4(d + 256 * i + 8 * lane, from(i) + ca);
+            cp4(d + 256 * i + 8 * lane + 4, from(i) + cb);
+          }
+        }
+      } else if (!split) {
         const float* base = fin + (lane >> 4) * (long long)L.plane + n + p4;
 #pragma unroll
         for (int k = 0; k < 4; ++k) cp16(d + 512 * k + 16 * lane, base + 2ll * k * L.plane);
@@ -565,13 +664,20 @@ __device__ __forceinline__ void tile(const Lattice<float>& L, int cur, int strip
     __syncthreads();
   }
   // ---- collisions and streaming
-  for (int y = ya - 1 + warp; y <= yb; y += W) {
+  for (int y = (AA ? ya : ya - 1) + warp; y < (AA ? yb : yb + 1); y += W) {
     const int* fg = flags + (y - ya + M0);
     if (fg[0] & 2) continue;
     float2 v[9];
     float2* const pr = pop_row(y);
 #pragma unroll
-    for (int i = 0; i < 9; ++i) v[i] = pr[32 * i];
+    for (int i = 0; i < 9; ++i) {
+      if (AA == 2 && ex(i) != 0) {
+        const float* p = reinterpret_cast<const float*>(pr + 32 * i) - ex(i);
+        v[i] = make_float2(p[0], p[1]);
+      } else {
+        v[i] = pr[32 * i];
+      }
+    }
     float2 drho, jx, jy, Fx, Fy;
     moments(v, drho, jx, jy);
     const float2 rho = add_rn(splat<float2>(L.rho_ref), drho);
@@ -610,7 +716,27 @@ __device__ __forceinline__ void tile(const Lattice<float>& L, int cur, int strip
     const float2 r1 = right(v[1]), r5 = right(v[5]), r8 = right(v[8]);
     const float2 l3 = left(v[3]), l6 = left(v[6]), l7 = left(v[7]);
     const int n = y * L.pitch + c;
-    if (out1) {
+    if constexpr (AA == 1) {
+      // each node's own slot opp(i)
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        float* p = fin1 + opp(i) * (long long)L.plane + n;
+        if (out1) *reinterpret_cast<float2*>(p) = v[i];
+        else if (one) *p = v[i].x;
+      }
+    } else if constexpr (AA == 2) {
+      // slot i of x + e_i: the slots read
+      const uint8_t* kd = L.kind + y * L.pitch;
+      const bool w0 = (out1 || one) && kd[c] == KIND_FLUID, w1 = out1 && kd[c + 1] == KIND_FLUID;
+      const int nm = row_of(y - 1) * L.pitch, n0 = y * L.pitch, np = row_of(y + 1) * L.pitch;
+      const int cm = c == 0 ? L.nx - 1 : c - 1, c1 = c + 1 == L.nx ? 0 : c + 1, c2 = c1 + 1 == L.nx ? 0 : c1 + 1;
+#pragma unroll
+      for (int i = 0; i < 9; ++i) {
+        float* p = fin1 + i * (long long)L.plane + (ey(i) == 0 ? n0 : ey(i) > 0 ? np : nm);
+        if (w0) p[ex(i) == 0 ? c : ex(i) > 0 ? c1 : cm] = v[i].x;
+        if (w1) p[ex(i) == 0 ? c1 : ex(i) > 0 ? c2 : c] = v[i].y;
+      }
+    } else if (out1) {
       auto put = [&](int i, int at, float2 a) { *reinterpret_cast<float2*>(fout + (long long)i * L.plane + at) = a; };
       if (mid) {
         put(0, n, v[0]);
@@ -658,7 +784,7 @@ __device__ __forceinline__ void tile(const Lattice<float>& L, int cur, int strip
   __syncthreads();
   // ---- densities (psi) of the outputs; rows next to solids hold meaningless values where a source
   // is solid: the boundary phase forms the boundary nodes' densities
-  for (int y = ya + warp; y < yb; y += W) {
+  for (int y = ya + (AA ? 1 : 0) + warp; y < yb - (AA ? 1 : 0); y += W) {
     if (flags[y - ya + M0] & 2) continue;
     const float2* o = pop_row(y);
     const float2* d = o - 9 * 32;
@@ -667,19 +793,26 @@ __device__ __forceinline__ void tile(const Lattice<float>& L, int cur, int strip
     float2 q = add_rn(splat<float2>(L.rho_ref), sum);
     if (PSEUDO) q = psi_of(L, q);
     float* p = L.rho_next + y * L.pitch + c;
+    if constexpr (AA != 0) {
+      const bool first = c == x0, last = c + 1 == x0 + OUT - 1 || c + 1 == L.nx - 1;
+      if (out1 && !first && !last) *reinterpret_cast<float2*>(p) = q;
+      else if (out1 && !first) *p = q.x;
+      else if (out1 && !last) p[1] = q.y;
+      continue;
+    }
     if (out1) *reinterpret_cast<float2*>(p) = q;
     else if (one) *p = q.x;
   }
 }
 
-template <bool PSEUDO, int H, int W, int MINB>
+template <bool PSEUDO, int H, int W, int MINB, int AA = 0>
 __global__ void __launch_bounds__(32 * W, MINB) k_tile(const __grid_constant__ Lattice<float> L, int cur, int strips, int rows) {
   extern __shared__ __align__(16) char smem[];
   const int band = blockIdx.x / strips, strip = blockIdx.x - band * strips;
   const int ya = band * rows, yb = min(ya + rows, L.ny);
   grid_wait();
   grid_launch();
-  tile<PSEUDO, H, W>(L, cur, strip, ya, yb, smem);
+  tile<PSEUDO, H, W, AA>(L, cur, strip, ya, yb, smem);
 }
 template <int H, int W, int MINB>
 __global__ void __launch_bounds__(32 * W, MINB) k_tile_batch(const Lattice<float>* lat, const int4* items, int cur) {
@@ -694,9 +827,9 @@ __global__ void __launch_bounds__(32 * W, MINB) k_tile_batch(const Lattice<float
 }
 
 constexpr int BC_BLOCK = 64;
-template <bool PSEUDO>
+template <bool PSEUDO, int AA = 0>
 __global__ void __launch_bounds__(BC_BLOCK) k_bc_fused(const __grid_constant__ Lattice<float> L, int cur) {
-  links<PSEUDO, true>(L, cur, blockIdx.x * BC_BLOCK + threadIdx.x);
+  links<PSEUDO, true, AA>(L, cur, blockIdx.x * BC_BLOCK + threadIdx.x);
 }
 // item: (instance, first boundary node)
 __global__ void __launch_bounds__(BC_BLOCK) k_bc_batch(const Lattice<float>* lat, const int2* items, int cur) {
@@ -712,6 +845,83 @@ template <bool PSEUDO>
 __global__ void __launch_bounds__(SOLID_BLOCK) k_solids(const __grid_constant__ Lattice<float> L, int blocks2, int blocks1,
                                                         int steps) {
   solids<PSEUDO, SOLID_BLOCK>(L, blockIdx.x, blocks2, blocks1, steps);
+}
+// The solid layers of an AA lattice and, in blocks of their own, the densities its pass leaves: the
+// outermost rows of the bands (edge_rows of them) and columns of the strips, from the populations of
+// the state in slot order `cur`, which the links have completed.  A column of a large lattice is a
+// memory access of its own for each population (35 us of 2048 x 4096): there (WALK) the walks hand
+// those columns' populations on in aa_edge, and only the lattice's own ends are read that way.
+template <bool PSEUDO, bool WALK>
+__global__ void __launch_bounds__(SOLID_BLOCK) k_layers_aa(const __grid_constant__ Lattice<float> L, int blocks2, int blocks1,
+                                                           int cur, int strips, int rows, int edge_rows) {
+  const int blk = (int)blockIdx.x - (blocks2 + blocks1 + 1);
+  if (blk < 0) {
+    solids<PSEUDO, SOLID_BLOCK>(L, blockIdx.x, blocks2, blocks1, 1);
+    return;
+  }
+  unsigned e = (unsigned)blk * SOLID_BLOCK + threadIdx.x;
+  const unsigned in_rows = (unsigned)edge_rows * (unsigned)L.nx, ends = WALK ? 2u * L.ny : 0u;
+  int x = 0, y = L.ny;
+  const float* from = nullptr;
+  if (e < in_rows) {
+    const int k = (int)(e / (unsigned)L.nx), ya = (k >> 1) * rows;
+    x = (int)(e - (unsigned)k * L.nx);
+    y = k & 1 ? min(ya + rows, L.ny) - 1 : ya;
+  } else if ((e -= in_rows) < ends) {
+    y = (int)(e >> 1);
+    x = e & 1u ? L.nx - 1 : 0;
+  } else if (WALK) {
+    // the columns left (x) and right of boundary b between two strips
+    e -= ends;
+    const unsigned b = e / (unsigned)L.ny;
+    if ((int)b < strips - 1) {
+      y = (int)(e - b * L.ny);
+      x = (int)(b + 1) * OUT - 1;
+      from = L.aa_edge + 16ll * e;
+    }
+  } else {
+    y = (int)(e / (2u * strips));
+    const int k = (int)(e - (unsigned)y * (2u * strips));
+    // (the last column of a strip and the first of the next are neighbours in the list)
+    x = k == 2 * strips - 1 ? L.nx - 1 : ((k + 1) >> 1) * OUT - (k & 1);
+  }
+  const int n = y * L.pitch + x;
+  if (WALK && from) {
+    // not next to a solid node (a boundary node has its density from the links), nor an end or in an
+    // outermost row
+    const int ya = y / rows * rows;
+    bool all[4];   // all of a column's three nodes fluid: x - 1 .. x + 2
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      all[k] = true;
+#pragma unroll
+      for (int d = -1; d <= 1; ++d) all[k] &= L.kind[node_at(L, x - 1 + k, y + d)] == KIND_FLUID;
+    }
+    const bool inside = y > ya && y < min(ya + rows, L.ny) - 1;
+    const bool left = inside && all[0] && all[1] && all[2], right = inside && all[1] && all[2] && all[3] && x + 1 < L.nx - 1;
+    grid_wait();
+    grid_launch();
+    if (!left && !right) return;
+    // record of the strip left of the boundary, then of the one right of it
+    const float4* p = reinterpret_cast<const float4*>(from);
+    const float4 h0 = p[0], h1 = p[1], g0 = p[2], g1 = p[3];
+    auto put = [&](int at, float f0, float f1, float f3, float f24, float f5, float f7, float f6, float f8) {
+      const float sum = add_rn(f0, add_rn(add_rn(add_rn(f1, f3), f24), add_rn(add_rn(f5, f7), add_rn(f6, f8))));
+      const float r = add_rn(L.rho_ref, sum);
+      L.rho_next[at] = PSEUDO ? psi_of(L, r) : r;
+    };
+    if (left) put(n, h0.x, h0.y, g1.y, h0.z, h0.w, g1.w, g1.z, h1.x);
+    if (right) put(n + 1, g0.x, h1.y, g0.y, g0.z, h1.z, g1.x, g0.w, h1.w);
+    return;
+  }
+  const bool live = y < L.ny && L.kind[n] == KIND_FLUID;
+  grid_wait();
+  grid_launch();
+  if (!live) return;
+  float v[9];
+  load_pops(L, cur, x, y, v);
+  const float r = density_of(L, v);
+  L.rho_next[n] = PSEUDO ? psi_of(L, r) : r;
 }
 // item: (instance, its block)
 __global__ void __launch_bounds__(SOLID_BLOCK) k_solids_batch(const Lattice<float>* lat, const int2* items, int steps) {
@@ -780,8 +990,16 @@ __global__ void __launch_bounds__(32 * RO_W) k_fields_fused(const __grid_constan
     if (f0 || f1) {
       const float* __restrict__ f = L.f[cur] + n;
       float2 v[9], drho, jx, jy, Fx, Fy;
+      if (L.aa && cur == 1) {
+        float a[9], b[9];
+        load_pops(L, cur, ca, y, a);
+        load_pops(L, cur, cb, y, b);
 #pragma unroll
-      for (int i = 0; i < 9; ++i) v[i] = make_float2(f[i * (long long)L.plane + ca], f[i * (long long)L.plane + cb]);
+        for (int i = 0; i < 9; ++i) v[i] = make_float2(a[i], b[i]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) v[i] = make_float2(f[i * (long long)L.plane + ca], f[i * (long long)L.plane + cb]);
+      }
       moments(v, drho, jx, jy);
       const float2 rho = add_rn(splat<float2>(L.rho_ref), drho);
       const float2* q = s_rho + (y - ya + RR) * SP + HX / 2 + lane;
@@ -830,10 +1048,8 @@ template <bool PSEUDO>
 __device__ __forceinline__ void density(const Lattice<float>& L, int cur, int x, int y) {
   const int n = y * L.pitch + x;
   if (x >= L.nx || L.kind[n] != KIND_FLUID) return;
-  const float* __restrict__ f = L.f[cur] + n;
   float v[9];
-#pragma unroll
-  for (int i = 0; i < 9; ++i) v[i] = f[i * L.plane];
+  load_pops(L, cur, x, y, v);
   const float r = density_of(L, v);
   L.rho_next[n] = PSEUDO ? psi_of(L, r) : r;
 }
@@ -853,11 +1069,11 @@ __global__ void __launch_bounds__(64) k_density_batch(const Lattice<float>* lat,
 }
 __device__ __forceinline__ void boundary_density(const Lattice<float>& L, int cur, int b) {
   if (b >= L.n_bnodes) return;
-  const float* __restrict__ f = L.f[cur] + L.bnode[b];
+  const int n = L.bnode[b];
   float v[9];
-#pragma unroll
-  for (int i = 0; i < 9; ++i) v[i] = f[i * L.plane];
+  load_pops(L, cur, n % L.pitch, n / L.pitch, v);
   L.rho_b[b] = density_of(L, v);
+  if (L.aa) moments(v, L.bmom[3 * b], L.bmom[3 * b + 1], L.bmom[3 * b + 2]);
 }
 
 // the tile shapes: output rows at most, warps a block, blocks an SM
@@ -919,6 +1135,17 @@ PassPlan fused_tile_plan(int nx, int ny, int sms) {
   return p;
 }
 
+// ... of an AA lattice: the same walks; its tiles are of the first shape, whose bands leave fewer
+// outermost rows to k_layers_aa.  (separate passes / fused, us a step: 131 x 97 24.6 / 9.5, 512 x 512 30 / 15.7,
+// 1024 x 1024 46 / 33, 1600 x 2000 94 / 92, 2048 x 4096 198 / 172.)
+PassPlan fused_aa_plan(int nx, int ny, int sms) {
+  PassPlan p = fused_plan(nx, ny, sms);
+  if (p.kind != PassPlan::TILE_L) return p;
+  p.kind = PassPlan::TILE_M;
+  p.rows = TH_M;
+  return p;
+}
+
 bool fused_setup() {
   auto allow = [](const void* k, int bytes) {
     return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess;
@@ -929,6 +1156,12 @@ bool fused_setup() {
          allow((const void*)k_tile<false, TH_L, TW_L, TB_L>, Tile<false, TH_L>::BYTES) &&
          allow((const void*)k_tile<true, TH_L, TW_L, TB_L>, Tile<true, TH_L>::BYTES) &&
          allow((const void*)k_tile_batch<TH_L, TW_L, TB_L>, Tile<false, TH_L>::BYTES) &&
+         allow((const void*)k_tile<false, TH_M, TW_M, TB_M, 1>, Tile<false, TH_M>::BYTES) &&
+         allow((const void*)k_tile<false, TH_M, TW_M, TB_M, 2>, Tile<false, TH_M>::BYTES) &&
+         allow((const void*)k_tile<true, TH_M, TW_M, TB_M, 1>, Tile<true, TH_M>::BYTES) &&
+         allow((const void*)k_tile<true, TH_M, TW_M, TB_M, 2>, Tile<true, TH_M>::BYTES) &&
+         allow((const void*)k_walk<false, 1>, Reach<false>::BYTES) && allow((const void*)k_walk<false, 2>, Reach<false>::BYTES) &&
+         allow((const void*)k_walk<true, 1>, Reach<true>::BYTES) && allow((const void*)k_walk<true, 2>, Reach<true>::BYTES) &&
          allow((const void*)k_walk<false>, Reach<false>::BYTES) && allow((const void*)k_walk<true>, Reach<true>::BYTES);
 }
 
@@ -964,6 +1197,37 @@ cudaError_t launch_fused_step(const Lattice<float>& L, int cur, PassPlan plan, c
   if (e == cudaSuccess && L.n_bnodes > 0)
     e = launch_after(L.pseudo ? k_bc_fused<true> : k_bc_fused<false>, dim3(blocks_for(L.n_bnodes, BC_BLOCK)), BC_BLOCK, 0, s, L, cur);
   return e == cudaSuccess ? launch_solids(L, 1, s) : e;
+}
+
+// One lattice in AA order, from slot order cur
+cudaError_t launch_fused_step_aa(const Lattice<float>& L, int cur, PassPlan p, cudaStream_t s) {
+  const int strips = (L.nx + OUT - 1) / OUT, bands = (L.ny + p.rows - 1) / p.rows;
+  const dim3 grid((unsigned)(strips * bands)), nb(blocks_for(L.n_bnodes, BC_BLOCK));
+  const int b2 = (int)blocks_for(8 * L.n_s2, SOLID_BLOCK), b1 = (int)blocks_for(L.n_s1, SOLID_BLOCK);
+  const int edge_rows = 2 * bands;
+  // (strips <= nx / OUT + 1 and rows >= 2: at most twice the lattice's nodes, 32-bit)
+  const unsigned edge = (unsigned)edge_rows * (unsigned)L.nx +
+                        (p.kind == PassPlan::WALK ? strips + 1u : 2u * (unsigned)strips) * (unsigned)L.ny;
+  const dim3 layers((unsigned)(b2 + b1 + 1) + (edge + SOLID_BLOCK - 1) / SOLID_BLOCK);
+  auto tiles = [&](auto* k, int bytes) { return launch_after(k, grid, 32 * TW_M, bytes, s, L, cur, strips, p.rows); };
+  auto walks = [&](auto* k, int bytes) { return launch_after(k, grid, 32, bytes, s, L, cur, strips, p.rows); };
+  cudaError_t e;
+  if (p.kind == PassPlan::WALK) {
+    if (L.pseudo) e = cur ? walks(k_walk<true, 2>, Reach<true>::BYTES) : walks(k_walk<true, 1>, Reach<true>::BYTES);
+    else e = cur ? walks(k_walk<false, 2>, Reach<false>::BYTES) : walks(k_walk<false, 1>, Reach<false>::BYTES);
+  } else if (L.pseudo) e = cur ? tiles(k_tile<true, TH_M, TW_M, TB_M, 2>, Tile<true, TH_M>::BYTES)
+                        : tiles(k_tile<true, TH_M, TW_M, TB_M, 1>, Tile<true, TH_M>::BYTES);
+  else e = cur ? tiles(k_tile<false, TH_M, TW_M, TB_M, 2>, Tile<false, TH_M>::BYTES)
+               : tiles(k_tile<false, TH_M, TW_M, TB_M, 1>, Tile<false, TH_M>::BYTES);
+  if (e == cudaSuccess && L.n_bnodes > 0) {
+    auto bc = [&](auto* k) { return launch_after(k, nb, BC_BLOCK, 0, s, L, cur); };
+    if (L.pseudo) e = cur ? bc(k_bc_fused<true, 2>) : bc(k_bc_fused<true, 1>);
+    else e = cur ? bc(k_bc_fused<false, 2>) : bc(k_bc_fused<false, 1>);
+  }
+  if (e != cudaSuccess) return e;
+  auto* k = p.kind == PassPlan::WALK ? (L.pseudo ? k_layers_aa<true, true> : k_layers_aa<false, true>)
+                                     : (L.pseudo ? k_layers_aa<true, false> : k_layers_aa<false, false>);
+  return launch_after(k, layers, SOLID_BLOCK, 0, s, L, b2, b1, cur ^ 1, strips, p.rows, edge_rows);
 }
 
 // ---- batches

@@ -41,7 +41,7 @@ inline cudaError_t launch_after(void (*k)(P...), dim3 grid, int block, int smem,
 // us for 50 steps) -- and the loads behind it make one round.  The node's own populations stay in
 // registers for its density.  Leaves one compensation sum per warp, which solids
 // adds up.
-template <bool PSEUDO, bool PLANES, typename real>
+template <bool PSEUDO, bool PLANES, int AA = 0, typename real>
 __device__ __forceinline__ void links(const Lattice<real>& L, int cur, int b) {
   const bool live = b < L.n_bnodes;
   const int2 nd = live ? L.bnd[b] : make_int2(0, 0);
@@ -54,14 +54,26 @@ __device__ __forceinline__ void links(const Lattice<real>& L, int cur, int b) {
   real fl[9], ux = real(0), uy = real(0), r = real(1), inv_r = real(1), Fx = real(0), Fy = real(0);
   double carry = 0.0;
   auto load_state = [&]() {
+    if constexpr (AA != 0) {
+      // (the collision has overwritten the populations: the moments the step before left)
 #pragma unroll
-    for (int i = 0; i < 9; ++i) fl[i] = fin[i * L.plane + n];
+      for (int i = 0; i < 3; ++i) fl[i] = L.bmom[3 * b + i];
+    } else {
+#pragma unroll
+      for (int i = 0; i < 9; ++i) fl[i] = fin[i * L.plane + n];
+    }
     carry = L.carry[b];
   };
   real F[8];   // the links' force terms
   auto terms = [&]() {
     real drho, jx, jy;
-    moments(fl, drho, jx, jy);
+    if constexpr (AA != 0) {
+      drho = fl[0];
+      jx = fl[1];
+      jy = fl[2];
+    } else {
+      moments(fl, drho, jx, jy);
+    }
     r = L.rho_ref + drho;
     if constexpr (!PLANES) force_at<real, PSEUDO>(L, x, n / L.pitch, r, Fx, Fy);
     inv_r = real(1) / r;
@@ -86,8 +98,11 @@ __device__ __forceinline__ void links(const Lattice<real>& L, int cur, int b) {
     const int yp = !L.walls && n >= L.plane - L.pitch ? L.pitch - L.plane : L.pitch;
     auto nb = [&](int dx, int dy) { return n + (dx < 0 ? xm : dx > 0 ? xp : 0) + (dy < 0 ? ym : dy > 0 ? yp : 0); };
     real g[9], a[8], cc[8];
+    // Slots of the new state: f_i(x) in slot i of x, or (AA 1: the step from the natural order)
+    // slot opp(i) of x - e_i
+    auto own = [&](int i) { return AA == 1 ? opp(i) * L.plane + nb(-ex(i), -ey(i)) : i * L.plane + n; };
 #pragma unroll
-    for (int i = 0; i < 9; ++i) g[i] = fout[i * L.plane + n];
+    for (int i = 0; i < 9; ++i) g[i] = fout[own(i)];
     if constexpr (PLANES) {
       load_state();
       Fx = L.fx[n];
@@ -97,8 +112,8 @@ __device__ __forceinline__ void links(const Lattice<real>& L, int cur, int b) {
     for (int i = 1; i < 9; ++i) {
       a[i - 1] = cc[i - 1] = real(0);
       if (mask & (1u << (i - 1))) {
-        a[i - 1] = fout[i * L.plane + nb(ex(i), ey(i))];
-        cc[i - 1] = fout[opp(i) * L.plane + nb(-ex(i), -ey(i))];
+        a[i - 1] = fout[AA == 1 ? opp(i) * L.plane + n : i * L.plane + nb(ex(i), ey(i))];
+        cc[i - 1] = fout[AA == 1 ? i * L.plane + n : opp(i) * L.plane + nb(-ex(i), -ey(i))];
       }
     }
     if constexpr (PLANES) terms();
@@ -114,7 +129,7 @@ __device__ __forceinline__ void links(const Lattice<real>& L, int cur, int b) {
     for (int i = 1; i < 9; ++i) {
       if (!(mask & (1u << (i - 1)))) continue;
       g[opp(i)] = v[i - 1];
-      fout[opp(i) * L.plane + n] = v[i - 1];
+      fout[own(opp(i))] = v[i - 1];
     }
     if (L.bc == BC_PRESENT || L.bc == BC_MIBC) {
       const double t = (double)g[0] + sum + carry;
@@ -124,6 +139,7 @@ __device__ __forceinline__ void links(const Lattice<real>& L, int cur, int b) {
     } else {
       sum = 0.0;
     }
+    if constexpr (AA != 0) moments(g, L.bmom[3 * b], L.bmom[3 * b + 1], L.bmom[3 * b + 2]);
     const real rn = density_of(L, g);
     L.rho_b[b] = rn;
     L.rho_next[n] = PSEUDO ? psi_of(L, rn) : rn;

@@ -94,6 +94,9 @@ struct PassPlan {
 };
 PassPlan fused_plan(int nx, int ny, int sms);
 PassPlan fused_tile_plan(int nx, int ny, int sms);
+PassPlan fused_aa_plan(int nx, int ny, int sms);
+// the fused step of one lattice in AA order, from slot order cur (L.bmom: the boundary nodes' moments)
+cudaError_t launch_fused_step_aa(const Lattice<float>& L, int cur, PassPlan plan, cudaStream_t s);
 // ---- the FP64 step (lbm_fp64.cu): chemical-potential force, an equation of state, two lattices
 // one step from lattice cur, whose density plane is L.rho (and psi' in L.psip); the next into rho_next
 cudaError_t launch_fp64_step(const Lattice<double>& L, double* rho_next, int cur, cudaStream_t s);
