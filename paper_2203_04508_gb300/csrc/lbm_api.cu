@@ -457,7 +457,7 @@ bool fused(const lbm_ctx* c) {
   return c->fused_ok && !c->fp64 && c->cfg.layout == LBM_LAYOUT_AB && c->cfg.eos != LBM_EOS_NONE && !c->slab.on &&
          c->mu_kind < 0 && !c->collide_set;
 }
-// ... on one lattice in AA order?  (2048 x 4096 198 -> 172 us a step, 512 x 512 30 -> 15.7)
+// ... on one lattice in AA order?  (2048 x 4096 214 -> 178 us a step, 512 x 512 30 -> 15.4)
 bool fused_aa(const lbm_ctx* c) {
   return c->fused_ok && !c->fp64 && c->cfg.layout == LBM_LAYOUT_AA && c->cfg.eos != LBM_EOS_NONE && !c->slab.on &&
          c->mu_kind < 0 && !c->collide_set;
@@ -1924,13 +1924,10 @@ lbm_status fused_tables(lbm_batch* b) {
   int dev = 0, sms = 0;
   BCUDA(b, cudaGetDevice(&dev));
   BCUDA(b, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  long long tiles = 0, strip_rows = 0;
-  for (auto* c : b->ctx) {
-    tiles += fused_tiles(c->cfg.nx, c->cfg.ny);
-    strip_rows += fused_strip_rows(c->cfg.nx, c->cfg.ny);
-  }
+  long long strip_rows = 0;
+  for (auto* c : b->ctx) strip_rows += fused_strip_rows(c->cfg.nx, c->cfg.ny);
   FusedBatch& F = b->fb;
-  F.rows = fused_batch_rows(b->n, tiles, strip_rows, sms);
+  F.rows = fused_batch_rows(strip_rows, sms);
   std::vector<Lattice<float>> lats;
   for (int p = 0; p < 2; ++p)
     for (auto* c : b->ctx) lats.push_back(fused_lattice(c, c->Lf, p));

@@ -18,19 +18,24 @@
 // those nodes in two planes (the pass stores it in the rows next to solids).  The densities of
 // boundary nodes come from k_bc_fused, those of the solid layers from k_solids.
 //
-// On the 2048 x 4096 impact lattice a step takes 0.145 ms against 0.192 ms for the separate passes
-// (1024 x 1024 with 16 drops 33 against 45 us, 131 x 97 9.0 against 29 us); the pass itself 0.13 ms,
-// 661 MB of DRAM traffic.  What was tried on the way there: the density formed from the populations
-// at the start of the same pass instead of the end of the previous one (72 instead of 80 bytes a
-// node, but the populations of four more rows wait in shared memory for their collision: 10 warps
-// an SM instead of 12, 0.19 ms); 8-byte cp.async through L1 instead of 16-byte ones past it (the
-// L1 lines left beside 200 KB of shared memory bound the loads in flight: 0.20 against 0.15 ms);
-// one row an iteration, conditions inside (0.22 ms: divergent branches and short chains); four
-// columns a lane (half the shared-memory and store instructions, but 7 warps an SM: 0.20 ms).
+// On the 2048 x 4096 impact lattice a step takes 0.148 ms against 0.192 ms for the separate passes
+// (2048 x 2048 84 against 110 us, 1024 x 1024 with 16 drops 33 against 45, 131 x 97 9.0 against 29);
+// the pass itself 0.13 ms, 661 MB of DRAM traffic.  What bounds a walk is instruction issue: twelve
+// warps an SM (three in each quarter, which is what their registers allow) issue 0.6 instructions a
+// clock and scheduler, a third of them integer work and constants' moves; DRAM is at 55 %.  What was
+// tried on the way there: the density formed from the populations at the start of the same pass
+// instead of the end of the previous one (72 instead of 80 bytes a node, but the populations of four
+// more rows wait in shared memory for their collision: 0.19 ms); 8-byte cp.async through L1 instead
+// of 16-byte ones past it (the L1 lines left beside 200 KB of shared memory bound the loads in
+// flight: 0.20 against 0.15 ms); two rows an iteration with a second path for rows that hold solids
+// (0.143 ms on 2048 x 4096, but 1.6 times the code, which the instruction cache pays for: 92 against
+// 82 us on 1672 x 2453, 0.137 against 0.128 ms with the pseudopotential), and with three paths 0.175;
+// four columns a lane (half the shared-memory and store instructions, but 7 warps an SM: 0.20 ms);
+// sixteen warps of 128 registers (0.153 ms).
 //
 // Batches run the same kernels over flat lists of all instances' tiles (walks, where the instances
 // are large), links and layers, each block with its instance's descriptor in shared memory: 64
-// lattices of 128..768 take 398 us a step against 590 us for the persistent kernel (k_batch: six grid
+// lattices of 128..768 take 368 us a step against 590 us for the persistent kernel (k_batch: six grid
 // barriers a step, 890 instructions a node), 256 of 64..128 119 against 217 us.
 #include <algorithm>
 #include <vector>
@@ -45,12 +50,13 @@ namespace lbmgb {
 namespace {
 
 constexpr int FW = 64;                 // columns a warp holds
-constexpr int FD = 4;                  // rows of populations (and densities) requested ahead
+constexpr int FD = 4;                  // rows of populations in shared memory
+constexpr int AHEAD = 3;               // rows of populations and densities requested ahead
 constexpr int ROW_F = 9 * FW * 4;      // bytes of one row's populations in shared memory
 constexpr int HX = 4;                  // columns held on each side of the strip's outputs
 constexpr int OUT = FW - 2 * HX;       // output columns
 constexpr int SP = FW / 2 + 4;         // pairs of a density or chemical-potential row: two more each side
-constexpr int RHO_ROWS = 16, MU_ROWS = 8;   // rows of the two rings (psi: RHO_ROWS)
+constexpr int RHO_ROWS = 8, MU_ROWS = 4;   // rows of the two rings (psi: RHO_ROWS)
 constexpr int RHO_CHUNKS = SP / 2;     // 16-byte pieces of a density row
 
 // LEAD: rows between the newest density row and the collision
@@ -79,9 +85,10 @@ __device__ __forceinline__ int wrap_col(int c, int nx) {
 
 // The walk: one warp takes a strip up through a band of rows.  At row r it forms the chemical
 // potential of row r - 2, whose stencil is complete then, collides row r - 4 and completes the
-// density of row r - 5.  Rows arrive by cp.async FD rows ahead; densities and chemical potentials
+// density of row r - 5.  Rows arrive by cp.async three rows ahead; densities and chemical potentials
 // live in rings in shared memory that no other warp reads, so one __syncwarp a row is all the
-// synchronisation.
+// synchronisation.  All rows take one path, whose only branches are warp-wide: solid nodes' chemical
+// potential is chosen, not branched for, and the classes that decide are fetched two rows early.
 //
 // One warp: the populations streaming into the output columns of strip `strip` in rows [ya, yb),
 // and those nodes' density (psi), from the state in lattice `cur`.
@@ -92,7 +99,8 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
   const int lane = threadIdx.x & 31;
   const int x0 = strip * OUT, c = x0 - HX + 2 * lane;   // this lane's columns c, c + 1
   const bool mine = lane >= HX / 2 && lane < 32 - HX / 2;
-  const bool out1 = mine && c + 1 < L.nx, one = mine && c + 1 == L.nx;   // both outputs; the first only
+  // (with nx odd the last pair's second column is the row's padding, which nothing reads)
+  const bool out1 = mine && c < L.nx;
   const int ca = wrap_col(c, L.nx), cb = wrap_col(c + 1, L.nx);   // inside the lattice
   // Rows arrive in 16-byte pieces of four columns, straight into shared memory (not through L1,
   // which would bound the rows in flight).  With nx a multiple of four a wrapped piece stays one
@@ -167,23 +175,22 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
   // rows collided: ya - 1 .. yb (AA: the band's own); the newest density row r runs from rb to re
   const int ylo = AA ? ya : ya - 1, yhi = AA ? yb - 1 : yb;
   const int rb = ylo + (PSEUDO ? 1 : 0), re = yhi + LEAD;
-  // density row r + FD and the populations of the row FD above the one collided with row r
+  // density row r + AHEAD and the populations of the row AHEAD above the one collided with row r
   auto request = [&](int r) {
-    if (r + FD <= re) load_rho(r + FD);
-    const int y = r - LEAD + FD;
+    if (r + AHEAD <= re) load_rho(r + AHEAD);
+    const int y = r - LEAD + AHEAD;
     if (y >= ylo && y <= yhi) load_f(y);
     cp_commit();
   };
-  // the classes of columns c and c + 1 of the row, in bytes 0 and 1
-  auto kind_row = [&](int r) -> unsigned {
+  // The classes of columns c and c + 1 of a row.  (Two registers that nothing touches before the row's
+  // turn: combining them at once would wait for the loads.)
+  struct Kinds { unsigned a, b; };
+  auto kind_row = [&](int r) -> Kinds {
     const uint8_t* k = L.kind + row_of(r) * L.pitch;
-    if ((L.nx & 1) == 0) return *reinterpret_cast<const unsigned short*>(k + ca);
-    return k[ca] | ((unsigned)k[cb] << 8);
+    return {k[ca], k[cb]};
   };
   // bit 0 / 1: column c / c + 1 is fluid
-  auto fluid_bits = [](unsigned k) {
-    return ((k & 0xffu) == KIND_FLUID ? 1u : 0u) | ((k >> 8) == KIND_FLUID ? 2u : 0u);
-  };
+  auto fluid_bits = [](Kinds k) { return (k.a == KIND_FLUID ? 1u : 0u) | (k.b == KIND_FLUID ? 2u : 0u); };
   auto load_pops = [&](int y, float2 (&v)[9]) {
     const float2* d = fs + fslot(y);
 #pragma unroll
@@ -282,12 +289,11 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
         for (int i = 0; i < 9; ++i) {
           float* const p = fone + opp(i) * (long long)L.plane + n;
           if (out1) *reinterpret_cast<float2*>(p) = v[i];
-          else if (one) *p = v[i].x;
         }
       } else {
         // slot i of x + e_i: the slots read
         const int nm = row_of(y - 1) * L.pitch, n0 = y * L.pitch, np = row_of(y + 1) * L.pitch;
-        const bool w0 = (out1 || one) && (fl & 1u), w1 = out1 && (fl & 2u);
+        const bool w0 = out1 && (fl & 1u), w1 = out1 && (fl & 2u) && c + 1 < L.nx;
 #pragma unroll
         for (int i = 0; i < 9; ++i) {
           float* const p = fone + i * (long long)L.plane + (ey(i) == 0 ? n0 : ey(i) > 0 ? np : nm);
@@ -313,24 +319,6 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
         put(fout + 8ll * L.plane, n - L.pitch, r8);
         put(rout, n - L.pitch, q);
       }
-    } else if (one) {
-      auto put = [&](float* plane, int at, float a) { plane[at] = a; };
-      if (mid) {
-        put(fout, n, v[0].x);
-        put(fout + 1ll * L.plane, n, r1.x);
-        put(fout + 3ll * L.plane, n, l3.x);
-      }
-      if (up) {
-        put(fout + 2ll * L.plane, n + L.pitch, v[2].x);
-        put(fout + 5ll * L.plane, n + L.pitch, r5.x);
-        put(fout + 6ll * L.plane, n + L.pitch, l6.x);
-      }
-      if (dn) {
-        put(fout + 4ll * L.plane, n - L.pitch, v[4].x);
-        put(fout + 7ll * L.plane, n - L.pitch, l7.x);
-        put(fout + 8ll * L.plane, n - L.pitch, r8.x);
-        put(rout, n - L.pitch, q.x);
-      }
     }
     in.c0 = v[0];
     in.s13 = add_rn(r1, l3);
@@ -342,125 +330,69 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
     in.e6 = l6;
   };
 
-  // density rows below rb, then the first FD requests
-#pragma unroll
+  // density rows below rb, then the first requests
+#pragma unroll 1
   for (int k = 1; k <= (PSEUDO ? 2 : 4); ++k) load_rho(rb - k);
-#pragma unroll
-  for (int k = 0; k < FD; ++k) {
-    cp_commit();                       // (the group of walls that precedes a request is empty here)
-    request(rb - FD + k);
-  }
-  unsigned k0 = kind_row(rb), k1 = kind_row(rb + 1);   // of rows r, r + 1
+#pragma unroll 1
+  for (int k = AHEAD; k >= 1; --k) request(rb - k);
+  Kinds k0 = kind_row(rb), k1 = kind_row(rb + 1);   // of rows r, r + 1
   unsigned bits = 0;                   // fluid bits of this lane, two per row, the newest row lowest
   unsigned solid = 0, none = 0;        // per row: some column of the warp is not fluid / none is
-  // the two rows below the first: their classes decide about walls, and about the force rows
-#pragma unroll
-  for (int k = 2; k >= 1; --k) {
-    const unsigned fl = fluid_bits(kind_row(rb - k));
+  // the constant chemical potential of a row's solid nodes
+  auto walls_of = [&](int r, unsigned fl) {
+    float2 w = make_float2(0.f, 0.f);
+    const float* m = L.mu + row_of(r) * L.pitch;
+    if (!PSEUDO && !(fl & 1u)) w.x = m[ca];
+    if (!PSEUDO && !(fl & 2u)) w.y = m[cb];
+    return w;
+  };
+  // Rows r - 2 and r - 1 came before the loop: their classes and walls (w2, w1).  Own pairs of density
+  // rows r - 5, r - 6 and chemical-potential rows r - 5, r - 6 stay in registers: no neighbour needs
+  // them, and the rings get by with 8 and 4 rows.
+  float2 w2, w1, p5, p6, m5, m6;
+  p5 = p6 = m5 = m6 = make_float2(0.f, 0.f);
+  {
+    const unsigned f2 = fluid_bits(kind_row(rb - 2)), f1 = fluid_bits(kind_row(rb - 1));
+    bits = (f2 << 2) | f1;
+    solid = (__all_sync(0xffffffffu, f2 == 3u) ? 0u : 2u) | (__all_sync(0xffffffffu, f1 == 3u) ? 0u : 1u);
+    none = (__any_sync(0xffffffffu, f2 != 0u) ? 0u : 2u) | (__any_sync(0xffffffffu, f1 != 0u) ? 0u : 1u);
+    w2 = walls_of(rb - 2, f2);
+    w1 = walls_of(rb - 1, f1);
+  }
+#pragma unroll 1
+  for (int r = rb; r <= re; ++r) {
+    const int y = r - LEAD;
+    const unsigned fl = fluid_bits(k0);
     bits = (bits << 2) | fl;
     solid = (solid << 1) | (__all_sync(0xffffffffu, fl == 3u) ? 0u : 1u);
     none = (none << 1) | (__any_sync(0xffffffffu, fl != 0u) ? 0u : 1u);
-    if (!PSEUDO && fl != 3u) {
-      // (they take part in the first collisions: their walls now)
-      const float* m = L.mu + row_of(rb - k) * L.pitch;
-      float2* const w = ms + mslot(rb - k);
-      if (!(fl & 1u)) w->x = m[ca];
-      if (!(fl & 2u)) w->y = m[cb];
-    }
-  }
-  for (int r = rb; r <= re;) {
-    const int y = r - LEAD;
-    const bool all0 = __all_sync(0xffffffffu, k0 == 0u), all1 = __all_sync(0xffffffffu, k1 == 0u);   // (fluid is 0)
-    // groups are committed in the order walls(r - 2), request(r - 2), walls(r - 1), request(r - 1)
-    if (r < re && y >= ylo && all0 && all1 && !(solid & ((2u << LEAD) - 1u))) {
-      // Rows y - 1 .. r + 1 hold no solid node: the chemical potentials of rows r - 2 and r - 1 and
-      // the collisions of rows y and y + 1 in one run of instructions without branches, whose chains
-      // overlap.
-      bits = (bits << 4) | 15u;
-      solid <<= 2;
-      none <<= 2;
-      k0 = kind_row(min(r + 2, re));
-      k1 = kind_row(min(r + 3, re));
-      cp_wait<4>();                    // density rows r, r + 1 and population rows y, y + 1 are in
-      __syncwarp();
-      // the populations into registers; their slots take the rows FD above at once, which have two
-      // iterations' time to arrive
-      float2 w0[9], w1[9];
-      load_pops(y, w0);
-      load_pops(y + 1, w1);
-      cp_commit();
-      request(r);
-      cp_commit();
-      request(r + 1);
-      auto collide_stream = [&](float2 (&w)[9], int yy, auto&& force) {
-        float2 drho, jx, jy, Fx, Fy;
-        moments(w, drho, jx, jy);
-        const float2 rho = add_rn(splat<float2>(L.rho_ref), drho);
-        force(rho, Fx, Fy);
-        collide_node(L, w, rho, drho, jx, jy, Fx, Fy);
-        stream_row(w, yy, 3u);
-      };
-      if constexpr (PSEUDO) {
-        collide_stream(w0, y, [&](float2 rho, float2& Fx, float2& Fy) { force_pp_at(rho, y, Fx, Fy); });
-        collide_stream(w1, y + 1, [&](float2 rho, float2& Fx, float2& Fy) { force_pp_at(rho, y + 1, Fx, Fy); });
-      } else {
-        const float2 p6 = rs[rslot(r - 6)], p5 = rs[rslot(r - 5)], t0 = rs[rslot(r)], t1 = rs[rslot(r + 1)];
-        const float2* q4 = rs + rslot(r - 4);
-        const float2* q3 = rs + rslot(r - 3);
-        const float2* q2 = rs + rslot(r - 2);
-        const float2* q1 = rs + rslot(r - 1);
-        const float2 p4 = q4[0], p3 = q3[0], p2 = q2[0], p1 = q1[0];
-        const float2 mu0 = mu_at(q2[-1], p2, q2[1], p1, t0, p3, p4);
-        const float2 mu1 = mu_at(q1[-1], p1, q1[1], t0, t1, p2, p3);
-        const float2 m6 = ms[mslot(r - 6)], m5 = ms[mslot(r - 5)];
-        const float2* z4 = ms + mslot(r - 4);
-        const float2* z3 = ms + mslot(r - 3);
-        const float2 m4 = z4[0], m3 = z3[0];
-        const float2 dm0 = dx_of(z4[-1], m4, z4[1]), dr0 = dx_of(q4[-1], p4, q4[1]);
-        const float2 dm1 = dx_of(z3[-1], m3, z3[1]), dr1 = dx_of(q3[-1], p3, q3[1]);
-        ms[mslot(r - 2)] = mu0;
-        ms[mslot(r - 1)] = mu1;
-        collide_stream(w0, y, [&](float2 rho, float2& Fx, float2& Fy) {
-          Fx = force_cp(rho, L.gx, dm0, dr0);
-          Fy = force_cp(rho, L.gy, diff4_of(m3, m5, mu0, m6), diff4_of(p3, p5, p2, p6));
-        });
-        collide_stream(w1, y + 1, [&](float2 rho, float2& Fx, float2& Fy) {
-          Fx = force_cp(rho, L.gx, dm1, dr1);
-          Fy = force_cp(rho, L.gy, diff4_of(mu0, m4, mu1, m5), diff4_of(p2, p4, p1, p5));
-        });
-      }
-      r += 2;
-      continue;
-    }
-    // ---- one row, solids anywhere
-    const unsigned fl = fluid_bits(k0);
     k0 = k1;
     k1 = kind_row(min(r + 2, re));
-    bits = (bits << 2) | fl;
-    solid = (solid << 1) | (all0 ? 0u : 1u);
-    none = (none << 1) | (__any_sync(0xffffffffu, fl != 0u) ? 0u : 1u);
-    cp_wait<3>();                      // density row r, population row y, the walls of row r - 2
+    cp_wait<AHEAD - 1>();              // density row r and population row y are in
     __syncwarp();
-    if (!PSEUDO) {
-      if (!all0) {
-        // the walls' chemical potential into row r's place in the ring
-        const float* m = L.mu + row_of(r) * L.pitch;
-        float2* const w = ms + mslot(r);
-        if (!(fl & 1u)) cp4(&w->x, m + ca);
-        if (!(fl & 2u)) cp4(&w->y, m + cb);
+    request(r);
+    const float2 wn = walls_of(r, fl);
+    // chemical potential of row r - 2, the walls' where solid
+    float2 p4, p3, p2, mu;
+    auto chem = [&]() {
+      const float2* q = rs + rslot(r - 2);
+      const float2 p1 = rs[rslot(r - 1)], t0 = rs[rslot(r)];
+      p4 = rs[rslot(r - 4)];
+      p3 = rs[rslot(r - 3)];
+      p2 = q[0];
+      mu = mu_at(q[-1], p2, q[1], p1, t0, p3, p4);
+      if (!(bits & 16u)) mu.x = w2.x;
+      if (!(bits & 32u)) mu.y = w2.y;
+      ms[mslot(r - 2)] = mu;
+    };
+    if (y < ylo || (none & (1u << LEAD))) {
+      // nothing to collide
+      if (!PSEUDO) {
+        chem();
+        m6 = m5;
+        m5 = ms[mslot(r - 4)];
       }
-      if (!(none & 4u)) {
-        // chemical potential of row r - 2
-        const float2* q = rs + rslot(r - 2);
-        const float2 mu = mu_at(q[-1], q[0], q[1], rs[rslot(r - 1)], rs[rslot(r)], rs[rslot(r - 3)], rs[rslot(r - 4)]);
-        float2* const w = ms + mslot(r - 2);
-        if (bits & (1u << 4)) w->x = mu.x;
-        if (bits & (2u << 4)) w->y = mu.y;
-      }
-    }
-    cp_commit();
-    // collision and streaming of row y
-    if (y >= ylo && !(none & (1u << LEAD))) {
+    } else {
       float2 v[9];
       load_pops(y, v);
       float2 drho, jx, jy, Fx, Fy;
@@ -469,30 +401,39 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
       if constexpr (PSEUDO) {
         force_pp_at(rho, y, Fx, Fy);
       } else {
-        const float2* q = rs + rslot(y);
-        const float2* z = ms + mslot(y);
-        Fx = force_cp(rho, L.gx, dx_of(z[-1], z[0], z[1]), dx_of(q[-1], q[0], q[1]));
-        Fy = force_cp(rho, L.gy, diff4_of(ms[mslot(y + 1)], ms[mslot(y - 1)], ms[mslot(y + 2)], ms[mslot(y - 2)]),
-                      diff4_of(rs[rslot(y + 1)], rs[rslot(y - 1)], rs[rslot(y + 2)], rs[rslot(y - 2)]));
+        chem();
+        const float2* q = rs + rslot(r - 4);
+        const float2* z = ms + mslot(r - 4);
+        const float2 m4 = z[0], m3 = ms[mslot(r - 3)];
+        Fx = force_cp(rho, L.gx, dx_of(z[-1], m4, z[1]), dx_of(q[-1], p4, q[1]));
+        Fy = force_cp(rho, L.gy, diff4_of(m3, m5, mu, m6), diff4_of(p3, p5, p2, p6));
+        m6 = m5;
+        m5 = m4;
       }
-      if ((solid & (7u << (LEAD - 1))) && y >= ya && y < yb) {
+      const unsigned fy = (bits >> (2 * LEAD)) & 3u;
+      if (solid & (7u << (LEAD - 1))) {
         // next to a solid: the force for the boundary phase
-        const unsigned fy = (bits >> (2 * LEAD)) & 3u;
         const int n = y * L.pitch + c;
-        if ((out1 || one) && (fy & 1u)) { L.fx[n] = Fx.x; L.fy[n] = Fy.x; }
-        if (out1 && (fy & 2u)) { L.fx[n + 1] = Fx.y; L.fy[n + 1] = Fy.y; }
+        if (out1 && y >= ya && y < yb) {
+          if (fy & 1u) { L.fx[n] = Fx.x; L.fy[n] = Fy.x; }
+          if (fy & 2u) { L.fx[n + 1] = Fx.y; L.fy[n + 1] = Fy.y; }
+        }
       }
       collide_node(L, v, rho, drho, jx, jy, Fx, Fy);
-      stream_row(v, y, (bits >> (2 * LEAD)) & 3u);
+      stream_row(v, y, fy);
     }
-    request(r);
-    ++r;
+    p6 = p5;
+    p5 = p4;
+    w2 = w1;
+    w1 = wn;
   }
   cp_wait<0>();
 }
 
+// (152 registers: twelve warps an SM either way, and the schedule the compiler finds within them is 2 to
+// 4 % faster than its own choice)
 template <bool PSEUDO, int AA = 0>
-__global__ void __launch_bounds__(32) k_walk(const __grid_constant__ Lattice<float> L, int cur, int strips, int rows) {
+__global__ void __maxnreg__(152) k_walk(const __grid_constant__ Lattice<float> L, int cur, int strips, int rows) {
   extern __shared__ __align__(16) char smem[];
   const int band = blockIdx.x / strips, strip = blockIdx.x - band * strips;
   const int ya = band * rows, yb = min(ya + rows, L.ny);
@@ -545,7 +486,7 @@ __device__ __forceinline__ void tile(const Lattice<float>& L, int cur, int strip
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int x0 = strip * OUT, c = x0 - HX + 2 * lane;
   const bool mine = lane >= HX / 2 && lane < 32 - HX / 2;
-  const bool out1 = mine && c + 1 < L.nx, one = mine && c + 1 == L.nx;
+  const bool out1 = mine && c < L.nx;   // (both columns: walk)
   const int ca = wrap_col(c, L.nx), cb = wrap_col(c + 1, L.nx);
   const bool split = (L.nx & 3) != 0 && (x0 - 2 * HX < 0 || x0 + OUT + 2 * HX > L.nx);
   const float* __restrict__ fin = L.f[cur];
@@ -658,7 +599,6 @@ __device__ __forceinline__ void tile(const Lattice<float>& L, int cur, int strip
       if (L.mu_out && m >= ya && m < yb) {
         float* p = L.mu_out + m * L.pitch + c;
         if (out1) *reinterpret_cast<float2*>(p) = v;
-        else if (one) *p = v.x;
       }
     }
     __syncthreads();
@@ -705,9 +645,6 @@ __device__ __forceinline__ void tile(const Lattice<float>& L, int cur, int strip
       if (out1) {
         *reinterpret_cast<float2*>(L.fx + nf) = Fx;
         *reinterpret_cast<float2*>(L.fy + nf) = Fy;
-      } else if (one) {
-        L.fx[nf] = Fx.x;
-        L.fy[nf] = Fy.x;
       }
     }
     collide_node(L, v, rho, drho, jx, jy, Fx, Fy);
@@ -722,12 +659,11 @@ __device__ __forceinline__ void tile(const Lattice<float>& L, int cur, int strip
       for (int i = 0; i < 9; ++i) {
         float* p = fin1 + opp(i) * (long long)L.plane + n;
         if (out1) *reinterpret_cast<float2*>(p) = v[i];
-        else if (one) *p = v[i].x;
       }
     } else if constexpr (AA == 2) {
       // slot i of x + e_i: the slots read
       const uint8_t* kd = L.kind + y * L.pitch;
-      const bool w0 = (out1 || one) && kd[c] == KIND_FLUID, w1 = out1 && kd[c + 1] == KIND_FLUID;
+      const bool w0 = out1 && kd[c] == KIND_FLUID, w1 = out1 && c + 1 < L.nx && kd[c + 1] == KIND_FLUID;
       const int nm = row_of(y - 1) * L.pitch, n0 = y * L.pitch, np = row_of(y + 1) * L.pitch;
       const int cm = c == 0 ? L.nx - 1 : c - 1, c1 = c + 1 == L.nx ? 0 : c + 1, c2 = c1 + 1 == L.nx ? 0 : c1 + 1;
 #pragma unroll
@@ -752,23 +688,6 @@ __device__ __forceinline__ void tile(const Lattice<float>& L, int cur, int strip
         put(4, n - L.pitch, v[4]);
         put(7, n - L.pitch, l7);
         put(8, n - L.pitch, r8);
-      }
-    } else if (one) {
-      auto put = [&](int i, int at, float a) { fout[(long long)i * L.plane + at] = a; };
-      if (mid) {
-        put(0, n, v[0].x);
-        put(1, n, r1.x);
-        put(3, n, l3.x);
-      }
-      if (up) {
-        put(2, n + L.pitch, v[2].x);
-        put(5, n + L.pitch, r5.x);
-        put(6, n + L.pitch, l6.x);
-      }
-      if (dn) {
-        put(4, n - L.pitch, v[4].x);
-        put(7, n - L.pitch, l7.x);
-        put(8, n - L.pitch, r8.x);
       }
     }
     // what the densities of rows y - 1, y and y + 1 are summed from, in place of the populations
@@ -801,7 +720,6 @@ __device__ __forceinline__ void tile(const Lattice<float>& L, int cur, int strip
       continue;
     }
     if (out1) *reinterpret_cast<float2*>(p) = q;
-    else if (one) *p = q.x;
   }
 }
 
@@ -1094,28 +1012,33 @@ inline unsigned blocks_for(int n, int b) { return (unsigned)((n + b - 1) / b); }
 
 }  // namespace
 
-long long fused_tiles(int nx, int ny) { return (long long)((nx + OUT - 1) / OUT) * ((ny + TH_M - 1) / TH_M); }
+static long long fused_tiles(int nx, int ny) { return (long long)((nx + OUT - 1) / OUT) * ((ny + TH_M - 1) / TH_M); }
 constexpr int MIN_TILE_ROWS = 2;
 
 // How the pass runs on a lattice of nx x ny, counted in tiles of 14 rows:
-//   from 28 tiles an SM on the walk wins, whose rows are formed twice only at the bands' ends and
-//   whose loads run through all of its rows (walk / tiles, us a step: 1024 x 1536 50.3 / 43.4,
-//   1600 x 2048 75.8 / 74.7, 2048 x 2048 90.6 / 90.7, 2048 x 3072 118 / 130, 2048 x 4096 145 / 175).
-//   A walk takes as many rows as give every SM 24 warps: two waves of what fits at once, so that the
-//   warps whose rows hold solid nodes, which take longer, do not set the pass's time alone (one wave:
-//   175 against 157 us on 2048 x 4096).
+//   from 10 tiles an SM on the walk wins, whose rows are formed twice only at the bands' ends and
+//   whose loads run through all of its rows (walk / tiles, us a step: 1001 x 1024 (8.8 tiles) 35.8 /
+//   32.0, 1024 x 1024 (9.3) 32.6 / 33.2, 1201 x 1300 (13.5) 43.4 / 46.0, 1024 x 1536 (13.8) 37.1 / 45.2,
+//   1200 x 2200 (22.7) 57 / 67, 2048 x 4096 148 / 175).  A walk takes as many rows as give every SM the
+//   twelve warps that fit at once (one wave / two: 1671 x 2453 87 / 92, 2048 x 2048 84 / 87), but where
+//   that is more than 64 rows half as many, so that the walks that take longer (strips at an end with
+//   nx % 4 != 0, rows with solids) do not set the pass's time alone (2048 x 4096 151 / 148).
 //   below, tiles of at most 14 rows and eight warps, or (from 6 tiles an SM) 10 rows and four warps,
-//   of which five fit an SM and so overlap their phases better (1024 x 1536 44.9 / 43.4, 800 x 800
-//   21.7 / 22.8).  The bands have equal heights and as many as give every SM the same number of tiles
-//   (500 x 300 13.0 -> 11.8, 96 x 96 10.3 -> 8.2).
+//   of which five fit an SM and so overlap their phases better (800 x 800 21.7 / 22.8).  The bands have
+//   equal heights and as many as give every SM the same number of tiles (500 x 300 13.0 -> 11.8, 96 x 96
+//   10.3 -> 8.2).
 PassPlan fused_plan(int nx, int ny, int sms) {
   const int strips = (nx + OUT - 1) / OUT;
   const long long tiles = fused_tiles(nx, ny);
   PassPlan p;
-  if (tiles >= 28LL * sms) {
+  if (tiles >= 10LL * sms) {
     p.kind = PassPlan::WALK;
-    const long long bands = std::max(1LL, 24LL * sms / strips);
-    p.rows = std::max(16, (int)((ny + bands - 1) / bands));
+    auto rows = [&](int per_sm) {
+      const long long bands = std::max(1LL, (long long)per_sm * sms / strips);
+      return std::max(8, (int)((ny + bands - 1) / bands));
+    };
+    p.rows = rows(12);
+    if (p.rows > 64) p.rows = rows(24);
     return p;
   }
   p.kind = tiles >= 6LL * sms ? PassPlan::TILE_L : PassPlan::TILE_M;
@@ -1136,8 +1059,8 @@ PassPlan fused_tile_plan(int nx, int ny, int sms) {
 }
 
 // ... of an AA lattice: the same walks; its tiles are of the first shape, whose bands leave fewer
-// outermost rows to k_layers_aa.  (separate passes / fused, us a step: 131 x 97 24.6 / 9.5, 512 x 512 30 / 15.7,
-// 1024 x 1024 46 / 33, 1600 x 2000 94 / 92, 2048 x 4096 198 / 172.)
+// outermost rows to k_layers_aa.  (separate passes / fused, us a step: 131 x 97 24.6 / 9.3, 512 x 512
+// 30 / 15.4, 1024 x 1024 46 / 33, 1600 x 2000 95 / 80, 2048 x 4096 214 / 178.)
 PassPlan fused_aa_plan(int nx, int ny, int sms) {
   PassPlan p = fused_plan(nx, ny, sms);
   if (p.kind != PassPlan::TILE_L) return p;
@@ -1249,14 +1172,13 @@ void fused_batch_caps(int nx, int ny, long long bnodes, long long s1, long long 
   *bc += (bnodes + BC_BLOCK - 1) / BC_BLOCK;
   *solid += (8 * s2 + SOLID_BLOCK - 1) / SOLID_BLOCK + (s1 + SOLID_BLOCK - 1) / SOLID_BLOCK + 1;
 }
-// Rows a warp of the batch walks, or 0 for tiles.  Small lattices are better off in tiles however
-// many there are (64 lattices of 128..768: 407 us a step in tiles, 446 walked -- a quarter of their
-// rows hold solid nodes, and a walk through such rows is slow), so the batch walks where its mean
-// lattice would on its own.
-int fused_batch_rows(int n, long long tiles, long long strip_rows, int sms) {
-  if (tiles < 28LL * sms * n) return 0;
-  const long long rows = (strip_rows + 24LL * sms - 1) / (24LL * sms);
-  return rows < 32 ? 32 : (int)rows;
+// Rows a warp of the batch walks, or 0 for tiles: 64 walks an SM, several waves that even out the
+// instances' widths and solids (48 / 64 / 96: 367 / 364 / 375 us a step on 64 lattices of 128..768), if
+// that leaves them 20 rows (walk / tiles, with its rows: 64 of 128..768 (30 rows) 368 / 401, 60 of
+// 200..400 (11) 196 / 180, 12 of 500..768 (11) 152 / 133, 256 of 64..128 (5) 144 / 121).
+int fused_batch_rows(long long strip_rows, int sms) {
+  const long long rows = strip_rows / (64LL * sms);
+  return rows < 20 ? 0 : (int)rows;
 }
 long long fused_strip_rows(int nx, int ny) { return (long long)((nx + OUT - 1) / OUT) * ny; }
 

@@ -118,9 +118,8 @@ struct FusedBatch {
   const int2* solid;              // (instance, block)
   int n_pass, n_bc, n_solid, rows;   // rows > 0: walks of about that many rows, 0: tiles
 };
-long long fused_tiles(int nx, int ny);
 long long fused_strip_rows(int nx, int ny);
-int fused_batch_rows(int n, long long tiles, long long strip_rows, int sms);
+int fused_batch_rows(long long strip_rows, int sms);
 void fused_batch_items(int k, int nx, int ny, int n_bnodes, int n_s1, int n_s2, int rows, std::vector<int4>* pass,
                        std::vector<int2>* bc, std::vector<int2>* solid);
 void fused_batch_caps(int nx, int ny, long long bnodes, long long s1, long long s2, long long* pass, long long* bc,

@@ -109,7 +109,7 @@ def test_fused_batch_equals_the_persistent_kernel_and_single_lattices(walk):
     import paper_2203_04508_gb300 as G
     scs = [S.small_parity(), _box(64, 70, walls=1), _box(117, 61), S.e1_flat_drop(0.3, 60.0, nx=90, ny=75, r0=18.0)]
     if walk:
-        scs = [_box(2100, 2001, walls=1), _box(2000, 2100)]
+        scs = [_box(2100, 2001, walls=1), _box(2000, 2100), _box(1999, 2300)]
     a, b = (G.Batch([sc.physics() for sc in scs]) for _ in range(2))
     b.set_spin_limit((1 << 22) + 1)
     for batch in (a, b):
