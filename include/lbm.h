@@ -194,11 +194,12 @@ lbm_status lbm_init(lbm_ctx* ctx, const lbm_init_spec* init);
  * chemical potential (Eq. 12); nonideal force (Eq. 9) with exact-difference forcing
  * (Eqs. 13-14), collision (Eq. 4) and streaming (Eq. 5); then every cut link by Eq. 16
  * (q < 1/2) or Eq. 17 (q >= 1/2) with the per-node compensation of Eq. 18 accumulated in FP64.
- * FP32 lattices on two population lattices with an equation of state (not slabs) run the fused
- * step: one pass over the populations, then the links, then the solid layers.  Others, and a
- * lattice whose kernels the caller chose (lbm_set_collide_kernel, lbm_set_mu_kernel), run the
- * separate passes, the density pass of the next state overlapping the links on a second stream
- * the context creates on first use (ordered with the context's stream by events).  Both give the
+ * FP32 lattices with an equation of state (on two population lattices or one; not slabs) run the
+ * fused step: one pass over the populations, then the links, then the solid layers.  FP64 ones on two
+ * population lattices with the chemical-potential force run four kernels: chemical potential,
+ * collision, links, density with the solid layers.  Others, and a lattice whose kernels the caller
+ * chose (lbm_set_collide_kernel, lbm_set_mu_kernel), run the separate passes, the density pass of the next state overlapping the links on a second stream
+ * the context creates on first use (ordered with the context's stream by events).  All give the
  * same values, bit for bit.  No device memory is allocated; to the caller the work is on the
  * context's stream. */
 lbm_status lbm_step(lbm_ctx* ctx, int64_t n);
@@ -409,14 +410,14 @@ lbm_status lbm_batch_build_links(lbm_batch* b);
 /* lbm_init for every instance with specs[k] (n specs).  Synchronises. */
 lbm_status lbm_batch_init(lbm_batch* b, const lbm_init_spec* specs);
 
-/* Advances every instance n steps.  Where all of them run the fused step (lbm_step: FP32, two
- * population lattices, an equation of state) its three kernels run over flat lists of all
+/* Advances every instance n steps.  Where all of them run the fused step on two population
+ * lattices (lbm_step) its three kernels run over flat lists of all
  * instances' work, captured into CUDA graphs on first use; a batch whose poll budget the caller
  * set (lbm_batch_set_spin_limit, other than the default) and every other batch runs ONE cooperative
  * launch of a persistent kernel (captured for this n), to which the tile shape and the schedule
- * below belong.  Both give the same values, bit for bit.  In the persistent kernel each step runs the phases of lbm_step over all
- * instances' work, separated by grid barriers; per-instance compensation sums go to each
- * instance's ring as with lbm_step.  Asynchronous; lbm_batch_check reports a barrier timeout. */
+ * below belong.  Both give the same values, bit for bit.  In the persistent kernel each step runs the
+ * phases of lbm_step over all instances' work, separated by grid barriers; per-instance
+ * compensation sums go to each instance's ring as with lbm_step.  Asynchronous; lbm_batch_check reports a barrier timeout. */
 lbm_status lbm_batch_step(lbm_batch* b, int64_t n);
 
 /* Synchronises and returns LBM_ETIMEOUT if a grid-barrier wait of the last launches gave up

@@ -14,8 +14,10 @@
 //                   kernel on large FP32 lattices, one tile per block otherwise
 //   k_bc            every cut link by Eq. 16 / Eq. 17, the per-node compensation of Eq. 18
 //                   accumulated in FP64, and the deterministic domain sum of that step
-// launch_step issues them one after another on one stream (used by the reverse sweep's
-// recomputation and by the per-phase timing).  lbm_step uses launch_step_overlap instead: the
+// These are the separate passes: most lattices step by the fused kernels (lbm_fused.cu) or the FP64
+// ones (lbm_fp64.cu).  launch_step issues the phases one after another on one stream (used by the
+// reverse sweep's recomputation where the fused step does not apply, and by the per-phase timing).
+// Otherwise lbm_step uses launch_step_overlap: the
 // step starts at the chemical potential (none for the pseudopotential force, whose psi the
 // previous step formed), and after the collide the next state's density pass runs on a second
 // stream while k_bc and the next state's solid layers run on the first (same values).
