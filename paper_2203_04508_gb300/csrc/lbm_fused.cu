@@ -808,15 +808,17 @@ __global__ void __launch_bounds__(SOLID_BLOCK) k_layers_aa(const __grid_constant
     // not next to a solid node (a boundary node has its density from the links), nor an end or in an
     // outermost row
     const int ya = y / rows * rows;
+    const bool inside = y > ya && y < min(ya + rows, L.ny) - 1;   // (rows y - 1 and y + 1 exist)
     bool all[4];   // all of a column's three nodes fluid: x - 1 .. x + 2
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      all[k] = true;
+      all[k] = inside;
+      if (inside) {
 #pragma unroll
-      for (int d = -1; d <= 1; ++d) all[k] &= L.kind[node_at(L, x - 1 + k, y + d)] == KIND_FLUID;
+        for (int d = -1; d <= 1; ++d) all[k] &= L.kind[node_at(L, x - 1 + k, y + d)] == KIND_FLUID;
+      }
     }
-    const bool inside = y > ya && y < min(ya + rows, L.ny) - 1;
-    const bool left = inside && all[0] && all[1] && all[2], right = inside && all[1] && all[2] && all[3] && x + 1 < L.nx - 1;
+    const bool left = all[0] && all[1] && all[2], right = all[1] && all[2] && all[3] && x + 1 < L.nx - 1;
     grid_wait();
     grid_launch();
     if (!left && !right) return;

@@ -18,6 +18,9 @@ SHAPES.update({
     "walked_a_column_more_2297x2301": lambda: _box(2297, 2301),
     "walked_whole_strips_2296x2310": lambda: _box(2296, 2310, walls=1),
     "walked_pseudo": lambda: _box(2360, 2290, **PSEUDO),
+    "walked_two_narrow_strips_57x10701": lambda: _box(57, 10701, walls=1, x0=[28.0], y0=[60.0], r0=[9.0], cx=[30.2],
+                                                      cy=[5000.4], r=[11.0], dmu_w=[0.02]),
+    "walked_narrowest_5x21300": lambda: _box(5, 21300, r0=[3.0]),
 })
 
 
@@ -38,7 +41,7 @@ def test_aa_step_equals_two_lattices(name):
     b = G.Lattice(sc.physics(), precision=G.LBM_FP32, layout=G.LBM_LAYOUT_AA)
     b.init_droplets(sc.droplets())
     assert b.launches_per_step() <= 3
-    for n in (1, 2, 10) if a.nx > 2000 else (1, 2, 11, 16):
+    for n in (1, 2, 10) if a.nx * a.ny > 100000 else (1, 2, 11, 16):
         a.step(n)
         b.step(n)
         assert np.array_equal(a.populations(), b.populations()), n
