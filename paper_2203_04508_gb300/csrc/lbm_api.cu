@@ -1449,6 +1449,7 @@ lbm_status lbm_save(lbm_ctx* c, const char* path) {
   h.config_hash = config_hash(c);
   h.steps = c->steps;
   h.n_bnodes = (uint64_t)c->n_bnodes;
+  if (!c->slab.on) CUDA_OK(c, c->fp64 ? launch_settle(c->Ld, c->cur, c->stream) : launch_settle(c->Lf, c->cur, c->stream));
   lbm_status ms = resolve_mass0(c);
   if (ms != LBM_OK) return ms;
   // the steps queued on the context's stream finish before the state is copied out (the copies

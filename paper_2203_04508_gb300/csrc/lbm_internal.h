@@ -42,6 +42,8 @@ cudaError_t launch_step_overlap(const Lattice<real>& Lt, const Lattice<real>& Ln
 template <typename real> int launches_per_step_overlap(const Lattice<real>& L);
 // one double into page-locked host memory (its device address dst), in stream order
 cudaError_t launch_copy8(const double* src, double* dst, cudaStream_t s);
+// zero where lattice cur holds no population (before it is stored)
+template <typename real> cudaError_t launch_settle(const Lattice<real>& L, int cur, cudaStream_t s);
 // density and velocity of a state whose density and chemical potential are in L's planes
 template <typename real>
 cudaError_t launch_fields_of(const Lattice<real>& L, int cur, real* rho, real* vx, real* vy, cudaStream_t s);

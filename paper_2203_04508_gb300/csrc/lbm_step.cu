@@ -1023,6 +1023,24 @@ __global__ void __launch_bounds__(NODE_BLOCK) k_column(Lattice<real> L, int cur,
 
 // Populations i0 <= i < i1 of the current state as absolute values, population i into the
 // dense plane i - i0 of `out` (0 at non-fluid nodes).
+// Zero into the slots of lattice `cur` that no population of the method occupies -- a row's padding,
+// and slot i of a solid node x whose x - e_i is no fluid node -- where the fused step may have left
+// values of its own: a stored lattice holds the same bytes whichever kernels advanced it.
+template <typename real>
+__global__ void k_settle(Lattice<real> L, int cur) {
+  const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (n >= L.plane) return;
+  const int y = (int)(n / L.pitch), x = (int)(n - (long long)y * L.pitch);
+  if (x < L.nx && L.kind[n] == KIND_FLUID) return;
+  real* f = L.f[cur];
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    const int ys = y - ey(i);
+    const bool in = x < L.nx && (!L.walls || (ys >= 0 && ys < L.ny));
+    if (!in || L.kind[node_at(L, x - ex(i), ys)] != KIND_FLUID) f[i * (long long)L.plane + n] = real(0);
+  }
+}
+
 template <typename real>
 __global__ void k_populations(Lattice<real> L, int cur, real* out, int i0, int i1) {
   const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1560,6 +1578,12 @@ cudaError_t launch_macro(const Lattice<real>& L, int cur, cudaStream_t s) {
 }
 
 template <typename real>
+cudaError_t launch_settle(const Lattice<real>& L, int cur, cudaStream_t s) {
+  k_settle<real><<<grid_for(L.plane, NODE_BLOCK), NODE_BLOCK, 0, s>>>(L, cur);
+  return cudaGetLastError();
+}
+
+template <typename real>
 cudaError_t launch_fields_of(const Lattice<real>& L, int cur, real* r, real* vx, real* vy, cudaStream_t s) {
   k_fields<real><<<grid_for(L.plane, NODE_BLOCK), NODE_BLOCK, 0, s>>>(L, cur, r, vx, vy);
   return cudaGetLastError();
@@ -1624,6 +1648,7 @@ cudaError_t launch_init(const Lattice<real>& L, const double* drops, int n_drop,
   template cudaError_t launch_step_overlap<real>(const Lattice<real>&, const Lattice<real>&, int, cudaStream_t, \
                                                  cudaStream_t, cudaEvent_t, cudaEvent_t);                  \
   template int launches_per_step_overlap<real>(const Lattice<real>&);                                   \
+  template cudaError_t launch_settle<real>(const Lattice<real>&, int, cudaStream_t);                      \
   template cudaError_t launch_fields_of<real>(const Lattice<real>&, int, real*, real*, real*, cudaStream_t); \
   template cudaError_t launch_fields<real>(const Lattice<real>&, int, real*, real*, real*, cudaStream_t); \
   template cudaError_t launch_populations<real>(const Lattice<real>&, int, real*, int, int, cudaStream_t); \

@@ -126,3 +126,23 @@ def test_fused_batch_equals_the_persistent_kernel_and_single_lattices(walk):
         assert np.array_equal(b.instances[k].populations(), pops), k
         assert a.instances[k].mass() == one.mass() == b.instances[k].mass()
         assert np.array_equal(a.instances[k].dM_history(), one.dM_history())
+
+
+@pytest.mark.parametrize("layout", [0, 1])
+@pytest.mark.parametrize("steps", [4, 7])
+def test_a_stored_lattice_holds_the_bytes_of_the_separate_passes(layout, steps, tmp_path):
+    """A checkpoint keeps the lattice as stored, padding and solid nodes' slots too."""
+    import paper_2203_04508_gb300 as G
+    files = []
+    for k, sc in enumerate((S.small_parity(), _box(121, 60))):
+        for kind in (None, 0):
+            lat = G.Lattice(sc.physics(), precision=G.LBM_FP32, layout=layout)
+            lat.init_droplets(sc.droplets())
+            if kind is not None:
+                lat.set_collide_kernel(kind)
+            lat.step(steps)
+            path = tmp_path / f"{k}_{kind}.ckpt"
+            lat.save(str(path))
+            files.append(path.read_bytes())
+    assert files[0] == files[1]
+    assert files[2] == files[3]
