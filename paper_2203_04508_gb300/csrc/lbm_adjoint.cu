@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK) k_adj_solid(Lattice<real> L, AdjBuf
 // recomputation left -- populations, density, chemical potential -- and the geometry is complete
 // before the sweep of a segment begins, so each kernel fetches its share before it waits for the
 // one it follows, and only lambda is read behind the wait.  They replace a chain of six whose
-// latency was what a 512 x 512 lattice paid for: 100 steps with their recomputation took 6.3 ms and take 3.1.
+// latency was what a 512 x 512 lattice paid for: 100 steps with their recomputation took 6.3 ms and take 3.0.
 
 // adds v to grad[k] (k < 0: nothing); a warp whose nodes all belong to one body adds once
 __device__ __forceinline__ void add_by_body(double* grad, int k, double v) {
@@ -391,7 +391,7 @@ __device__ __forceinline__ void add_by_body(double* grad, int k, double v) {
 }
 
 // k_adj_bc with the links by node (as the fused step's): one round of loads instead of one a link
-constexpr int AL_BLOCK = 64;
+constexpr int AL_BLOCK = 32;
 __global__ void __launch_bounds__(AL_BLOCK) k_adj_links(const __grid_constant__ Lattice<float> L,
                                                         const __grid_constant__ AdjBuffers A) {
   const int b = blockIdx.x * AL_BLOCK + threadIdx.x;
@@ -503,26 +503,23 @@ __global__ void __launch_bounds__(AL_BLOCK) k_adj_links(const __grid_constant__ 
   lF[L.plane + n] = lFy;
 }
 
-// k_adj_collide: a node a thread
+// k_adj_collide: a node a thread.  Latency and its loads are what it costs: sixteen blocks an SM (32
+// registers instead of 40: a 512 x 512 lattice is one wave instead of 1.1), and what the geometry says
+// of a node in one word (MOVES_) instead of ten bytes: 100 reverse steps of 512 x 512 with their
+// recomputation 3.17 -> 2.96 ms.
 constexpr int AC_BLOCK = 128;
-__global__ void __launch_bounds__(AC_BLOCK) k_adj_nodes(const __grid_constant__ Lattice<float> L,
+constexpr unsigned MOVES_BC = 1u << 9, MOVES_BNODE = 1u << 10, MOVES_FLUID = 1u << 11;   // bits 0-8: directions that stream to a fluid node
+__global__ void __launch_bounds__(AC_BLOCK, 16) k_adj_nodes(const __grid_constant__ Lattice<float> L,
                                                         const __grid_constant__ AdjBuffers A) {
   const int x = blockIdx.x * AC_BLOCK + threadIdx.x, y = blockIdx.y, n = y * L.pitch + x;
-  const bool live = x < L.nx && L.kind[n] == KIND_FLUID;
+  const unsigned to = x < L.nx ? A.moves[n] : 0u;
+  const bool live = to & MOVES_FLUID;
   const int xm = x == 0 ? L.nx - 1 : -1, xp = x == L.nx - 1 ? 1 - L.nx : 1;
   const int ym = !L.walls && y == 0 ? L.plane - L.pitch : -L.pitch;
   const int yp = !L.walls && y == L.ny - 1 ? L.pitch - L.plane : L.pitch;
   auto nb = [&](int i) { return n + (ex(i) < 0 ? xm : ex(i) > 0 ? xp : 0) + (ey(i) < 0 ? ym : ey(i) > 0 ? yp : 0); };
-  unsigned to = 0;   // directions whose population streams to a fluid node
   float f[9], r = 1.f, drho = 0.f, jx = 0.f, jy = 0.f, Fx = 0.f, Fy = 0.f;
-  if (live) {
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      const bool in = !L.walls || (y + ey(i) >= 0 && y + ey(i) < L.ny);
-      if (in && L.kind[nb(i)] == KIND_FLUID) to |= 1u << i;
-    }
-    node_state(L, x, y, f, r, drho, jx, jy, Fx, Fy);
-  }
+  if (live) node_state(L, x, y, f, r, drho, jx, jy, Fx, Fy);
   grid_wait();
   grid_launch();
   if (!live) return;
@@ -531,19 +528,18 @@ __global__ void __launch_bounds__(AC_BLOCK) k_adj_nodes(const __grid_constant__ 
   float* lout = static_cast<float*>(A.lam_out);
   float* lbc = static_cast<float*>(A.lam_bc);
   float* lF = static_cast<float*>(A.lamF);
-  const uint8_t t = A.bct[n];
   float lt[9];
 #pragma unroll
   for (int i = 0; i < 9; ++i) lt[i] = to & (1u << i) ? lin[i * L.plane + nb(i)] + lrp[nb(i)] : 0.f;
   float lrho = 0, ljx = 0, ljy = 0, lFx = 0, lFy = 0;
-  if (t & 1) {
+  if (to & MOVES_BC) {
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
       lt[i] += lbc[i * L.plane + n];
       lbc[i * L.plane + n] = 0.f;
     }
   }
-  if (t & 2) {
+  if (to & MOVES_BNODE) {
     const float* lrj = static_cast<const float*>(A.lrj);
     lrho = lrj[n];
     ljx = lrj[L.plane + n];
@@ -729,6 +725,23 @@ __global__ void k_adj_geometry(Lattice<float> L, float* winv, double2* dqdc, int
   }
 }
 
+// moves of every node, once a sweep
+__global__ void __launch_bounds__(ADJ_BLOCK) k_adj_moves(Lattice<float> L, const uint8_t* bct, uint16_t* moves) {
+  const long long n = (long long)blockIdx.x * ADJ_BLOCK + threadIdx.x;
+  if (n >= L.plane) return;
+  const int y = (int)(n / L.pitch), x = (int)(n - (long long)y * L.pitch);
+  unsigned m = 0;
+  if (x < L.nx && L.kind[n] == KIND_FLUID) {
+    m = MOVES_FLUID | (bct[n] & 1 ? MOVES_BC : 0u) | (bct[n] & 2 ? MOVES_BNODE : 0u);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const bool in = !L.walls || (y + ey(i) >= 0 && y + ey(i) < L.ny);
+      if (in && L.kind[node_at(L, x + ex(i), y + ey(i))] == KIND_FLUID) m |= 1u << i;
+    }
+  }
+  moves[n] = (uint16_t)m;
+}
+
 // ---- set-up, objective, seeds ------------------------------------------------------------
 // bct bit 0: node may receive boundary contributions to its post-collision adjoint (x1 or x2 of
 // a cut link); bit 1: boundary node (local moment and force adjoints from its links)
@@ -883,7 +896,9 @@ cudaError_t adj_export(const Lattice<real>& L, const real* lam, const real* Lrho
   return cudaGetLastError();
 }
 
-cudaError_t adj_geometry(const Lattice<float>& L, float* winv, double2* dqdc, int n_cyl, cudaStream_t s) {
+cudaError_t adj_geometry(const Lattice<float>& L, const uint8_t* bct, float* winv, double2* dqdc, uint16_t* moves, int n_cyl,
+                         cudaStream_t s) {
+  k_adj_moves<<<(unsigned)((L.plane + ADJ_BLOCK - 1) / ADJ_BLOCK), ADJ_BLOCK, 0, s>>>(L, bct, moves);
   const int n = L.n_s2 > L.n_bnodes ? L.n_s2 : L.n_bnodes;
   if (n > 0) k_adj_geometry<<<list_grid(n), ADJ_BLOCK, 0, s>>>(L, winv, dqdc, n_cyl);
   return cudaGetLastError();

@@ -2259,7 +2259,7 @@ namespace {
 // restore the forward state afterwards.
 struct AdjLayout {
   long long n, every, nseg;
-  size_t ckpt, ckcarry, seg, segrho, segmu, lam0, lam1, lam_bc, lrj, lamF, Lmu, Lrho, winv, dqdc, bct, ring, ctr, carry, grad;
+  size_t ckpt, ckcarry, seg, segrho, segmu, lam0, lam1, lam_bc, lrj, lamF, Lmu, Lrho, winv, moves, dqdc, bct, ring, ctr, carry, grad;
   size_t state;   // bytes of one population lattice (9 planes)
   size_t total;
 };
@@ -2291,6 +2291,7 @@ AdjLayout make_adj_layout(const lbm_ctx* c, long long n, long long every) {
   A.Lmu = take(pl);
   A.Lrho = take(pl);
   A.winv = take(c->fp64 ? 0 : pl);
+  A.moves = take(c->fp64 ? 0 : (size_t)y.plane * 2);
   A.dqdc = take(c->fp64 || c->cfg.n_cyl == 0 ? 0 : (size_t)y.cap.bnodes * 8 * 16);
   A.bct = take((size_t)y.plane);
   A.ring = take((size_t)(DM_RING + 1) * 8);
@@ -2382,9 +2383,8 @@ lbm_status adjoint(lbm_ctx* c, const Lattice<real>& L, const void* drho, const v
   }
   real* lam[2] = {(real*)(w + A.lam0), (real*)(w + A.lam1)};
   CUDA_OK(c, adj_seed(L, lam[0], s_rho, s_f, st));
-  CUDA_OK(c, cudaMemsetAsync(lam[1], 0, 9 * pl, st));
   CUDA_OK(c, cudaMemsetAsync(w + A.lam_bc, 0, 9 * pl, st));
-  CUDA_OK(c, cudaMemsetAsync(w + A.lamF, 0, 2 * pl, st));
+  // (lam[1] and lamF are read at fluid nodes only, which a step writes before it reads them)
   CUDA_OK(c, cudaMemsetAsync(w + A.grad, 0, (size_t)(3 * c->cfg.n_cyl + 1) * 8, st));
   CUDA_OK(c, adj_flags(L, (uint8_t*)(w + A.bct), st));
   AdjBuffers B{};
@@ -2396,7 +2396,9 @@ lbm_status adjoint(lbm_ctx* c, const Lattice<real>& L, const void* drho, const v
   B.winv = w + A.winv;
   if constexpr (sizeof(real) == 4) {
     B.dqdc = (const double2*)(w + A.dqdc);
-    CUDA_OK(c, adj_geometry(L, (float*)(w + A.winv), (double2*)(w + A.dqdc), c->cfg.n_cyl, st));
+    B.moves = (const uint16_t*)(w + A.moves);
+    CUDA_OK(c, adj_geometry(L, (const uint8_t*)(w + A.bct), (float*)(w + A.winv), (double2*)(w + A.dqdc),
+                            (uint16_t*)(w + A.moves), c->cfg.n_cyl, st));
   }
   B.bct = (const uint8_t*)(w + A.bct);
   B.grad = (double*)(w + A.grad);

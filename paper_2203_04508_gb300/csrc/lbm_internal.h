@@ -227,11 +227,12 @@ struct AdjBuffers {
   void* lam_out;        // 9 planes: dJ/df^t
   void* lam_bc;         // 9 planes: boundary contributions to dJ/d(post-collision f), zero between steps
   void* lrj;            // 3 planes: dJ/d(delta rho, jx, jy) of the link rule at boundary nodes
-  void* lamF;           // 2 planes: dJ/dF (zero off the fluid)
+  void* lamF;           // 2 planes: dJ/dF at fluid nodes
   void* Lmu;            // dJ/dmu
   void* Lrho;           // dJ/drho (the density plane); between steps the density share of lambda
   bool first;           // FP32: the step follows work other than a reverse step: nothing of it starts early
   const void* winv;     // FP32: 1 / sum of Eq. 15's weights at second-layer nodes, by node
+  const uint16_t* moves;   // FP32: what the geometry says of each node (k_adj_nodes)
   const double2* dqdc;  // FP32: dq/dc of the link of boundary node b in direction i at (i - 1) bcap + b
   const uint8_t* bct;   // per node: bit 0 lam_bc may be non-zero, bit 1 boundary node
   double* grad;         // dJ/d dmu per cylinder, dJ/d dmu of the walls, dJ/d(cx, cy) per cylinder
@@ -240,8 +241,9 @@ struct AdjBuffers {
 // blocks of the objective's reduction over a plane of `plane` nodes (at most one per 256
 // nodes): it leaves 4 partial sums per block in `red`
 unsigned objective_blocks(long long plane);
-// FP32: winv and dqdc of a sweep
-cudaError_t adj_geometry(const Lattice<float>& L, float* winv, double2* dqdc, int n_cyl, cudaStream_t s);
+// FP32: winv, dqdc and moves of a sweep (after adj_flags)
+cudaError_t adj_geometry(const Lattice<float>& L, const uint8_t* bct, float* winv, double2* dqdc, uint16_t* moves, int n_cyl,
+                         cudaStream_t s);
 template <typename real> cudaError_t adj_flags(const Lattice<real>& L, uint8_t* bct, cudaStream_t s);
 template <typename real>
 cudaError_t objective_sums(const Lattice<real>& L, int cur, int body, uint8_t* touch, double* red, double rg,
