@@ -480,6 +480,15 @@ cudaError_t leave_fused(lbm_ctx* c) {
   return cudaMemcpyAsync(c->ws + c->lay.mu2, c->ws + c->lay.mu, c->lay.plane * c->lay.sz, cudaMemcpyDeviceToDevice, c->stream);
 }
 
+// Is the caller capturing the stream?  What is issued then is recorded and not run: the planes of the
+// current state stay as they are, and a recorded launch must not count on them.
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  (void)cudaGetLastError();   // (the default stream while another is captured)
+  return false;
+}
+
 // descriptors of a step from lattice `cur`: its density in plane `cur`, the boundary densities
 // into rho_b, and the next state's density plane
 template <typename real>
@@ -1311,9 +1320,11 @@ namespace {
 
 // Queues the fields of the current state into device-writable arrays: from the planes the fused step
 // keeps (formed first for a new state) in one launch, or through the separate passes.  The arrays of
-// a pair of columns are written together where they are 8-byte aligned.
+// a pair of columns are written together where they are 8-byte aligned.  A read-out that is recorded
+// forms everything from the populations: a replay may find another state in them.
 cudaError_t queue_fields(lbm_ctx* c, void* r, void* u, void* v) {
-  if (fused_any(c) && (((uintptr_t)r | (uintptr_t)u | (uintptr_t)v) & 7) == 0) {
+  const bool recorded = capturing(c->stream);
+  if (!recorded && fused_any(c) && (((uintptr_t)r | (uintptr_t)u | (uintptr_t)v) & 7) == 0) {
     if (!c->rho_ok) {
       cudaError_t e = launch_fused_prepare(fused_lattice(c, c->Lf, c->cur ^ 1), c->cur, c->stream);
       if (e != cudaSuccess) return e;
@@ -1321,7 +1332,7 @@ cudaError_t queue_fields(lbm_ctx* c, void* r, void* u, void* v) {
     }
     return launch_fused_fields(fused_lattice(c, c->Lf, c->cur), c->cur, (float*)r, (float*)u, (float*)v, c->stream);
   }
-  if (step64(c) && c->rho_ok) {
+  if (!recorded && step64(c) && c->rho_ok) {
     // the planes of the current state are complete but for its chemical potential
     Lattice<double> Lt, Ln;
     step_lattices(c, c->Ld, c->cur, Lt, Ln);
