@@ -417,7 +417,9 @@ lbm_status lbm_batch_init(lbm_batch* b, const lbm_init_spec* specs);
  * launch of a persistent kernel (captured for this n), to which the tile shape and the schedule
  * below belong.  Both give the same values, bit for bit.  In the persistent kernel each step runs the
  * phases of lbm_step over all instances' work, separated by grid barriers; per-instance
- * compensation sums go to each instance's ring as with lbm_step.  Asynchronous; lbm_batch_check reports a barrier timeout. */
+ * compensation sums go to each instance's ring as with lbm_step.  On a stream that the caller is
+ * capturing the persistent kernel is recorded, for a state of the present lattice parity (an odd n
+ * changes it with every replay).  Asynchronous; lbm_batch_check reports a barrier timeout. */
 lbm_status lbm_batch_step(lbm_batch* b, int64_t n);
 
 /* Synchronises and returns LBM_ETIMEOUT if a grid-barrier wait of the last launches gave up

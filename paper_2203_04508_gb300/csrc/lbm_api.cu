@@ -156,6 +156,9 @@ struct lbm_ctx {
   // (planes rho, rho2), computing the next one while the boundary phase runs; false until a
   // step or an explicit density pass has put it there
   bool rho_ok = false;
+  // the caller has captured a batch step of this lattice: its replays change the state unseen, so no
+  // call counts on the planes an earlier one left
+  bool replayed = false;
   cudaStream_t side = nullptr;                      // second stream of the overlapped step
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   cudaEvent_t ev_user = nullptr;                    // orders a read-out with a stream of the caller's
@@ -489,6 +492,9 @@ bool capturing(cudaStream_t s) {
   return false;
 }
 
+// Do the planes hold the density of the current state?
+bool planes_current(const lbm_ctx* c) { return c->rho_ok && !c->replayed; }
+
 // descriptors of a step from lattice `cur`: its density in plane `cur`, the boundary densities
 // into rho_b, and the next state's density plane
 template <typename real>
@@ -591,11 +597,10 @@ lbm_status do_step(lbm_ctx* c, const Lattice<real>& L, long long n) {
   if (n <= 0) return LBM_OK;
   lbm_status sst = step_streams(c);
   if (sst != LBM_OK) return sst;
-  if (!c->rho_ok && fused_any(c)) {
+  if (!planes_current(c) && fused_any(c)) {
     if constexpr (sizeof(real) == 4) CUDA_OK(c, launch_fused_prepare(fused_lattice(c, L, c->cur ^ 1), c->cur, c->stream));
     c->rho_ok = true;
-  }
-  if (!c->rho_ok) {
+  } else if (!planes_current(c)) {
     // density of the current lattice and its solid layers, which the overlapped step expects
     Lattice<real> Lt, Ln;
     step_lattices(c, L, c->cur, Lt, Ln);
@@ -646,7 +651,7 @@ lbm_status profile_steps(lbm_ctx* c, const Lattice<real>& L, long long n, double
     // one another (chemical potential, collide, boundary links, the next state's solid layers,
     // the densities the collide left), the density planes alternating as lbm_step keeps them
     Lattice<real> Lt, Ln;
-    if (!c->rho_ok) {
+    if (!planes_current(c)) {
       step_lattices(c, L, c->cur, Lt, Ln);
       CUDA_OK(c, launch_phase(Lt, c->cur, 0, c->stream));
       CUDA_OK(c, launch_phase(Lt, c->cur, 1, c->stream));
@@ -1325,14 +1330,14 @@ namespace {
 cudaError_t queue_fields(lbm_ctx* c, void* r, void* u, void* v) {
   const bool recorded = capturing(c->stream);
   if (!recorded && fused_any(c) && (((uintptr_t)r | (uintptr_t)u | (uintptr_t)v) & 7) == 0) {
-    if (!c->rho_ok) {
+    if (!planes_current(c)) {
       cudaError_t e = launch_fused_prepare(fused_lattice(c, c->Lf, c->cur ^ 1), c->cur, c->stream);
       if (e != cudaSuccess) return e;
       c->rho_ok = true;
     }
     return launch_fused_fields(fused_lattice(c, c->Lf, c->cur), c->cur, (float*)r, (float*)u, (float*)v, c->stream);
   }
-  if (!recorded && step64(c) && c->rho_ok) {
+  if (!recorded && step64(c) && planes_current(c)) {
     // the planes of the current state are complete but for its chemical potential
     Lattice<double> Lt, Ln;
     step_lattices(c, c->Ld, c->cur, Lt, Ln);
@@ -1976,7 +1981,7 @@ lbm_status fused_tables(lbm_batch* b) {
 // n fused steps of every instance: graphs of STEPS_LONG, two and one steps, as lbm_step's
 lbm_status fused_batch_step(lbm_batch* b, long long n) {
   bool ready = true;
-  for (auto* c : b->ctx) ready &= c->rho_ok;
+  for (auto* c : b->ctx) ready &= planes_current(c);
   if (!ready) BCUDA(b, launch_fused_batch_prepare(b->fb, b->cur, b->stream));
   int cur = b->cur;
   auto run = [&](int steps) -> lbm_status {
@@ -2087,9 +2092,11 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t n) {
   if (n <= 0) return n == 0 ? LBM_OK : LBM_EINVAL;
   if (n > (1LL << 30)) return bfail(b, LBM_EINVAL, "too many steps in one launch");
   const int flip = (int)(n & 1);
-  // the fused step where every instance runs it, unless the caller bounds the persistent kernel's
-  // waits (the fused step has none)
-  bool all_fused = b->fused && b->spin_limit == BATCH_SPIN_DEFAULT;
+  // The fused step where every instance runs it, unless the caller bounds the persistent kernel's
+  // waits (the fused step has none) or records the step: graphs are not replayed into a capture, and the
+  // persistent kernel takes any number of steps in one launch.
+  const bool recorded = capturing(b->stream);
+  bool all_fused = b->fused && b->spin_limit == BATCH_SPIN_DEFAULT && !recorded;
   for (int k = 0; k < b->n && all_fused; ++k) all_fused = fused(b->ctx[k]);
   if (all_fused) {
     lbm_status st = fused_batch_step(b, n);
@@ -2103,7 +2110,7 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t n) {
     return LBM_OK;
   }
   b->dev.spin_limit = b->spin_limit;
-  if (b->use_graph && (b->graph_steps != n || b->graph_cur != b->cur || !b->graph)) {
+  if (b->use_graph && !recorded && (b->graph_steps != n || b->graph_cur != b->cur || !b->graph)) {
     if (b->graph) { cudaGraphExecDestroy(b->graph); b->graph = nullptr; }
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
@@ -2124,13 +2131,14 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t n) {
       b->graph_cur = b->cur;
     }
   }
-  if (b->use_graph && b->graph) BCUDA(b, cudaGraphLaunch(b->graph, b->stream));
+  if (b->use_graph && b->graph && !recorded) BCUDA(b, cudaGraphLaunch(b->graph, b->stream));
   else BCUDA(b, launch_batch(b->dev, b->fp64, b->grid, (int)n, b->cur, b->stream));
   b->cur ^= flip;
   for (int k = 0; k < b->n; ++k) {
     b->ctx[k]->cur ^= flip;
     b->ctx[k]->steps += n;
     b->ctx[k]->rho_ok = false;
+    b->ctx[k]->replayed |= recorded;
   }
   return LBM_OK;
 }

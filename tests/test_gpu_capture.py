@@ -66,3 +66,35 @@ def test_a_recorded_read_out_leaves_the_state_and_reads_what_it_finds(precision,
     b.step(3)
     assert np.array_equal(a.populations(), b.populations())
 
+
+@pytest.mark.parametrize("warm", [0, 4])
+@pytest.mark.parametrize("precision", [FP32, FP64])
+def test_a_recorded_batch_step(precision, warm):
+    """lbm_batch_step under the caller's capture, replayed between steps that are not recorded."""
+    import paper_2203_04508_gb300 as G
+    import torch
+    scs = [S.small_parity(), S.small_parity(seed=11, nx=97, ny=83)]
+    a, b = (G.Batch([sc.physics() for sc in scs], precision=precision) for _ in range(2))
+    for batch in (a, b):
+        batch.init([sc.droplets() for sc in scs])
+        batch.step(warm)
+        batch.synchronize()
+
+    def same():
+        for x, y in zip(a.instances, b.instances):
+            assert np.array_equal(x.populations(), y.populations())
+            for u, v in zip(x.fields(), y.fields()):
+                assert np.array_equal(u, v)
+
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=a.stream):
+        a.step(4)
+    for between in (0, 6, 2):
+        graph.replay()
+        torch.cuda.synchronize()
+        b.step(4)
+        same()
+        a.step(between)
+        b.step(between)
+        same()
+    a.check()
