@@ -541,7 +541,8 @@ __device__ __forceinline__ void force_at(const Lattice<real>& L, int x, int y, r
 //   w_i rho [3 e.du + 4.5 (e.du)(e.(2u+du)) - 1.5 du.(2u+du)].
 template <typename real>
 __device__ __forceinline__ real edm_term(int i, real r, real ux, real uy, real dux, real duy) {
-  // (products rounded explicitly: every kernel that evaluates a link gets the same bits)
+  // (products rounded explicitly, the arguments' by the caller: every kernel that evaluates a link gets
+  // the same bits; products by 2 and by the directions' components are exact)
   const real ax = real(2) * ux + dux, ay = real(2) * uy + duy;
   const real edu = real(ex(i)) * dux + real(ey(i)) * duy;
   const real e2u = real(ex(i)) * ax + real(ey(i)) * ay;
@@ -620,7 +621,7 @@ __device__ __forceinline__ void odd_split(V Jx, V Jy, V& px, V& py, V& pd, V& pa
 __device__ __forceinline__ void collide_bgk64(const Lattice<double>& L, double (&f)[9], double r, double drho, double jx,
                                               double jy, double Fx, double Fy) {
   const double keep = 1.0 - L.omega, inv_r = 1.0 / r, nk = -keep;
-  const double Jx = jx + Fx, Jy = jy + Fy;
+  const double Jx = add_rn(jx, Fx), Jy = add_rn(jy, Fy);
   const double q = div36(drho), qw = fma(nk, q, q);
   const double vx = Jx * inv_r, vy = Jy * inv_r, ux = (nk * jx) * inv_r, uy = (nk * jy) * inv_r;
   const double X = fma(Jx, vx, jx * ux), Y = fma(Jy, vy, jy * uy), Z = fma(Jx, vy, jx * uy), S = X + Y;

@@ -77,9 +77,9 @@ __device__ __forceinline__ void links(const Lattice<real>& L, int cur, int b) {
     r = L.rho_ref + drho;
     if constexpr (!PLANES) force_at<real, PSEUDO>(L, x, n / L.pitch, r, Fx, Fy);
     inv_r = real(1) / r;
-    ux = jx * inv_r;
-    uy = jy * inv_r;
-    const real dux = Fx * inv_r, duy = Fy * inv_r;
+    ux = mul_rn(jx, inv_r);
+    uy = mul_rn(jy, inv_r);
+    const real dux = mul_rn(Fx, inv_r), duy = mul_rn(Fy, inv_r);
 #pragma unroll
     for (int i = 1; i < 9; ++i) F[i - 1] = mask & (1u << (i - 1)) ? edm_term<real>(i, r, ux, uy, dux, duy) : real(0);
   };
@@ -213,14 +213,26 @@ __device__ __forceinline__ void solids(const Lattice<real>& L, int blk, int bloc
     if (steps) {
       // k_bc's blocks of eight warps: their warps' sums in block_sum's tree, then the blocks'
       const int warps = (L.n_bnodes + 31) / 32, chunks = (warps + 7) / 8;
-      double v = 0.0;
-      for (int k = threadIdx.x; k < chunks; k += BLOCK) {
-        double w[8];
+      constexpr int SUM_BLOCK = 256, PARTS = SUM_BLOCK / BLOCK;   // k_bc's last block; each thread's share of it
+      static_assert(PARTS == 1 || PARTS == 2, "block_sum's tree over 8 warps begins with pairs (j, j + 4)");
+      double v[PARTS];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) w[j] = 8 * k + j < warps ? L.partials[8 * k + j] : 0.0;
-        v += ((w[0] + w[4]) + (w[2] + w[6])) + ((w[1] + w[5]) + (w[3] + w[7]));
+      for (int p = 0; p < PARTS; ++p) {
+        v[p] = 0.0;
+        for (int k = threadIdx.x + p * BLOCK; k < chunks; k += SUM_BLOCK) {
+          double w[8];
+#pragma unroll
+          for (int j = 0; j < 8; ++j) w[j] = 8 * k + j < warps ? L.partials[8 * k + j] : 0.0;
+          v[p] += ((w[0] + w[4]) + (w[2] + w[6])) + ((w[1] + w[5]) + (w[3] + w[7]));
+        }
+        if constexpr (PARTS == 2) {
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) v[p] += __shfl_down_sync(0xffffffffu, v[p], o);
+        }
       }
-      const double total = block_sum(v, red);
+      double mine = v[0];
+      if constexpr (PARTS == 2) mine = (threadIdx.x & 31) == 0 ? v[0] + v[1] : 0.0;
+      const double total = block_sum(mine, red);
       if (threadIdx.x == 0) {
         const unsigned long long st = *L.step_ctr;
         L.dM_ring[st % DM_RING] = total;

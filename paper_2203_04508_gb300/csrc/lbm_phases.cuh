@@ -429,7 +429,8 @@ __device__ __forceinline__ double phase_bc(const Lattice<real>& L, int cur, int 
   real Fx, Fy;
   force_at<real, PSEUDO>(L, x, y, r, Fx, Fy);
   const real inv_r = real(1) / r;
-  const real ux = jx * inv_r, uy = jy * inv_r, dux = Fx * inv_r, duy = Fy * inv_r;
+  // (explicit products, which no compiler fuses into edm_term's sums: links() gets the same bits)
+  const real ux = mul_rn(jx, inv_r), uy = mul_rn(jy, inv_r), dux = mul_rn(Fx, inv_r), duy = mul_rn(Fy, inv_r);
   double sum = 0.0;
   for (int l = l0; l < l1; ++l) {
     const int k = l - l0;
