@@ -305,7 +305,7 @@ lbm_status lbm_launches_per_step(lbm_ctx* ctx, int64_t* n);
  * persistent block at least 16 tiles, kind 0 otherwise; kind 2 runs only when set (on GB300 its
  * added density work slows a collide kernel that is already bound by instruction issue more
  * than the separate density pass costs).  Setting a kind, the current one too, makes lbm_step run
- * the separate passes instead of the fused step.  Setting a kind the lattice cannot run returns
+ * the separate passes instead of the fused step until lbm_reset_kernels.  Setting a kind the lattice cannot run returns
  * LBM_EINVAL.  Call after lbm_build_links; the step graphs are captured again.  A
  * bounded wait of kind 1 or 2 that gives up is reported as LBM_ETIMEOUT by the next lbm_mass. */
 lbm_status lbm_set_collide_kernel(lbm_ctx* ctx, int32_t kind);
@@ -318,10 +318,15 @@ lbm_status lbm_get_collide_kernel(lbm_ctx* ctx, int32_t* kind);
  * only) row sweeps, a thread walking down a column of four-node groups with the stencil's rows
  * in registers.  The default is 2 for FP32 lattices of at least four 512 x 16-node blocks per
  * SM, else 1.  All three give the same bits.  Setting a kind makes lbm_step run the separate
- * passes instead of the fused step.  Call
+ * passes instead of the fused step until lbm_reset_kernels.  Call
  * after lbm_build_links; the step graphs are captured again.  LBM_EINVAL for another value or
  * for 2 on an FP64 lattice. */
 lbm_status lbm_set_mu_kernel(lbm_ctx* ctx, int32_t kind);
+
+/* Undoes lbm_set_collide_kernel and lbm_set_mu_kernel: lbm_step runs again what lbm_build_links chose
+ * (the fused step where the lattice has one).  Call after lbm_build_links; the step graphs are captured
+ * again. */
+lbm_status lbm_reset_kernels(lbm_ctx* ctx);
 
 /* Polls before the TMA-pipelined kernel's wait for a tile's loads gives up (default 2^22, a
  * second or more); 0 makes every such wait give up at once, to test the timeout path.  A block

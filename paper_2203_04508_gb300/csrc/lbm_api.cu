@@ -181,6 +181,7 @@ struct lbm_ctx {
   long long spin_limit = 1LL << 22;   // polls before a pipelined kernel's wait gives up
   int mu_kind = -1;                   // chemical-potential pass (-1: the precision's default)
   bool collide_set = false;           // lbm_set_collide_kernel was called
+  int collide_default = 1;            // what lbm_build_links chose
   bool fused_ok = false;              // the fused step's kernels can run on this device
   PassPlan plan, tile_plan, aa_plan;           // how the fused step's pass runs on this lattice; without the walk
   long long n_near = 0;               // entries of the near list, built where the fused density +
@@ -1111,6 +1112,7 @@ lbm_status lbm_build_links(lbm_ctx* c) {
     // bound by instruction issue) and the step 0.31 ms against 0.21 ms.
     const long long tiles = (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8);
     c->collide_kind = (c->tma_ok && tiles >= 16LL * c->tma.blocks[g.force_model == LBM_FORCE_PSEUDO ? 1 : 0]) ? 1 : 0;
+    c->collide_default = c->collide_kind;
     refresh(c);
     int dev = 0, sms = 0;
     c->fused_ok = cudaGetDevice(&dev) == cudaSuccess &&
@@ -1288,6 +1290,22 @@ lbm_status lbm_set_mu_kernel(lbm_ctx* c, int32_t kind) {
     lbm_status st = near_list(c);
     if (st != LBM_OK) return st;
   }
+  for (auto& gr : c->graph)
+    if (gr) { cudaGraphExecDestroy(gr); gr = nullptr; }
+  for (auto& a : c->adj_graphs) cudaGraphExecDestroy(a.exec);
+  c->adj_graphs.clear();
+  refresh(c);
+  return LBM_OK;
+}
+
+lbm_status lbm_reset_kernels(lbm_ctx* c) {
+  if (!c || !c->built) return LBM_ESTATE;
+  if (c->mu_kind < 0 && !c->collide_set) return LBM_OK;
+  c->mu_kind = -1;
+  c->collide_set = false;
+  c->collide_kind = c->collide_default;
+  // the density (and psi) planes are formed anew; the walls' chemical potential has stayed in the first mu plane
+  c->rho_ok = false;
   for (auto& gr : c->graph)
     if (gr) { cudaGraphExecDestroy(gr); gr = nullptr; }
   for (auto& a : c->adj_graphs) cudaGraphExecDestroy(a.exec);

@@ -220,12 +220,18 @@ class Lattice:
         """0: the plain collide kernel; 1: the TMA-pipelined one (FP32); 2: the TMA-pipelined column
         sweeps that also form the next state's density (FP32, chemical-potential force, lattices of
         whole 32 x 8 tiles; slower on GB300, so never the default).  lbm_build_links picks 1 on large
-        lattices, 0 otherwise."""
+        lattices, 0 otherwise.  Setting a kind, the current one too, makes step() run the separate
+        passes instead of the fused step, until reset_kernels()."""
         self._c(self.lib.lbm_set_collide_kernel(self.ctx, int(kind)))
 
     def set_mu_kernel(self, kind: int):
-        """Chemical-potential pass: 0 per node, 1 row vectors, 2 row sweeps (FP32); same bits."""
+        """Chemical-potential pass: 0 per node, 1 row vectors, 2 row sweeps (FP32); same bits.  Setting
+        one makes step() run the separate passes, until reset_kernels()."""
         self._c(self.lib.lbm_set_mu_kernel(self.ctx, int(kind)))
+
+    def reset_kernels(self):
+        """Back to the step that lbm_build_links chose, after set_collide_kernel / set_mu_kernel."""
+        self._c(self.lib.lbm_reset_kernels(self.ctx))
 
     def set_spin_limit(self, polls: int):
         """Polls before the pipelined kernel's waits give up (0: at once, to test that path)."""
