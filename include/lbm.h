@@ -415,26 +415,31 @@ lbm_status lbm_batch_build_links(lbm_batch* b);
 /* lbm_init for every instance with specs[k] (n specs).  Synchronises. */
 lbm_status lbm_batch_init(lbm_batch* b, const lbm_init_spec* specs);
 
-/* Advances every instance n steps.  Where all of them run the fused step on two population
- * lattices (lbm_step) its three kernels run over flat lists of all
- * instances' work, captured into CUDA graphs on first use; a batch whose poll budget the caller
- * set (lbm_batch_set_spin_limit, other than the default) and every other batch runs ONE cooperative
- * launch of a persistent kernel (captured for this n), to which the tile shape and the schedule
- * below belong.  Both give the same values, bit for bit.  In the persistent kernel each step runs the
- * phases of lbm_step over all instances' work, separated by grid barriers; per-instance
- * compensation sums go to each instance's ring as with lbm_step.  On a stream that the caller is
- * capturing the persistent kernel is recorded, for a state of the present lattice parity (an odd n
- * changes it with every replay).  Asynchronous; lbm_batch_check reports a barrier timeout. */
+/* Advances every instance n steps.  Where all of them run the fused step on two population lattices
+ * (lbm_step), its three kernels run over flat lists of all instances' work, captured into CUDA graphs
+ * on first use.  Every other batch, and one set to it by lbm_batch_set_kernel, runs ONE cooperative
+ * launch of a persistent kernel (captured for this n), to which the tile shape, the schedule and the
+ * poll budget below belong: each step runs the phases of lbm_step over all instances' work,
+ * separated by grid barriers.  Both give the same values, bit for bit; the compensation sums go to
+ * each instance's ring as with lbm_step.  On a stream that the caller is capturing the persistent
+ * kernel is recorded, for a state of the present lattice parity (an odd n changes it with every
+ * replay).  Asynchronous; lbm_batch_check reports a barrier timeout. */
 lbm_status lbm_batch_step(lbm_batch* b, int64_t n);
 
 /* Synchronises and returns LBM_ETIMEOUT if a grid-barrier wait of the last launches gave up
  * (the kernel then left without finishing its steps). */
 lbm_status lbm_batch_check(lbm_batch* b);
 
-/* Polls before a grid-barrier wait gives up (default 2^22, about a second or more); 0 makes
- * every wait give up at once (used to test the timeout path).  Another value than the default makes
- * lbm_batch_step run the persistent kernel (the fused step waits for nothing).  Clears the error
- * flag. */
+/* 1: lbm_batch_step runs the persistent kernel; 0 (the default): the fused step where all instances
+ * run it.  LBM_EINVAL for other values. */
+lbm_status lbm_batch_set_kernel(lbm_batch* b, int32_t kind);
+/* What lbm_batch_step runs now: 0 the fused step, 1 the persistent kernel.  After
+ * lbm_batch_build_links. */
+lbm_status lbm_batch_get_kernel(lbm_batch* b, int32_t* kind);
+
+/* Polls before a grid-barrier wait of the persistent kernel gives up (default 2^22, about a second
+ * or more).  The fused step waits for nothing and keeps to any budget but 0, which makes every wait give
+ * up at once: the persistent kernel runs then, to test the timeout path.  Clears the error flag. */
 lbm_status lbm_batch_set_spin_limit(lbm_batch* b, int64_t polls);
 
 /* Shape of the node tiles of the persistent kernel: 2^log2w nodes wide and 256 / 2^log2w

@@ -86,6 +86,8 @@ _SIGS = {
     "lbm_batch_step": (I32, [P, I64]),
     "lbm_batch_check": (I32, [P]),
     "lbm_batch_set_spin_limit": (I32, [P, I64]),
+    "lbm_batch_set_kernel": (I32, [P, I32]),
+    "lbm_batch_get_kernel": (I32, [P, C.POINTER(I32)]),
     "lbm_batch_instance": (I32, [P, I32, C.POINTER(P)]),
     "lbm_batch_set_tile": (I32, [P, I32]),
     "lbm_batch_set_schedule": (I32, [P, I32]),

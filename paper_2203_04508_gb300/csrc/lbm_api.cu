@@ -1756,8 +1756,6 @@ void lbm_destroy(lbm_ctx* c) {
 // ---------------------------------------------------------------------------------------
 // Batched lattices
 // ---------------------------------------------------------------------------------------
-constexpr long long BATCH_SPIN_DEFAULT = 1LL << 22;
-
 struct lbm_batch {
   int n = 0;
   bool fp64 = false;
@@ -1783,7 +1781,8 @@ struct lbm_batch {
   cudaGraphExec_t graph = nullptr;
   long long graph_steps = -1;
   int graph_cur = -1;
-  long long spin_limit = BATCH_SPIN_DEFAULT;
+  long long spin_limit = 1LL << 22;
+  bool persistent = false;   // lbm_batch_set_kernel: the persistent kernel even where the fused step runs
   int tile_log2w = BATCH_TILE_LOG2W_DEFAULT;
   int cur = 0;
   std::string err;
@@ -1996,6 +1995,14 @@ lbm_status fused_tables(lbm_batch* b) {
   return LBM_OK;
 }
 
+// Does lbm_batch_step run the fused step?  Where every instance runs it, unless the caller chose the
+// persistent kernel, or asked its waits to give up at once (the fused step has none that could).
+bool batch_fused(const lbm_batch* b) {
+  bool all = b->fused && !b->persistent && b->spin_limit > 0;
+  for (int k = 0; k < b->n && all; ++k) all = fused(b->ctx[k]);
+  return all;
+}
+
 // n fused steps of every instance: graphs of STEPS_LONG, two and one steps, as lbm_step's
 lbm_status fused_batch_step(lbm_batch* b, long long n) {
   bool ready = true;
@@ -2110,13 +2117,10 @@ lbm_status lbm_batch_step(lbm_batch* b, int64_t n) {
   if (n <= 0) return n == 0 ? LBM_OK : LBM_EINVAL;
   if (n > (1LL << 30)) return bfail(b, LBM_EINVAL, "too many steps in one launch");
   const int flip = (int)(n & 1);
-  // The fused step where every instance runs it, unless the caller bounds the persistent kernel's
-  // waits (the fused step has none) or records the step: graphs are not replayed into a capture, and the
-  // persistent kernel takes any number of steps in one launch.
+  // A step that is recorded takes the persistent kernel: graphs are not replayed into a capture, and it
+  // runs any number of steps in one launch.
   const bool recorded = capturing(b->stream);
-  bool all_fused = b->fused && b->spin_limit == BATCH_SPIN_DEFAULT && !recorded;
-  for (int k = 0; k < b->n && all_fused; ++k) all_fused = fused(b->ctx[k]);
-  if (all_fused) {
+  if (!recorded && batch_fused(b)) {
     lbm_status st = fused_batch_step(b, n);
     if (st != LBM_OK) return st;
     b->cur ^= flip;
@@ -2179,6 +2183,19 @@ lbm_status lbm_batch_set_spin_limit(lbm_batch* b, int64_t polls) {
     BCUDA(b, cudaMemsetAsync(b->dev.err, 0, sizeof(int), b->stream));
     BCUDA(b, cudaStreamSynchronize(b->stream));
   }
+  return LBM_OK;
+}
+
+lbm_status lbm_batch_set_kernel(lbm_batch* b, int32_t kind) {
+  if (!b || b->ctx.empty()) return LBM_ESTATE;
+  if (kind != 0 && kind != 1) return bfail(b, LBM_EINVAL, "batch kernel must be 0 (default) or 1 (persistent), not %d", kind);
+  b->persistent = kind == 1;
+  return LBM_OK;
+}
+
+lbm_status lbm_batch_get_kernel(lbm_batch* b, int32_t* kind) {
+  if (!b || !b->tables || !kind) return LBM_ESTATE;
+  *kind = batch_fused(b) ? 0 : 1;
   return LBM_OK;
 }
 

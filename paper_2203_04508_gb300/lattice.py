@@ -329,7 +329,8 @@ class _InstanceView(Lattice):
 
 
 class Batch:
-    """Many independent lattices advanced together by the persistent batched kernel."""
+    """Many independent lattices advanced together: by the fused step's kernels over all instances' work
+    (FP32, two population lattices) or by one persistent kernel."""
 
     def __init__(self, physics: list, precision: int = _abi.LBM_FP32, stream=None,
                  layout: int = _abi.LBM_LAYOUT_AB):
@@ -388,7 +389,19 @@ class Batch:
         self._check(self.lib.lbm_batch_check(self.b))
 
     def set_spin_limit(self, polls: int):
+        """Polls before a grid-barrier wait of the persistent kernel gives up (0: at once, to test that
+        path; such a batch runs the persistent kernel)."""
         self._check(self.lib.lbm_batch_set_spin_limit(self.b, int(polls)))
+
+    def set_kernel(self, kind: int):
+        """1: step() runs the persistent kernel; 0: the fused step where all instances run it."""
+        self._check(self.lib.lbm_batch_set_kernel(self.b, int(kind)))
+
+    def kernel(self) -> int:
+        """What step() runs now: 0 the fused step, 1 the persistent kernel."""
+        k = C.c_int32()
+        self._check(self.lib.lbm_batch_get_kernel(self.b, C.byref(k)))
+        return k.value
 
     def set_tile(self, log2w: int):
         """Node-tile shape of the persistent kernel: 2^log2w x 256/2^log2w (log2w in 4..8)."""

@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 
 import scenarios as S
+from test_gpu_fused_step import _box
 
 pytestmark = pytest.mark.gpu
 
@@ -50,3 +51,65 @@ def test_reset_goes_back_to_the_default_step(precision, layout, over):
                 assert np.array_equal(u, v)
     b.reset_kernels()   # nothing to undo
     assert b.launches_per_step() == launches
+
+
+def _batch(precision=FP32, layout=AB, walked=False):
+    import paper_2203_04508_gb300 as G
+    scs = [S.small_parity(), S.small_parity(seed=11, nx=97, ny=83)]
+    if walked:   # large enough for the batch's walks
+        scs = [_box(2100, 2001, walls=1), _box(2000, 2100), _box(1999, 2300)]
+    b = G.Batch([sc.physics() for sc in scs], precision=precision, layout=layout)
+    b.init([sc.droplets() for sc in scs])
+    return scs, b
+
+
+def test_a_poll_budget_does_not_choose_the_batch_kernel():
+    """Any budget but zero leaves the fused step, which waits for nothing, in place."""
+    _, b = _batch()
+    assert b.kernel() == 0
+    for polls in (1, 100, (1 << 22) - 1, (1 << 22) + 1, 1 << 30):
+        b.set_spin_limit(polls)
+        assert b.kernel() == 0
+    b.step(3)
+    b.check()
+    b.set_spin_limit(0)
+    assert b.kernel() == 1
+    b.set_spin_limit(1 << 22)
+    assert b.kernel() == 0
+    b.instances[1].set_mu_kernel(1)
+    assert b.kernel() == 1
+    b.instances[1].reset_kernels()
+    assert b.kernel() == 0
+    for kw in (dict(precision=FP64), dict(layout=AA)):
+        assert _batch(**kw)[1].kernel() == 1
+
+
+@pytest.mark.parametrize("walked", [False, True])
+def test_the_persistent_kernel_by_choice_and_after_a_timeout(walked):
+    """The persistent kernel against the fused step (tiles and walks) over changes between them, and
+    again after its barriers gave up."""
+    from paper_2203_04508_gb300 import LbmError
+    scs, a = _batch(walked=walked)
+    b = _batch(walked=walked)[1]
+    if b.info()["grid"] >= 2:
+        b.set_spin_limit(0)
+        b.step(3)
+        with pytest.raises(LbmError):
+            b.check()
+        b.set_spin_limit(1 << 22)
+        b.init([sc.droplets() for sc in scs])
+    for n, kind in ((1, 1), (13, 0), (2, 1), (5, 1), (8, 0)):
+        b.set_kernel(kind)
+        assert b.kernel() == kind
+        a.step(n)
+        b.step(n)
+        b.check()
+        for x, y in zip(a.instances, b.instances):
+            assert np.array_equal(x.populations(), y.populations())
+            assert x.mass() == y.mass()
+            for u, v in zip(x.fields(), y.fields()):
+                assert np.array_equal(u, v)
+    for x, y in zip(a.instances, b.instances):
+        assert np.array_equal(x.dM_history(), y.dM_history())
+    with pytest.raises(LbmError):
+        b.set_kernel(2)
