@@ -457,7 +457,8 @@ lbm_status lbm_batch_set_tile(lbm_batch* b, int32_t log2w);
  * identical results.  Default 2.  LBM_EINVAL for other values.  Synchronises. */
 lbm_status lbm_batch_set_schedule(lbm_batch* b, int32_t groups);
 
-/* Autotuner of tile shape and schedule: times `steps` steps of the batch with each tile shape
+/* Autotuner of the persistent kernel's tile shape and schedule (the fused step has neither; the trials
+ * run the persistent kernel on a batch of either kind): times `steps` steps with each tile shape
  * under the current schedule, then with the fastest shape under both schedules (CUDA events on
  * the batch's stream, each after one untimed launch of the same length), and keeps the fastest
  * combination.  Writes the chosen log2w and groups (either pointer may be NULL) and the seven

@@ -2248,6 +2248,9 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int64_t steps, int32_t* chosen_log2w
   int best = b->tile_log2w, best_g = b->groups;
   double best_ms = 1e300;
   lbm_status st = LBM_OK;
+  // the persistent kernel's shapes are timed on it, whichever kernel the batch's steps run
+  const bool chosen = b->persistent;
+  b->persistent = true;
   // tile shapes under the current schedule, then both schedules with the fastest shape
   for (int lw = BATCH_TILE_LOG2W_MIN; lw <= BATCH_TILE_LOG2W_MAX && st == LBM_OK; ++lw) {
     float t = 0.f;
@@ -2265,6 +2268,7 @@ lbm_status lbm_batch_autotune(lbm_batch* b, int64_t steps, int32_t* chosen_log2w
     if (ms) ms[5 + g - 1] = t;
     if (st == LBM_OK && t < best_ms) { best_ms = t; best_g = g; }
   }
+  b->persistent = chosen;
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   if (st != LBM_OK) return st;

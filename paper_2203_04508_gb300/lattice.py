@@ -413,8 +413,8 @@ class Batch:
         self._check(self.lib.lbm_batch_set_schedule(self.b, int(groups)))
 
     def autotune(self, steps: int = 20):
-        """Times every tile shape, then both schedules with the fastest shape, over `steps`
-        steps each (the instances advance 14 * steps steps) and keeps the fastest; returns
+        """Tile shape and schedule of the persistent kernel (the fused step has neither): times every
+        tile shape, then both schedules with the fastest shape, over `steps` steps of it each (the instances advance 14 * steps steps) and keeps the fastest; returns
         {"log2w", "tile", "groups", "ms": {tile or schedule: ms}}."""
         chosen, groups = C.c_int32(), C.c_int32()
         ms = np.zeros(7)

@@ -113,3 +113,30 @@ def test_the_persistent_kernel_by_choice_and_after_a_timeout(walked):
         assert np.array_equal(x.dM_history(), y.dM_history())
     with pytest.raises(LbmError):
         b.set_kernel(2)
+
+
+def test_the_autotuner_times_the_persistent_kernel():
+    """Its shapes are the persistent kernel's: on a batch whose steps are fused the trials run that
+    kernel all the same -- with a budget of one poll its barriers give up, which only they can."""
+    from paper_2203_04508_gb300 import LbmError
+    scs, b = _batch()
+    if b.info()["grid"] < 2:
+        pytest.skip("a one-block grid never waits")
+    b.set_spin_limit(1)
+    assert b.kernel() == 0
+    with pytest.raises(LbmError) as e:
+        b.autotune(2)
+    assert e.value.status == 6
+    assert b.kernel() == 0
+    b.set_spin_limit(1 << 22)
+    b.init([sc.droplets() for sc in scs])
+    r = b.autotune(2)
+    assert b.kernel() == 0
+    tiles = {k: v for k, v in r["ms"].items() if "x" in k}
+    assert r["ms"][r["tile"]] == min(tiles.values())
+    b.init([sc.droplets() for sc in scs])
+    a = _batch()[1]
+    a.step(9)
+    b.step(9)
+    for x, y in zip(a.instances, b.instances):
+        assert np.array_equal(x.populations(), y.populations())
