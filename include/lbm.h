@@ -277,10 +277,12 @@ lbm_status lbm_last_dM(lbm_ctx* ctx, double* dM);
  * waits for the stream. */
 lbm_status lbm_last_dM_async(lbm_ctx* ctx, double* dM);
 
-/* Advances n steps like lbm_step, launching the five phases of the separate passes one by one
- * (the same values, bit for bit) with CUDA events on the context's stream between them, and adds each phase's device time (ms) to ms5:
- * [0] density, [1] solid layers (Eq. 15), [2] chemical potential, [3] force + collision +
- * streaming, [4] boundary links (Eqs. 16-18).  Synchronises after every step. */
+/* Advances n steps like lbm_step, launching its kernels one by one with CUDA events on the context's
+ * stream between them, and adds each phase's device time (ms) to ms5: [0] density, [1] solid layers
+ * (Eq. 15), [2] chemical potential, [3] force + collision + streaming, [4] boundary links (Eqs. 16-18).
+ * Of the fused step (lbm_step) [3] is the whole pass, the next state's density and the chemical
+ * potential with it, and [0] and [2] are zero; of the FP64 step of four kernels [0] holds the solid layers
+ * too and [1] is zero.  Synchronises after every step. */
 lbm_status lbm_profile_steps(lbm_ctx* ctx, int64_t n, double* ms5);
 
 /* EOS summary (host FP64): Tc, rho_c, T, alpha, rho_g, rho_l, mu_sat, p_sat. */

@@ -528,17 +528,17 @@ Lattice<float> fused_lattice(const lbm_ctx* c, const Lattice<float>& L, int cur)
   return F;
 }
 
-// Issues one step from lattice `cur` on the context's stream.
+// Issues one step from lattice `cur` on the context's stream (of the fused and FP64 steps: its `parts`).
 template <typename real>
-cudaError_t issue_step(lbm_ctx* c, const Lattice<real>& L, int cur) {
+cudaError_t issue_step(lbm_ctx* c, const Lattice<real>& L, int cur, unsigned parts = PART_ALL) {
   if constexpr (sizeof(real) == 4) {
-    if (fused(c)) return launch_fused_step(fused_lattice(c, L, cur), cur, c->plan, c->stream);
-    if (fused_aa(c)) return launch_fused_step_aa(fused_lattice(c, L, cur), cur, c->aa_plan, c->stream);
+    if (fused(c)) return launch_fused_step(fused_lattice(c, L, cur), cur, c->plan, c->stream, parts);
+    if (fused_aa(c)) return launch_fused_step_aa(fused_lattice(c, L, cur), cur, c->aa_plan, c->stream, parts);
   }
   Lattice<real> Lt, Ln;
   step_lattices(c, L, cur, Lt, Ln);
   if constexpr (sizeof(real) == 8) {
-    if (step64(c)) return launch_fp64_step(Lt, Ln.rho, cur, c->stream);
+    if (step64(c)) return launch_fp64_step(Lt, Ln.rho, cur, c->stream, parts);
   }
   return launch_step_overlap(Lt, Ln, cur, c->stream, c->side, c->ev_fork, c->ev_join);
 }
@@ -593,24 +593,31 @@ lbm_status prepare_steps(lbm_ctx* c, const Lattice<real>& L, long long n) {
   return LBM_OK;
 }
 
+// The planes a step starts from: the density of the current state and its solid layers.
 template <typename real>
-lbm_status do_step(lbm_ctx* c, const Lattice<real>& L, long long n) {
-  if (n <= 0) return LBM_OK;
-  lbm_status sst = step_streams(c);
-  if (sst != LBM_OK) return sst;
-  if (!planes_current(c) && fused_any(c)) {
+lbm_status form_planes(lbm_ctx* c, const Lattice<real>& L) {
+  if (planes_current(c)) return LBM_OK;
+  if (fused_any(c)) {
     if constexpr (sizeof(real) == 4) CUDA_OK(c, launch_fused_prepare(fused_lattice(c, L, c->cur ^ 1), c->cur, c->stream));
-    c->rho_ok = true;
-  } else if (!planes_current(c)) {
-    // density of the current lattice and its solid layers, which the overlapped step expects
+  } else {
     Lattice<real> Lt, Ln;
     step_lattices(c, L, c->cur, Lt, Ln);
     CUDA_OK(c, launch_phase(Lt, c->cur, 0, c->stream));
     CUDA_OK(c, launch_phase(Lt, c->cur, 1, c->stream));
     // the step that forms mu with the next density starts from this state's mu
     if (L.mu_kernel == 3) CUDA_OK(c, launch_phase(Lt, c->cur, 2, c->stream));
-    c->rho_ok = true;
   }
+  c->rho_ok = true;
+  return LBM_OK;
+}
+
+template <typename real>
+lbm_status do_step(lbm_ctx* c, const Lattice<real>& L, long long n) {
+  if (n <= 0) return LBM_OK;
+  lbm_status sst = step_streams(c);
+  if (sst != LBM_OK) return sst;
+  lbm_status pst = form_planes(c, L);
+  if (pst != LBM_OK) return pst;
   auto graph_of = [&](int p, int steps, cudaGraphExec_t* out) { return step_graph(c, L, p, steps, out); };
   if (n >= STEPS_LONG && c->stream != nullptr) {
     cudaGraphExec_t gl;
@@ -643,10 +650,40 @@ lbm_status do_step(lbm_ctx* c, const Lattice<real>& L, long long n) {
 
 template <typename real>
 lbm_status profile_steps(lbm_ctx* c, const Lattice<real>& L, long long n, double* ms) {
+  static const char* const phase_name[5] = {"density", "solid layers", "chemical potential", "collide", "boundary"};
   cudaEvent_t ev[6];
   for (auto& e : ev) CUDA_OK(c, cudaEventCreate(&e));
   for (int k = 0; k < 5; ++k) ms[k] = 0.0;
   lbm_status st = LBM_OK;
+  if (fused_any(c) || step64(c)) {
+    // the kernels lbm_step runs, in their order, and the phase each is counted as
+    struct Part { unsigned part; int phase; };
+    static const Part fused_parts[] = {{PART_PASS, 3}, {PART_LINKS, 4}, {PART_LAYERS, 1}};
+    static const Part fp64_parts[] = {{PART_MU, 2}, {PART_PASS, 3}, {PART_LINKS, 4}, {PART_LAYERS, 0}};
+    const Part* parts = fused_any(c) ? fused_parts : fp64_parts;
+    const int count = fused_any(c) ? 3 : 4;
+    if (n > 0) st = form_planes(c, L);
+    for (long long s = 0; s < n && st == LBM_OK; ++s) {
+      cudaError_t e = cudaSuccess;
+      for (int k = 0; k < count && e == cudaSuccess; ++k) {
+        LBM_RANGE(phase_name[parts[k].phase]);
+        cudaEventRecord(ev[k], c->stream);
+        e = issue_step(c, L, c->cur, parts[k].part);
+      }
+      if (e == cudaSuccess) e = cudaEventRecord(ev[count], c->stream);
+      if (e == cudaSuccess) e = cudaEventSynchronize(ev[count]);
+      if (e != cudaSuccess) { st = fail(c, LBM_ECUDA, "step failed: %s", cudaGetErrorString(e)); break; }
+      for (int k = 0; k < count; ++k) {
+        float t = 0.f;
+        cudaEventElapsedTime(&t, ev[k], ev[k + 1]);
+        ms[parts[k].phase] += t;
+      }
+      c->cur ^= 1;
+      c->steps += 1;
+    }
+    for (auto& e : ev) cudaEventDestroy(e);
+    return st;
+  }
   if (step_sweeps(L, c->cur)) {
     // the collide kernel forms most of the next density: the phases in the order they depend on
     // one another (chemical potential, collide, boundary links, the next state's solid layers,
@@ -660,7 +697,6 @@ lbm_status profile_steps(lbm_ctx* c, const Lattice<real>& L, long long n, double
     }
     static const int order[5] = {2, 3, 4, 1, 0};
     for (long long s = 0; s < n && st == LBM_OK; ++s) {
-      static const char* const phase_name[5] = {"density", "solid layers", "chemical potential", "collide", "boundary"};
       step_lattices(c, L, c->cur, Lt, Ln);
       for (int k = 0; k < 5; ++k) {
         LBM_RANGE(phase_name[order[k]]);
@@ -684,7 +720,6 @@ lbm_status profile_steps(lbm_ctx* c, const Lattice<real>& L, long long n, double
     return st;
   }
   for (long long s = 0; s < n && st == LBM_OK; ++s) {
-    static const char* const phase_name[5] = {"density", "solid layers", "chemical potential", "collide", "boundary"};
     for (int ph = 0; ph < 5; ++ph) {
       LBM_RANGE(phase_name[ph]);
       cudaEventRecord(ev[ph], c->stream);

@@ -100,17 +100,17 @@ cudaError_t launch_fp64_mu(const Lattice<double>& L, cudaStream_t s) {
   return launch_after(k64_mu, dim3((unsigned)(per_row * L.ny)), D_BLOCK, 0, s, L, per_row);
 }
 
-cudaError_t launch_fp64_step(const Lattice<double>& Lt, double* rho_next, int cur, cudaStream_t s) {
+cudaError_t launch_fp64_step(const Lattice<double>& Lt, double* rho_next, int cur, cudaStream_t s, unsigned parts) {
   Lattice<double> L = Lt;
   L.rho_next = rho_next;
   const auto blocks = [](int n, int per) { return (n + per - 1) / per; };
   const int per_row = blocks(L.nx, D_BLOCK), b2 = blocks(8 * L.n_s2, D_BLOCK), b1 = blocks(L.n_s1, D_BLOCK);
-  cudaError_t e = launch_fp64_mu(L, s);
+  cudaError_t e = parts & PART_MU ? launch_fp64_mu(L, s) : cudaSuccess;
   const int across = blocks(L.nx, DC_X), grid = across * blocks(L.ny, D_BLOCK / DC_X);
-  if (e == cudaSuccess) e = launch_after(k64_collide, dim3((unsigned)grid), D_BLOCK, 0, s, L, cur, across);
-  if (e == cudaSuccess && L.n_bnodes > 0)
+  if (e == cudaSuccess && (parts & PART_PASS)) e = launch_after(k64_collide, dim3((unsigned)grid), D_BLOCK, 0, s, L, cur, across);
+  if (e == cudaSuccess && L.n_bnodes > 0 && (parts & PART_LINKS))
     e = launch_after(k64_links, dim3((unsigned)blocks(L.n_bnodes, DB_BLOCK)), DB_BLOCK, 0, s, L, cur);
-  if (e == cudaSuccess)
+  if (e == cudaSuccess && (parts & PART_LAYERS))
     e = launch_after(k64_state, dim3((unsigned)(b2 + b1 + 1 + per_row * L.ny)), D_BLOCK, 0, s, L, cur ^ 1, b2, b1, per_row);
   return e;
 }

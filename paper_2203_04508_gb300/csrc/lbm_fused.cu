@@ -1117,15 +1117,15 @@ static cudaError_t launch_pass(const Lattice<float>& L, int cur, PassPlan p, cud
                   : launch_after(k_walk<false>, dim3((unsigned)(strips * bands)), 32, Reach<false>::BYTES, s, L, cur, strips, p.rows);
 }
 
-cudaError_t launch_fused_step(const Lattice<float>& L, int cur, PassPlan plan, cudaStream_t s) {
-  cudaError_t e = launch_pass(L, cur, plan, s);
-  if (e == cudaSuccess && L.n_bnodes > 0)
+cudaError_t launch_fused_step(const Lattice<float>& L, int cur, PassPlan plan, cudaStream_t s, unsigned parts) {
+  cudaError_t e = parts & PART_PASS ? launch_pass(L, cur, plan, s) : cudaSuccess;
+  if (e == cudaSuccess && L.n_bnodes > 0 && (parts & PART_LINKS))
     e = launch_after(L.pseudo ? k_bc_fused<true> : k_bc_fused<false>, dim3(blocks_for(L.n_bnodes, BC_BLOCK)), BC_BLOCK, 0, s, L, cur);
-  return e == cudaSuccess ? launch_solids(L, 1, s) : e;
+  return e == cudaSuccess && (parts & PART_LAYERS) ? launch_solids(L, 1, s) : e;
 }
 
 // One lattice in AA order, from slot order cur
-cudaError_t launch_fused_step_aa(const Lattice<float>& L, int cur, PassPlan p, cudaStream_t s) {
+cudaError_t launch_fused_step_aa(const Lattice<float>& L, int cur, PassPlan p, cudaStream_t s, unsigned parts) {
   const int strips = (L.nx + OUT - 1) / OUT, bands = (L.ny + p.rows - 1) / p.rows;
   const dim3 grid((unsigned)(strips * bands)), nb(blocks_for(L.n_bnodes, BC_BLOCK));
   const int b2 = (int)blocks_for(8 * L.n_s2, SOLID_BLOCK), b1 = (int)blocks_for(L.n_s1, SOLID_BLOCK);
@@ -1136,20 +1136,21 @@ cudaError_t launch_fused_step_aa(const Lattice<float>& L, int cur, PassPlan p, c
   const dim3 layers((unsigned)(b2 + b1 + 1) + (edge + SOLID_BLOCK - 1) / SOLID_BLOCK);
   auto tiles = [&](auto* k, int bytes) { return launch_after(k, grid, 32 * TW_M, bytes, s, L, cur, strips, p.rows); };
   auto walks = [&](auto* k, int bytes) { return launch_after(k, grid, 32, bytes, s, L, cur, strips, p.rows); };
-  cudaError_t e;
-  if (p.kind == PassPlan::WALK) {
+  cudaError_t e = cudaSuccess;
+  if (!(parts & PART_PASS)) {
+  } else if (p.kind == PassPlan::WALK) {
     if (L.pseudo) e = cur ? walks(k_walk<true, 2>, Reach<true>::BYTES) : walks(k_walk<true, 1>, Reach<true>::BYTES);
     else e = cur ? walks(k_walk<false, 2>, Reach<false>::BYTES) : walks(k_walk<false, 1>, Reach<false>::BYTES);
   } else if (L.pseudo) e = cur ? tiles(k_tile<true, TH_M, TW_M, TB_M, 2>, Tile<true, TH_M>::BYTES)
                         : tiles(k_tile<true, TH_M, TW_M, TB_M, 1>, Tile<true, TH_M>::BYTES);
   else e = cur ? tiles(k_tile<false, TH_M, TW_M, TB_M, 2>, Tile<false, TH_M>::BYTES)
                : tiles(k_tile<false, TH_M, TW_M, TB_M, 1>, Tile<false, TH_M>::BYTES);
-  if (e == cudaSuccess && L.n_bnodes > 0) {
+  if (e == cudaSuccess && L.n_bnodes > 0 && (parts & PART_LINKS)) {
     auto bc = [&](auto* k) { return launch_after(k, nb, BC_BLOCK, 0, s, L, cur); };
     if (L.pseudo) e = cur ? bc(k_bc_fused<true, 2>) : bc(k_bc_fused<true, 1>);
     else e = cur ? bc(k_bc_fused<false, 2>) : bc(k_bc_fused<false, 1>);
   }
-  if (e != cudaSuccess) return e;
+  if (e != cudaSuccess || !(parts & PART_LAYERS)) return e;
   auto* k = p.kind == PassPlan::WALK ? (L.pseudo ? k_layers_aa<true, true> : k_layers_aa<false, true>)
                                      : (L.pseudo ? k_layers_aa<true, false> : k_layers_aa<false, false>);
   return launch_after(k, layers, SOLID_BLOCK, 0, s, L, b2, b1, cur ^ 1, strips, p.rows, edge_rows);

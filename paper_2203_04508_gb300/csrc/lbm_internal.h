@@ -97,18 +97,22 @@ struct PassPlan {
 PassPlan fused_plan(int nx, int ny, int sms);
 PassPlan fused_tile_plan(int nx, int ny, int sms);
 PassPlan fused_aa_plan(int nx, int ny, int sms);
+// the kernels of the fused and the FP64 step, to launch one by one (per-phase timing): the pass (FP64: the
+// collision), the links, the solid layers (FP64: the new state's density and layers); FP64 only: the
+// chemical potential
+enum StepPart : unsigned { PART_PASS = 1, PART_LINKS = 2, PART_LAYERS = 4, PART_MU = 8, PART_ALL = 15 };
 // the fused step of one lattice in AA order, from slot order cur (L.bmom: the boundary nodes' moments)
-cudaError_t launch_fused_step_aa(const Lattice<float>& L, int cur, PassPlan plan, cudaStream_t s);
+cudaError_t launch_fused_step_aa(const Lattice<float>& L, int cur, PassPlan plan, cudaStream_t s, unsigned parts = PART_ALL);
 // ---- the FP64 step (lbm_fp64.cu): chemical-potential force, an equation of state, two lattices
 // one step from lattice cur, whose density plane is L.rho (and psi' in L.psip); the next into rho_next
-cudaError_t launch_fp64_step(const Lattice<double>& L, double* rho_next, int cur, cudaStream_t s);
+cudaError_t launch_fp64_step(const Lattice<double>& L, double* rho_next, int cur, cudaStream_t s, unsigned parts = PART_ALL);
 // the chemical potential of such a state
 cudaError_t launch_fp64_mu(const Lattice<double>& L, cudaStream_t s);
 int launches_fp64(const Lattice<double>& L);
 // the solid layers of a new state in lattice cur, where the fused step expects them
 cudaError_t launch_fused_prepare(const Lattice<float>& L, int cur, cudaStream_t s);
 // one step from lattice cur (L.rho_b, L.fx and L.fy set)
-cudaError_t launch_fused_step(const Lattice<float>& L, int cur, PassPlan plan, cudaStream_t s);
+cudaError_t launch_fused_step(const Lattice<float>& L, int cur, PassPlan plan, cudaStream_t s, unsigned parts = PART_ALL);
 int fused_launches(const Lattice<float>& L);
 // density and velocity of the state in lattice cur, whose density (psi) plane L names (L.rho or L.mu)
 cudaError_t launch_fused_fields(const Lattice<float>& L, int cur, float* r, float* vx, float* vy, cudaStream_t s);

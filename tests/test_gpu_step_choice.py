@@ -53,6 +53,31 @@ def test_reset_goes_back_to_the_default_step(precision, layout, over):
     assert b.launches_per_step() == launches
 
 
+@pytest.mark.parametrize("precision,layout,over", [(FP32, AB, {}), (FP32, AA, {}), (FP32, AB, PSEUDO), (FP64, AB, {})])
+def test_profiled_steps_run_the_kernels_of_the_step(precision, layout, over):
+    """lbm_profile_steps times what lbm_step runs: the fused step has no density or chemical-potential
+    kernel of its own, the FP64 one no layer kernel; the values and the state are lbm_step's."""
+    import paper_2203_04508_gb300 as G
+    sc = S.small_parity().with_(**over)
+    a, b = (G.Lattice(sc.physics(), precision=precision, layout=layout) for _ in range(2))
+    for lat in (a, b):
+        lat.init_droplets(sc.droplets())
+    for n in (3, 4, 1):
+        a.step(n)
+        ms = b.profile_steps(n)
+        zero = {0, 2} if precision == FP32 else {1}
+        assert all((v == 0.0) == (k in zero) for k, v in enumerate(ms)), ms
+        assert np.array_equal(a.populations(), b.populations())
+        assert a.mass() == b.mass()
+        a.step(2)
+        b.step(2)
+        assert np.array_equal(a.populations(), b.populations())
+    assert np.array_equal(a.dM_history(), b.dM_history())
+    b.set_collide_kernel(0)      # the separate passes' five phases
+    ms = b.profile_steps(2)
+    assert (ms[[0, 1, 3, 4]] > 0).all()
+
+
 def _batch(precision=FP32, layout=AB, walked=False):
     import paper_2203_04508_gb300 as G
     scs = [S.small_parity(), S.small_parity(seed=11, nx=97, ny=83)]
