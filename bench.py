@@ -19,14 +19,14 @@ exchanged over NCCL every few steps (strong scaling); rank 0 prints one JSON lin
 Before the clock starts the graphs that the timed steps launch are captured (lbm_prepare_steps),
 so that no capture happens inside the timed region; nothing is stepped by it.
 
-Besides the contract keys the line carries: `roofline` (the collide kernel's algorithmic bytes
-over its CUDA-event time, against the measured HBM copy bandwidth, with the per-phase times),
+Besides the contract keys the line carries: `roofline` (the algorithmic bytes of the kernel that moves
+the populations -- the fused step's pass, the one the timed steps launch -- over its CUDA-event time, against the measured HBM copy bandwidth, with the per-phase times),
 `cpu_baseline` (the oracle on the host cores), `e2e` (through the C-ABI with host buffers),
 `clocks`, `fp64` (the same workload with FP64 populations: MLUPS and the FP32/FP64 speed
 ratio; the drop's interface on the centre line in FP32 and FP64 over 10000 steps; the 128 x 128
 FP64 case's mass change with the present scheme and IBC), `batched` (256 instances of
-128^2..768^2 in one persistent launch against the same instances stepped one by one; the
-autotuned tile shape; the same comparison on 1024 instances of 64^2..128^2), and `adjoint` (512 x 512, 4000 steps, checkpoint every 200: forward,
+128^2..768^2 advanced together against the same instances stepped one by one; the persistent kernel's
+autotuned tile shape, which the AA batch uses; the same comparison on 1024 instances of 64^2..128^2), and `adjoint` (512 x 512, 4000 steps, checkpoint every 200: forward,
 checkpointed forward and reverse-sweep times, one reverse step against one forward step, and
 the gradient), and `bc_comparison` (the boundary schemes of the paper's Sec. 4.3-4.4 on
 reduced-size drops: late per-step compensation and spurious currents), and `paper_runs` (the
@@ -55,17 +55,28 @@ sys.path.insert(0, ROOT)
 
 METRIC = "MLUPS & % HBM roofline, FP32 vs FP64 oracle; batched and adjoint cost ratio"
 UNIT = "MLUPS"
-# algorithmic bytes of the fused force + collision + streaming kernel: per fluid node read 9
-# and write 9 FP32 populations (72 B) and read rho and mu (8 B); per lattice node its class
-# byte (1 B)
+# algorithmic bytes of the kernel that moves the populations: per fluid node read 9 and write 9 FP32
+# populations (72 B), and 8 B more -- the fused step's pass reads this state's density (psi) and writes the
+# next one's, the separate collide kernel reads rho and mu; per lattice node its class byte (1 B)
 COLLIDE_BYTES_PER_FLUID_NODE = 80
 COLLIDE_BYTES_PER_NODE = 1
-# the pseudopotential variant reads psi only (4 B) besides the populations
+# the separate pseudopotential kernel reads psi only (4 B) besides the populations
 PSEUDO_COLLIDE_BYTES_PER_FLUID_NODE = 76
 STEP_BYTES_PER_NODE = 72
 # y-slabs of one lattice over several GPUs: halo refresh period (the halo is 8 rows per step)
 SLAB_EXCHANGE_EVERY = 4
 FALLBACK_HBM_GBS = 6800.0
+
+
+def profiled_kernel(lat, phase_ms, pseudo):
+    """(name, algorithmic bytes per fluid node, fused?) of the kernel behind phase_ms[3]: the fused step's
+    pass, which has no density kernel beside it, or the collide kernel of the separate passes."""
+    if phase_ms[0] == 0.0:
+        name = "psi" if pseudo else "chemical potential"
+        return (f"k_walk, k_tile on smaller lattices ({name}, force + collide + stream + the next density)",
+                COLLIDE_BYTES_PER_FLUID_NODE, True)
+    return (collide_kernel_name(lat.collide_kernel(), pseudo),
+            PSEUDO_COLLIDE_BYTES_PER_FLUID_NODE if pseudo else COLLIDE_BYTES_PER_FLUID_NODE, False)
 
 
 def collide_kernel_name(kind, pseudo):
@@ -100,8 +111,7 @@ def workload(name):
 
 def run_batched(G, torch, rank, world, steps, small=False):
     """Batched workload: seed-random droplet-on-cylinder instances of 128^2..768^2 (small:
-    1024 instances of 64^2..128^2), advanced together by the persistent kernel (one launch for
-    all steps), against the same instances each advanced by its own lbm_step graph launches,
+    1024 instances of 64^2..128^2), advanced together by the fused step over all instances, against the same instances each advanced by its own lbm_step graph launches,
     issued one lattice after another (each lattice has its own stream)."""
     import scenarios as S
     scs = S.c4_batch(seed=5, n=1024, nmin=64, nmax=128) if small else S.c4_batch()
@@ -111,7 +121,8 @@ def run_batched(G, torch, rank, world, steps, small=False):
     nodes = sum(sc.nodes for sc in scs)
     b = G.Batch([sc.physics() for sc in scs], precision=G.LBM_FP32)
     b.init([sc.droplets() for sc in scs])
-    # the library's autotuner picks the node-tile shape on this batch, then a fresh start
+    # the library's autotuner picks the persistent kernel's node-tile shape on this batch (for the AA
+    # batch below, which that kernel advances), then a fresh start
     tuned = b.autotune(10)
     b.init([sc.droplets() for sc in scs])
     b.step(2)
@@ -124,10 +135,11 @@ def run_batched(G, torch, rank, world, steps, small=False):
     b.check()
     ms_b = e0.elapsed_time(e1)
     info = b.info()
+    kernel = ("fused step", "persistent")[b.kernel()]
     ws_b = b.workspace.numel()
     del b
     torch.cuda.empty_cache()
-    # the same batch with one population lattice per instance in AA order (same tile shape)
+    # the same batch with one population lattice per instance in AA order (the persistent kernel)
     ba = G.Batch([sc.physics() for sc in scs], precision=G.LBM_FP32, layout=G.LBM_LAYOUT_AA)
     ba.init([sc.droplets() for sc in scs])
     ba.set_tile(int(tuned["log2w"]))
@@ -162,7 +174,7 @@ def run_batched(G, torch, rank, world, steps, small=False):
     return {"instances": len(scs), "nodes": nodes, "steps": steps, "ms_batched": round(ms_b, 3),
             "mlups_batched": round(nodes * steps / ms_b / 1e3, 1), "ms_looped": round(ms_l, 3),
             "mlups_looped": round(nodes * steps / ms_l / 1e3, 1), "speedup": round(ms_l / ms_b, 3),
-            "persistent_grid": info["grid"], "graph_captured": info["graph"],
+            "kernel": kernel, "persistent_grid": info["grid"], "graph_captured": info["graph"],
             "tile": tuned["tile"], "schedule": "two groups" if tuned["groups"] == 2 else "lockstep",
             "autotune_ms_per_10_steps": tuned["ms"],
             "workspace_GB": round(ws_b / 1e9, 3),
@@ -319,7 +331,6 @@ def run_pseudopotential(G, torch, steps, ms_chempot):
     lat = G.Lattice(sc.physics(), precision=G.LBM_FP32)
     lat.init_droplets(sc.droplets())
     fluid = lat.counts()["fluid"]
-    kname = collide_kernel_name(lat.collide_kernel(), pseudo=True)
     lat.step(20)
     lat.synchronize()
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -330,17 +341,18 @@ def run_pseudopotential(G, torch, steps, ms_chempot):
     ms = e0.elapsed_time(e1) / steps
     n_prof = max(10, min(100, steps // 5))
     phase_ms = lat.profile_steps(n_prof) / n_prof
+    kname, node_bytes, fused = profiled_kernel(lat, phase_ms, pseudo=True)
     M, M0, _ = lat.mass()
     del lat
     torch.cuda.empty_cache()
     peak, peak_src = measured_peak()
-    coll_bytes = PSEUDO_COLLIDE_BYTES_PER_FLUID_NODE * fluid + COLLIDE_BYTES_PER_NODE * sc.nodes
+    coll_bytes = node_bytes * fluid + COLLIDE_BYTES_PER_NODE * sc.nodes
     collide_ms = float(phase_ms[3])
     achieved = coll_bytes / (collide_ms / 1e3) / 1e9
     return {"workload": "c3 geometry 2048x4096, pseudopotential force, CS T=0.7Tc, k=1, FP32",
             "roofline": {"bound": "hbm", "kernel": kname,
                          "achieved": round(achieved, 1), "peak": peak, "peak_source": peak_src, "unit": "GB/s",
-                         "frac": round(achieved / peak, 4), "traffic": recorded_traffic("c3pp"),
+                         "frac": round(achieved / peak, 4), "traffic": None if fused else recorded_traffic("c3pp"),
                          "algorithmic_bytes_per_launch": coll_bytes, "launch_ms": round(collide_ms, 5)},
             "steps": steps, "ms_per_step": round(ms, 5), "mlups": round(sc.nodes / ms / 1e3, 1),
             "phase_ms": {k: round(float(v), 5) for k, v in zip(("rho", "solid", "psi", "collide", "bc"), phase_ms)},
@@ -808,8 +820,6 @@ def main():
         scs = S.c4_batch()[:args.batch_instances]
         b = G.Batch([x.physics() for x in scs], precision=G.LBM_FP32)
         b.init([x.droplets() for x in scs])
-        b.set_tile(5)
-        b.set_schedule(1)   # 32 x 8 tiles in lockstep: the autotuner's choice on the 256-lattice mix
         b.step(args.warmup)
         b.synchronize()
         b.check()
@@ -817,7 +827,7 @@ def main():
         b.synchronize()
         b.check()
         print(json.dumps({"mode": "batch", "instances": len(scs), "nodes": sum(x.nodes for x in scs),
-                          "tile": "32x8", "schedule": "lockstep", "steps": args.steps, "warmup": args.warmup}))
+                          "kernel": ("fused step", "persistent")[b.kernel()], "steps": args.steps, "warmup": args.warmup}))
         return
 
     sc, wname = workload(args.workload)
@@ -850,7 +860,6 @@ def main():
                           "launches_per_step": lat.launches_per_step(), "mass_drift": M / M0 - 1}))
         return
     lps = lat.launches_per_step()
-    collide_name = collide_kernel_name(lat.collide_kernel(), pseudo=False)
     flush = None
     if args.workload == "c2":
         flush = torch.empty(256 * 1024 * 1024 // 4, dtype=torch.float32, device="cuda")
@@ -902,10 +911,11 @@ def main():
     n_prof = max(10, min(200, args.steps // 10))
     if world == 1:
         phase_ms = lat.profile_steps(n_prof) / n_prof
+        collide_name, node_bytes, fused = profiled_kernel(lat, phase_ms, pseudo=args.workload == "c3pp")
         collide_ms = float(phase_ms[3])
-        coll_bytes = COLLIDE_BYTES_PER_FLUID_NODE * counts["fluid"] + COLLIDE_BYTES_PER_NODE * sc.nodes
+        coll_bytes = node_bytes * counts["fluid"] + COLLIDE_BYTES_PER_NODE * sc.nodes
         achieved = coll_bytes / (collide_ms / 1e3) / 1e9
-        traffic = recorded_traffic(args.workload)
+        traffic = None if fused else recorded_traffic(args.workload)
         M, M0, _ = lat.mass()
     else:
         M, M0, _ = dslab.mass()
@@ -966,7 +976,7 @@ def main():
     batched = None
     if args.batch_steps > 0:
         batched = run_batched(G, torch, rank, world, args.batch_steps)
-        # many small lattices, where one persistent launch replaces thousands of launches
+        # many small lattices, where a batch's few launches a step replace thousands
         small = run_batched(G, torch, rank, world, args.batch_steps, small=True) if world == 1 else None
         if world > 1:
             t = torch.tensor([batched["ms_batched"], batched["ms_looped"]], device="cuda", dtype=torch.float64)
