@@ -73,11 +73,16 @@ bool sweep_shape(const lbm_config* c) {
          c->ny % 8 == 0 && c->layout != LBM_LAYOUT_AA;
 }
 
+// nodes of a padded row: whole 128-byte lines
+long long row_pitch(const lbm_config* c) {
+  const long long per_line = c->precision == LBM_FP64 ? 16 : 32;
+  return (c->nx + per_line - 1) / per_line * per_line;
+}
+
 Layout make_layout(const lbm_config* c) {
   Layout L{};
   L.sz = c->precision == LBM_FP64 ? 8 : 4;
-  const int per_line = (int)(128 / L.sz);
-  L.pitch = (c->nx + per_line - 1) / per_line * per_line;
+  L.pitch = (int)row_pitch(c);
   L.plane = (long long)L.pitch * c->ny;
   L.cap = list_caps(c);
   size_t o = 0;
@@ -416,6 +421,8 @@ lbm_status validate(const lbm_config* g, char* msg) {
   auto bad = [&](const char* m) { std::snprintf(msg, 256, "%s", m); return LBM_EINVAL; };
   if (g->nx < 5 || g->ny < 5) return bad("nx and ny must be at least 5");
   if ((long long)g->nx * g->ny > 200000000LL) return bad("lattice larger than 2e8 nodes (32-bit plane offsets)");
+  // (rows are padded to 128 bytes: a narrow lattice's planes hold up to 6.4 times its nodes)
+  if (9 * row_pitch(g) * g->ny > INT_MAX) return bad("lattice's nine padded planes exceed 32-bit offsets");
   if (g->walls != 0 && g->walls != 1) return bad("walls must be 0 or 1");
   if (g->walls) {
     if (!(g->y_bottom >= 1.0 && g->y_bottom < 2.0)) return bad("y_bottom must lie in [1, 2)");
