@@ -39,7 +39,7 @@ struct Lattice {
   real* rho_b;                  // if set: the boundary phase leaves the density of each
                                 // boundary node's final populations here (one per node)
   real* mu;                     // chemical potential minus k^2 mu_sat (constant at solids)
-  real* rho_next;               // fused step (FP32): the next state's density (psi) plane
+  real* rho_next;               // fused and FP64 steps: the next state's density (psi) plane
   real* mu_out;                 // ... if set (tiles): this state's chemical potential is kept here
   real* aa_edge;                // ... in AA order, walked: what the strips left and right of a boundary between
                                 // two hand on of their outermost columns, 2 x 8 values a row, by boundary
@@ -604,20 +604,11 @@ __device__ __forceinline__ void odd_split(V Jx, V Jy, V& px, V& py, V& pd, V& pa
   py = fma_rn(half, Jy, fma_rn(d, n12, npd));
 }
 
-// The second-order part w_i rho (4.5 (e_i.v)^2 - 1.5 v^2) of f^eq from X = Jx vx, Y = Jy vy,
-// Z = Jx vy (J = rho v): X/3 - Y/6 and Y/3 - X/6 on the axes, (X + Y)/12 +- Z/4 on the two
-// diagonals, -2 (X + Y)/3 at rest; the rounded constants are exact multiples of one another, so
-// the parts sum to zero.
-//
-// Every operation is rounded explicitly (add_rn ... fma_rn), so that no kernel's compiler fuses
-// them differently, and no product enters a plain sum (ptxas fuses mul.rn.f32x2 with a following
-// add.rn.f32x2): all kernels that collide a node, or two at once, get the same bits.
-// Opposite directions share their even and odd parts, f~_i = w_i delta rho + (even +- odd).
-// BGK in FP64, whose instructions are what it costs (two lanes an SM and clock): f~ = (1 - 1/tau) f +
-// [f^eq(rho, u') - (1 - 1/tau) f^eq(rho, u)], the difference formed in delta rho, j and the three
+// collide_node's BGK branch in FP64, whose instructions are what it costs (two lanes an SM and clock):
+// f~ = (1 - 1/tau) f + [f^eq(rho, u') - (1 - 1/tau) f^eq(rho, u)], the difference formed in delta rho, j and the three
 // second-order products before it is spread over the directions: 45 operations instead of 93 (a node's
-// collision with its force: 160 -> 105; 512 x 512: 129 -> 101 us a step).  1/tau enters as 1 - (1 - 1/tau) only, so mass and momentum balance whatever the rounding
-// of either.
+// collision with its force: 160 -> 105; 512 x 512: 129 -> 101 us a step).  1/tau enters as
+// 1 - (1 - 1/tau) only, so mass and momentum balance whatever the rounding of either.
 __device__ __forceinline__ void collide_bgk64(const Lattice<double>& L, double (&f)[9], double r, double drho, double jx,
                                               double jy, double Fx, double Fy) {
   const double keep = 1.0 - L.omega, inv_r = 1.0 / r, nk = -keep;
@@ -641,6 +632,15 @@ __device__ __forceinline__ void collide_bgk64(const Lattice<double>& L, double (
   f[8] = fma(keep, f[8], e6 - pa);
 }
 
+// The second-order part w_i rho (4.5 (e_i.v)^2 - 1.5 v^2) of f^eq from X = Jx vx, Y = Jy vy,
+// Z = Jx vy (J = rho v): X/3 - Y/6 and Y/3 - X/6 on the axes, (X + Y)/12 +- Z/4 on the two
+// diagonals, -2 (X + Y)/3 at rest; the rounded constants are exact multiples of one another, so
+// the parts sum to zero.
+//
+// Every operation is rounded explicitly (add_rn ... fma_rn), so that no kernel's compiler fuses
+// them differently, and no product enters a plain sum (ptxas fuses mul.rn.f32x2 with a following
+// add.rn.f32x2): all kernels that collide a node, or two at once, get the same bits.
+// Opposite directions share their even and odd parts, f~_i = w_i delta rho + (even +- odd).
 template <typename V, typename real>
 __device__ __forceinline__ void collide_node(const Lattice<real>& L, V (&f)[9], V r, V drho, V jx, V jy, V Fx, V Fy) {
   if constexpr (sizeof(real) == 8) {

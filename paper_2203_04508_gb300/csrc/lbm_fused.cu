@@ -466,6 +466,11 @@ __global__ void __launch_bounds__(32) k_walk_batch(const Lattice<float>* lat, co
 // The same pass by tiles: a block of W warps takes the OUT output columns of a strip in H rows; its
 // density rows (five more on each side) and population rows (one more) arrive together, then all
 // chemical-potential rows, all collisions and all densities are formed side by side.
+
+// the tile shapes: output rows at most, warps a block, blocks an SM
+constexpr int TH_M = 14, TW_M = 8, TB_M = 3;
+constexpr int TH_L = 10, TW_L = 4, TB_L = 5;
+
 template <bool PSEUDO, int H>
 struct Tile {
   static constexpr int MR = PSEUDO ? 0 : 3;              // chemical-potential rows beyond the outputs
@@ -995,10 +1000,6 @@ __device__ __forceinline__ void boundary_density(const Lattice<float>& L, int cu
   L.rho_b[b] = density_of(L, v);
   if (L.aa) moments(v, L.bmom[3 * b], L.bmom[3 * b + 1], L.bmom[3 * b + 2]);
 }
-
-// the tile shapes: output rows at most, warps a block, blocks an SM
-constexpr int TH_M = 14, TW_M = 8, TB_M = 3;
-constexpr int TH_L = 10, TW_L = 4, TB_L = 5;
 __global__ void __launch_bounds__(128) k_boundary_density(const __grid_constant__ Lattice<float> L, int cur) {
   boundary_density(L, cur, blockIdx.x * blockDim.x + threadIdx.x);
 }

@@ -364,16 +364,12 @@ __global__ void k_fill_links(GeomParams g, const uint8_t* kind, int n_bnodes, Ge
     o.lq64[l] = qb;
     ((real*)o.lq)[l] = (real)qb;
     o.lx2f[l] = (ok2 && kind[m2] == KIND_FLUID) ? 1 : 0;
-    if (o.bnd) {
-      mask |= (1u << (i - 1)) | (o.lx2f[l] ? 1u << (i + 7) : 0u);
-      ((real*)o.bq)[(i - 1) * (long long)o.bcap + b] = (real)qb;
-    }
+    mask |= (1u << (i - 1)) | (o.lx2f[l] ? 1u << (i + 7) : 0u);
+    ((real*)o.bq)[(i - 1) * (long long)o.bcap + b] = (real)qb;
     ++l;
   }
-  if (o.bnd) {
-    o.bnd[b] = make_int2(n, x);
-    o.bmask[b] = (unsigned short)mask;
-  }
+  o.bnd[b] = make_int2(n, x);
+  o.bmask[b] = (unsigned short)mask;
 }
 
 // Entry j of a solid-layer list (node[j] of class cls): the mask of its neighbours of class

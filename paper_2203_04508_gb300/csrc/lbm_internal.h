@@ -177,7 +177,7 @@ struct GeomOut {
   int* s1nb;                                // 8 per first-layer entry: neighbours' boundary index
   int* s2nb;                                // 8 per second-layer entry: neighbours' first-layer index
   void* lq;   void* s1winv; void* s2winv;   // precision-typed
-  int2* bnd; unsigned short* bmask; void* bq; int bcap;   // links by boundary node (FP32; null otherwise)
+  int2* bnd; unsigned short* bmask; void* bq; int bcap;   // links by boundary node
   void* mu;                                 // precision-typed plane
   int fp64;
   int n_bnodes, n_s1, n_s2;                 // list lengths (from the counts)

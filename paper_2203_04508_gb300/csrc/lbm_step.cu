@@ -1021,8 +1021,6 @@ __global__ void __launch_bounds__(NODE_BLOCK) k_column(Lattice<real> L, int cur,
   out[j] = (double)density_of(L, fl);
 }
 
-// Populations i0 <= i < i1 of the current state as absolute values, population i into the
-// dense plane i - i0 of `out` (0 at non-fluid nodes).
 // Zero into the slots of lattice `cur` that no population of the method occupies -- a row's padding,
 // and slot i of a solid node x whose x - e_i is no fluid node -- where the fused step may have left
 // values of its own: a stored lattice holds the same bytes whichever kernels advanced it.
@@ -1041,6 +1039,8 @@ __global__ void k_settle(Lattice<real> L, int cur) {
   }
 }
 
+// Populations i0 <= i < i1 of the current state as absolute values, population i into the
+// dense plane i - i0 of `out` (0 at non-fluid nodes).
 template <typename real>
 __global__ void k_populations(Lattice<real> L, int cur, real* out, int i0, int i1) {
   const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
