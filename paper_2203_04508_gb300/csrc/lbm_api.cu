@@ -468,7 +468,7 @@ bool fused(const lbm_ctx* c) {
   return c->fused_ok && !c->fp64 && c->cfg.layout == LBM_LAYOUT_AB && c->cfg.eos != LBM_EOS_NONE && !c->slab.on &&
          c->mu_kind < 0 && !c->collide_set;
 }
-// ... on one lattice in AA order?  (2048 x 4096 214 -> 178 us a step, 512 x 512 30 -> 15.4)
+// ... on one lattice in AA order?  (2048 x 4096 206 -> 172 us a step, 512 x 512 30 -> 15.4)
 bool fused_aa(const lbm_ctx* c) {
   return c->fused_ok && !c->fp64 && c->cfg.layout == LBM_LAYOUT_AA && c->cfg.eos != LBM_EOS_NONE && !c->slab.on &&
          c->mu_kind < 0 && !c->collide_set;

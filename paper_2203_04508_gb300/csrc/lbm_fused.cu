@@ -18,7 +18,7 @@
 // those nodes in two planes (the pass stores it in the rows next to solids).  The densities of
 // boundary nodes come from k_bc_fused, those of the solid layers from k_solids.
 //
-// On the 2048 x 4096 impact lattice a step takes 0.148 ms against 0.192 ms for the separate passes
+// On the 2048 x 4096 impact lattice a step takes 0.147 ms against 0.192 ms for the separate passes
 // (2048 x 2048 84 against 110 us, 1024 x 1024 with 16 drops 33 against 45, 131 x 97 9.0 against 29);
 // the pass itself 0.13 ms, 661 MB of DRAM traffic.  What bounds a walk is instruction issue: twelve
 // warps an SM (three in each quarter, which is what their registers allow) issue 0.6 instructions a
@@ -430,8 +430,8 @@ __device__ __forceinline__ void walk(const Lattice<float>& L, int cur, int strip
   cp_wait<0>();
 }
 
-// (152 registers: twelve warps an SM either way, and the schedule the compiler finds within them is 2 to
-// 4 % faster than its own choice)
+// (A limit of 152 registers, of which the variants take 128 to 148: twelve warps an SM with or without
+// it, and the schedule the compiler finds within it is 2 to 4 % faster than the one it finds alone.)
 template <bool PSEUDO, int AA = 0>
 __global__ void __maxnreg__(152) k_walk(const __grid_constant__ Lattice<float> L, int cur, int strips, int rows) {
   extern __shared__ __align__(16) char smem[];
@@ -1063,7 +1063,7 @@ PassPlan fused_tile_plan(int nx, int ny, int sms) {
 
 // ... of an AA lattice: the same walks; its tiles are of the first shape, whose bands leave fewer
 // outermost rows to k_layers_aa.  (separate passes / fused, us a step: 131 x 97 24.6 / 9.3, 512 x 512
-// 30 / 15.4, 1024 x 1024 46 / 33, 1600 x 2000 95 / 80, 2048 x 4096 214 / 178.)
+// 30 / 15.4, 1024 x 1024 46 / 33, 1600 x 2000 95 / 80, 2048 x 4096 206 / 172.)
 PassPlan fused_aa_plan(int nx, int ny, int sms) {
   PassPlan p = fused_plan(nx, ny, sms);
   if (p.kind != PassPlan::TILE_L) return p;

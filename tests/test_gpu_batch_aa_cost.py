@@ -12,7 +12,7 @@ AB, AA = 0, 1
 
 
 def test_a_batch_in_aa_order_costs_what_the_persistent_kernel_costs_on_two_lattices():
-    """At most 1.12 times (measured 1.00 to 1.01; 1.23 when the collide phase addressed every slot for
+    """At most 1.12 times (measured 1.00 to 1.01; 1.22 when the collide phase addressed every slot for
     itself).  Timed in turn, the best of five, so that clocks and neighbours do not decide."""
     import torch
     if not torch.cuda.is_available():
